@@ -325,6 +325,20 @@ struct ff_acc {
     __device__ __forceinline__ ff value() const { return two_sum(s, t); }
 };
 
+// A float as a double from its bits: GB300 converts at the FP64 rate (1/64 of
+// the FP32 rate), while moving the exponent and the mantissa takes a few
+// integer operations.  Subnormals, infinities and NaN take the conversion.
+__device__ __forceinline__ double widen(float v) {
+    const unsigned b = __float_as_uint(v);
+    if (((b >> 23) & 0xFFu) - 1u < 254u)
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
+    if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
+    return (double)v;
+}
+
+// a float-float value as a double: one FP64 addition
+__device__ __forceinline__ double widen(ff a) { return __dadd_rn(widen(a.hi), widen(a.lo)); }
+
 // The potential at an interior fluid cell (c) and at its 18 D3Q19
 // neighbours, named by their offsets (xpym: x + 1, y - 1, ...).
 struct Psi19 {

@@ -144,6 +144,31 @@ struct FbPsi {
     float Ex, Ey, Ez, k2e;
 };
 
+// psi at an interior cell and its 18 neighbours; sx, sy, sz: the offsets of
+// the steps +1, 0, -1 along each axis (wrapped), p the cell's own value.
+__device__ __forceinline__ Psi19 load_psi19(const float* __restrict__ p, const int (&sx)[3], const int (&sy)[3],
+                                            const int (&sz)[3]) {
+    return Psi19{__ldg(p),
+                 __ldg(p + sx[0]),
+                 __ldg(p + sx[2]),
+                 __ldg(p + sy[0]),
+                 __ldg(p + sy[2]),
+                 __ldg(p + sz[0]),
+                 __ldg(p + sz[2]),
+                 __ldg(p + sx[0] + sy[0]),
+                 __ldg(p + sx[2] + sy[2]),
+                 __ldg(p + sx[0] + sy[2]),
+                 __ldg(p + sx[2] + sy[0]),
+                 __ldg(p + sx[0] + sz[0]),
+                 __ldg(p + sx[2] + sz[2]),
+                 __ldg(p + sx[0] + sz[2]),
+                 __ldg(p + sx[2] + sz[0]),
+                 __ldg(p + sy[0] + sz[0]),
+                 __ldg(p + sy[2] + sz[2]),
+                 __ldg(p + sy[0] + sz[2]),
+                 __ldg(p + sy[2] + sz[0])};
+}
+
 // SLIP: the grid has free-slip faces (a separate instance, so that the
 // common no-slip/periodic form keeps its register count).  FBPSI: the body
 // force of an interior fluid cell (no obstacle or wall among its D3Q19
@@ -189,29 +214,8 @@ __device__ __forceinline__ void lbm_cell(const Grid& g, const Streams<S>& P, con
     if (!(fl & F_NEAR19)) {
         // all 18 pull sources are fluid cells inside the (periodic) domain
         if constexpr (FBPSI) {
-            // psi(x + d) at offset sx[1 - dx] + sy[1 - dy] + sz[1 - dz]
-            const float* ps = fp.psi + c;
-            const Psi19 p{__ldg(ps),
-                          __ldg(ps + sx[0]),
-                          __ldg(ps + sx[2]),
-                          __ldg(ps + sy[0]),
-                          __ldg(ps + sy[2]),
-                          __ldg(ps + sz[0]),
-                          __ldg(ps + sz[2]),
-                          __ldg(ps + sx[0] + sy[0]),
-                          __ldg(ps + sx[2] + sy[2]),
-                          __ldg(ps + sx[0] + sy[2]),
-                          __ldg(ps + sx[2] + sy[0]),
-                          __ldg(ps + sx[0] + sz[0]),
-                          __ldg(ps + sx[2] + sz[2]),
-                          __ldg(ps + sx[0] + sz[2]),
-                          __ldg(ps + sx[2] + sz[0]),
-                          __ldg(ps + sy[0] + sz[0]),
-                          __ldg(ps + sy[2] + sz[2]),
-                          __ldg(ps + sy[0] + sz[2]),
-                          __ldg(ps + sy[2] + sz[0])};
             float f0, f1, f2;
-            body_force_iso(p, fp.Ex, fp.Ey, fp.Ez, fp.k2e, f0, f1, f2);
+            body_force_iso(load_psi19(fp.psi + c, sx, sy, sz), fp.Ex, fp.Ey, fp.Ez, fp.k2e, f0, f1, f2);
             fx = f0 + ax;
             fy = f1 + ay;
             fz = f2 + az;
@@ -758,25 +762,127 @@ __global__ void k_set_pdf(long long N, long long ps, const double* src, S* dst) 
     dst[(long long)q * ps + (i - (long long)q * N)] = Store<S>::from_f(q, src[i]);
 }
 
-template <class S, class C = typename Store<S>::C>
-__global__ void k_moments(long long N, long long ps, const S* f, const C* fb, double ax, double ay, double az,
-                          double* rho, double* u) {
-    long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// Density or velocity of the FP64 form: rho = sum f, u = sum c f - f_b / 2
+// (the collision keeps rho and adds exactly f_b).
+template <bool RHO>
+__global__ void __launch_bounds__(256) k_moments(long long N, long long ps, const double* __restrict__ f,
+                                                 const double* __restrict__ fb, double ax, double ay, double az,
+                                                 double* __restrict__ out) {
+    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     double r = 0.0, j0 = 0.0, j1 = 0.0, j2 = 0.0;
+#pragma unroll
     for (int q = 0; q < 19; q++) {
-        double v = Store<S>::to_f(q, f[(long long)q * ps + c]);
-        r += v;
-        j0 += cx(q) * v;
-        j1 += cy(q) * v;
-        j2 += cz(q) * v;
+        if (!RHO && q == 0) continue;
+        const double v = f[(long long)q * ps + c];
+        if (RHO) {
+            r += v;
+            continue;
+        }
+        if (cx(q)) j0 += cx(q) > 0 ? v : -v;
+        if (cy(q)) j1 += cy(q) > 0 ? v : -v;
+        if (cz(q)) j2 += cz(q) > 0 ? v : -v;
     }
-    // collision keeps rho and adds exactly f_b, so u = sum c f - f_b / 2
-    if (rho) rho[c] = r;
-    if (u) {
-        u[c] = j0 - 0.5 * ((double)fb[c] + ax);
-        u[N + c] = j1 - 0.5 * ((double)fb[N + c] + ay);
-        u[2 * N + c] = j2 - 0.5 * ((double)fb[2 * N + c] + az);
+    if (RHO) {
+        out[c] = r;
+    } else {
+        out[c] = j0 - 0.5 * (fb[c] + ax);
+        out[N + c] = j1 - 0.5 * (fb[N + c] + ay);
+        out[2 * N + c] = j2 - 0.5 * (fb[2 * N + c] + az);
+    }
+}
+
+// Density or velocity of the reduced forms.  The stored deviations are
+// summed in float-float (TwoSum, about 48 bits) and widened to FP64 once per
+// value: summed in FP64, the 100 FP64 operations a cell bound the kernel at
+// 1/64 of the FP32 rate (density, velocity and potential of a 320^3 MIXED32
+// state: 13.5 ms, in float-float 1.21 ms, 0.49 of the copy rate).  The
+// deviations carry no
+// w_q, so the sums hold more bits of the velocity than FP64 sums of
+// w_q + dev do.  FP16 storage: the axis and the diagonal streams are summed
+// apart and take their weight as a float-float product.  FBPSI: the body
+// force of an interior cell is formed from psi as the stream-collide forms
+// it (cells next to obstacles read the stored field, obstacle cells have
+// none), so the whole field is neither stored nor read back.
+struct Accel3 {
+    ff a[3];  // - accel / 2
+};
+
+template <class S, bool RHO, bool FBPSI>
+__global__ void __launch_bounds__(256) k_moments_ff(Grid g, const S* __restrict__ f, const float* __restrict__ fb,
+                                                    const uint8_t* __restrict__ flags, FbPsi fp, Accel3 acc,
+                                                    double* __restrict__ out) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
+    if (x >= g.nx || y >= g.ny) return;
+    const int c = x + g.nx * (y + g.ny * z);
+    constexpr bool kHalf = sizeof(S) == 2;
+    // the weights of FP16 storage: dev = h w_q / 2^12
+    constexpr float wa = (float)(1.0 / 18.0 / kHalfScale), wa2 = (float)(1.0 / 18.0 / kHalfScale - (double)wa);
+    constexpr float wd = 0.5f * wa, wd2 = 0.5f * wa2;
+    auto ld = [&](int q) -> float { return (float)__ldg(f + (size_t)q * g.ps + c); };
+    if constexpr (RHO) {
+        ff_acc s{0.0f, 0.0f}, d{0.0f, 0.0f};
+#pragma unroll
+        for (int q = 1; q < 19; q++) {
+            if (kHalf && !(q <= 3 || (q >= 10 && q <= 12)))
+                d.add(ld(q), 0.0f);
+            else
+                s.add(ld(q), 0.0f);
+        }
+        ff v;
+        if constexpr (kHalf) {
+            s.add(6.0f * ld(0), 0.0f);  // (w_0 = 6 w_1; an 11-bit value times 6 is exact)
+            v = ff_add(ff_mul(s.value(), {wa, wa2}), ff_mul(d.value(), {wd, wd2}));
+        } else {
+            s.add(ld(0), 0.0f);
+            v = s.value();
+        }
+        out[c] = 1.0 + widen(v);
+    } else {
+        ff_acc s[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, d[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+#pragma unroll
+        for (int q = 1; q < 19; q++) {
+            const float v = ld(q);
+            const int cq[3] = {cx(q), cy(q), cz(q)};
+#pragma unroll
+            for (int a = 0; a < 3; a++)
+                if (cq[a]) {
+                    if (kHalf && !(q <= 3 || (q >= 10 && q <= 12)))
+                        d[a].add(cq[a] > 0 ? v : -v, 0.0f);
+                    else
+                        s[a].add(cq[a] > 0 ? v : -v, 0.0f);
+                }
+        }
+        const size_t N = (size_t)g.N;
+        float b[3];
+        bool stored = true;
+        if constexpr (FBPSI) {
+            const uint8_t fl = flags[c];
+            stored = (fl & (F_SOLID | F_NEAR19)) == F_NEAR19;
+            b[0] = b[1] = b[2] = 0.0f;
+            if (!(fl & (F_SOLID | F_NEAR19))) {
+                const int nx = g.nx, nxy = g.nx * g.ny;
+                const int sx[3] = {(x == nx - 1 ? 0 : x + 1) - x, 0, (x == 0 ? nx - 1 : x - 1) - x};
+                const int sy[3] = {((y == g.ny - 1 ? 0 : y + 1) - y) * nx, 0, ((y == 0 ? g.ny - 1 : y - 1) - y) * nx};
+                const int sz[3] = {((z == g.nz - 1 ? 0 : z + 1) - z) * nxy, 0, ((z == 0 ? g.nz - 1 : z - 1) - z) * nxy};
+                body_force_iso(load_psi19(fp.psi + c, sx, sy, sz), fp.Ex, fp.Ey, fp.Ez, fp.k2e, b[0], b[1], b[2]);
+            }
+        }
+        if (stored) {
+#pragma unroll
+            for (int a = 0; a < 3; a++) b[a] = fb[a * N + c];
+        }
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            ff v;
+            if constexpr (kHalf)
+                v = ff_add(ff_mul(s[a].value(), {wa, wa2}), ff_mul(d[a].value(), {wd, wd2}));
+            else
+                v = s[a].value();
+            v = ff_add(ff_add_f(v, -0.5f * b[a]), acc.a[a]);
+            out[a * N + c] = widen(v);
+        }
     }
 }
 
@@ -1095,16 +1201,38 @@ cudaError_t launch_set_pdf(es_ctx* c, const double* src) {
 }
 
 cudaError_t launch_get_moments(es_ctx* c, double* rho, double* u) {
-    const cudaError_t err = materialize_body_force(c);
-    if (err != cudaSuccess) return err;
+    const Grid& g = c->g;
     const double* a = c->P.accel;
+    if (!mixed(c)) {
+        const double *f = (const double*)c->pdf[c->cur], *fb = (const double*)c->fb;
+        if (rho) k_moments<true><<<blocks_for(g.N, 256), 256, 0, c->stream>>>(g.N, g.ps, f, fb, a[0], a[1], a[2], rho);
+        if (u) k_moments<false><<<blocks_for(g.N, 256), 256, 0, c->stream>>>(g.N, g.ps, f, fb, a[0], a[1], a[2], u);
+        count(c, (rho ? 1 : 0) + (u ? 1 : 0));
+        return cudaGetLastError();
+    }
+    const bool lazy = c->fb_lazy;
+    if (u && lazy) {
+        const cudaError_t err = launch_body_force_near(c);
+        if (err != cudaSuccess) return err;
+    }
+    const double k2e = c->S.kappa * c->S.kappa * c->S.eps;
+    const FbPsi fp{c->psi32, (float)c->P.E_ext[0], (float)c->P.E_ext[1], (float)c->P.E_ext[2], (float)k2e};
+    Accel3 acc;
+    for (int k = 0; k < 3; k++) acc.a[k] = ff_from_double(-0.5 * a[k]);
+    const dim3 blk(32, 8), grd((g.nx + 31) / 32, (g.ny + 7) / 8, g.nz);
     dispatch_store(c, [&](auto tag) {
         using S = decltype(tag);
-        using C = typename Store<S>::C;
-        k_moments<S><<<blocks_for(c->g.N, 256), 256, 0, c->stream>>>(c->g.N, c->g.ps, (const S*)c->pdf[c->cur],
-                                                                     (const C*)c->fb, a[0], a[1], a[2], rho, u);
+        if constexpr (!std::is_same<S, double>::value) {
+            const S* f = (const S*)c->pdf[c->cur];
+            const float* fb = (const float*)c->fb;
+            if (rho) k_moments_ff<S, true, false><<<grd, blk, 0, c->stream>>>(g, f, fb, c->flags, fp, acc, rho);
+            if (u && lazy)
+                k_moments_ff<S, false, true><<<grd, blk, 0, c->stream>>>(g, f, fb, c->flags, fp, acc, u);
+            else if (u)
+                k_moments_ff<S, false, false><<<grd, blk, 0, c->stream>>>(g, f, fb, c->flags, fp, acc, u);
+        }
     });
-    count(c);
+    count(c, (rho ? 1 : 0) + (u ? 1 : 0));
     return cudaGetLastError();
 }
 

@@ -2557,7 +2557,7 @@ __global__ void k_split_psi(int N, const double* __restrict__ src, float* __rest
 
 __global__ void k_join_psi(int N, const float* __restrict__ hi, const float* __restrict__ lo, double* __restrict__ dst) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < N) dst[c] = (double)hi[c] + (double)lo[c];
+    if (c < N) dst[c] = widen(ff{hi[c], lo[c]});
 }
 
 // --- EDL field and body force (Sec. 5.6) ---
