@@ -50,6 +50,52 @@ void launch_pdl(const es_ctx* c, void (*kernel)(KArgs...), dim3 grid, dim3 block
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);  // (errors: cudaGetLastError)
 }
 
+// The share of an x-y plane that a block takes in the residual, restriction
+// and prolongation kernels, whose threads own a span of a row: tw spans of th
+// rows (thread t: span t % tw of row t / tw).  Rows are rarely a multiple of
+// 32 spans (of 8 cells: 16 at nx = 128, 36 at nx = 288), and a fixed 32 x 8
+// shape then leaves up to half of the lanes idle; the shape with the fewest
+// blocks is taken, 32 x 8 where it is as good (512^3).  288 x 576 x 288, with
+// 32 x 8 / so: restriction 154 / 123 us, residual update 412 / 338 us,
+// prolongation 57 / 49 us.  The half sweeps keep 32 x 8: they are bound by
+// the latency of their near-boundary cells, and the fewer blocks cost as much
+// as the full lanes gain (98 / 96 us there, 12.1 / 14.4 us at 96^3).
+struct Tile {
+    int tw, th;
+    unsigned inv;  // ceil(2^16 / tw): t / tw = (t inv) >> 16 for t < 256, tw <= 64
+};
+
+constexpr int kTileThreads = 256;
+
+Tile plane_tile(int nspan, int nrows, int threads = kTileThreads) {
+    Tile best{32, threads / 32, 2048};
+    if (nspan < 1) return best;  // (a level without such spans: not launched)
+    auto blocks = [&](const Tile& t) {
+        return (long long)((nspan + t.tw - 1) / t.tw) * ((nrows + t.th - 1) / t.th);
+    };
+    for (int k = (nspan + 63) / 64; k <= (nspan + 3) / 4; k++) {
+        const int tw = (nspan + k - 1) / k;
+        const Tile t{tw, threads / tw, (65536u + tw - 1) / tw};
+        if (blocks(t) < blocks(best)) best = t;
+    }
+    return best;
+}
+
+dim3 tile_grid(const Tile& t, int nspan, int nrows, int nz) {
+    return dim3((nspan + t.tw - 1) / t.tw, (nrows + t.th - 1) / t.th, nz);
+}
+
+// Span and row of this thread; false when it has none (span and row are then
+// valid ones, so that its loads need no guards).
+__device__ __forceinline__ bool tile_at(const Tile& t, int nspan, int nrows, int tid, int& span, int& row) {
+    const int ty = (int)(((unsigned)tid * t.inv) >> 16);
+    span = (int)blockIdx.x * t.tw + (tid - ty * t.tw);
+    row = (int)blockIdx.y * t.th + ty;
+    const bool on = ty < t.th && span < nspan && row < nrows;
+    if (!on) span = row = 0;
+    return on;
+}
+
 __device__ __forceinline__ bool wrap_axis(int v, int n, int per, int& out) {
     if (v < 0 || v >= n) {
         if (!per) return false;
@@ -366,7 +412,7 @@ __global__ void __launch_bounds__(256, 2) k_outer_residual_ff(Grid g, ff diag0, 
                                                            const float* __restrict__ psi_lo,
                                                            const uint8_t* __restrict__ st0,
                                                            float* __restrict__ r_out,
-                                                           double* __restrict__ partial, int zc,
+                                                           double* __restrict__ partial, int zc, Tile tl,
                                                            const int* __restrict__ gate) {
     static_assert(!SPLIT || W == 4, "the split store takes 4-cell spans");
     if (gate && *gate == 0) return;  // (uniform over the grid: the patched residual runs instead)
@@ -374,14 +420,12 @@ __global__ void __launch_bounds__(256, 2) k_outer_residual_ff(Grid g, ff diag0, 
     const int half = (int)(g.N >> 1);
     float acc = 0.0f;
     const int nx = g.nx, ny = g.ny, nz = g.nz;
-    const int xs = W * (blockIdx.x * 32 + threadIdx.x);
-    const int y = blockIdx.y * 8 + threadIdx.y;
-    const bool lane_on = xs < nx;
-    const int xq = lane_on ? xs : 0;  // (inactive lanes read a valid span)
+    int span, y;
+    const bool lane_on = tile_at(tl, nx / W, ny, threadIdx.x, span, y);
+    const int xs = W * span, xq = xs;  // (inactive lanes read a valid span)
     const int z0 = (int)blockIdx.z * zc;
     const int z1 = z0 + zc < nz ? z0 + zc : nz;
-    // y is the same for the 32 lanes of a warp, so the march is warp-uniform
-    if (y < ny && z0 < z1) {
+    if (lane_on && z0 < z1) {
         // unguarded loads: beyond a wall only near-boundary cells would read,
         // and those are formed from memory by near_residual_ff
         int ym, yp, xl, xr;
@@ -497,9 +541,9 @@ __global__ void __launch_bounds__(256, 2) k_outer_residual_ff(Grid g, ff diag0, 
     // double per block
     float v = acc;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) swarp[threadIdx.y] = v;
+    if ((threadIdx.x & 31) == 0) swarp[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
+    if (threadIdx.x == 0) {
         double tot = 0.0;
         for (int w = 0; w < 8; w++) tot += (double)swarp[w];
         partial[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = tot;
@@ -1671,12 +1715,13 @@ __global__ void __launch_bounds__(128) k_prolong(Level<T> L, const uint8_t* __re
 template <class T, class E, bool SPLIT = false>
 __global__ void __launch_bounds__(256) k_prolong_v(Level<T> L, const uint8_t* __restrict__ st, E* __restrict__ e,
                                                    int cnx, int cny, const uint8_t* __restrict__ cst,
-                                                   const T* __restrict__ ce, EAcc<T, E> A, int half = 0,
+                                                   const T* __restrict__ ce, EAcc<T, E> A, Tile tl, int half = 0,
                                                    int chalf = 0) {
     pdl_wait();
-    const int xs = 4 * (blockIdx.x * 32 + threadIdx.x);
-    const int y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
-    if (xs >= L.nx || y >= L.ny) return;
+    int span, y;
+    const int z = blockIdx.z;
+    if (!tile_at(tl, L.nx / 4, L.ny, threadIdx.x, span, y)) return;
+    const int xs = 4 * span;
     const int c = xs + L.nx * (y + L.ny * z);
     const int C = (xs >> 1) + cnx * ((y >> 1) + cny * (z >> 1));
     const unsigned sw = *reinterpret_cast<const unsigned*>(st + c);
@@ -1733,12 +1778,13 @@ __device__ __forceinline__ void store_coarse4(float* __restrict__ crhs, int C, i
 __global__ void __launch_bounds__(256) k_prolong_black_rb(Level<float> L, const uint8_t* __restrict__ st,
                                                           float* __restrict__ e, int half, int cnx, int cny,
                                                           const uint8_t* __restrict__ cst,
-                                                          const float* __restrict__ ce, int chalf) {
+                                                          const float* __restrict__ ce, int chalf, Tile tl) {
     pdl_wait();
     const int nxh = L.nx >> 1;
-    const int X0 = 4 * (blockIdx.x * 32 + threadIdx.x);
-    const int y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
-    if (X0 >= nxh || y >= L.ny) return;
+    int X0, y;
+    const int z = blockIdx.z;
+    if (!tile_at(tl, L.nx >> 3, L.ny, threadIdx.x, X0, y)) return;
+    X0 *= 4;
     const int O = (1 + y + z) & 1;
     float* eb = e + half + nxh * (y + L.ny * z) + X0;
     const uint2 sw = *reinterpret_cast<const uint2*>(st + L.nx * (y + L.ny * z) + 2 * X0);
@@ -1809,13 +1855,12 @@ __global__ void __launch_bounds__(256) k_restrict_v(Level<T> L, T inv_diag0, T i
                                                     const T* __restrict__ rhs, const E* __restrict__ e,
                                                     const T* __restrict__ near_res, int cnx,
                                                     int cny, const uint8_t* __restrict__ cst, T* __restrict__ crhs,
-                                                    EAcc<T, E> A, int half = 0, int red_only = 0) {
+                                                    EAcc<T, E> A, Tile tl, int half = 0, int red_only = 0) {
     pdl_wait();
-    const int cx_warp = 2 * (blockIdx.x * 32);
-    const int cxs = cx_warp + 2 * threadIdx.x;
-    const int cy = blockIdx.y * 8 + threadIdx.y, cz = blockIdx.z;
-    if (cy >= cny) return;  // whole warps
-    const bool lane_on = cxs < cnx;
+    int span, cy;
+    const int cz = blockIdx.z;
+    if (!tile_at(tl, cnx / 2, cny, threadIdx.x, span, cy)) return;
+    const int cxs = 2 * span;
     const int nx = L.nx, ny = L.ny, nz = L.nz;
     const int xs = 2 * cxs;
     T sum0 = (T)0, sum1 = (T)0;
@@ -1832,7 +1877,7 @@ __global__ void __launch_bounds__(256) k_restrict_v(Level<T> L, T inv_diag0, T i
             if (!wrap_axis(y + 1, ny, L.per[1], yp)) yp = y;
             if (!wrap_axis(z - 1, nz, L.per[2], zm)) zm = z;
             if (!wrap_axis(z + 1, nz, L.per[2], zp)) zp = z;
-            const int xq = lane_on ? xs : 0;
+            const int xq = xs;
             if (!wrap_axis(xq - 1, nx, L.per[0], xl)) xl = xq;
             if (!wrap_axis(xq + 4, nx, L.per[0], xr)) xr = xq;
             const int rym = nx * (ym + ny * z), ryp = nx * (yp + ny * z);
@@ -1866,7 +1911,7 @@ __global__ void __launch_bounds__(256) k_restrict_v(Level<T> L, T inv_diag0, T i
                 ES_ELD(A, f, 0, e + rzp + xq);
                 ES_VLD(r, 0, rhs + row + xq);
             }
-            const unsigned sw = lane_on ? *reinterpret_cast<const unsigned*>(st + row + xs) : 0x02020202u;
+            const unsigned sw = *reinterpret_cast<const unsigned*>(st + row + xs);
             T res[4];
             unsigned near_bits = 0;
 #pragma unroll
@@ -1900,7 +1945,6 @@ __global__ void __launch_bounds__(256) k_restrict_v(Level<T> L, T inv_diag0, T i
             sum0 += res[0] + res[1];
             sum1 += res[2] + res[3];
         }
-    if (!lane_on) return;
     const int C = cxs + cnx * (cy + cny * cz);
     const T v0 = ((cst[C] & ST_KIND) == ST_UNKNOWN) ? sum0 / (T)8 : (T)0;
     const T v1 = ((cst[C + 1] & ST_KIND) == ST_UNKNOWN) ? sum1 / (T)8 : (T)0;
@@ -1910,9 +1954,9 @@ __global__ void __launch_bounds__(256) k_restrict_v(Level<T> L, T inv_diag0, T i
 }
 
 // Residual + restriction from the colour-split finest level (float,
-// nx % 8 == 0).  A block of 32 x 8 threads covers 128 coarse cells of two
-// coarse rows; the 4 warps of a coarse row take one fine row of the
-// children each (threadIdx.y = 4 * row + 2 dk + dj), so a thread forms the
+// nx % 8 == 0).  A block covers 64 spans of four coarse cells (tl), and its
+// four quarters take one fine row of the children each (quarter 2 dk + dj),
+// so a thread forms the
 // residuals of 8 fine cells: in a fine row, the two children of coarse
 // cell X are the compact cells X of the two colours (x = 2X and 2X+1), so
 // it loads 4 compact cells of each colour, the same places of the four
@@ -1925,16 +1969,15 @@ __global__ void __launch_bounds__(256) k_restrict_rb(Level<float> L, float inv_h
                                                      const float* __restrict__ rhs, const float* __restrict__ e,
                                                      const float* __restrict__ near_res, int cnx, int cny,
                                                      const uint8_t* __restrict__ cst, float* __restrict__ crhs,
-                                                     int half, int chalf) {
+                                                     int half, int chalf, Tile tl) {
     pdl_wait();
-    __shared__ float4 part[8][32];
-    const int X0 = 4 * (blockIdx.x * 32 + threadIdx.x);
-    const int crow = threadIdx.y >> 2, sub = threadIdx.y & 3;
-    const int cy = blockIdx.y * 2 + crow, cz = blockIdx.z;
-    const bool row_on = cy < cny;
-    const bool lane_on = X0 < cnx && row_on;
-    const int Xq = X0 < cnx ? X0 : 0;
-    const int cyq = row_on ? cy : 0;  // (rows past the end compute on a valid row; nothing is stored)
+    __shared__ float4 part[4][64];
+    const int sub = threadIdx.x >> 6, t = threadIdx.x & 63;
+    int X0, cy;
+    const int cz = blockIdx.z;
+    const bool lane_on = tile_at(tl, cnx / 4, cny, t, X0, cy);
+    X0 *= 4;
+    const int Xq = X0, cyq = cy;  // (threads without a span compute on a valid one; nothing is stored)
     const int nx = L.nx, ny = L.ny, nz = L.nz, nxh = nx >> 1;
     const int dk = sub >> 1, dj = sub & 1;
     const int y = 2 * cyq + dj, z = 2 * cz + dk;
@@ -2002,13 +2045,13 @@ __global__ void __launch_bounds__(256) k_restrict_rb(Level<float> L, float inv_h
         const unsigned sv = ((j < 4 ? sw.x : sw.y) >> (8 * (j & 3))) & 0xFFu;
         if ((sv & (ST_KIND | ST_NEAR)) == (ST_UNKNOWN | ST_NEAR)) res[j] = near_res[rown + j];
     }
-    part[threadIdx.y][threadIdx.x] = make_float4(res[0] + res[1], res[2] + res[3], res[4] + res[5], res[6] + res[7]);
+    part[sub][t] = make_float4(res[0] + res[1], res[2] + res[3], res[4] + res[5], res[6] + res[7]);
     __syncthreads();
     if (sub != 0 || !lane_on) return;
     float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int q = 0; q < 4; q++) {  // q = 2 dk + dj: dk outer, dj inner
-        const float4 p = part[4 * crow + q][threadIdx.x];
+        const float4 p = part[q][t];
         sum[0] += p.x;
         sum[1] += p.y;
         sum[2] += p.z;
@@ -2045,19 +2088,19 @@ __global__ void __launch_bounds__(256, 2) k_residual_update_rb(Level<float> L, f
                                                                const uint8_t* __restrict__ st,
                                                                float* __restrict__ rhs, const float* __restrict__ e,
                                                                const float* __restrict__ near_res, int half,
-                                                               double* __restrict__ partial, int zc,
+                                                               double* __restrict__ partial, int zc, Tile tl,
                                                                float* __restrict__ psi_hi, float* __restrict__ psi_lo) {
     __shared__ float swarp[8];
     const int nx = L.nx, ny = L.ny, nz = L.nz, nxh = nx >> 1;
-    const int X0 = 4 * (blockIdx.x * 32 + threadIdx.x);
-    const int y = blockIdx.y * 8 + threadIdx.y;
-    const bool lane_on = X0 < nxh;
-    const int Xq = lane_on ? X0 : 0;
+    int X0, y;
+    const bool lane_on = tile_at(tl, nx >> 3, ny, threadIdx.x, X0, y);
+    X0 *= 4;
+    const int Xq = X0;
     const float k2h2 = L.diag0 - 6.0f;  // (exact: diag0 in [6, 12))
     const int z0 = (int)blockIdx.z * zc;
     const int z1 = z0 + zc < nz ? z0 + zc : nz;
     float acc = 0.0f;
-    if (y < ny && z0 < z1) {
+    if (lane_on && z0 < z1) {
         int ym, yp, il, ir;
         if (!wrap_axis(y - 1, ny, L.per[1], ym)) ym = y;
         if (!wrap_axis(y + 1, ny, L.per[1], yp)) yp = y;
@@ -2161,7 +2204,7 @@ __global__ void __launch_bounds__(256, 2) k_residual_update_rb(Level<float> L, f
                 for (int j = 0; j < 8; j++)
                     if ((near >> j) & 1u) out[j] = near_res[rown + j];
             }
-            if (lane_on) {
+            {
 #pragma unroll
                 for (int j = 0; j < 8; j++) acc = __fmaf_rn(out[j], out[j], acc);
                 vst(rhs + pe * half + rowh + X0, out[0], out[2], out[4], out[6]);
@@ -2215,9 +2258,9 @@ __global__ void __launch_bounds__(256, 2) k_residual_update_rb(Level<float> L, f
     }
     float v = acc;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) swarp[threadIdx.y] = v;
+    if ((threadIdx.x & 31) == 0) swarp[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
+    if (threadIdx.x == 0) {
         double tot = 0.0;
         for (int w = 0; w < 8; w++) tot += (double)swarp[w];
         partial[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = tot;
@@ -2236,29 +2279,29 @@ __global__ void __launch_bounds__(256, 2) k_residual_update_rb(Level<float> L, f
 // the black rows (y, z+1), (y-1, z) and (y+1, z), one halo value, the red
 // e and rhs of (y, z) and the state bytes (about 7 bytes per fine cell),
 // and the loads of plane z+1 are issued before plane z is formed.  The two
-// warps of a coarse row (dj = 0, 1) meet in shared memory after each pair
+// threads of a coarse span (dj = 0, 1) meet in shared memory after each pair
 // of fine planes, and the 4 red children are added in the order of
 // k_restrict_v (dk outer, dj inner).  Near-boundary red children come from
 // k_near_residual (red segments).  chalf != 0: the coarse right-hand side
 // is stored colour-split (chalf: half the coarse cells).
-constexpr int kRestrictRows = 4;  // coarse rows per block (2 warps each)
+constexpr int kRestrictSpans = 128;  // spans of four coarse cells per block (two threads each)
 
-__global__ void __launch_bounds__(32 * 2 * kRestrictRows)
+__global__ void __launch_bounds__(2 * kRestrictSpans)
     k_restrict_red_rb(Level<float> L, float inv_h2, const uint8_t* __restrict__ st, const float* __restrict__ rhs,
                       const float* __restrict__ e, const float* __restrict__ near_res, int cnx, int cny, int cnz,
-                      const uint8_t* __restrict__ cst, float* __restrict__ crhs, int half, int chalf, int czc) {
+                      const uint8_t* __restrict__ cst, float* __restrict__ crhs, int half, int chalf, int czc,
+                      Tile tl) {
     pdl_wait();
-    __shared__ float4 part[2][kRestrictRows][4][32];  // (coarse-plane parity, coarse row, 2 dk + dj, lane)
+    __shared__ float4 part[2][4][kRestrictSpans];  // (coarse-plane parity, 2 dk + dj, span)
     const int nxh = L.nx >> 1, ny = L.ny, nz = L.nz;
-    const int X0 = 4 * (blockIdx.x * 32 + threadIdx.x);
-    const int dj = threadIdx.y & 1, row = threadIdx.y >> 1;
-    const int cy = blockIdx.y * kRestrictRows + row;
+    const int dj = threadIdx.x / kRestrictSpans, t = threadIdx.x % kRestrictSpans;
+    int X0, cy;
+    const bool lane_on = tile_at(tl, cnx / 4, cny, t, X0, cy);
+    X0 *= 4;
     const int cz0 = (int)blockIdx.z * czc;
     const int cz1 = cz0 + czc < cnz ? cz0 + czc : cnz;
-    const bool row_on = cy < cny;
-    const bool lane_on = X0 < cnx && row_on;
-    const int iq = X0 < cnx ? X0 : 0;
-    const int y = 2 * (row_on ? cy : 0) + dj;  // (rows past the end march a valid row; nothing is stored)
+    const int iq = X0;
+    const int y = 2 * cy + dj;  // (threads without a span march a valid row; nothing is stored)
     const float* eo = e + half;  // black
     int ym, yp, il, ir;
     if (!wrap_axis(y - 1, ny, L.per[1], ym)) ym = y;
@@ -2320,9 +2363,9 @@ __global__ void __launch_bounds__(32 * 2 * kRestrictRows)
             res[k] = R[k] - (L.diag0 * Cr[k] - o) * inv_h2;
         }
         const int dk = z & 1, par = (z >> 1) & 1;
-        part[par][row][2 * dk + dj][threadIdx.x] = make_float4(res[0], res[1], res[2], res[3]);
+        part[par][2 * dk + dj][t] = make_float4(res[0], res[1], res[2], res[3]);
         if (dk == 1) {
-            // (both warps of every row reach this together: whole planes, same bounds)
+            // (every thread reaches this together: whole planes, same bounds)
             __syncthreads();
             if (dj == 0 && lane_on) {
                 // per fine row k_restrict_v adds (even child + odd child), one
@@ -2330,7 +2373,7 @@ __global__ void __launch_bounds__(32 * 2 * kRestrictRows)
                 float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
-                    const float4 p = part[par][row][q][threadIdx.x];
+                    const float4 p = part[par][q][t];
                     sum[0] += p.x;
                     sum[1] += p.y;
                     sum[2] += p.z;
@@ -3065,7 +3108,8 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
     {
         ProfScope ps_r(c, "restrict", l, b_grid);
         if (vec) {
-            dim3 rgrd((m[0] / 2 + 31) / 32, (m[1] + 7) / 8, m[2]);
+            const Tile rt = plane_tile(m[0] / 2, m[1]);
+            const dim3 rgrd = tile_grid(rt, m[0] / 2, m[1], m[2]);
             T* scratch = (T*)c->e2[l];  // (the fused sweep's second iterate; free between sweeps)
             const dim3 ngrd(near_grid_x(c), 2 * kNearSegs);
             const int* cnt = c->near_count + 2 * kNearSegs * l;
@@ -3076,27 +3120,28 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
                     launch_pdl(c, k_near_residual<T, E, RbMap>, dim3(ngrd.x, kNearSegs), 256, 0, L, st, rhs, e,
                                c->near_list[l], cnt, c->near_cap[l], (T)1 / L.h2, scratch, A, rb);
                     // coarse planes per block: up to 8, about 16 blocks per SM in all
-                    const int qx = (m[0] / 4 + 31) / 32, qy = (m[1] + kRestrictRows - 1) / kRestrictRows;
-                    int czc = (int)((long long)qx * qy * m[2] / (16LL * c->n_sm));
+                    const Tile qt = plane_tile(m[0] / 4, m[1], kRestrictSpans);
+                    dim3 qgrd = tile_grid(qt, m[0] / 4, m[1], m[2]);
+                    int czc = (int)((long long)qgrd.x * qgrd.y * m[2] / (16LL * c->n_sm));
                     czc = czc < 1 ? 1 : (czc > 8 ? 8 : czc);
-                    const dim3 qgrd(qx, qy, (m[2] + czc - 1) / czc);
-                    launch_pdl(c, k_restrict_red_rb, qgrd, dim3(32, 2 * kRestrictRows), 0, L, (T)1 / L.h2, st, rhs, e,
-                               scratch, m[0], m[1], m[2], c->st[l + 1], (T*)c->rhs[l + 1], rb.half, chalf, czc);
+                    qgrd.z = (m[2] + czc - 1) / czc;
+                    launch_pdl(c, k_restrict_red_rb, qgrd, 2 * kRestrictSpans, 0, L, (T)1 / L.h2, st, rhs, e, scratch,
+                               m[0], m[1], m[2], c->st[l + 1], (T*)c->rhs[l + 1], rb.half, chalf, czc, qt);
                     done = true;
                 } else if (split) {
                     launch_pdl(c, k_near_residual<T, E, RbMap>, ngrd, 256, 0, L, st, rhs, e, c->near_list[l], cnt,
                                c->near_cap[l], (T)1 / L.h2, scratch, A, rb);
-                    const dim3 qgrd((m[0] / 4 + 31) / 32, (m[1] + 1) / 2, m[2]);
-                    launch_pdl(c, k_restrict_rb, qgrd, vblk, 0, L, (T)1 / L.h2, st, rhs, e, scratch, m[0], m[1],
-                               c->st[l + 1], (T*)c->rhs[l + 1], rb.half, chalf);
+                    const Tile qt = plane_tile(m[0] / 4, m[1], 64);
+                    launch_pdl(c, k_restrict_rb, tile_grid(qt, m[0] / 4, m[1], m[2]), 256, 0, L, (T)1 / L.h2, st, rhs,
+                               e, scratch, m[0], m[1], c->st[l + 1], (T*)c->rhs[l + 1], rb.half, chalf, qt);
                     done = true;
                 }
             }
             if (!done) {
                 launch_pdl(c, k_near_residual<T, E>, ngrd, 256, 0, L, st, rhs, e, c->near_list[l], cnt, c->near_cap[l],
                            (T)1 / L.h2, scratch, A, NatMap{});
-                launch_pdl(c, k_restrict_v<T, E>, rgrd, vblk, 0, L, inv_diag0, (T)1 / L.h2, st, rhs, e, scratch, m[0],
-                           m[1], c->st[l + 1], (T*)c->rhs[l + 1], A, 0, red_only ? 1 : 0);
+                launch_pdl(c, k_restrict_v<T, E>, rgrd, kTileThreads, 0, L, inv_diag0, (T)1 / L.h2, st, rhs, e,
+                           scratch, m[0], m[1], c->st[l + 1], (T*)c->rhs[l + 1], A, rt, 0, red_only ? 1 : 0);
             }
             count(c, 2);
         } else if constexpr (kNative) {
@@ -3117,21 +3162,23 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
         bool done = false;
         if constexpr (kNative && std::is_same<T, float>::value) {
             if (black_only) {
-                const dim3 bgrd((L.nx / 8 + 31) / 32, (L.ny + 7) / 8, L.nz);
-                launch_pdl(c, k_prolong_black_rb, bgrd, vblk, 0, L, st, e, rb.half, m[0], m[1], c->st[l + 1],
-                           (const T*)c->e[l + 1], chalf);
+                const Tile st8 = plane_tile(L.nx / 8, L.ny);
+                launch_pdl(c, k_prolong_black_rb, tile_grid(st8, L.nx / 8, L.ny, L.nz), kTileThreads, 0, L, st, e,
+                           rb.half, m[0], m[1], c->st[l + 1], (const T*)c->e[l + 1], chalf, st8);
                 done = true;
             } else if (split) {
-                launch_pdl(c, k_prolong_v<T, E, true>, vgrd, vblk, 0, L, st, e, m[0], m[1], c->st[l + 1],
-                           (const T*)c->e[l + 1], A, rb.half, chalf);
+                const Tile vt = plane_tile(L.nx / W, L.ny);
+                launch_pdl(c, k_prolong_v<T, E, true>, tile_grid(vt, L.nx / W, L.ny, L.nz), kTileThreads, 0, L, st, e, m[0], m[1], c->st[l + 1],
+                           (const T*)c->e[l + 1], A, vt, rb.half, chalf);
                 done = true;
             }
         }
         if (done) {
-        } else if (vec)
-            launch_pdl(c, k_prolong_v<T, E>, vgrd, vblk, 0, L, st, e, m[0], m[1], c->st[l + 1], (const T*)c->e[l + 1],
-                       A, 0, 0);
-        else if constexpr (kNative)
+        } else if (vec) {
+            const Tile vt = plane_tile(L.nx / W, L.ny);
+            launch_pdl(c, k_prolong_v<T, E>, tile_grid(vt, L.nx / W, L.ny, L.nz), kTileThreads, 0, L, st, e, m[0],
+                       m[1], c->st[l + 1], (const T*)c->e[l + 1], A, vt, 0, 0);
+        } else if constexpr (kNative)
             launch_pdl(c, k_prolong<T>, full, blk, 0, L, st, e, m[0], m[1], c->st[l + 1], (const T*)c->e[l + 1]);
     }
     count(c);
@@ -3229,18 +3276,19 @@ __global__ void __launch_bounds__(256) k_flip_patch(Grid g, ff diag0, WallFF wal
 // layout and partial slots of k_outer_residual_ff<4, true> (zc planes a
 // block), for the patched residual.  gate: 1 when the full residual runs
 // instead.
-__global__ void __launch_bounds__(256) k_rhs_norm_rb(Grid g, const float* __restrict__ r, int zc,
+__global__ void __launch_bounds__(256) k_rhs_norm_rb(Grid g, const float* __restrict__ r, int zc, Tile tl,
                                                      double* __restrict__ partial, const int* __restrict__ gate) {
     if (*gate != 0) return;
     __shared__ float swarp[8];
     const int half = (int)(g.N >> 1);
     const int nx = g.nx, ny = g.ny, nz = g.nz;
-    const int xs = 4 * (blockIdx.x * 32 + threadIdx.x);
-    const int y = blockIdx.y * 8 + threadIdx.y;
+    int span, y;
+    const bool lane_on = tile_at(tl, nx / 4, ny, threadIdx.x, span, y);
+    const int xs = 4 * span;
     const int z0 = (int)blockIdx.z * zc;
     const int z1 = z0 + zc < nz ? z0 + zc : nz;
     float acc = 0.0f;
-    if (xs < nx && y < ny)
+    if (lane_on)
         for (int z = z0; z < z1; z++) {
             const Q4<float> q = rb_ld4(r, half, xs + nx * (y + ny * z), (xs + y + z) & 1);
             acc = __fmaf_rn(q.v0, q.v0, acc);
@@ -3250,9 +3298,9 @@ __global__ void __launch_bounds__(256) k_rhs_norm_rb(Grid g, const float* __rest
         }
     float v = acc;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) swarp[threadIdx.y] = v;
+    if ((threadIdx.x & 31) == 0) swarp[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
+    if (threadIdx.x == 0) {
         double tot = 0.0;
         for (int w = 0; w < 8; w++) tot += (double)swarp[w];
         partial[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = tot;
@@ -3582,10 +3630,12 @@ cudaError_t launch_outer_residual(es_ctx* c, bool patch) {
             if (c->S.pot_bc[f] == ES_POT_DIRICHLET) mask |= 1 << f;
         }
         const int W = (c->g.nx % 4) == 0 ? 4 : 1;
-        const int gx = (c->g.nx / W + 31) / 32, gy = (c->g.ny + 7) / 8;
+        const Tile tl = plane_tile(c->g.nx / W, c->g.ny);
+        dim3 grd = tile_grid(tl, c->g.nx / W, c->g.ny, 1);
+        const int gx = grd.x, gy = grd.y;
         int gz, zc;
         res_march_grid(c, gx, gy, c->g.nz, gz, zc);
-        const dim3 grd(gx, gy, gz), blk(32, 8);
+        grd.z = gz;
         const dim3 ngrd(near_grid_x(c), 2 * kNearSegs);
         const ff d0 = ff_from_double(diag0);
         float* r = (float*)c->rhs[0];
@@ -3598,13 +3648,13 @@ cudaError_t launch_outer_residual(es_ctx* c, bool patch) {
             k_outer_residual_near_ff<RbMap><<<ngrd, 256, 0, c->stream>>>(
                 c->g, d0, wall, mask, c->psi32, c->psi_lo, c->st[0], c->owner, (const float2*)c->pbc,
                 c->near_list[0], c->near_count, c->near_cap[0], r, rb);
-            k_outer_residual_ff<4, true><<<grd, blk, 0, c->stream>>>(c->g, d0, c->psi32, c->psi_lo, c->st[0], r,
-                                                                      c->partial, zc, gate);
+            k_outer_residual_ff<4, true><<<grd, kTileThreads, 0, c->stream>>>(c->g, d0, c->psi32, c->psi_lo, c->st[0],
+                                                                               r, c->partial, zc, tl, gate);
             if (patch) {
                 k_flip_patch<RbMap><<<2 * c->n_sm, 256, 0, c->stream>>>(
                     c->g, d0, wall, mask, c->psi32, c->psi_lo, c->st[0], c->owner, (const float2*)c->pbc,
                     c->flip_list, c->flip_count, c->flip_cap, r, rb, c->d_moved);
-                k_rhs_norm_rb<<<grd, blk, 0, c->stream>>>(c->g, r, zc, c->partial, c->d_moved);
+                k_rhs_norm_rb<<<grd, kTileThreads, 0, c->stream>>>(c->g, r, zc, tl, c->partial, c->d_moved);
                 count(c, 2);
             }
         } else {
@@ -3612,11 +3662,11 @@ cudaError_t launch_outer_residual(es_ctx* c, bool patch) {
                 c->g, d0, wall, mask, c->psi32, c->psi_lo, c->st[0], c->owner, (const float2*)c->pbc,
                 c->near_list[0], c->near_count, c->near_cap[0], r, NatMap{});
             if (W == 4)
-                k_outer_residual_ff<4, false><<<grd, blk, 0, c->stream>>>(c->g, d0, c->psi32, c->psi_lo, c->st[0],
-                                                                           r, c->partial, zc, nullptr);
+                k_outer_residual_ff<4, false><<<grd, kTileThreads, 0, c->stream>>>(
+                    c->g, d0, c->psi32, c->psi_lo, c->st[0], r, c->partial, zc, tl, nullptr);
             else
-                k_outer_residual_ff<1, false><<<grd, blk, 0, c->stream>>>(c->g, d0, c->psi32, c->psi_lo, c->st[0],
-                                                                           r, c->partial, zc, nullptr);
+                k_outer_residual_ff<1, false><<<grd, kTileThreads, 0, c->stream>>>(
+                    c->g, d0, c->psi32, c->psi_lo, c->st[0], r, c->partial, zc, tl, nullptr);
         }
         k_finalize_norm<<<1, 1024, 0, c->stream>>>(c->partial, gx * gy * gz, c->d_norm);
         count(c, 3);
@@ -3741,23 +3791,26 @@ cudaError_t launch_correct(es_ctx* c) {
 // (8), the state byte, and with the correction psi in and out (16).
 cudaError_t launch_residual_update(es_ctx* c, bool correct) {
     Level<float> L = level_desc<float>(c, 0);
-    const int N = (int)c->g.N, nxh = L.nx / 2;
+    const int N = (int)c->g.N;
     ProfScope ps(c, correct ? "residual_update_correct" : "residual_update", -1, (double)N * (correct ? 29.0 : 13.0));
     float* scratch = (float*)c->e2[0];
     const dim3 ngrd(near_grid_x(c), 2 * kNearSegs);
     k_near_residual<float, float, RbMap><<<ngrd, 256, 0, c->stream>>>(
         L, c->st[0], (const float*)c->rhs[0], (const float*)c->e[0], c->near_list[0], c->near_count,
         c->near_cap[0], 1.0f / L.h2, scratch, EAcc<float, float>{1.0f, 1.0f}, RbMap{N / 2});
-    const int gx = (nxh / 4 + 31) / 32, gy = (L.ny + 7) / 8;
+    const Tile tl = plane_tile(L.nx / 8, L.ny);
+    dim3 grd = tile_grid(tl, L.nx / 8, L.ny, 1);
+    const int gx = grd.x, gy = grd.y;
     int gz, zc;
     res_march_grid(c, gx, gy, L.nz, gz, zc);
+    grd.z = gz;
     if (correct)
-        k_residual_update_rb<true><<<dim3(gx, gy, gz), dim3(32, 8), 0, c->stream>>>(
-            L, 1.0f / L.h2, c->st[0], (float*)c->rhs[0], (const float*)c->e[0], scratch, N / 2, c->partial, zc,
+        k_residual_update_rb<true><<<grd, kTileThreads, 0, c->stream>>>(
+            L, 1.0f / L.h2, c->st[0], (float*)c->rhs[0], (const float*)c->e[0], scratch, N / 2, c->partial, zc, tl,
             c->psi32, c->psi_lo);
     else
-        k_residual_update_rb<false><<<dim3(gx, gy, gz), dim3(32, 8), 0, c->stream>>>(
-            L, 1.0f / L.h2, c->st[0], (float*)c->rhs[0], (const float*)c->e[0], scratch, N / 2, c->partial, zc,
+        k_residual_update_rb<false><<<grd, kTileThreads, 0, c->stream>>>(
+            L, 1.0f / L.h2, c->st[0], (float*)c->rhs[0], (const float*)c->e[0], scratch, N / 2, c->partial, zc, tl,
             nullptr, nullptr);
     k_finalize_norm<<<1, 1024, 0, c->stream>>>(c->partial, gx * gy * gz, c->d_norm);
     count(c, 3);
