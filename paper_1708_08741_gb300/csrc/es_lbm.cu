@@ -122,8 +122,7 @@ Trt<C> trt(double le, double lo) {
 //   d = (1 + lambda_o)/2 m + w c.g,               g = -3 lambda_o u + 3 ao F
 // (ae, ao = 1 + lambda / 2; w_2 = w_1 / 2 folded into h, K and g): 139
 // operations a cell instead of 357 (a 160 x 136 x 152 FP64 step: 1.88 ms
-// before, 0.96 ms now).  The MIXED32 kernel, which issues on most
-// cycles, gains from the same count: 3.89 -> 3.72 ms at 512^3.
+// before, 0.96 ms now).
 template <class C, class Put>
 __device__ __forceinline__ void collide(const C (&f)[19], C fx, C fy, C fz, const Trt<C>& R, Put&& put) {
     C p[10], m[10];
@@ -176,10 +175,11 @@ __device__ __forceinline__ void collide(const C (&f)[19], C fx, C fy, C fz, cons
     }
 }
 
-// The same collision term by term, for FP16 populations: their rounding
-// after every step decides the form's error, and with these operations the
-// 32^3 sphere's velocity after 100 steps is 8.6e-5 from the FP64 oracle, with
-// those of collide() 1.2e-4 (the FP16 kernel's time is the same either way).
+// The same collision term by term, for the reduced forms, whose rounding is
+// what decides their error: with these operations the FP16 form's 32^3
+// sphere is 8.6e-5 from the FP64 oracle's velocity after 100 steps, with those
+// of collide() 1.2e-4, and their FP32 kernels are bound by HBM (512^3 MIXED32:
+// 3.89 ms against 3.85).
 template <class C, class Put>
 __device__ __forceinline__ void collide_direct(const C (&f)[19], C fx, C fy, C fz, C lam_e, C lam_o, Put&& put) {
     // moments (Eq. MacroscopVel) with the modified velocity (Eq. modified_velocity)
@@ -369,7 +369,7 @@ __device__ __forceinline__ void lbm_cell(const Grid& g, const Streams<S>& P, con
     }
 
     auto put = [&](int q, C v) { P.dst[q][c] = St::st(q, v); };
-    if constexpr (std::is_same<S, __half>::value)
+    if constexpr (sizeof(C) == 4)
         collide_direct<C>(f, fx, fy, fz, R.lam_e, R.lam_o, put);
     else
         collide<C>(f, fx, fy, fz, R, put);
