@@ -3,6 +3,8 @@
 
 #include <cuda_fp16.h>
 
+#include <utility>
+
 #include "es_internal.cuh"
 
 namespace es {
@@ -370,6 +372,33 @@ __device__ __forceinline__ void body_force_iso(const Psi19& p, float Ex, float E
     f0 = __fmul_rn(rho_e, __fsub_rn(Ex, g0));
     f1 = __fmul_rn(rho_e, __fsub_rn(Ey, g1));
     f2 = __fmul_rn(rho_e, __fsub_rn(Ez, g2));
+}
+
+// Programmatic dependent launch for the V-cycle's chain of kernels: a
+// kernel launched by launch_pdl may be scheduled while the one before it
+// on the stream drains, and waits here (before touching memory) until that
+// one has completed and its writes are visible; launched plainly, the wait
+// returns at once.  It then lets the next kernel be scheduled in turn (that
+// one waits here for this one's end); what a kernel reads before its wait was
+// therefore written by the kernel before the last one or earlier.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... KArgs, typename... Args>
+void launch_pdl(const es_ctx* c, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);  // (errors: cudaGetLastError)
 }
 
 // host-side split of a double into float-float

@@ -28,28 +28,6 @@ namespace {
 
 constexpr int kRedThreads = 256;
 
-// Programmatic dependent launch for the V-cycle's chain of kernels: a
-// kernel launched by launch_pdl may be scheduled while the one before it
-// on the stream drains, and waits here (before touching memory) until that
-// one has completed and its writes are visible; launched plainly, the wait
-// returns at once.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-template <typename... KArgs, typename... Args>
-void launch_pdl(const es_ctx* c, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = c->stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);  // (errors: cudaGetLastError)
-}
-
 // The share of an x-y plane that a block takes in the residual, restriction
 // and prolongation kernels, whose threads own a span of a row: tw spans of th
 // rows (thread t: span t % tw of row t / tw).  Rows are rarely a multiple of
@@ -308,42 +286,53 @@ __device__ __forceinline__ float near_residual_ff(const Grid& g, ff diag0, const
                                                   const float2* __restrict__ pbc, int x, int y, int z) {
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     const int c = x + nx * (y + ny * z);
-    HiSum hs = {0.0f, 0.0f};
-    float lo = 0.0f;
-    int dk = 0;
     const int g3[3] = {x, y, z}, n3[3] = {nx, ny, nz}, stride[3] = {1, nx, nx * ny};
+    // (all loads that depend on the cell only are issued before the first is used)
+    unsigned kind[6], wallf = 0;
+    int own[6];
+    float ph[6], pl[6];
 #pragma unroll
     for (int k = 0; k < 6; k++) {
-        const int ax = k >> 1, side = (k & 1) ? 1 : -1;
-        int q = g3[ax] + side;
+        const int ax = k >> 1;
+        int q = g3[ax] + ((k & 1) ? 1 : -1);
         if (q < 0 || q >= n3[ax]) {
-            if (!g.per[ax]) {
-                const int face = 2 * ax + (side > 0 ? 1 : 0);
-                if ((pot_dir_mask >> face) & 1) {
-                    dk += 1;
-                    hs.add(wall.hi[face]);
-                    lo = __fadd_rn(lo, wall.lo[face]);
-                } else {
-                    dk -= 1;
-                }
-                continue;
-            }
+            if (!g.per[ax]) wallf |= 1u << k;
             q = q < 0 ? q + n3[ax] : q - n3[ax];
         }
         const int nb = c + (q - g3[ax]) * stride[ax];
-        const uint8_t kk = st0[nb] & ST_KIND;
-        if (kk == ST_UNKNOWN) {
-            hs.add(psi_hi[nb]);
-            lo = __fadd_rn(lo, psi_lo[nb]);
+        kind[k] = st0[nb];
+        own[k] = owner[nb];
+        ph[k] = psi_hi[nb];
+        pl[k] = psi_lo[nb];
+    }
+    const float hc = psi_hi[c], lc = psi_lo[c];
+    float2 bv[6];
+#pragma unroll
+    for (int k = 0; k < 6; k++)
+        bv[k] = !((wallf >> k) & 1u) && (kind[k] & ST_KIND) != ST_UNKNOWN ? pbc[own[k]] : make_float2(0.0f, 0.0f);
+    HiSum hs = {0.0f, 0.0f};
+    float lo = 0.0f;
+    int dk = 0;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        if ((wallf >> k) & 1u) {
+            if ((pot_dir_mask >> k) & 1) {
+                dk += 1;
+                hs.add(wall.hi[k]);
+                lo = __fadd_rn(lo, wall.lo[k]);
+            } else {
+                dk -= 1;
+            }
+        } else if ((kind[k] & ST_KIND) == ST_UNKNOWN) {
+            hs.add(ph[k]);
+            lo = __fadd_rn(lo, pl[k]);
         } else {
-            dk += kk == ST_DIR ? 1 : -1;
-            const float2 bv = pbc[owner[nb]];
-            hs.add(bv.x);
-            lo = __fadd_rn(lo, bv.y);
+            dk += (kind[k] & ST_KIND) == ST_DIR ? 1 : -1;
+            hs.add(bv[k].x);
+            lo = __fadd_rn(lo, bv[k].y);
         }
     }
     const ff dg = ff_add_f(diag0, (float)dk);
-    const float hc = psi_hi[c], lc = psi_lo[c];
     const float p = __fmul_rn(dg.hi, hc);
     float t = __fmaf_rn(dg.hi, hc, -p);
     t = __fmaf_rn(dg.hi, lc, t);
@@ -651,6 +640,102 @@ struct RbMap {
     __device__ __forceinline__ int operator()(int c, int col) const { return col * half + (c >> 1); }
 };
 
+// The six faces of a near-boundary unknown cell (x-, x+, y-, y+, z-, z+): two
+// bits each -- 0 an unknown neighbour, 1 the diagonal moves by +1 (Dirichlet),
+// otherwise by -1 (Neumann, zero flux) -- and the neighbours' cell indices
+// (beyond a wall: some valid cell).  All state bytes are loaded before the
+// first is tested: tested one by one, each face waited for its state and then
+// for its value, twelve round trips to L2 in a row that set the time of the
+// small half sweeps.
+template <class T>
+__device__ __forceinline__ unsigned near_faces(const Level<T>& L, const uint8_t* __restrict__ st, int x, int y, int z,
+                                               int (&nb)[6]) {
+    const int v[3] = {x, y, z}, n3[3] = {L.nx, L.ny, L.nz}, stride[3] = {1, L.nx, L.nx * L.ny};
+    const int c = x + L.nx * (y + L.ny * z);
+    unsigned kind[6], wall = 0;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const int a = k >> 1;
+        int p = v[a] + ((k & 1) ? 1 : -1);
+        if (p < 0 || p >= n3[a]) {
+            if (!L.per[a]) wall |= 1u << k;
+            p = p < 0 ? p + n3[a] : p - n3[a];
+        }
+        nb[k] = c + (p - v[a]) * stride[a];
+        kind[k] = st[nb[k]];
+    }
+    unsigned code = 0;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const unsigned f = ((wall >> k) & 1u) ? (L.pot_bc[k] == ES_POT_DIRICHLET ? 1u : 2u) : (kind[k] & ST_KIND);
+        code |= f << (2 * k);
+    }
+    return code;
+}
+
+// The diagonal at such a cell and the sum of its unknown neighbours' values
+// v, face by face.
+template <class T>
+__device__ __forceinline__ void near_sums(unsigned code, T diag0, const T (&v)[6], T& diag, T& off) {
+    T dg = diag0, o = (T)0;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const unsigned f = (code >> (2 * k)) & 3u;
+        if (f == 0u)
+            o += v[k];
+        else
+            dg += f == 1u ? (T)1 : (T)-1;
+    }
+    diag = dg;
+    off = o;
+}
+
+// The face code of near_faces for a cell whose neighbours' state bytes (low
+// byte of s*) are at hand; wyz: wall_codes of its row.
+template <class T>
+__device__ __forceinline__ unsigned wall_codes(const Level<T>& L, int y, int z) {
+    auto w = [&](bool on, int f) { return !on ? 0u : (L.pot_bc[f] == ES_POT_DIRICHLET ? 1u : 2u) << (2 * f); };
+    return w(!L.per[1] && y == 0, 2) | w(!L.per[1] && y == L.ny - 1, 3) | w(!L.per[2] && z == 0, 4) |
+           w(!L.per[2] && z == L.nz - 1, 5);
+}
+
+template <class T>
+__device__ __forceinline__ unsigned span_faces(const Level<T>& L, unsigned wyz, int x, unsigned sl, unsigned sr,
+                                               unsigned su, unsigned sd, unsigned sm, unsigned sp) {
+    auto w = [&](int f) { return L.pot_bc[f] == ES_POT_DIRICHLET ? 1u : 2u; };
+    const unsigned f0 = !L.per[0] && x == 0 ? w(0) : (sl & ST_KIND);
+    const unsigned f1 = !L.per[0] && x == L.nx - 1 ? w(1) : (sr & ST_KIND);
+    auto pick = [&](int f, unsigned s) { return ((wyz >> (2 * f)) & 3u) ? (wyz & (3u << (2 * f))) : (s & ST_KIND) << (2 * f); };
+    return f0 | (f1 << 2) | pick(2, su) | pick(3, sd) | pick(4, sm) | pick(5, sp);
+}
+
+// The state bytes around an 8-cell span (natural x = x0 .. x0 + 7 of row
+// (y, z), its own bytes at st + at) for its near-boundary cells.
+struct Span8 {
+    uint2 u, d, m, p;  // rows (y-1, z), (y+1, z), (y, z-1), (y, z+1)
+    unsigned l, r;     // the cells left and right of the span
+    template <class T>
+    __device__ __forceinline__ Span8(const Level<T>& L, const uint8_t* __restrict__ st, int at, int y, int z, int ym,
+                                     int yp, int iq) {
+        const int plane = L.nx * L.ny;
+        auto ld = [&](int o) { return *reinterpret_cast<const uint2*>(st + o); };
+        u = ld(at + (ym - y) * L.nx);
+        d = ld(at + (yp - y) * L.nx);
+        m = ld(z > 0 ? at - plane : (L.per[2] ? at + (L.nz - 1) * plane : at));
+        p = ld(z + 1 < L.nz ? at + plane : (L.per[2] ? at - (L.nz - 1) * plane : at));
+        const int x0 = 2 * iq;
+        l = st[at + (x0 > 0 ? -1 : (L.per[0] ? L.nx - 1 : 0))];
+        r = st[at + (x0 + 8 < L.nx ? 8 : (L.per[0] ? 8 - L.nx : 7))];
+    }
+    static __device__ __forceinline__ unsigned byte(const uint2& w, int j) { return (j < 4 ? w.x : w.y) >> (8 * (j & 3)); }
+    // face code of cell x0 + j; own: the span's own state bytes
+    template <class T>
+    __device__ __forceinline__ unsigned faces(const Level<T>& L, unsigned wyz, int x0, int j, const uint2& own) const {
+        return span_faces(L, wyz, x0 + j, j == 0 ? l : byte(own, j - 1), j == 7 ? r : byte(own, j + 1), byte(u, j),
+                          byte(d, j), byte(m, j), byte(p, j));
+    }
+};
+
 // Diagonal and off-diagonal sum of level l at an unknown cell.  With
 // READ = false only the diagonal is formed (off = 0, e is not touched).
 template <class T, bool READ = true, class E = T, class M = NatMap>
@@ -678,29 +763,14 @@ __device__ __forceinline__ void level_stencil(const Level<T>& L, const uint8_t* 
         off = o;
         return;
     }
-    T dg = L.diag0;
-    T o = (T)0;
-    const int v[3] = {x, y, z}, n3[3] = {L.nx, L.ny, L.nz}, stride[3] = {1, nx, nxy};
-    for (int a = 0; a < 3; a++)
-        for (int side = -1; side <= 1; side += 2) {
-            int p = v[a] + side;
-            if (p < 0 || p >= n3[a]) {
-                if (!L.per[a]) {
-                    dg += (L.pot_bc[2 * a + (side > 0 ? 1 : 0)] == ES_POT_DIRICHLET) ? (T)1 : (T)-1;
-                    continue;
-                }
-                p = p < 0 ? p + n3[a] : p - n3[a];
-            }
-            const int nb = c + (p - v[a]) * stride[a];
-            const uint8_t k = st[nb] & ST_KIND;
-            if (k == ST_UNKNOWN) {
-                if (READ) o += A.ld(e + m(nb, ncol));
-            } else {
-                dg += (k == ST_DIR) ? (T)1 : (T)-1;
-            }
-        }
-    diag = dg;
-    off = o;
+    int nb[6];
+    const unsigned code = near_faces(L, st, x, y, z, nb);
+    T v[6] = {(T)0, (T)0, (T)0, (T)0, (T)0, (T)0};
+    if (READ) {
+#pragma unroll
+        for (int k = 0; k < 6; k++) v[k] = A.ld(e + m(nb[k], ncol));
+    }
+    near_sums(code, L.diag0, v, diag, off);
 }
 
 // One red (colour 0) or black (1) Gauss-Seidel / SOR half sweep,
@@ -772,13 +842,13 @@ __device__ __forceinline__ T near_gs(const Level<T>& L, const uint8_t* __restric
                                      const EAcc<T, E>& A = EAcc<T, E>{(T)1, (T)1}, M m = M{}) {
     const int cidx = x + L.nx * (y + L.ny * z);
     const int col = (x + y + z) & 1;
-    const uint8_t s = st[cidx];
+    const T r = rhs[m(cidx, col)];
     T diag, off;
     if (first == 1)
-        level_stencil<T, false, E, M>(L, st, e, x, y, z, s, diag, off, A, m);
+        level_stencil<T, false, E, M>(L, st, e, x, y, z, ST_NEAR, diag, off, A, m);
     else
-        level_stencil<T, true, E, M>(L, st, e, x, y, z, s, diag, off, A, m);
-    const T gs = (L.h2 * rhs[m(cidx, col)] + off) / diag;
+        level_stencil<T, true, E, M>(L, st, e, x, y, z, ST_NEAR, diag, off, A, m);
+    const T gs = (L.h2 * r + off) / diag;
     return first ? omega * gs : ((T)1 - omega) * A.ld(e + m(cidx, col)) + omega * gs;
 }
 
@@ -795,25 +865,47 @@ struct NearWork {
 // half-sweep launch after their interior spans: with at least kNearSegs
 // blocks, block b serves segment b % kNearSegs together with the other
 // blocks of that residue; with fewer, block b serves segments b, b + nblk, ...
+// The list is the mapping's, at least two kernels back, so a thread looks up
+// its first cell (most have none or one) before it waits for the kernel
+// before this one (near_first).
+struct NearShare {
+    int nblk, b, tid, nth;
+    bool many;
+    __device__ __forceinline__ NearShare() {
+        nblk = (int)(gridDim.x * gridDim.y * gridDim.z);
+        b = ((int)blockIdx.z * (int)gridDim.y + (int)blockIdx.y) * (int)gridDim.x + (int)blockIdx.x;
+        tid = (int)((threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x);
+        nth = (int)(blockDim.x * blockDim.y * blockDim.z);
+        many = nblk >= kNearSegs;
+    }
+    __device__ __forceinline__ int seg0() const { return many ? b % kNearSegs : b; }
+    __device__ __forceinline__ int start() const { return (many ? b / kNearSegs : 0) * nth + tid; }
+};
+
+// This thread's first cell, or -1.
+__device__ __forceinline__ int near_first(const NearWork& nw, int colour) {
+    const NearShare s;
+    if (s.seg0() >= kNearSegs) return -1;
+    const int k = colour * kNearSegs + s.seg0(), i = s.start();
+    return i < nw.count[k] ? nw.list[(size_t)k * nw.cap + i] : -1;
+}
+
 template <class T, class E, class M>
-__device__ __forceinline__ void near_share(const Level<T>& L, const NearWork& nw, const T* __restrict__ rhs, E* e,
-                                           int colour, int first, T omega, const EAcc<T, E>& A, M m) {
-    const int nblk = (int)(gridDim.x * gridDim.y * gridDim.z);
-    const int b = ((int)blockIdx.z * (int)gridDim.y + (int)blockIdx.y) * (int)gridDim.x + (int)blockIdx.x;
-    const bool many = nblk >= kNearSegs;
-    const int tid = (int)((threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x);
-    const int nth = (int)(blockDim.x * blockDim.y * blockDim.z);
-    for (int seg = many ? b % kNearSegs : b; seg < kNearSegs; seg += many ? kNearSegs : nblk) {
-        const int sb = many ? b / kNearSegs : 0;
-        const int nsb = many ? (nblk - seg + kNearSegs - 1) / kNearSegs : 1;  // blocks on this segment
+__device__ __forceinline__ void near_share(const Level<T>& L, const NearWork& nw, int cc, const T* __restrict__ rhs,
+                                           E* e, int colour, int first, T omega, const EAcc<T, E>& A, M m) {
+    const NearShare s;
+    if (cc < 0 && s.many) return;
+    for (int seg = s.seg0(); seg < kNearSegs; seg += s.many ? kNearSegs : s.nblk) {
+        const int nsb = s.many ? (s.nblk - seg + kNearSegs - 1) / kNearSegs : 1;  // blocks on this segment
         const int k = colour * kNearSegs + seg;
         const int n = nw.count[k];
         const int* list = nw.list + (size_t)k * nw.cap;
-        for (int i = sb * nth + tid; i < n; i += nsb * nth) {
-            const int cc = list[i];
+        for (int i = s.start(); i < n; i += nsb * s.nth) {
+            if (cc < 0) cc = list[i];
             const int x = cc % L.nx, yz = cc / L.nx;
             const int yy = yz % L.ny, zz = yz / L.ny;
             A.st(e + m(cc, colour), near_gs<T, E, M>(L, nw.st, rhs, e, x, yy, zz, first, omega, A, m));
+            cc = -1;
         }
     }
 }
@@ -833,11 +925,13 @@ template <class T, int W, bool INLINE_NEAR, class E = T>
 __global__ void __launch_bounds__(256) k_smooth_v(Level<T> L, T inv_diag0, const uint8_t* __restrict__ st,
                                                   const T* __restrict__ rhs, E* __restrict__ e, int colour,
                                                   int first, T omega, EAcc<T, E> A, NearWork nw) {
+    int cc0 = -1;
+    if constexpr (!INLINE_NEAR) cc0 = near_first(nw, colour);
     pdl_wait();
     const int xs = W * (blockIdx.x * 32 + threadIdx.x);
     const int y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
     if (y < L.ny) smooth_v_span<T, W, INLINE_NEAR, E>(L, inv_diag0, st, rhs, e, colour, first, omega, A, xs, y, z);
-    if constexpr (!INLINE_NEAR) near_share<T, E, NatMap>(L, nw, rhs, e, colour, first, omega, A, NatMap{});
+    if constexpr (!INLINE_NEAR) near_share<T, E, NatMap>(L, nw, cc0, rhs, e, colour, first, omega, A, NatMap{});
 }
 
 template <class T, int W, bool INLINE_NEAR, class E>
@@ -1106,9 +1200,10 @@ __global__ void __launch_bounds__(256, 4) k_smooth_rb(Level<T> L, T inv_diag0, c
                                                       int wpr, const T* __restrict__ rhs, T* __restrict__ e,
                                                       int colour, int first, T omega, int half, NearWork nw,
                                                       int zc) {
+    const int cc0 = near_first(nw, colour);
     pdl_wait();
-    const int i0 = 4 * (blockIdx.x * 32 + threadIdx.x);
-    const int y = blockIdx.y * 8 + threadIdx.y;
+    const int i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (y < L.ny && i0 < (L.nx >> 1)) {
         const int z0 = (int)blockIdx.z * zc;
         const int z1 = z0 + zc < L.nz ? z0 + zc : L.nz;
@@ -1126,7 +1221,7 @@ __global__ void __launch_bounds__(256, 4) k_smooth_rb(Level<T> L, T inv_diag0, c
             rb_march<T, 0, false>(L, inv_diag0, mcol, wpr, rcol, eo, es, colour, omega, i0, y, z0, z1);
     }
     // the near-boundary cells, shared out to the blocks
-    near_share<T, T, RbMap>(L, nw, rhs, e, colour, first, omega, EAcc<T, T>{(T)1, (T)1}, RbMap{half});
+    near_share<T, T, RbMap>(L, nw, cc0, rhs, e, colour, first, omega, EAcc<T, T>{(T)1, (T)1}, RbMap{half});
 }
 
 __device__ __forceinline__ bool axis_ok(int v, int n, int per, int& w) {
@@ -1373,6 +1468,7 @@ __global__ void __launch_bounds__(256) k_smooth_rb_bulk(Level<T> L, T inv_diag0,
                                                         int wpr, const T* __restrict__ rhs, T* __restrict__ e,
                                                         int colour, int first, T omega, int half, NearWork nw,
                                                         BulkShape B, int* status) {
+    const int cc0 = near_first(nw, colour);
     pdl_wait();
     extern __shared__ __align__(16) unsigned char bsm[];
     __shared__ __align__(8) uint64_t bars[kBulkSlots];
@@ -1407,7 +1503,7 @@ __global__ void __launch_bounds__(256) k_smooth_rb_bulk(Level<T> L, T inv_diag0,
         return;
     }
     // the colour's near-boundary cells, shared out as in k_smooth_rb
-    near_share<T, T, RbMap>(L, nw, rhs, e, colour, first, omega, EAcc<T, T>{(T)1, (T)1}, RbMap{half});
+    near_share<T, T, RbMap>(L, nw, cc0, rhs, e, colour, first, omega, EAcc<T, T>{(T)1, (T)1}, RbMap{half});
 }
 
 template <class T>
@@ -1812,12 +1908,6 @@ __global__ void __launch_bounds__(256) k_prolong_black_rb(Level<float> L, const 
     vst(eb, v[0], v[1], v[2], v[3]);
 }
 
-// Vectorized residual + restriction: a thread owns 2 coarse cells of a
-// coarse row, i.e. a 4 x 2 x 2 block of fine cells (nx % 4 == 0).  For each
-// of its 4 fine rows it loads the row (with one cell of x halo from the
-// neighbouring vectors) and the 4 neighbour rows as 16-byte vectors, forms
-// the residuals and adds them to the coarse sums in the children order
-// (dk, dj, di) of the scalar kernel.
 template <class T, class E = T, class M = NatMap>
 __device__ __forceinline__ T near_residual(const Level<T>& L, const uint8_t* __restrict__ st,
                                            const T* __restrict__ rhs, const E* __restrict__ e, int x, int y, int z,
@@ -1825,13 +1915,13 @@ __device__ __forceinline__ T near_residual(const Level<T>& L, const uint8_t* __r
     const int cidx = x + L.nx * (y + L.ny * z);
     const int sc = m(cidx, (x + y + z) & 1);
     T diag, off;
-    level_stencil<T, true, E, M>(L, st, e, x, y, z, st[cidx], diag, off, A, m);
+    level_stencil<T, true, E, M>(L, st, e, x, y, z, ST_NEAR, diag, off, A, m);
     return rhs[sc] - (diag * A.ld(e + sc) - off) * inv_h2;
 }
 
-// The residual at the near-boundary unknown cells of a level, from its
-// near-cell list (both colours), into a scratch array that the restriction
-// then reads for those children.
+// The residual at the near-boundary unknown cells of a large colour-split
+// level, from its near-cell list, into a scratch array that the restriction
+// and the residual update then read for those cells.
 template <class T, class E, class M = NatMap>
 __global__ void __launch_bounds__(256) k_near_residual(Level<T> L, const uint8_t* __restrict__ st,
                                                        const T* __restrict__ rhs, const E* __restrict__ e,
@@ -1849,12 +1939,20 @@ __global__ void __launch_bounds__(256) k_near_residual(Level<T> L, const uint8_t
     }
 }
 
+// Vectorized residual + restriction: a thread owns 2 coarse cells of a
+// coarse row, i.e. a 4 x 2 x 2 block of fine cells (nx % 4 == 0).  For each
+// of its 4 fine rows it loads the row (with one cell of x halo from the
+// neighbouring vectors) and the 4 neighbour rows as 16-byte vectors, forms
+// the residuals and adds them to the coarse sums in the children order
+// (dk, dj, di) of the scalar kernel.
 // SPLIT: e and rhs of this level in the colour-split layout (float).
-template <class T, class E, bool SPLIT = false>
+// INLINE_NEAR: near-boundary children load their neighbours' state bytes
+// here; else they come from k_near_residual, run just before (see
+// restrict_inline).
+template <class T, class E, bool INLINE_NEAR, bool SPLIT = false>
 __global__ void __launch_bounds__(256) k_restrict_v(Level<T> L, T inv_diag0, T inv_h2, const uint8_t* __restrict__ st,
                                                     const T* __restrict__ rhs, const E* __restrict__ e,
-                                                    const T* __restrict__ near_res, int cnx,
-                                                    int cny, const uint8_t* __restrict__ cst, T* __restrict__ crhs,
+                                                    const T* __restrict__ near_res, int cnx, int cny, const uint8_t* __restrict__ cst, T* __restrict__ crhs,
                                                     EAcc<T, E> A, Tile tl, int half = 0, int red_only = 0) {
     pdl_wait();
     int span, cy;
@@ -1931,10 +2029,29 @@ __global__ void __launch_bounds__(256) k_restrict_v(Level<T> L, T inv_diag0, T i
                 o += f[i];
                 res[i] = r[i] - (L.diag0 * c[i + 1] - o) * inv_h2;
             }
-            // near-boundary children: formed by k_near_residual just before
+            if constexpr (!INLINE_NEAR) {
 #pragma unroll
-            for (int i = 0; i < 4; i++)
-                if ((near_bits >> i) & 1u) res[i] = near_res[row + xq + i];
+                for (int i = 0; i < 4; i++)
+                    if ((near_bits >> i) & 1u) res[i] = near_res[row + xq + i];
+            } else if (near_bits) {  // (Sec. 5.4: the values are in registers)
+                const unsigned su = *reinterpret_cast<const unsigned*>(st + rym + xq);
+                const unsigned sd = *reinterpret_cast<const unsigned*>(st + ryp + xq);
+                const unsigned sm = *reinterpret_cast<const unsigned*>(st + rzm + xq);
+                const unsigned sp = *reinterpret_cast<const unsigned*>(st + rzp + xq);
+                const unsigned sl = st[row + xl], sr = st[row + xr];
+                const unsigned wyz = wall_codes(L, y, z);
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    if (!((near_bits >> i) & 1u)) continue;
+                    const unsigned code = span_faces(L, wyz, xq + i, i == 0 ? sl : (sw >> (8 * (i - 1))),
+                                                     i == 3 ? sr : (sw >> (8 * (i + 1))), su >> (8 * i), sd >> (8 * i),
+                                                     sm >> (8 * i), sp >> (8 * i));
+                    const T v[6] = {c[i], c[i + 2], a[i], b[i], d[i], f[i]};
+                    T dg, o;
+                    near_sums(code, L.diag0, v, dg, o);
+                    res[i] = r[i] - (dg * c[i + 1] - o) * inv_h2;
+                }
+            }
             if (red_only) {
                 // (after a Gauss-Seidel black half sweep the black residuals
                 // vanish: see k_restrict_red_rb)
@@ -1964,12 +2081,11 @@ __global__ void __launch_bounds__(256) k_restrict_v(Level<T> L, T inv_diag0, T i
 // the right-hand sides, all as 16-byte vectors.  The four partial sums of
 // a coarse cell are then added through shared memory in the order of
 // k_restrict_v (dk outer, dj inner), whose arithmetic this repeats exactly;
-// near-boundary children come from k_near_residual.
+// near-boundary children load their neighbours' state bytes as well.
 __global__ void __launch_bounds__(256) k_restrict_rb(Level<float> L, float inv_h2, const uint8_t* __restrict__ st,
                                                      const float* __restrict__ rhs, const float* __restrict__ e,
-                                                     const float* __restrict__ near_res, int cnx, int cny,
-                                                     const uint8_t* __restrict__ cst, float* __restrict__ crhs,
-                                                     int half, int chalf, Tile tl) {
+                                                     int cnx, int cny, const uint8_t* __restrict__ cst,
+                                                     float* __restrict__ crhs, int half, int chalf, Tile tl) {
     pdl_wait();
     __shared__ float4 part[4][64];
     const int sub = threadIdx.x >> 6, t = threadIdx.x & 63;
@@ -2000,6 +2116,9 @@ __global__ void __launch_bounds__(256) k_restrict_rb(Level<float> L, float inv_h
     const float hl = E1[rowh + il], hr = E0[rowh + ir];
     const uint2 sw = *reinterpret_cast<const uint2*>(st + nx * (y + ny * z) + 2 * Xq);
     float res[8];
+    const int at = nx * (y + ny * z) + 2 * Xq;
+    const unsigned wyz = wall_codes(L, y, z);
+    unsigned near = 0;
     // even-x children (A): x neighbours B[k-1] (or the halo), B[k]
     ES_VLD(r, 0, rhs + pe * half + rowh + Xq);
     ES_VLD(a, 0, E1 + hym + Xq);
@@ -2010,7 +2129,11 @@ __global__ void __launch_bounds__(256) k_restrict_rb(Level<float> L, float inv_h
     for (int k = 0; k < 4; k++) {
         const unsigned sv = ((k < 2 ? sw.x : sw.y) >> (16 * (k & 1))) & 0xFFu;
         res[2 * k] = 0.0f;
-        if ((sv & (ST_KIND | ST_NEAR)) != ST_UNKNOWN) continue;
+        if ((sv & ST_KIND) != ST_UNKNOWN) continue;
+        if (sv & ST_NEAR) {
+            near |= 1u << k;
+            continue;
+        }
         float o = k == 0 ? hl : B[k - 1];
         o += B[k];
         o += a[k];
@@ -2019,6 +2142,18 @@ __global__ void __launch_bounds__(256) k_restrict_rb(Level<float> L, float inv_h
         o += f[k];
         res[2 * k] = r[k] - (L.diag0 * A[k] - o) * inv_h2;
     }
+    if (near) {
+        const Span8 S(L, st, at, y, z, ym, yp, Xq);
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (!((near >> k) & 1u)) continue;
+            const float v[6] = {k == 0 ? hl : B[k - 1], B[k], a[k], b[k], d[k], f[k]};
+            float dg, o;
+            near_sums(S.faces(L, wyz, 2 * Xq, 2 * k, sw), L.diag0, v, dg, o);
+            res[2 * k] = r[k] - (dg * A[k] - o) * inv_h2;
+        }
+    }
+    near = 0;
     // odd-x children (B): x neighbours A[k], A[k+1] (or the halo)
     ES_VLD(r, 0, rhs + (pe ^ 1) * half + rowh + Xq);
     ES_VLD(a, 0, E0 + hym + Xq);
@@ -2029,7 +2164,11 @@ __global__ void __launch_bounds__(256) k_restrict_rb(Level<float> L, float inv_h
     for (int k = 0; k < 4; k++) {
         const unsigned sv = ((k < 2 ? sw.x : sw.y) >> (16 * (k & 1) + 8)) & 0xFFu;
         res[2 * k + 1] = 0.0f;
-        if ((sv & (ST_KIND | ST_NEAR)) != ST_UNKNOWN) continue;
+        if ((sv & ST_KIND) != ST_UNKNOWN) continue;
+        if (sv & ST_NEAR) {
+            near |= 1u << k;
+            continue;
+        }
         float o = A[k];
         o += k == 3 ? hr : A[k + 1];
         o += a[k];
@@ -2038,12 +2177,16 @@ __global__ void __launch_bounds__(256) k_restrict_rb(Level<float> L, float inv_h
         o += f[k];
         res[2 * k + 1] = r[k] - (L.diag0 * B[k] - o) * inv_h2;
     }
-    // near-boundary children: formed by k_near_residual just before
-    const int rown = nx * (y + ny * z) + 2 * Xq;
+    if (near) {
+        const Span8 S(L, st, at, y, z, ym, yp, Xq);
 #pragma unroll
-    for (int j = 0; j < 8; j++) {
-        const unsigned sv = ((j < 4 ? sw.x : sw.y) >> (8 * (j & 3))) & 0xFFu;
-        if ((sv & (ST_KIND | ST_NEAR)) == (ST_UNKNOWN | ST_NEAR)) res[j] = near_res[rown + j];
+        for (int k = 0; k < 4; k++) {
+            if (!((near >> k) & 1u)) continue;
+            const float v[6] = {A[k], k == 3 ? hr : A[k + 1], a[k], b[k], d[k], f[k]};
+            float dg, o;
+            near_sums(S.faces(L, wyz, 2 * Xq, 2 * k + 1, sw), L.diag0, v, dg, o);
+            res[2 * k + 1] = r[k] - (dg * B[k] - o) * inv_h2;
+        }
     }
     part[sub][t] = make_float4(res[0] + res[1], res[2] + res[3], res[4] + res[5], res[6] + res[7]);
     __syncthreads();
@@ -2281,11 +2424,16 @@ __global__ void __launch_bounds__(256, 2) k_residual_update_rb(Level<float> L, f
 // and the loads of plane z+1 are issued before plane z is formed.  The two
 // threads of a coarse span (dj = 0, 1) meet in shared memory after each pair
 // of fine planes, and the 4 red children are added in the order of
-// k_restrict_v (dk outer, dj inner).  Near-boundary red children come from
+// k_restrict_v (dk outer, dj inner).  Near-boundary red children:
+// INLINE_NEAR (levels of up to near_list_cells cells) loads their neighbours'
+// state bytes here, which saves the launch of k_near_residual ahead of it
+// (17 -> 11-15 us at 96^3 .. 128^3); on larger levels its registers (113
+// against 74) cost more (249 -> 357 us at 512^3), and the children come from
 // k_near_residual (red segments).  chalf != 0: the coarse right-hand side
 // is stored colour-split (chalf: half the coarse cells).
 constexpr int kRestrictSpans = 128;  // spans of four coarse cells per block (two threads each)
 
+template <bool INLINE_NEAR>
 __global__ void __launch_bounds__(2 * kRestrictSpans)
     k_restrict_red_rb(Level<float> L, float inv_h2, const uint8_t* __restrict__ st, const float* __restrict__ rhs,
                       const float* __restrict__ e, const float* __restrict__ near_res, int cnx, int cny, int cnz,
@@ -2344,6 +2492,7 @@ __global__ void __launch_bounds__(2 * kRestrictSpans)
         // the black row with its halo: ox[0] left of X0 (O = 0), ox[5] right of X0+3 (O = 1)
         const float ox[6] = {O == 0 ? h : 0.0f, X[0], X[1], X[2], X[3], O == 1 ? h : 0.0f};
         float res[4];
+        unsigned near = 0;
 #pragma unroll
         for (int k = 0; k < 4; k++) {
             const int bit = 2 * k + O;
@@ -2351,7 +2500,10 @@ __global__ void __launch_bounds__(2 * kRestrictSpans)
             res[k] = 0.0f;
             if ((sv & ST_KIND) != ST_UNKNOWN) continue;
             if (sv & ST_NEAR) {
-                res[k] = near_res[rown + bit];
+                if constexpr (INLINE_NEAR)
+                    near |= 1u << k;
+                else
+                    res[k] = near_res[rown + bit];
                 continue;
             }
             float o = O == 0 ? ox[k] : ox[k + 1];  // (left, right, y-, y+, z-, z+ as k_restrict_v)
@@ -2361,6 +2513,21 @@ __global__ void __launch_bounds__(2 * kRestrictSpans)
             o += D[k];
             o += F[k];
             res[k] = R[k] - (L.diag0 * Cr[k] - o) * inv_h2;
+        }
+        // near-boundary red children (Sec. 5.4): the values are in
+        // registers, the neighbours' state bytes are loaded here
+        if (INLINE_NEAR && near) {
+            const Span8 S(L, st, rown, y, z, ym, yp, iq);
+            const unsigned wyz = wall_codes(L, y, z);
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (!((near >> k) & 1u)) continue;
+                const float v[6] = {O == 0 ? ox[k] : ox[k + 1], O == 0 ? ox[k + 1] : ox[k + 2], A[k], B[k], D[k], F[k]};
+                float dg, o;
+                near_sums(O == 0 ? S.faces(L, wyz, 2 * iq, 2 * k, sw) : S.faces(L, wyz, 2 * iq, 2 * k + 1, sw), L.diag0,
+                          v, dg, o);
+                res[k] = R[k] - (dg * Cr[k] - o) * inv_h2;
+            }
         }
         const int dk = z & 1, par = (z >> 1) & 1;
         part[par][2 * dk + dj][t] = make_float4(res[0], res[1], res[2], res[3]);
@@ -2795,12 +2962,34 @@ __global__ void __launch_bounds__(256) k_body_force_near(Grid g, Solver s, float
         const int c = seg[i];
         const int x = c % g.nx, yz = c / g.nx, y = yz % g.ny, z = yz / g.ny;
         const float pc = psi[c];
-        const float g0 = 0.5f * (face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 0, 1) -
-                                 face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 0, -1));
-        const float g1 = 0.5f * (face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 1, 1) -
-                                 face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 1, -1));
-        const float g2 = 0.5f * (face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 2, 1) -
-                                 face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 2, -1));
+        // (as face_value_f; all loads that depend on the cell only first)
+        const int g3[3] = {x, y, z}, n3[3] = {g.nx, g.ny, g.nz}, stride[3] = {1, g.nx, g.nx * g.ny};
+        unsigned kind[6], wallf = 0;
+        int own[6];
+        float v[6];
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            const int ax = k >> 1;
+            int q = g3[ax] + ((k & 1) ? 1 : -1);
+            if (q < 0 || q >= n3[ax]) {
+                if (!g.per[ax]) wallf |= 1u << k;
+                q = q < 0 ? q + n3[ax] : q - n3[ax];
+            }
+            const int nb = c + (q - g3[ax]) * stride[ax];
+            kind[k] = st0[nb];
+            own[k] = owner[nb];
+            v[k] = psi[nb];
+        }
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            if ((wallf >> k) & 1u)
+                v[k] = s.pot_bc[k] == ES_POT_DIRICHLET ? wall2.v2[k] - pc : pc;
+            else if ((kind[k] & ST_KIND) != ST_UNKNOWN) {
+                const float b = pbc[own[k]].x;
+                v[k] = (kind[k] & ST_KIND) == ST_DIR ? b - pc : pc + b;
+            }
+        }
+        const float g0 = 0.5f * (v[1] - v[0]), g1 = 0.5f * (v[3] - v[2]), g2 = 0.5f * (v[5] - v[4]);
         const float rho_e = -k2e * pc;
         fb[c] = rho_e * (Ex - g0);
         fb[(size_t)g.N + c] = rho_e * (Ey - g1);
@@ -2850,6 +3039,18 @@ size_t coarse_smem_bytes(const es_ctx* c, size_t tsize) {
 // pass over the near-cell list.
 long long inline_near_cells(const es_ctx* c) {
     return c->P.near_list_cells > 0 ? (long long)c->P.near_list_cells : (long long)ES_NEAR_LIST_CELLS;
+}
+
+// Whether the restriction of a natural level of Nl cells forms its
+// near-boundary children itself (saving the launch of k_near_residual and its
+// serial chain of loads) or takes them from that pass.  FP64: the pass packs
+// those cells into full warps, and a warp costs the FP64 pipe the same
+// whatever its lanes do, so from 2^18 cells on the pass wins (16^3 .. 32^3:
+// 23 -> 18 us inline, 64^3 the same, 128^3 54 -> 68 us).
+template <class T>
+bool restrict_inline(const es_ctx* c, int Nl) {
+    const long long most = inline_near_cells(c);
+    return Nl <= (sizeof(T) == 8 && most > (1 << 18) ? (1 << 18) : most);
 }
 
 // Launch shape of the fused sweep: 128 x 12 output tiles, and the z extent
@@ -2969,7 +3170,16 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
                 // near-boundary cells from the list
                 // planes per block: up to 16, keeping about eight blocks per
                 // SM in all
-                const int gx = (L.nx / 8 + 31) / 32, gy = (L.ny + 7) / 8;
+                // rows of at most half a block's width take a narrower, taller
+                // block, as long as every SM still gets about six (128^3,
+                // 16 spans: a V-cycle 272 -> 250 us; at 96^3, where four an
+                // SM would be left, 208 -> 215 us)
+                int bx = 32;
+                while (bx > 8 && L.nx / 8 <= bx / 2 &&
+                       (long long)((L.ny + 512 / bx - 1) / (512 / bx)) * L.nz >= 6LL * c->n_sm)
+                    bx /= 2;
+                const dim3 sblk(bx, 256 / bx);
+                const int gx = (L.nx / 8 + bx - 1) / bx, gy = (L.ny + 256 / bx - 1) / (256 / bx);
                 int zc = (int)((long long)gx * gy * L.nz / (8LL * c->n_sm));
                 zc = zc < 1 ? 1 : (zc > 16 ? 16 : zc);
                 const dim3 sgrd(gx, gy, (L.nz + zc - 1) / zc);
@@ -3016,7 +3226,7 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
                         launch_pdl(c, k_smooth_rb_bulk<T>, bgrd, 256, bsm, L, inv_diag0, rbmask, rb_wpr, rhs, e, col,
                                    fs, omega, rb.half, nw, bs, c->d_status);
                     else
-                        launch_pdl(c, k_smooth_rb<T>, sgrd, vblk, 0, L, inv_diag0, rbmask, rb_wpr, rhs, e, col, fs,
+                        launch_pdl(c, k_smooth_rb<T>, sgrd, sblk, 0, L, inv_diag0, rbmask, rb_wpr, rhs, e, col, fs,
                                    omega, rb.half, nw, zc);
                 }
                 count(c, 2);
@@ -3110,40 +3320,48 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
         if (vec) {
             const Tile rt = plane_tile(m[0] / 2, m[1]);
             const dim3 rgrd = tile_grid(rt, m[0] / 2, m[1], m[2]);
-            T* scratch = (T*)c->e2[l];  // (the fused sweep's second iterate; free between sweeps)
-            const dim3 ngrd(near_grid_x(c), 2 * kNearSegs);
-            const int* cnt = c->near_count + 2 * kNearSegs * l;
             bool done = false;
             if constexpr (kNative && std::is_same<T, float>::value) {
                 if (split && red_only) {
-                    // (red near cells only: the first kNearSegs segments)
-                    launch_pdl(c, k_near_residual<T, E, RbMap>, dim3(ngrd.x, kNearSegs), 256, 0, L, st, rhs, e,
-                               c->near_list[l], cnt, c->near_cap[l], (T)1 / L.h2, scratch, A, rb);
                     // coarse planes per block: up to 8, about 16 blocks per SM in all
                     const Tile qt = plane_tile(m[0] / 4, m[1], kRestrictSpans);
                     dim3 qgrd = tile_grid(qt, m[0] / 4, m[1], m[2]);
                     int czc = (int)((long long)qgrd.x * qgrd.y * m[2] / (16LL * c->n_sm));
                     czc = czc < 1 ? 1 : (czc > 8 ? 8 : czc);
                     qgrd.z = (m[2] + czc - 1) / czc;
-                    launch_pdl(c, k_restrict_red_rb, qgrd, 2 * kRestrictSpans, 0, L, (T)1 / L.h2, st, rhs, e, scratch,
-                               m[0], m[1], m[2], c->st[l + 1], (T*)c->rhs[l + 1], rb.half, chalf, czc, qt);
+                    const bool inl = Nl <= inline_near_cells(c);
+                    T* scratch = (T*)c->e2[l];  // (the fused sweep's second iterate; free between sweeps)
+                    if (!inl) {  // (red near cells only: the first kNearSegs segments)
+                        launch_pdl(c, k_near_residual<T, E, RbMap>, dim3(near_grid_x(c), kNearSegs), 256, 0, L, st, rhs,
+                                   e, c->near_list[l], c->near_count + 2 * kNearSegs * l, c->near_cap[l],
+                                   (T)1 / L.h2, scratch, A, rb);
+                        count(c);
+                    }
+                    launch_pdl(c, inl ? k_restrict_red_rb<true> : k_restrict_red_rb<false>, qgrd, 2 * kRestrictSpans, 0,
+                               L, (T)1 / L.h2, st, rhs, e, scratch, m[0], m[1], m[2], c->st[l + 1],
+                               (T*)c->rhs[l + 1], rb.half, chalf, czc, qt);
                     done = true;
                 } else if (split) {
-                    launch_pdl(c, k_near_residual<T, E, RbMap>, ngrd, 256, 0, L, st, rhs, e, c->near_list[l], cnt,
-                               c->near_cap[l], (T)1 / L.h2, scratch, A, rb);
                     const Tile qt = plane_tile(m[0] / 4, m[1], 64);
                     launch_pdl(c, k_restrict_rb, tile_grid(qt, m[0] / 4, m[1], m[2]), 256, 0, L, (T)1 / L.h2, st, rhs,
-                               e, scratch, m[0], m[1], c->st[l + 1], (T*)c->rhs[l + 1], rb.half, chalf, qt);
+                               e, m[0], m[1], c->st[l + 1], (T*)c->rhs[l + 1], rb.half, chalf, qt);
                     done = true;
                 }
             }
             if (!done) {
-                launch_pdl(c, k_near_residual<T, E>, ngrd, 256, 0, L, st, rhs, e, c->near_list[l], cnt, c->near_cap[l],
-                           (T)1 / L.h2, scratch, A, NatMap{});
-                launch_pdl(c, k_restrict_v<T, E>, rgrd, kTileThreads, 0, L, inv_diag0, (T)1 / L.h2, st, rhs, e,
-                           scratch, m[0], m[1], c->st[l + 1], (T*)c->rhs[l + 1], A, rt, 0, red_only ? 1 : 0);
+                const bool inl = restrict_inline<T>(c, Nl);
+                T* scratch = (T*)c->e2[l];  // (the fused sweep's second iterate; free between sweeps)
+                if (!inl) {
+                    launch_pdl(c, k_near_residual<T, E>, dim3(near_grid_x(c), 2 * kNearSegs), 256, 0, L, st, rhs, e,
+                               c->near_list[l], c->near_count + 2 * kNearSegs * l, c->near_cap[l], (T)1 / L.h2,
+                               scratch, A, NatMap{});
+                    count(c);
+                }
+                launch_pdl(c, inl ? k_restrict_v<T, E, true> : k_restrict_v<T, E, false>, rgrd, kTileThreads, 0, L,
+                           inv_diag0, (T)1 / L.h2, st, rhs, e, scratch, m[0], m[1], c->st[l + 1],
+                           (T*)c->rhs[l + 1], A, rt, 0, red_only ? 1 : 0);
             }
-            count(c, 2);
+            count(c);
         } else if constexpr (kNative) {
             dim3 cgrid((m[0] + 127) / 128, m[1], m[2]);
             launch_pdl(c, k_residual_restrict<T>, cgrid, blk, 0, L, st, rhs, e, m[0], m[1], c->st[l + 1],
