@@ -162,6 +162,7 @@ size_t field_bytes(const es_params* P, int n, size_t* per_level) {
     b += res_partial_slots(P->dims[0], P->dims[1], 0) * 8 + 64;
     b += (size_t)kFlipCap * 4 + 3 * 256;  // flipped-cell list, its count, the moved flag
     if (colour_split(P)) b += (size_t)4 * kLocalCells * 4 + 1024;  // the local correction's scratch
+    b += tail_code_bytes(P);
     return b;
 }
 
@@ -352,6 +353,7 @@ int es_create_with_allocator(const es_params* params, const es_particle* parts, 
     c->e_scale = 1.0f;
     c->mapped_once = false;
 
+    c->tail_l0 = c->L;
     const long long N = c->g.N;
     const size_t s = mixed(c) ? 4 : 8;
     const int np1 = n > 0 ? n : 1;
@@ -411,6 +413,10 @@ int es_create_with_allocator(const es_params* params, const es_particle* parts, 
     c->local_meta = c->rb0 ? A(1024) : nullptr;
     c->res_valid = false;
     c->res_age = 0;
+    {
+        const size_t b = tail_code_bytes(params);
+        c->tail_codes = b ? (unsigned char*)A(b) : nullptr;
+    }
     c->rb_wpr = (c->g.nx + 63) / 64;
     c->rbmask = c->rb0 ? (uint32_t*)A((size_t)2 * c->g.ny * c->g.nz * c->rb_wpr * 4) : nullptr;
     c->rb_wpr1 = (c->ln[1][0] + 63) / 64;
@@ -430,6 +436,7 @@ int es_create_with_allocator(const es_params* params, const es_particle* parts, 
         delete c;
         return fail(nullptr, ES_ENOMEM, "pinned host allocation failed");
     }
+    tail_setup(c);
     // initial state: fluid at rest, psi = 0, no obstacle cells
     cudaError_t e = cudaSuccess;
     std::vector<DParticle> hp(np1);
@@ -463,6 +470,7 @@ int es_create_with_allocator(const es_params* params, const es_particle* parts, 
     if (e == cudaSuccess) e = launch_init_flags(c);
     if (e == cudaSuccess) e = launch_coarse_states(c);
     if (e == cudaSuccess) e = launch_near_lists(c);
+    if (e == cudaSuccess) e = launch_tail_codes(c);
     if (e == cudaSuccess) e = launch_fill_rest(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
@@ -491,6 +499,7 @@ int es_map_particles(es_ctx* c) {
     ES_CUDA(c, launch_map(c));
     ES_CUDA(c, launch_coarse_states(c));
     ES_CUDA(c, launch_near_lists(c));
+    ES_CUDA(c, launch_tail_codes(c));
     return ES_OK;
 }
 

@@ -163,6 +163,8 @@ struct es_ctx {
     cudaGraphExec_t vgraph[2];          // the V-cycle from zero / warm-started, captured on first use
     unsigned long long vgraph_kernels[2];  // kernel launches in each graph
     bool vgraph_off;                    // capture failed once: launch directly
+    int tail_l0;                        // first level that k_tail takes (L: none)
+    unsigned char* tail_codes;          // its levels' stencil codes, block by block
     cudaEvent_t ev_sync;                // orders the context's stream against a batched launch
     bool bulk_smem_set;                 // the staged half sweep's shared-memory size is set
     int bulk_blocks;                    // resident staged half-sweep blocks per SM; 0 = not queried
@@ -202,6 +204,14 @@ cudaError_t launch_near_lists(es_ctx* c);
 // solver (es_solver.cu)
 cudaError_t launch_outer_residual(es_ctx* c, bool patch = false);  // patch: see k_flip_patch
 cudaError_t launch_vcycle(es_ctx* c, int warm);
+// the coarse levels of the V-cycle in one launch (es_tail.cu)
+size_t tail_code_bytes(const es_params* P);
+void tail_setup(es_ctx* c);
+// its first level's right-hand side and correction colour-split as well: the
+// level above is, and the rows are whole spans
+bool tail_split(const es_ctx* c);
+cudaError_t launch_tail_codes(es_ctx* c);
+cudaError_t launch_tail(es_ctx* c, int warm);
 cudaError_t launch_split_psi(es_ctx* c, const double* src);  // MIXED32: psi = src
 cudaError_t launch_join_psi(es_ctx* c, double* dst);         // MIXED32: dst = psi
 cudaError_t launch_correct(es_ctx* c);
@@ -259,6 +269,13 @@ inline int near_grid_x(const es_ctx* c) {
 // Levels 0 and 1 may be stored colour-split (e and rhs: one colour's cells,
 // then the other's, each in natural order; the states stay natural).
 inline bool split_level(const es_ctx* c, int l) { return (l == 0 && c->rb0) || (l == 1 && c->rb1); }
+
+// Levels of up to this many cells (and what follows them) go to k_tail: in
+// FP32 what the shared memory of 16 blocks holds (64^3: a half sweep 2.3 us
+// there, about 4 launched); in FP64 what 16 SMs' FP64 pipes finish sooner than
+// separate launches over all SMs (32^3: 2.7 us against 5; 64^3 would be bound
+// by the pipes at about 20 us, against 15 launched).
+constexpr long long kTailCells32 = 1 << 18, kTailCells64 = 40 * 1024;
 
 constexpr int kFlipCap = 1 << 16;
 // cells of the local correction's region and ring: at most 16 flipped cells, boxes of radius 9

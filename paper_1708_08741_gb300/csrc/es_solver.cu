@@ -3133,7 +3133,7 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
     const int rb_wpr = l == 0 ? c->rb_wpr : c->rb_wpr1;
     // half the cells of the next level when it is split too (its right-hand
     // side is restricted, and its correction prolonged, in that layout)
-    const int chalf = split && l + 1 < c->L && split_level(c, l + 1)
+    const int chalf = split && l + 1 < c->L && (split_level(c, l + 1) || (l + 1 == c->tail_l0 && tail_split(c)))
                           ? c->ln[l + 1][0] * c->ln[l + 1][1] * c->ln[l + 1][2] / 2
                           : 0;
     const RbMap rb{Nl / 2};
@@ -3406,6 +3406,7 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
 
 template <class T>
 cudaError_t vcycle_level(es_ctx* c, int l, int warm) {
+    if (l == c->tail_l0) return launch_tail(c, warm);
     if constexpr (std::is_same<T, float>::value)
         if (l == 0 && c->P.mg_storage == ES_MG_FP16) return vcycle_impl<float, __half>(c, l, warm);
     return vcycle_impl<T, T>(c, l, warm);

@@ -1,0 +1,43 @@
+"""The coarse levels of the V-cycle in one cluster launch against the same
+levels launched one by one (near_list_cells = 1 keeps every level out of it)."""
+import numpy as np
+import pytest
+
+import paper_1708_08741_gb300 as es
+from paper_1708_08741_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+CASES = [  # dims, periodic, levels, nu1, nu2, omega
+    ((32, 32, 32), (1, 1, 1), 3, 2, 2, 1.0),
+    ((64, 64, 64), (1, 1, 1), 4, 2, 2, 1.0),
+    ((64, 64, 64), (1, 1, 0), 5, 1, 2, 1.0),
+    ((42, 24, 36), (0, 1, 1), 2, 2, 2, 1.0),   # 21 cells a row on the coarser level
+    ((36, 44, 26), (1, 1, 0), 2, 2, 1, 1.0),
+    ((48, 40, 56), (1, 1, 1), 3, 2, 0, 1.0),
+    ((40, 24, 32), (0, 0, 0), 3, 1, 1, 1.3),
+    ((128, 16, 24), (1, 1, 1), 3, 0, 2, 1.0),
+    ((96, 96, 48), (1, 1, 0), 4, 2, 2, 1.0),   # only the coarser levels fit
+    ((24, 20, 28), (1, 1, 1), 1, 2, 2, 1.7),   # one level: sweeps only
+]
+
+
+@pytest.mark.parametrize("precision", [es.ES_FP64, es.ES_MIXED32])
+@pytest.mark.parametrize("dims,periodic,levels,nu1,nu2,omega", CASES)
+def test_cluster_levels_match_separate_launches(precision, dims, periodic, levels, nu1, nu2, omega):
+    """FP64: two V-cycles, the same iteration up to the rounding of a few sums
+    (each below 1e-15 of the iterate, contracted by the cycle): 1e-12.
+    MIXED32: both iterations end below 1e-10 of the first residual, so the
+    potentials differ by at most 2e-10 cond(A) < 2e-10 (12 + kappa^2) / kappa^2 = 3e-8."""
+    wl = W.mixed_box(dims=dims, periodic=periodic, levels=levels, n_spheres=3, radius=3.2)
+    wl.omega, wl.nu1, wl.nu2, wl.coarse_sweeps, wl.max_cycles = omega, nu1, nu2, 12, 300
+    out = []
+    for lists in (0, 1):
+        sim = es.Simulation(wl, precision, overrides=dict(near_list_cells=lists))
+        sim.map_particles()
+        sim.solve(forced_cycles=2 if precision == es.ES_FP64 else -1)
+        out.append(sim.field(es.FIELD_PSI))
+        sim.close()
+    diff = np.linalg.norm(out[0] - out[1]) / np.linalg.norm(out[1])
+    assert np.linalg.norm(out[1]) > 0
+    assert diff < (1e-12 if precision == es.ES_FP64 else 3e-8), diff
