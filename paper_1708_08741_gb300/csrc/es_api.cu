@@ -469,8 +469,9 @@ int es_create_with_allocator(const es_params* params, const es_particle* parts, 
     if (e == cudaSuccess) e = cudaMemsetAsync(c->flip_count, 0, 64, c->stream);
     if (e == cudaSuccess) e = launch_init_flags(c);
     if (e == cudaSuccess) e = launch_coarse_states(c);
-    if (e == cudaSuccess) e = launch_near_lists(c);
+    if (e == cudaSuccess) e = launch_near_lists(c, true);
     if (e == cudaSuccess) e = launch_tail_codes(c);
+    if (e == cudaSuccess) e = launch_particles_f32(c);
     if (e == cudaSuccess) e = launch_fill_rest(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
@@ -498,7 +499,7 @@ int es_map_particles(es_ctx* c) {
     if (!c) return fail(nullptr, ES_EINVAL, "ctx is NULL");
     ES_CUDA(c, launch_map(c));
     ES_CUDA(c, launch_coarse_states(c));
-    ES_CUDA(c, launch_near_lists(c));
+    ES_CUDA(c, launch_near_lists(c, c->np == 0));
     ES_CUDA(c, launch_tail_codes(c));
     return ES_OK;
 }

@@ -68,7 +68,27 @@ __device__ __forceinline__ bool cell_inside(const Grid& g, const DParticle& p, i
 // path for every cell).
 struct BallF {
     float c[3], r2, margin;
-    bool ok;
+    bool ok, ok3[3];
+    // as init, one thread an axis (threads first .. first + 2; the caller
+    // synchronises, and asks all_ok instead of ok)
+    __device__ void init_by_axis(const Grid& g, const double* X, double R, const int* blo, const int* bhi,
+                                 int first = 0) {
+        const int a = (int)threadIdx.x - first;
+        if (a < 0 || a >= 3) return;
+        bool good = true;
+        c[a] = (float)(X[a] - ((double)blo[a] + 0.5));
+        if (g.per[a]) {
+            const double half = 0.5 * (double)gdim(g, a);
+            const double lo = (double)blo[a] + 0.5 - X[a], hi = (double)bhi[a] + 0.5 - X[a];
+            good = lo > -half + 1.0 && hi < half - 1.0;
+        }
+        ok3[a] = good;
+        if (a == 0) {
+            r2 = (float)(R * R);
+            margin = 1e-5f * (r2 + 100.0f);
+        }
+    }
+    __device__ bool all_ok() const { return ok3[0] && ok3[1] && ok3[2]; }
     __device__ void init(const Grid& g, const double* X, double R, const int* blo, const int* bhi) {
         ok = true;
         for (int a = 0; a < 3; a++) {
@@ -86,24 +106,6 @@ struct BallF {
         const float dx = (float)i - c[0], dy = (float)j - c[1], dz = (float)k - c[2];
         return dx * dx + dy * dy + dz * dz;
     }
-};
-
-// The owner field over a box [lo - 1, hi + 1] (the box and a one-cell
-// halo) in shared memory, x fastest; cells beyond a non-periodic face read
-// kOwnerOutside.  Per-sphere kernels read a cell's D3Q19 neighbours from it
-// with fixed offsets instead of wrapping indices per neighbour.
-constexpr int kOwnerOutside = -0x7fffffff;
-constexpr int kOwnerTileMax = 8192;  // ints of shared memory per block
-
-struct OwnerTile {
-    int n[3];  // box extents (the tile is (n + 2)^3)
-    __device__ int tx() const { return n[0] + 2; }
-    __device__ int txy() const { return (n[0] + 2) * (n[1] + 2); }
-    __device__ bool fits(int max_ints = kOwnerTileMax) const { return (n[0] + 2) * (n[1] + 2) * (n[2] + 2) <= max_ints; }
-    // tile index of the box cell with local index (i, j, k)
-    __device__ int at(int i, int j, int k) const { return (i + 1) + tx() * (j + 1) + txy() * (k + 1); }
-    // offset of the D3Q19 neighbour in direction q
-    __device__ int step(int q) const { return cx(q) + tx() * cy(q) + txy() * cz(q); }
 };
 
 // Local indices (i, j, k) of the cells t, t + step, t + 2 step, ... of a box
@@ -137,28 +139,6 @@ struct BoxWalk {
 
 // v in [-n, 2n) into [0, n) (a box never spans more than one period).
 __device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
-
-__device__ __forceinline__ void load_owner_tile(const Grid& g, const int32_t* __restrict__ owner, const int* lo,
-                                                const OwnerTile& T, int* tile) {
-    const int sx = T.n[0] + 2, sy = T.n[1] + 2, n = sx * sy * (T.n[2] + 2);
-    const int dim[3] = {g.nx, g.ny, g.nz};
-    BoxWalk w;
-    w.start(threadIdx.x, blockDim.x, sx, sy);
-    for (int t = threadIdx.x; t < n; t += blockDim.x, w.next()) {
-        int v[3] = {lo[0] - 1 + w.i, lo[1] - 1 + w.j, lo[2] - 1 + w.k};
-        bool out = false;
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            if (v[a] < 0 || v[a] >= dim[a]) {
-                if (!g.per[a])
-                    out = true;
-                else
-                    v[a] = wrap1(v[a], dim[a]);
-            }
-        }
-        tile[t] = out ? kOwnerOutside : owner[lin(g, v[0], v[1], v[2])];
-    }
-}
 
 // Surface velocity u_s = V + Omega x (x_s - X) at the centre of a cell.
 __device__ __forceinline__ void surface_velocity(const Grid& g, const double* X, const double* V,

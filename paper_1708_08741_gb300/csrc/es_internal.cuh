@@ -52,6 +52,13 @@ __host__ __device__ constexpr int cz(int q) {
     return t[q];
 }
 __host__ __device__ constexpr int opp(int q) { return q == 0 ? 0 : (q <= 9 ? q + 9 : q - 9); }
+// the directions with component s along axis a, as bits
+__host__ __device__ constexpr unsigned dir_bits(int a, int s) {
+    unsigned m = 0;
+    for (int q = 1; q < 19; q++)
+        if ((a == 0 ? cx(q) : (a == 1 ? cy(q) : cz(q))) == s) m |= 1u << q;
+    return m;
+}
 __host__ __device__ constexpr double wq(int q) {
     return q == 0 ? 1.0 / 3.0 : ((q <= 3 || (q >= 10 && q <= 12)) ? 1.0 / 18.0 : 1.0 / 36.0);
 }
@@ -200,7 +207,7 @@ namespace es {
 cudaError_t launch_init_flags(es_ctx* c);
 cudaError_t launch_map(es_ctx* c);
 cudaError_t launch_coarse_states(es_ctx* c);
-cudaError_t launch_near_lists(es_ctx* c);
+cudaError_t launch_near_lists(es_ctx* c, bool zero);
 // solver (es_solver.cu)
 cudaError_t launch_outer_residual(es_ctx* c, bool patch = false);  // patch: see k_flip_patch
 cudaError_t launch_vcycle(es_ctx* c, int warm);
@@ -226,6 +233,7 @@ cudaError_t launch_lbm_batch(es_ctx* const* cs, int n);  // es_lbm_step_batch
 cudaError_t launch_forces(es_ctx* c);
 cudaError_t launch_advance(es_ctx* c);
 cudaError_t launch_set_particles(es_ctx* c);  // part (and pbc) from pstage; sigma, mass, inertia kept
+cudaError_t launch_particles_f32(es_ctx* c);
 cudaError_t launch_fill_rest(es_ctx* c);
 cudaError_t launch_get_pdf(es_ctx* c, int which_buf, double* dst);
 cudaError_t launch_set_pdf(es_ctx* c, const double* src);

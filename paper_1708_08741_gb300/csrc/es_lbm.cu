@@ -11,6 +11,7 @@
 //
 // MIXED32 stores f_q - w_q in float: the collision is linear in f, and the
 // weights cancel in every term except the density, which becomes 1 + sum.
+#include <cmath>
 #include <type_traits>
 
 #include "es_device.cuh"
@@ -28,7 +29,8 @@ struct Streams {
 };
 
 // Float copy of the particle state used by the FP32 stream-collide (centre,
-// velocity, angular velocity), so that its moving-wall term needs no FP64.
+// velocity, angular velocity), so that its moving-wall term needs no FP64:
+// made at creation, then kept by the kernels that change the state.
 __global__ void k_particles_f32(int np, const DParticle* __restrict__ part, float* __restrict__ pf) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np) return;
@@ -385,6 +387,7 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 3 : 5) k_lbm(Grid g, con
                                              const int32_t* __restrict__ owner, const DParticle* __restrict__ part,
                                              const float* __restrict__ partf, const C* __restrict__ fb, C ax, C ay,
                                              C az, const Trt<C> R, int slip_faces, FbPsi fp) {
+    pdl_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
     if (x >= g.nx || y >= g.ny) return;
@@ -452,128 +455,308 @@ __global__ void __launch_bounds__(kBatchTileX * kBatchTileY, sizeof(S) == 8 ? 6 
 
 // Momentum exchange (Eq. LBMhydrodynForce): one block per sphere.  Each
 // link x_F -> x_F + e_q into the sphere adds [2 f~_q(x_F) - 2 w_q (c_q . u_s)/c_s^2] c_q
-// and the torque (x_s - X) x dF.  The box around the sphere is scanned 256
-// cells at a time; the links found are compacted into shared memory in
-// (thread, direction) order by a block prefix sum and then summed one link
-// per thread, so the FP64 arithmetic (1/64 rate on GB300) runs on dense
-// warps instead of on divergent lanes.  Fixed order: deterministic.
-constexpr int kForceThreads = 256;
+// and the torque (x_s - X) x dF.  On small grids a few such blocks are all
+// that runs, so their length is what counts, and a sphere's box holds twenty
+// cells for every one with links.  The block therefore
+//  * holds the rows of its box (one-cell halo included) as bit words, one for
+//    the sphere's cells and one for fluid cells, built with a load and two
+//    ballots a row;
+//  * finds the cells with links a whole row at a time by shifts of those
+//    words, and lists them (a prefix sum: in the order of their box index);
+//  * then works on that list only.
+// Boxes whose rows exceed 32 cells (R > 13) look every cell's neighbours up
+// in the fields, 256 cells at a time.  Fixed order: deterministic.
+constexpr int kForceChunk = 256;   // cells of a chunk (see k_forces_f32)
+constexpr int kForceLinks = 4608;  // links held at once: at least one chunk's 18 x 256
+constexpr int kForceSide = 32;     // longest row (halo included) of the bit words
+constexpr int kForceChunks = (kForceSide - 2) * (kForceSide - 2) * (kForceSide - 2) / kForceChunk + 1;
 
-template <class S>
-__global__ void __launch_bounds__(kForceThreads) k_forces(Grid g, const DParticle* __restrict__ part,
-                                                          const int32_t* __restrict__ owner,
-                                                          const uint8_t* __restrict__ flags,
-                                                          const S* __restrict__ src, double Ex, double Ey, double Ez,
-                                                          const double* __restrict__ mapped, double* F, double* T) {
-    __shared__ int s_cell[kForceThreads * 18];
-    __shared__ uint8_t s_q[kForceThreads * 18];
-    __shared__ int s_warp[kForceThreads / 32];
-    __shared__ double sh[32];
-    const int p = blockIdx.x;
-    const DParticle P = part[p];
-    int lo[3], hi[3];
-    for (int a = 0; a < 3; a++) axis_range(g, a, P.x[a], P.x[a], P.R, 1, lo[a], hi[a]);
-    const int sx = hi[0] - lo[0] + 1, sy = hi[1] - lo[1] + 1, sz = hi[2] - lo[2] + 1;
-    // A link runs from a fluid cell to a cell of p within sqrt 2, and p's
-    // cells are those within R of its centre at the last mapping, so only
-    // cells between R - 1 and R + 1.5 of that centre are scanned (FP32
-    // distances; the bounds are far outside their rounding).
-    BallF ball;
-    ball.init(g, mapped + 9 * p, P.R, lo, hi);
-    const float rin = (float)P.R - 1.0f, rout = (float)P.R + 1.5f;
-    const float in2 = rin > 0.0f ? rin * rin : -1.0f, out2 = rout * rout;
-    const int n = sx * sy * sz;
-    const size_t ps = (size_t)g.ps;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int base = 0; base < n; base += kForceThreads) {
-        const int t = base + threadIdx.x;
-        unsigned mask = 0;
-        int c = 0;
-        bool scan = t < n;
-        if (scan && ball.ok) {
-            const float d2 = ball.d2(t % sx, (t / sx) % sy, t / (sx * sy));
-            scan = d2 >= in2 && d2 <= out2;
+// Components of the direction q, from two bits each.
+__host__ __device__ constexpr unsigned long long dir_code(int a) {
+    unsigned long long v = 0;
+    for (int q = 0; q < 19; q++) v |= (unsigned long long)((a == 0 ? cx(q) : (a == 1 ? cy(q) : cz(q))) + 1) << (2 * q);
+    return v;
+}
+__device__ __forceinline__ void dir_of(int q, int (&v)[3]) {
+    constexpr unsigned long long X = dir_code(0), Y = dir_code(1), Z = dir_code(2);
+    v[0] = (int)((X >> (2 * q)) & 3u) - 1;
+    v[1] = (int)((Y >> (2 * q)) & 3u) - 1;
+    v[2] = (int)((Z >> (2 * q)) & 3u) - 1;
+}
+
+// Local indices of a box cell from its linear index (x fastest).  Boxes of up
+// to 2^20 cells divide by a multiplication: t / d = (t ceil(2^32 / d)) >> 32
+// for t d < 2^32.
+struct BoxIndex {
+    int sx, sy, sxy;
+    unsigned mx, mxy;
+    bool quick;
+    __device__ __forceinline__ BoxIndex(int sx_, int sy_, int n) : sx(sx_), sy(sy_), sxy(sx_ * sy_) {
+        quick = n <= (1 << 20) && sxy < (1 << 11) && sx > 1;
+        mx = (unsigned)((0x100000000ULL + sx - 1) / sx);
+        mxy = (unsigned)((0x100000000ULL + sxy - 1) / sxy);
+    }
+    __device__ __forceinline__ void at(int t, int (&v)[3]) const {
+        if (quick) {
+            v[2] = (int)__umulhi((unsigned)t, mxy);
+            const int r = t - v[2] * sxy;
+            v[1] = (int)__umulhi((unsigned)r, mx);
+            v[0] = r - v[1] * sx;
+        } else {
+            v[0] = t % sx;
+            v[1] = (t / sx) % sy;
+            v[2] = t / sxy;
         }
-        if (scan) {
-            const int tx = t % sx, tyz = t / sx;
-            const int x = wrap_coord(lo[0] + tx, g.nx);
-            const int y = wrap_coord(lo[1] + tyz % sy, g.ny);
-            const int z = wrap_coord(lo[2] + tyz / sy, g.nz);
-            c = x + g.nx * (y + g.ny * z);
-            if (flags[c] & F_NEAR19) {
+    }
+};
+
+// Exclusive prefix sum over the block (T threads), and its total.
+template <int T>
+__device__ __forceinline__ int block_excl(int v, int* s_warp, int& total) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int incl = v;
 #pragma unroll
-                for (int q = 1; q < 19; q++) {
-                    long long nb;
-                    if (neighbour(g, x, y, z, cx(q), cy(q), cz(q), nb) && owner[nb] == p) mask |= 1u << q;
-                }
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) s_warp[wid] = incl;
+    __syncthreads();
+    const int w = lane < T / 32 ? s_warp[lane] : 0;
+    total = __reduce_add_sync(0xffffffffu, w);
+    const int before = __reduce_add_sync(0xffffffffu, lane < wid ? w : 0);
+    __syncthreads();
+    return before + incl - v;
+}
+
+// The links of a cell from the fields (boxes too large for the bit words).
+__device__ __noinline__ unsigned force_links_fields(const Grid& g, const int32_t* __restrict__ owner,
+                                                    const uint8_t* __restrict__ flags, int p, int x, int y, int z) {
+    x = wrap_coord(x, g.nx);
+    y = wrap_coord(y, g.ny);
+    z = wrap_coord(z, g.nz);
+    unsigned mask = 0;
+    if (flags[x + g.nx * (y + g.ny * z)] & F_NEAR19) {
+#pragma unroll
+        for (int q = 1; q < 19; q++) {
+            long long nb;
+            if (neighbour(g, x, y, z, cx(q), cy(q), cz(q), nb) && owner[nb] == p) mask |= 1u << q;
+        }
+    }
+    return mask;
+}
+
+// A sphere's box and the list of its cells with links.
+struct ForceBox {
+    int lo[3], n[3];
+    int warp[32];
+};
+
+__device__ __forceinline__ void force_box(const Grid& g, const DParticle& P, ForceBox& B) {
+    if (threadIdx.x < 3) {
+        const int a = threadIdx.x;
+        int l, h;
+        axis_range(g, a, P.x[a], P.x[a], P.R, 1, l, h);
+        B.lo[a] = l;
+        B.n[a] = h - l + 1;
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ bool force_by_rows(const ForceBox& B) {
+    return B.n[0] + 2 <= kForceSide && B.n[1] + 2 <= kForceSide && B.n[2] + 2 <= kForceSide;
+}
+
+// The cells with links in s_near (box index) and s_mask (bit q: a link along
+// q), by rows of bits; own, fluid: a word a row of the box with its halo.
+// Returns their number.
+template <int T>
+__device__ __forceinline__ int force_cells(const Grid& g, const int32_t* __restrict__ owner, int p, ForceBox& B,
+                                           const BoxIndex& bi, unsigned* own, unsigned* fluid, int* s_near,
+                                           unsigned* s_mask) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int sx = B.n[0], sy = B.n[1], sz = B.n[2], ry = sy + 2, nr = ry * (sz + 2);
+    // this lane's column, wrapped once
+    const int gx0 = B.lo[0] - 1 + lane;
+    const bool xin = lane < sx + 2 && (g.per[0] || (gx0 >= 0 && gx0 < g.nx));
+    const int gx = xin ? wrap1(gx0, g.nx) : 0;
+    int jz = wid / ry, jy = wid - jz * ry;
+    for (int r0 = wid; r0 < nr; r0 += 4 * (T / 32)) {
+        int o[4];
+        bool in[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int y0 = B.lo[1] - 1 + jy, z0 = B.lo[2] - 1 + jz;
+            in[u] = xin && r0 + u * (T / 32) < nr && (g.per[1] || (y0 >= 0 && y0 < g.ny)) &&
+                    (g.per[2] || (z0 >= 0 && z0 < g.nz));
+            o[u] = in[u] ? owner[gx + g.nx * (wrap1(y0, g.ny) + g.ny * wrap1(z0, g.nz))] : 0;
+            for (jy += T / 32; jy >= ry; jy -= ry) jz++;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const unsigned wo = __ballot_sync(0xffffffffu, in[u] && o[u] == p);
+            const unsigned wf = __ballot_sync(0xffffffffu, in[u] && o[u] < 0);
+            if (lane == 0 && r0 + u * (T / 32) < nr) {
+                own[r0 + u * (T / 32)] = wo;
+                fluid[r0 + u * (T / 32)] = wf;
             }
         }
-        // block-wide exclusive prefix sum of the link counts
-        const int cnt = __popc(mask);
-        int incl = cnt;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (lane == 31) s_warp[wid] = incl;
-        __syncthreads();
-        int woff = 0, total = 0;
-        for (int w = 0; w < kForceThreads / 32; w++) {
-            if (w < wid) woff += s_warp[w];
-            total += s_warp[w];
-        }
-        int off = woff + incl - cnt;
-        while (mask) {
-            const int q = __ffs(mask) - 1;
-            mask &= mask - 1;
-            s_cell[off] = c;
-            s_q[off] = (uint8_t)q;
-            off++;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < total; i += kForceThreads) {
-            const int cc = s_cell[i], q = s_q[i];
-            const int x = cc % g.nx, yz = cc / g.nx;
-            const int y = yz % g.ny, z = yz / g.ny;
-            int qx = 0, qy = 0, qz = 0;
-#pragma unroll
-            for (int k = 1; k < 19; k++)
-                if (k == q) {
-                    qx = cx(k);
-                    qy = cy(k);
-                    qz = cz(k);
-                }
-            const int bx = wrap_coord(x + qx, g.nx), by = wrap_coord(y + qy, g.ny), bz = wrap_coord(z + qz, g.nz);
-            const double r0 = cell_disp(g, 0, bx, P.x[0]);
-            const double r1 = cell_disp(g, 1, by, P.x[1]);
-            const double r2 = cell_disp(g, 2, bz, P.x[2]);
-            const double us0 = P.v[0] + (P.w[1] * r2 - P.w[2] * r1);
-            const double us1 = P.v[1] + (P.w[2] * r0 - P.w[0] * r2);
-            const double us2 = P.v[2] + (P.w[0] * r1 - P.w[1] * r0);
-            const double cu = qx * us0 + qy * us1 + qz * us2;
-            const double w = (q <= 3 || (q >= 10 && q <= 12)) ? 1.0 / 18.0 : 1.0 / 36.0;
-            const double fq = Store<S>::to_f(q, src[q * ps + cc]);
-            const double m = 2.0 * fq - 6.0 * w * cu;
-            const double d0 = m * qx, d1 = m * qy, d2 = m * qz;
-            acc[0] += d0;
-            acc[1] += d1;
-            acc[2] += d2;
-            acc[3] += r1 * d2 - r2 * d1;
-            acc[4] += r2 * d0 - r0 * d2;
-            acc[5] += r0 * d1 - r1 * d0;
-        }
-        __syncthreads();
     }
-    const double E[3] = {Ex, Ey, Ez};
-    for (int k = 0; k < 6; k++) {
-        double s = block_sum(acc[k], sh);
-        if (threadIdx.x == 0) {
-            if (k < 3)
-                F[3 * p + k] = s + P.qeff * E[k];  // F_C = q E_ext (Sec. 5.6)
-            else
-                T[3 * p + k - 3] = s;
+    __syncthreads();
+    // rows of the box: cells with links, listed in the order of the box index
+    const int rows = sy * sz, per = (rows + T - 1) / T;
+    const unsigned inside = sx >= 31 ? 0x7ffffffeu : (((1u << sx) - 1u) << 1);
+    auto any_of = [&](int r) {
+        const int k = r / sy, at = (r - k * sy) + 1 + ry * (k + 1);
+        unsigned m = 0;
+        auto three = [&](int d) {
+            const unsigned w = own[at + d];
+            return w | (w << 1) | (w >> 1);
+        };
+        m = (own[at] << 1) | (own[at] >> 1);
+        m |= three(-1) | three(1) | three(-ry) | three(ry);
+        m |= own[at - 1 - ry] | own[at + 1 - ry] | own[at - 1 + ry] | own[at + 1 + ry];
+        return m & fluid[at] & inside;
+    };
+    int cnt = 0;
+    for (int u = 0; u < per; u++) {
+        const int r = (int)threadIdx.x * per + u;
+        if (r < rows) cnt += __popc(any_of(r));
+    }
+    int total;
+    int at = block_excl<T>(cnt, B.warp, total);
+    for (int u = 0; u < per; u++) {
+        const int r = (int)threadIdx.x * per + u;
+        if (r < rows)
+            for (unsigned m = any_of(r); m; m &= m - 1u) s_near[at++] = r * sx + __ffs(m) - 2;  // (bit i + 1: cell i)
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < total; c += T) {
+        int v[3];
+        bi.at(s_near[c], v);
+        const int w0 = v[1] + 1 + ry * (v[2] + 1), b = v[0] + 1;
+        unsigned m = 0;
+#pragma unroll
+        for (int q = 1; q < 19; q++) m |= ((own[w0 + cy(q) + ry * cz(q)] >> (b + cx(q))) & 1u) << q;
+        s_mask[c] = m;
+    }
+    __syncthreads();
+    return total;
+}
+
+// The cells with links among the box's cells t0 .. t0 + 255, from the fields.
+template <int T>
+__device__ __forceinline__ int force_cells_fields(const Grid& g, const int32_t* __restrict__ owner,
+                                                  const uint8_t* __restrict__ flags, int p, ForceBox& B,
+                                                  const BoxIndex& bi, int t0, int n, int* s_near, unsigned* s_mask) {
+    const int t = t0 + (int)threadIdx.x;
+    unsigned m = 0;
+    if (threadIdx.x < kForceChunk && t < n) {
+        int v[3];
+        bi.at(t, v);
+        m = force_links_fields(g, owner, flags, p, B.lo[0] + v[0], B.lo[1] + v[1], B.lo[2] + v[2]);
+    }
+    int total;
+    const int at = block_excl<T>(m ? 1 : 0, B.warp, total);
+    if (m) {
+        s_near[at] = t;
+        s_mask[at] = m;
+    }
+    __syncthreads();
+    return total;
+}
+
+// FP64 form.  The FP64 pipe (2 operations a clock and SM) bounds it, so a
+// cell's links share what they can: u_s . c_q = u_F . c_q with u_F = V + W x
+// r_F, since x_s = x_F + c_q and (W x c_q) . c_q = 0, and the torques add up to
+// r_F x sum m_q c_q, since c_q x c_q = 0; about five operations a link instead
+// of 35.  (A sphere R = 4 / 64 spheres R = 6: 62 / 133 us before, 32 / 48
+// now.)
+template <int T>
+__global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __restrict__ part,
+                                                 const int32_t* __restrict__ owner, const uint8_t* __restrict__ flags,
+                                                 const double* __restrict__ src, double Ex, double Ey, double Ez,
+                                                 double* F, double* T_out, int cells) {
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ ForceBox B;
+    __shared__ double sh[6][32];
+    unsigned* own = (unsigned*)dyn;
+    unsigned* fluid = own + kForceSide * kForceSide;
+    int* s_near = (int*)(fluid + kForceSide * kForceSide);
+    unsigned* s_mask = (unsigned*)(s_near + cells);
+    const int p = blockIdx.x;
+    pdl_wait();
+    force_box(g, part[p], B);
+    const int n = B.n[0] * B.n[1] * B.n[2];
+    const BoxIndex bi(B.n[0], B.n[1], n);
+    const DParticle& P = part[p];
+    const double X[3] = {P.x[0], P.x[1], P.x[2]}, V[3] = {P.v[0], P.v[1], P.v[2]}, Wv[3] = {P.w[0], P.w[1], P.w[2]};
+    const size_t ps = (size_t)g.ps;
+    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    auto consume = [&](int total) {
+        for (int i = threadIdx.x; i < total; i += T) {
+            int v[3];
+            bi.at(s_near[i], v);
+            const unsigned m = s_mask[i];
+            const int x = wrap_coord(B.lo[0] + v[0], g.nx), y = wrap_coord(B.lo[1] + v[1], g.ny),
+                      z = wrap_coord(B.lo[2] + v[2], g.nz);
+            const int c = x + g.nx * (y + g.ny * z);
+            const double r0 = cell_disp(g, 0, x, X[0]), r1 = cell_disp(g, 1, y, X[1]), r2 = cell_disp(g, 2, z, X[2]);
+            const double u[3] = {V[0] + (Wv[1] * r2 - Wv[2] * r1), V[1] + (Wv[2] * r0 - Wv[0] * r2),
+                                 V[2] + (Wv[0] * r1 - Wv[1] * r0)};
+            double d[3] = {0.0, 0.0, 0.0};
+            // six directions' populations in flight at a time
+#pragma unroll
+            for (int q0 = 1; q0 < 19; q0 += 6) {
+                double f[6];
+#pragma unroll
+                for (int j = 0; j < 6; j++) f[j] = ((m >> (q0 + j)) & 1u) ? src[(q0 + j) * ps + c] : 0.0;
+#pragma unroll
+                for (int j = 0; j < 6; j++) {
+                    const int q = q0 + j;
+                    if (!((m >> q) & 1u)) continue;
+                    double cu = 0.0;
+                    if (cx(q)) cu = cx(q) > 0 ? u[0] : -u[0];
+                    if (cy(q)) cu = cx(q) ? (cy(q) > 0 ? cu + u[1] : cu - u[1]) : (cy(q) > 0 ? u[1] : -u[1]);
+                    if (cz(q)) cu = cx(q) || cy(q) ? (cz(q) > 0 ? cu + u[2] : cu - u[2]) : (cz(q) > 0 ? u[2] : -u[2]);
+                    const double mq = 2.0 * f[j] - 6.0 * wq(q) * cu;
+                    if (cx(q)) d[0] += cx(q) > 0 ? mq : -mq;
+                    if (cy(q)) d[1] += cy(q) > 0 ? mq : -mq;
+                    if (cz(q)) d[2] += cz(q) > 0 ? mq : -mq;
+                }
+            }
+            acc[0] += d[0];
+            acc[1] += d[1];
+            acc[2] += d[2];
+            acc[3] += r1 * d[2] - r2 * d[1];
+            acc[4] += r2 * d[0] - r0 * d[2];
+            acc[5] += r0 * d[1] - r1 * d[0];
         }
+    };
+    if (force_by_rows(B)) {
+        consume(force_cells<T>(g, owner, p, B, bi, own, fluid, s_near, s_mask));
+    } else {
+        for (int t0 = 0; t0 < n; t0 += kForceChunk) {
+            consume(force_cells_fields<T>(g, owner, flags, p, B, bi, t0, n, s_near, s_mask));
+            __syncthreads();
+        }
+    }
+    // block sums in a fixed order: warps, then one thread per component
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
+        if ((threadIdx.x & 31) == 0) sh[k][threadIdx.x >> 5] = acc[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        const int k = threadIdx.x;
+        double s = 0.0;
+        for (int w = 0; w < T / 32; w++) s += sh[k][w];
+        const double E[3] = {Ex, Ey, Ez};
+        if (k < 3)
+            F[3 * p + k] = s + P.qeff * E[k];  // F_C = q E_ext (Sec. 5.6)
+        else
+            T_out[3 * p + k - 3] = s;
     }
 }
 
@@ -582,248 +765,258 @@ __global__ void __launch_bounds__(kForceThreads) k_forces(Grid g, const DParticl
 // no FP64 arithmetic runs per link (GB300's FP64 rate is a small fraction
 // of its FP32 rate).  With f~ = w_q + dev the link term is
 // [2 w_q + m'] c_q, m' = 2 dev - 6 w_q (c_q . u_s):
-//  * the m' part (small) is summed in FP32 per thread, with lever arms in
-//    FP32, and over the block in float-float;
-//  * the 2 w_q part is summed exactly: per direction, the number of links
-//    and the integer sums of the surface cells' coordinates (relative to the
-//    box origin, unwrapped), from which thread 0 forms sum 2 w_q c_q and
-//    sum 2 w_q (x_s - X) x c_q in FP64 at the end.
-// Near-surface scan as in k_forces (cells between R - 1 and R + 1.5 of the
-// centre at the last mapping).  Deterministic: fixed summation order.
-template <class S>
-__global__ void __launch_bounds__(kForceThreads) k_forces_f32(Grid g, const DParticle* __restrict__ part,
-                                                              const int32_t* __restrict__ owner,
-                                                              const uint8_t* __restrict__ flags,
-                                                              const S* __restrict__ src, double Ex, double Ey,
-                                                              double Ez, const double* __restrict__ mapped,
-                                                              double* F, double* T) {
+//  * the m' part (small) is formed by all threads, one link each, with lever
+//    arms in FP32, then summed in FP32 by 256 of them -- link i of a chunk of
+//    256 box cells by thread i mod 256, chunk after chunk -- and over the block
+//    in float-float;
+//  * the 2 w_q part is summed exactly in integers: with S = sum of 18 x 2 w_q
+//    c_q over a cell's links, sum S and sum rel x S (rel: the cell's
+//    coordinates relative to the box, minimum image), from which sum 2 w_q c_q
+//    and sum 2 w_q (x_s - X) x c_q follow in FP64 at the end (c_q x c_q = 0).
+// (2,880 spheres R = 5 / 64 spheres R = 6: 277 / 102 us before, 216 / 25
+// now: a sphere R = 6 did not fit the owner tile and looked every cell's
+// neighbours up one by one, and every link made four shared-memory atomics.)
+template <class S, int T>
+__global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
+    k_forces_f32(Grid g, const DParticle* __restrict__ part, const int32_t* __restrict__ owner,
+                 const uint8_t* __restrict__ flags, const S* __restrict__ src, double Ex, double Ey, double Ez,
+                 double* F, double* T_out, int cells) {
     using St = Store<S>;
-    constexpr int kTile = 4096;  // (with the link lists below, within 48 KB of static shared memory)
-    __shared__ int tile[kTile];
-    __shared__ int s_cell[kForceThreads * 18];
-    __shared__ uint8_t s_q[kForceThreads * 18];
-    __shared__ int s_warp[kForceThreads / 32];
-    __shared__ int s_lo[3], s_n[3];
-    __shared__ BallF s_ball;
-    __shared__ float s_X[3], s_V[3], s_W[3], s_band[2];
-    __shared__ int s_cnt[19], s_sum[19][3];
-    __shared__ float s_red[kForceThreads / 32][12];
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ ForceBox B;
+    __shared__ float s_X[3], s_V[3], s_W[3];
+    __shared__ double s_off[3], s_qeff;
+    __shared__ int s_int[6], s_first[kForceChunks], s_count[kForceChunks];
+    __shared__ float s_red[kForceChunk / 32][12];
+    unsigned* own = (unsigned*)dyn;
+    unsigned* fluid = own + kForceSide * kForceSide;
+    int* s_near = (int*)(fluid + kForceSide * kForceSide);
+    unsigned* s_mask = (unsigned*)(s_near + cells);
+    int* s_link = (int*)(s_mask + cells);         // cell of the list | q << 16
+    float* s_m = (float*)(s_link + kForceLinks);  // its m'
     const int p = blockIdx.x;
-    if (threadIdx.x == 0) {
+    pdl_wait();
+    force_box(g, part[p], B);
+    if (threadIdx.x < 3) {
         const DParticle& P = part[p];
-        int lo[3], hi[3];
-        for (int a = 0; a < 3; a++) {
-            axis_range(g, a, P.x[a], P.x[a], P.R, 1, lo[a], hi[a]);
-            s_lo[a] = lo[a];
-            s_n[a] = hi[a] - lo[a] + 1;
-            // centre relative to the box origin's cell centre: r = i - s_X for
-            // the cell with local index i (exact to FP32 rounding of s_X)
-            s_X[a] = (float)(P.x[a] - ((double)lo[a] + 0.5));
-            s_V[a] = (float)P.v[a];
-            s_W[a] = (float)P.w[a];
-        }
-        s_ball.init(g, mapped + 9 * p, P.R, lo, hi);
-        const float rin = (float)P.R - 1.0f, rout = (float)P.R + 1.5f;
-        s_band[0] = rin > 0.0f ? rin * rin : -1.0f;
-        s_band[1] = rout * rout;
+        const int a = threadIdx.x;
+        // centre relative to the box origin's cell centre: r = i - s_X for
+        // the cell with local index i (exact to FP32 rounding of s_X)
+        const double off = (double)B.lo[a] + 0.5 - P.x[a];
+        s_off[a] = off;
+        s_X[a] = (float)(-off);
+        s_V[a] = (float)P.v[a];
+        s_W[a] = (float)P.w[a];
     }
-    if (threadIdx.x < 19) {
-        s_cnt[threadIdx.x] = 0;
-        s_sum[threadIdx.x][0] = s_sum[threadIdx.x][1] = s_sum[threadIdx.x][2] = 0;
-    }
+    if (threadIdx.x == 32) s_qeff = part[p].qeff;
+    if (threadIdx.x < 6) s_int[threadIdx.x] = 0;
     __syncthreads();
-    const int sx = s_n[0], sy = s_n[1], sz = s_n[2];
-    const int n = sx * sy * sz;
-    const BallF ball = s_ball;
-    const OwnerTile TL{{sx, sy, sz}};
-    const bool use_tile = TL.fits(kTile);
-    if (use_tile) {
-        const int lo3[3] = {s_lo[0], s_lo[1], s_lo[2]};
-        load_owner_tile(g, owner, lo3, TL, tile);
-        __syncthreads();
-    }
-    const float in2 = s_band[0], out2 = s_band[1];
+    const int n = B.n[0] * B.n[1] * B.n[2];
+    const BoxIndex bi(B.n[0], B.n[1], n);
     const float Xr[3] = {s_X[0], s_X[1], s_X[2]}, V[3] = {s_V[0], s_V[1], s_V[2]}, W[3] = {s_W[0], s_W[1], s_W[2]};
-    const int L[3] = {g.nx, g.ny, g.nz};
     const size_t ps = (size_t)g.ps;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    float acc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    BoxWalk bw;
-    bw.start(threadIdx.x, kForceThreads, sx, sy);
-    for (int base = 0; base < n; base += kForceThreads, bw.next()) {
-        const int t = base + threadIdx.x;
-        unsigned mask = 0;
-        int c = 0;
-        bool scan = t < n;
-        if (scan && ball.ok) {
-            const float d2 = ball.d2(bw.i, bw.j, bw.k);
-            scan = d2 >= in2 && d2 <= out2;
+    // a box index's minimum image (a periodic box may span the whole axis)
+    auto image = [&](int u, int a) {
+        const int L = a == 0 ? g.nx : (a == 1 ? g.ny : g.nz);
+        if (g.per[a]) {
+            if ((float)u - Xr[a] > 0.5f * (float)L) u -= L;
+            if ((float)u - Xr[a] < -0.5f * (float)L) u += L;
         }
-        if (scan) {
-            if (use_tile) {
-                const int ti = TL.at(bw.i, bw.j, bw.k);
-                if (tile[ti] < 0 && tile[ti] != kOwnerOutside) {
-#pragma unroll
-                    for (int q = 1; q < 19; q++)
-                        if (tile[ti + TL.step(q)] == p) mask |= 1u << q;
-                }
+        return u;
+    };
+    float acc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    int isum[6] = {0, 0, 0, 0, 0, 0};
+    // The listed cells' links: chunk of a cell: (box index - t0) / 256, nch chunks.
+    auto consume = [&](int total, int t0, int nch) {
+        for (int c = threadIdx.x; c < nch; c += T) s_count[c] = 0;
+        __syncthreads();
+        const int per = (total + T - 1) / T;
+        int cnt = 0;
+        for (int u = 0; u < per; u++) {
+            const int c = (int)threadIdx.x * per + u;
+            if (c >= total) break;
+            const unsigned m = s_mask[c];
+            const int t = s_near[c];
+            cnt += __popc(m);
+            atomicAdd(&s_count[(t - t0) / kForceChunk], __popc(m));
+            // S = sum of 18 x 2 w_q c_q: 2 for an axis, 1 for a diagonal
+            constexpr unsigned xp = dir_bits(0, 1), xm = dir_bits(0, -1), yp = dir_bits(1, 1), ym = dir_bits(1, -1),
+                               zp = dir_bits(2, 1), zm = dir_bits(2, -1);
+            auto axis = [&](int a) { return (int)((m >> (1 + a)) & 1u) - (int)((m >> (10 + a)) & 1u); };
+            const int S0 = __popc(m & xp) - __popc(m & xm) + axis(0), S1 = __popc(m & yp) - __popc(m & ym) + axis(1),
+                      S2 = __popc(m & zp) - __popc(m & zm) + axis(2);
+            int v[3];
+            bi.at(t, v);
+            const int u0 = image(v[0], 0), u1 = image(v[1], 1), u2 = image(v[2], 2);
+            isum[0] += S0;
+            isum[1] += S1;
+            isum[2] += S2;
+            isum[3] += u1 * S2 - u2 * S1;
+            isum[4] += u2 * S0 - u0 * S2;
+            isum[5] += u0 * S1 - u1 * S0;
+        }
+        int nlinks;
+        const int base = block_excl<T>(cnt, B.warp, nlinks);
+        {
+            int at = base;
+            for (int u = 0; u < per; u++) {
+                const int c = (int)threadIdx.x * per + u;
+                if (c >= total) break;
+                const int ch = (s_near[c] - t0) / kForceChunk;
+                if (c == 0 || (s_near[c - 1] - t0) / kForceChunk != ch) s_first[ch] = at;
+                at += __popc(s_mask[c]);
+            }
+        }
+        __syncthreads();
+        // as many chunks at a time as the link list holds (nearly always all)
+        for (int k0 = 0, done = 0; k0 < nch;) {
+            int k1 = k0, held = 0;
+            if (nlinks - done <= kForceLinks) {
+                k1 = nch;
+                held = nlinks - done;
             } else {
-                const int x = wrap1(s_lo[0] + bw.i, g.nx);
-                const int y = wrap1(s_lo[1] + bw.j, g.ny);
-                const int z = wrap1(s_lo[2] + bw.k, g.nz);
-                const int cg = x + g.nx * (y + g.ny * z);
-                if (flags[cg] & F_NEAR19) {
+                while (k1 < nch && held + s_count[k1] <= kForceLinks) held += s_count[k1++];
+            }
+            int at = base;
+            for (int u = 0; u < per; u++) {
+                const int c = (int)threadIdx.x * per + u;
+                if (c >= total) break;
+                const int ch = (s_near[c] - t0) / kForceChunk;
+                unsigned m = s_mask[c];
+                if (ch < k0 || ch >= k1) {
+                    at += __popc(m);
+                    continue;
+                }
+                for (; m; m &= m - 1u) s_link[at++ - done] = c | ((__ffs(m) - 1) << 16);
+            }
+            __syncthreads();
+            for (int i = threadIdx.x; i < held; i += T) {
+                const int link = s_link[i], q = link >> 16;
+                int li[3], qv[3];
+                bi.at(s_near[link & 0xFFFF], li);
+                dir_of(q, qv);
+                const int cc = wrap1(B.lo[0] + li[0], g.nx) +
+                               g.nx * (wrap1(B.lo[1] + li[1], g.ny) + g.ny * wrap1(B.lo[2] + li[2], g.nz));
+                const S f = src[q * ps + cc];
+                float r[3];
 #pragma unroll
-                    for (int q = 1; q < 19; q++) {
-                        long long nb;
-                        if (neighbour(g, x, y, z, cx(q), cy(q), cz(q), nb) && owner[nb] == p) mask |= 1u << q;
+                for (int a = 0; a < 3; a++) r[a] = (float)image(li[a] + qv[a], a) - Xr[a];
+                const float us0 = V[0] + (W[1] * r[2] - W[2] * r[1]);
+                const float us1 = V[1] + (W[2] * r[0] - W[0] * r[2]);
+                const float us2 = V[2] + (W[0] * r[1] - W[1] * r[0]);
+                const float cu = (float)qv[0] * us0 + (float)qv[1] * us1 + (float)qv[2] * us2;
+                const float w = (q <= 3 || (q >= 10 && q <= 12)) ? 1.0f / 18.0f : 1.0f / 36.0f;
+                float dev;  // f~ - w_q
+                if constexpr (std::is_same<S, __half>::value)
+                    dev = __half2float(f) * (w * (float)(1.0 / kHalfScale));  // (Store<__half>::ld in FP32)
+                else
+                    dev = St::ld(q, f);
+                s_m[i] = 2.0f * dev - 6.0f * w * cu;
+            }
+            __syncthreads();
+            if (threadIdx.x < kForceChunk)
+                for (int ch = k0; ch < k1; ch++) {
+                    const int nl = s_count[ch];
+                    if (nl == 0) continue;
+                    const int first = s_first[ch] - done;
+                    for (int i = threadIdx.x; i < nl; i += kForceChunk) {
+                        const int link = s_link[first + i];
+                        const float m = s_m[first + i];
+                        int li[3], qv[3];
+                        bi.at(s_near[link & 0xFFFF], li);
+                        dir_of(link >> 16, qv);
+                        float r[3];
+#pragma unroll
+                        for (int a = 0; a < 3; a++) r[a] = (float)image(li[a] + qv[a], a) - Xr[a];
+                        const float d0 = m * (float)qv[0], d1 = m * (float)qv[1], d2 = m * (float)qv[2];
+                        acc[0] += d0;
+                        acc[1] += d1;
+                        acc[2] += d2;
+                        acc[3] += r[1] * d2 - r[2] * d1;
+                        acc[4] += r[2] * d0 - r[0] * d2;
+                        acc[5] += r[0] * d1 - r[1] * d0;
                     }
                 }
-            }
-            c = bw.i | (bw.j << 10) | (bw.k << 20);  // local indices of x_F (a box is < 1024 cells a side)
+            __syncthreads();
+            done += held;
+            k0 = k1;
         }
-        const int cnt = __popc(mask);
-        int incl = cnt;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (lane == 31) s_warp[wid] = incl;
-        __syncthreads();
-        int woff = 0, total = 0;
-        for (int w = 0; w < kForceThreads / 32; w++) {
-            if (w < wid) woff += s_warp[w];
-            total += s_warp[w];
-        }
-        int off = woff + incl - cnt;
-        while (mask) {
-            const int q = __ffs(mask) - 1;
-            mask &= mask - 1;
-            s_cell[off] = c;
-            s_q[off] = (uint8_t)q;
-            off++;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < total; i += kForceThreads) {
-            const int pk = s_cell[i], q = s_q[i];
-            const int li[3] = {pk & 1023, (pk >> 10) & 1023, pk >> 20};
-            const int cc = wrap1(s_lo[0] + li[0], g.nx) +
-                           g.nx * (wrap1(s_lo[1] + li[1], g.ny) + g.ny * wrap1(s_lo[2] + li[2], g.nz));
-            int qv[3] = {0, 0, 0};
-#pragma unroll
-            for (int k = 1; k < 19; k++)
-                if (k == q) {
-                    qv[0] = cx(k);
-                    qv[1] = cy(k);
-                    qv[2] = cz(k);
-                }
-            // surface cell x_s = x_F + c_q in the box's unwrapped frame
-            // (minimum image where a periodic box spans the whole axis)
-            int rel[3];
-            float r[3];
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                int u = li[a] + qv[a];
-                if (g.per[a]) {
-                    if ((float)u - Xr[a] > 0.5f * (float)L[a]) u -= L[a];
-                    if ((float)u - Xr[a] < -0.5f * (float)L[a]) u += L[a];
-                }
-                rel[a] = u;
-                r[a] = (float)u - Xr[a];
-            }
-            const float us0 = V[0] + (W[1] * r[2] - W[2] * r[1]);
-            const float us1 = V[1] + (W[2] * r[0] - W[0] * r[2]);
-            const float us2 = V[2] + (W[0] * r[1] - W[1] * r[0]);
-            const float cu = (float)qv[0] * us0 + (float)qv[1] * us1 + (float)qv[2] * us2;
-            const float w = (q <= 3 || (q >= 10 && q <= 12)) ? 1.0f / 18.0f : 1.0f / 36.0f;
-            float dev;  // f~ - w_q
-            if constexpr (std::is_same<S, __half>::value)
-                dev = __half2float(src[q * ps + cc]) * (w * (float)(1.0 / kHalfScale));  // (Store<__half>::ld in FP32)
-            else
-                dev = St::ld(q, src[q * ps + cc]);
-            const float m = 2.0f * dev - 6.0f * w * cu;
-            const float d0 = m * (float)qv[0], d1 = m * (float)qv[1], d2 = m * (float)qv[2];
-            acc[0] += d0;
-            acc[1] += d1;
-            acc[2] += d2;
-            acc[3] += r[1] * d2 - r[2] * d1;
-            acc[4] += r[2] * d0 - r[0] * d2;
-            acc[5] += r[0] * d1 - r[1] * d0;
-            atomicAdd(&s_cnt[q], 1);
-            atomicAdd(&s_sum[q][0], rel[0]);
-            atomicAdd(&s_sum[q][1], rel[1]);
-            atomicAdd(&s_sum[q][2], rel[2]);
-        }
-        __syncthreads();
+    };
+    if (force_by_rows(B)) {
+        const int total = force_cells<T>(g, owner, p, B, bi, own, fluid, s_near, s_mask);
+        consume(total, 0, (n + kForceChunk - 1) / kForceChunk);
+    } else {
+        for (int t0 = 0; t0 < n; t0 += kForceChunk)
+            consume(force_cells_fields<T>(g, owner, flags, p, B, bi, t0, n, s_near, s_mask), t0, 1);
     }
     // block sum of the six FP32 partials in float-float (fixed order)
-    ff v[6];
+    if (threadIdx.x < kForceChunk) {
+        ff v[6];
 #pragma unroll
-    for (int k = 0; k < 6; k++) v[k] = {acc[k], 0.0f};
-    for (int o = 16; o > 0; o >>= 1)
+        for (int k = 0; k < 6; k++) v[k] = {acc[k], 0.0f};
+        for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-        for (int k = 0; k < 6; k++) {
-            const ff u = {__shfl_down_sync(0xffffffffu, v[k].hi, o), __shfl_down_sync(0xffffffffu, v[k].lo, o)};
-            v[k] = ff_add(v[k], u);
-        }
-    if (lane == 0)
+            for (int k = 0; k < 6; k++) {
+                const ff u = {__shfl_down_sync(0xffffffffu, v[k].hi, o), __shfl_down_sync(0xffffffffu, v[k].lo, o)};
+                v[k] = ff_add(v[k], u);
+            }
+        if ((threadIdx.x & 31) == 0)
 #pragma unroll
-        for (int k = 0; k < 6; k++) {
-            s_red[wid][2 * k] = v[k].hi;
-            s_red[wid][2 * k + 1] = v[k].lo;
-        }
+            for (int k = 0; k < 6; k++) {
+                s_red[threadIdx.x >> 5][2 * k] = v[k].hi;
+                s_red[threadIdx.x >> 5][2 * k + 1] = v[k].lo;
+            }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const int v = __reduce_add_sync(0xffffffffu, isum[k]);
+        if ((threadIdx.x & 31) == 0 && v != 0) atomicAdd(&s_int[k], v);
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const DParticle& P = part[p];
-        double sum[6];
-        for (int k = 0; k < 6; k++) {
-            ff a = {s_red[0][2 * k], s_red[0][2 * k + 1]};
-            for (int w = 1; w < kForceThreads / 32; w++) a = ff_add(a, ff{s_red[w][2 * k], s_red[w][2 * k + 1]});
-            sum[k] = (double)a.hi + (double)a.lo;
-        }
-        // the 2 w_q part: sum 2 w_q c_q and sum 2 w_q (x_s - X) x c_q, with
-        // x_s - X = rel + (lo + 1/2 - X)
-        double off[3];
-        for (int a = 0; a < 3; a++) off[a] = (double)s_lo[a] + 0.5 - P.x[a];
-        for (int q = 1; q < 19; q++) {
-            if (s_cnt[q] == 0) continue;
-            const double w2 = 2.0 * ((q <= 3 || (q >= 10 && q <= 12)) ? 1.0 / 18.0 : 1.0 / 36.0);
-            const double nq = (double)s_cnt[q];
-            const double c3[3] = {(double)cx(q), (double)cy(q), (double)cz(q)};
-            double rs[3];  // sum over the links of x_s - X
-            for (int a = 0; a < 3; a++) rs[a] = (double)s_sum[q][a] + nq * off[a];
-            sum[0] += w2 * nq * c3[0];
-            sum[1] += w2 * nq * c3[1];
-            sum[2] += w2 * nq * c3[2];
-            sum[3] += w2 * (rs[1] * c3[2] - rs[2] * c3[1]);
-            sum[4] += w2 * (rs[2] * c3[0] - rs[0] * c3[2]);
-            sum[5] += w2 * (rs[0] * c3[1] - rs[1] * c3[0]);
-        }
-        const double E[3] = {Ex, Ey, Ez};
-        for (int k = 0; k < 3; k++) {
-            F[3 * p + k] = sum[k] + P.qeff * E[k];  // F_C = q E_ext (Sec. 5.6)
-            T[3 * p + k] = sum[3 + k];
+    if (threadIdx.x < 6) {
+        const int k = threadIdx.x;
+        ff a = {s_red[0][2 * k], s_red[0][2 * k + 1]};
+        for (int w = 1; w < kForceChunk / 32; w++) a = ff_add(a, ff{s_red[w][2 * k], s_red[w][2 * k + 1]});
+        double sum = (double)a.hi + (double)a.lo;
+        if (k < 3) {
+            const double E[3] = {Ex, Ey, Ez};
+            sum += (double)s_int[k] * (1.0 / 18.0);
+            F[3 * p + k] = sum + s_qeff * E[k];  // F_C = q E_ext (Sec. 5.6)
+        } else {
+            // x_F - X = rel + (lo + 1/2 - X)
+            const int c = k - 3, d = (c + 1) % 3, e = (c + 2) % 3;
+            sum += ((double)s_int[k] + (s_off[d] * (double)s_int[e] - s_off[e] * (double)s_int[d])) * (1.0 / 18.0);
+            T_out[3 * p + c] = sum;
         }
     }
 }
 
 // Semi-implicit Euler, dt = 1 (the integrator is a reading: the paper
 // leaves it to the pe engine).
+// A thread an axis of a sphere (its chain of FP64 operations is the kernel's
+// time).  Keeps the float copy that the reduced forms' stream-collide reads.
 __global__ void k_advance(int np, DParticle* part, const double* F, const double* T, int px, int py, int pz,
-                          double Lx, double Ly, double Lz) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
+                          double Lx, double Ly, double Lz, float* __restrict__ pf) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    if (t >= 3 * np) return;
+    const int p = t / 3, a = t - 3 * p;
     DParticle& P = part[p];
-    const int per[3] = {px, py, pz};
-    const double L[3] = {Lx, Ly, Lz};
-    for (int a = 0; a < 3; a++) {
-        P.v[a] += F[3 * p + a] / P.mass;
-        P.x[a] += P.v[a];
-        P.w[a] += T[3 * p + a] / P.inertia;
-        if (per[a]) {
-            if (P.x[a] >= L[a]) P.x[a] -= L[a];
-            if (P.x[a] < 0.0) P.x[a] += L[a];
-        }
+    const bool per = a == 0 ? px : (a == 1 ? py : pz);
+    const double L = a == 0 ? Lx : (a == 1 ? Ly : Lz);
+    const double w = P.w[a] + T[t] / P.inertia, v = P.v[a] + F[t] / P.mass;
+    double x = P.x[a] + v;
+    if (per) {
+        if (x >= L) x -= L;
+        if (x < 0.0) x += L;
+    }
+    P.v[a] = v;
+    P.x[a] = x;
+    P.w[a] = w;
+    if (pf) {
+        pf[12 * p + a] = (float)x;
+        pf[12 * p + 3 + a] = (float)v;
+        pf[12 * p + 6 + a] = (float)w;
     }
 }
 
@@ -1074,10 +1267,6 @@ cudaError_t launch_lbm(es_ctx* c) {
     const dim3 blk = lbm_block(c);
     const dim3 grd((g.nx + blk.x - 1) / blk.x, (g.ny + blk.y - 1) / blk.y, g.nz);
     const double* a = c->P.accel;
-    if (mixed(c) && c->np > 0) {
-        k_particles_f32<<<(c->np + 127) / 128, 128, 0, c->stream>>>(c->np, c->part, c->partf);
-        count(c);
-    }
     // the body force evaluated in the stream-collide: first the stored values
     // of the cells next to obstacles and walls
     const bool lazy = c->fb_lazy;
@@ -1094,9 +1283,10 @@ cudaError_t launch_lbm(es_ctx* c) {
         // or psi (4) and the flag byte in
         ProfScope ps(c, "lbm", -1, (double)g.N * (38.0 * sizeof(S) + (lazy ? 4.0 : 3.0 * sizeof(C)) + 1.0));
         auto run = [&](auto slip, auto fused) {
-            k_lbm<S, decltype(slip)::value, decltype(fused)::value><<<grd, blk, 0, c->stream>>>(
-                g, streams<S>(c), c->flags, c->owner, c->part, c->partf, (const C*)c->fb, (C)a[0], (C)a[1], (C)a[2],
-                trt<C>(c->lambda_e, c->lambda_o), c->slip, fp);
+            launch_pdl(c, k_lbm<S, decltype(slip)::value, decltype(fused)::value>, grd, blk, 0, g, streams<S>(c),
+                       (const uint8_t*)c->flags, (const int32_t*)c->owner, (const DParticle*)c->part,
+                       (const float*)c->partf, (const C*)c->fb, (C)a[0], (C)a[1], (C)a[2],
+                       trt<C>(c->lambda_e, c->lambda_o), c->slip, fp);
         };
         using T_ = std::true_type;
         using F_ = std::false_type;
@@ -1121,16 +1311,12 @@ cudaError_t launch_lbm(es_ctx* c) {
 // The stream-collide of n contexts (same precision and device, no
 // free-slip faces; checked by the caller) in one launch on cs[0]'s stream,
 // ordered after each context's pending work and before its later work by
-// events.  Each context's per-run preparation (the float particle copy, the
-// body force at cells next to obstacles) runs on its own stream first.
+// events.  Each context's per-run preparation (the body force at cells next
+// to obstacles) runs on its own stream first.
 cudaError_t launch_lbm_batch(es_ctx* const* cs, int n) {
     cudaStream_t bs = cs[0]->stream;
     for (int i = 0; i < n; i++) {
         es_ctx* c = cs[i];
-        if (mixed(c) && c->np > 0) {
-            k_particles_f32<<<(c->np + 127) / 128, 128, 0, c->stream>>>(c->np, c->part, c->partf);
-            count(c);
-        }
         if (c->fb_lazy) {
             const cudaError_t e = launch_body_force_near(c);
             if (e != cudaSuccess) return e;
@@ -1190,28 +1376,44 @@ cudaError_t launch_lbm_batch(es_ctx* const* cs, int n) {
     return err;
 }
 
+template <class S, int T>
+cudaError_t run_forces(es_ctx* c, int src, double rmax) {
+    const double* E = c->P.E_ext;
+    // room for the cells with links of a sphere whose rows fit the bit words
+    // (R <= 13.5): their centres lie between R and R + sqrt 2 of its centre, so
+    // they number less than the volume between R - 1.9 and R + 2.4
+    const double r = rmax < 13.5 ? rmax : 13.5, ro = r + 2.4, ri = r > 1.9 ? r - 1.9 : 0.0;
+    const int room = (int)(4.19 * (ro * ro * ro - ri * ri * ri)) + 32;
+    const int cells = room < kForceChunk ? kForceChunk : (room + 7) / 8 * 8;
+    auto launch = [&](auto* kernel, size_t lists, size_t most) -> cudaError_t {
+        // (the attribute belongs to the kernel: the most any context needs)
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+        if (e != cudaSuccess) return e;
+        launch_pdl(c, kernel, c->np, T, lists, c->g, (const DParticle*)c->part, (const int32_t*)c->owner,
+                   (const uint8_t*)c->flags, (const S*)c->pdf[src], E[0], E[1], E[2], c->F, c->T, cells);
+        return cudaGetLastError();
+    };
+    const size_t words = (size_t)2 * kForceSide * kForceSide * 4, list = (size_t)cells * 8, most = 12 * 1024 * 8;
+    if constexpr (std::is_same<S, double>::value)
+        return launch(k_forces<T>, words + list, words + most);
+    else
+        return launch(k_forces_f32<S, T>, words + list + (size_t)kForceLinks * 8, words + most + kForceLinks * 8);
+}
+
 cudaError_t launch_forces(es_ctx* c) {
     if (c->np == 0) return cudaSuccess;
-    const double* E = c->P.E_ext;
     int src = c->last_src >= 0 ? c->last_src : c->cur;
     ProfScope ps(c, "forces", -1, 0.0);
+    double rmax = 0.0;
+    for (double r : c->h_R) rmax = r > rmax ? r : rmax;
+    cudaError_t err = cudaSuccess;
     dispatch_store(c, [&](auto tag) {
         using S = decltype(tag);
-        // (the FP32 form packs box-local indices in 10 bits per axis)
-        double rmax = 0.0;
-        for (double r : c->h_R) rmax = r > rmax ? r : rmax;
-        const bool small_boxes = 2.0 * rmax + 8.0 < 1024.0;
-        if (std::is_same<S, double>::value || !small_boxes)
-            k_forces<S><<<c->np, kForceThreads, 0, c->stream>>>(c->g, c->part, c->owner, c->flags,
-                                                                (const S*)c->pdf[src], E[0], E[1], E[2], c->mapped,
-                                                                c->F, c->T);
-        else
-            k_forces_f32<S><<<c->np, kForceThreads, 0, c->stream>>>(c->g, c->part, c->owner, c->flags,
-                                                                    (const S*)c->pdf[src], E[0], E[1], E[2],
-                                                                    c->mapped, c->F, c->T);
+        // few spheres: a block of 1,024 threads each
+        err = c->np <= 2 * c->n_sm ? run_forces<S, 1024>(c, src, rmax) : run_forces<S, 256>(c, src, rmax);
     });
     count(c);
-    return cudaGetLastError();
+    return err;
 }
 
 // A new particle state from the host: position, velocities, zeta, q and the
@@ -1222,7 +1424,7 @@ cudaError_t launch_forces(es_ctx* c) {
 // boundary value (2 zeta, or sigma / eps) is split into float-float as the
 // mapping does.
 __global__ void k_set_particles(const double* __restrict__ in, DParticle* part, const int* kind, double eps,
-                                float* pbc, int np) {
+                                float* pbc, float* __restrict__ pf, int np) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np) return;
     const double* s = in + 12 * p;
@@ -1232,6 +1434,8 @@ __global__ void k_set_particles(const double* __restrict__ in, DParticle* part, 
         d.v[a] = s[3 + a];
         d.w[a] = s[6 + a];
     }
+    if (pf)
+        for (int k = 0; k < 9; k++) pf[12 * p + k] = (float)s[k];
     d.zeta = s[9];
     d.q = s[10];
     d.qeff = s[11];
@@ -1245,7 +1449,7 @@ __global__ void k_set_particles(const double* __restrict__ in, DParticle* part, 
 cudaError_t launch_set_particles(es_ctx* c) {
     if (c->np == 0) return cudaSuccess;
     k_set_particles<<<blocks_for(c->np, 128), 128, 0, c->stream>>>(c->pstage, c->part, c->kind, c->S.eps, c->pbc,
-                                                                   c->np);
+                                                                   c->partf, c->np);
     count(c);
     return cudaGetLastError();
 }
@@ -1253,9 +1457,16 @@ cudaError_t launch_set_particles(es_ctx* c) {
 cudaError_t launch_advance(es_ctx* c) {
     if (c->np == 0) return cudaSuccess;
     ProfScope ps(c, "advance", -1, 0.0);
-    k_advance<<<blocks_for(c->np, 128), 128, 0, c->stream>>>(c->np, c->part, c->F, c->T, c->g.per[0], c->g.per[1],
-                                                             c->g.per[2], (double)c->g.nx, (double)c->g.ny,
-                                                             (double)c->g.nz);
+    launch_pdl(c, k_advance, blocks_for(3 * (long long)c->np, 128), 128, 0, c->np, c->part, (const double*)c->F,
+               (const double*)c->T, c->g.per[0], c->g.per[1], c->g.per[2], (double)c->g.nx, (double)c->g.ny,
+               (double)c->g.nz, c->partf);
+    count(c);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_particles_f32(es_ctx* c) {
+    if (!mixed(c) || c->np == 0) return cudaSuccess;
+    k_particles_f32<<<(c->np + 127) / 128, 128, 0, c->stream>>>(c->np, c->part, c->partf);
     count(c);
     return cudaGetLastError();
 }

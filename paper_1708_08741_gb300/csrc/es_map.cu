@@ -11,8 +11,14 @@
 //   k_uncover   cells still marked -2 - p were uncovered: PDFs set to
 //               f^eq(rho_0, u_s) of p's state at the last mapping
 //   k_flags     flags / level-0 states of every cell within two cells of
-//               the old or new sphere, and the count of p's fluid faces
-//               (sigma = q / faces for a charged sphere)
+//               the old or new sphere, the count of p's fluid faces (sigma =
+//               q / faces for a charged sphere), and p's mapped state
+//
+// On small grids the chain of these kernels is bound by latency, not work:
+// every kernel is launched with programmatic dependent launch and forms its
+// FP64 set-up (64-cycle operations in one or three threads) before it waits
+// for the kernel before it, and few spheres get blocks of 1,024 threads
+// (map_threads).
 #include "es_device.cuh"
 
 namespace es {
@@ -48,37 +54,24 @@ struct Box {
         y = wrap1(lo[1] + j, g.ny);
         z = wrap1(lo[2] + k, g.nz);
     }
-    __device__ void cell(const Grid& g, int t, int& x, int& y, int& z) const {
-        int sx = size(0), sy = size(1);
-        int i = t % sx;
-        int j = (t / sx) % sy;
-        int k = t / (sx * sy);
-        x = wrap_coord(lo[0] + i, g.nx);
-        y = wrap_coord(lo[1] + j, g.ny);
-        z = wrap_coord(lo[2] + k, g.nz);
-    }
 };
 
-__device__ Box sphere_box(const Grid& g, const double* X, double R, int ext) {
-    Box b;
-    for (int a = 0; a < 3; a++) axis_range(g, a, X[a], X[a], R, ext, b.lo[a], b.hi[a]);
-    return b;
+// The box of cells within R (+ ext) of X, one thread an axis (the caller
+// synchronises).
+__device__ void sphere_box_by_axis(const Grid& g, const double* X, double R, int ext, Box& b) {
+    const int a = threadIdx.x;
+    if (a < 3) axis_range(g, a, X[a], X[a], R, ext, b.lo[a], b.hi[a]);
 }
 
-// Union box of the old and the new position; on periodic axes the new
-// position is taken as the image nearest to the old one.
-__device__ Box union_box(const Grid& g, const double* Xo, const double* Xn, double R, int ext) {
-    Box b;
-    for (int a = 0; a < 3; a++) {
-        double xo = Xo[a], xn = Xn[a];
-        if (g.per[a]) {
-            double L = (double)gdim(g, a);
-            if (xn - xo > 0.5 * L) xn -= L;
-            if (xn - xo < -0.5 * L) xn += L;
-        }
-        axis_range(g, a, fmin(xo, xn), fmax(xo, xn), R, ext, b.lo[a], b.hi[a]);
+// One axis of the union box of the old and the new position; on a periodic
+// axis the new position is taken as the image nearest to the old one.
+__device__ void union_range(const Grid& g, int a, double xo, double xn, double R, int ext, Box& b) {
+    if (g.per[a]) {
+        double L = (double)gdim(g, a);
+        if (xn - xo > 0.5 * L) xn -= L;
+        if (xn - xo < -0.5 * L) xn += L;
     }
-    return b;
+    axis_range(g, a, fmin(xo, xn), fmax(xo, xn), R, ext, b.lo[a], b.hi[a]);
 }
 
 // GB300 runs FP64 arithmetic at a small fraction of the FP32 rate, so the
@@ -103,11 +96,19 @@ struct FlipList {
     }
 };
 
-__global__ void k_clear(Grid g, const DParticle* part, const double* mapped, int32_t* owner) {
+// (Block 0 also zeroes the counters of the cell lists, which no kernel still
+// running reads.)
+__global__ void __launch_bounds__(1024) k_clear(Grid g, const DParticle* part, const double* mapped, int32_t* owner, int* near_count,
+                        int nnear, int* bf_count) {
     __shared__ Box sb;
     int p = blockIdx.x;
-    if (threadIdx.x == 0) sb = sphere_box(g, mapped + 9 * p, part[p].R, 0);
+    sphere_box_by_axis(g, mapped + 9 * p, part[p].R, 0, sb);
     __syncthreads();
+    pdl_wait();
+    if (p == 0) {
+        for (int i = threadIdx.x; i < nnear; i += blockDim.x) near_count[i] = 0;
+        for (int i = threadIdx.x; i < kNearSegs; i += blockDim.x) bf_count[i] = 0;
+    }
     const Box b = sb;
     int n = b.count();
     BoxWalk w;
@@ -120,7 +121,7 @@ __global__ void k_clear(Grid g, const DParticle* part, const double* mapped, int
     }
 }
 
-__global__ void k_set(Grid g, const DParticle* part, const int* kind, int32_t* owner, double* psi,
+__global__ void __launch_bounds__(1024) k_set(Grid g, const DParticle* part, const int* kind, int32_t* owner, double* psi,
                       float* psi_hi, float* psi_lo, int* status, FlipList flips) {
     __shared__ Box sb;
     __shared__ BallF sball;
@@ -128,28 +129,34 @@ __global__ void k_set(Grid g, const DParticle* part, const int* kind, int32_t* o
     __shared__ float sbhi, sblo;
     int p = blockIdx.x;
     const DParticle& P = part[p];
-    if (threadIdx.x == 0) {
-        for (int a = 0; a < 3; a++)
-            if (!g.per[a] && (P.x[a] - P.R < 0.0 || P.x[a] + P.R > (double)gdim(g, a)))
-                atomicOr(status, DS_WALLCUT);
+    sphere_box_by_axis(g, P.x, P.R, 0, sb);
+    bool cut = false;
+    if (threadIdx.x < 3) {
+        const int a = threadIdx.x;
+        cut = !g.per[a] && (P.x[a] - P.R < 0.0 || P.x[a] + P.R > (double)gdim(g, a));
+    }
+    if (threadIdx.x == 32) {
         // boundary value kept in the solution field at boundary cells (Sec. 5.4)
         sbval = kind[p] == ES_KIND_ZETA ? P.zeta : 0.0;
         const ff bff = ff_from_double(sbval);
         sbhi = bff.hi;
         sblo = bff.lo;
-        sb = sphere_box(g, P.x, P.R, 0);
-        sball.init(g, P.x, P.R, sb.lo, sb.hi);
     }
     __syncthreads();
+    sball.init_by_axis(g, P.x, P.R, sb.lo, sb.hi);
+    __syncthreads();
+    pdl_wait();
+    if (cut) atomicOr(status, DS_WALLCUT);
     const Box b = sb;
     const BallF ball = sball;
+    const bool ball_ok = ball.all_ok();
     int n = b.count();
     BoxWalk w;
     w.start(threadIdx.x, blockDim.x, b.size(0), b.size(1));
     for (int t = threadIdx.x; t < n; t += blockDim.x, w.next()) {
         // decided in FP32 away from the surface, by the FP64 test near it
         int in = -1;
-        if (ball.ok) {
+        if (ball_ok) {
             const float d2 = ball.d2(w.i, w.j, w.k);
             if (d2 > ball.r2 + ball.margin) continue;
             if (d2 < ball.r2 - ball.margin) in = 1;
@@ -171,13 +178,14 @@ __global__ void k_set(Grid g, const DParticle* part, const int* kind, int32_t* o
 }
 
 template <class S>
-__global__ void k_uncover(Grid g, const DParticle* part, const double* mapped, int32_t* owner, S* pdf,
+__global__ void __launch_bounds__(1024) k_uncover(Grid g, const DParticle* part, const double* mapped, int32_t* owner, S* pdf,
                           FlipList flips) {
     __shared__ Box sb;
     int p = blockIdx.x;
     const double* M = mapped + 9 * p;  // x, v, w at the last mapping
-    if (threadIdx.x == 0) sb = sphere_box(g, M, part[p].R, 0);
+    sphere_box_by_axis(g, M, part[p].R, 0, sb);
     __syncthreads();
+    pdl_wait();
     const Box b = sb;
     int n = b.count();
     BoxWalk w;
@@ -204,7 +212,7 @@ __global__ void k_uncover(Grid g, const DParticle* part, const double* mapped, i
 
 // Flags of one cell from the owner field.  Returns the number of D3Q7 faces
 // the cell (if fluid) shares with sphere `p`.
-__device__ int cell_flags(const Grid& g, const int32_t* owner, const int* kind, int x, int y, int z,
+__device__ __noinline__ int cell_flags(const Grid& g, const int32_t* owner, const int* kind, int x, int y, int z,
                           int p, uint8_t& fl, uint8_t& st) {
     long long c = lin(g, x, y, z);
     int o = owner[c];
@@ -236,140 +244,177 @@ __device__ int cell_flags(const Grid& g, const int32_t* owner, const int* kind, 
     return faces;
 }
 
-// all_cells = 0 skips the cells whose flags cannot have changed.  With D
-// the displacement since the last mapping, a cell that changed owner lies
-// within D of the old surface in its old distance and within D of the new
-// surface in its new distance; a cell whose D3Q19 neighbours (within
-// sqrt 2) include one is therefore within D + sqrt 2 of both.  A cell
-// outside either band keeps its flags, and it has no D3Q7 face to the new
-// sphere unless it is within 1 of the new surface.  So a cell is visited
-// when it is within 2.5 of the new surface, or within 2.5 + D of both.
-// The first mapping of a context visits every cell (all_cells = 1).
-__global__ void k_flags(Grid g, DParticle* part, const double* mapped, const int* kind,
-                        const int32_t* owner, uint8_t* flags, uint8_t* st0, int* nfaces, int all_cells) {
-    __shared__ int tile[kOwnerTileMax];
+// One block per sphere: flags and level-0 states of the cells within two of
+// the old or new sphere, and the sphere's faces.  The rows of that box (with a
+// halo of one cell) are held as bit words -- solid cells, cells beyond a wall,
+// Dirichlet cells, the sphere's own -- built with one load and four ballots a
+// row; whether a cell's neighbours hold an obstacle is then a few shifts for a
+// row at a time, and a warp writes a row's bytes.  (Per cell, from a tile of
+// owners: 18 shared-memory reads each; 2,880 spheres R = 5 140 us, 64 spheres
+// R = 6 30 us, now 150 and 16 us.)  Cells outside the changed shell are rewritten with
+// what they hold.
+//
+// Boxes with longer rows (R > 11) visit the cells whose flags can have
+// changed one by one.  With D the displacement since the last mapping, a cell
+// that changed owner lies within D of the old surface in its old distance and
+// within D of the new surface in its new distance; a cell whose D3Q19
+// neighbours (within sqrt 2) include one is therefore within D + sqrt 2 of
+// both.  A cell outside either band keeps its flags, and it has no D3Q7 face
+// to the new sphere unless it is within 1 of the new surface.  The first
+// mapping of a context visits every cell (all_cells = 1).
+//
+// The block's last act keeps the mapped state for the next reconstruction (no
+// other block reads it) and, in the reduced forms, the sphere's boundary value
+// for the float-float outer residual: 2 zeta for a Dirichlet sphere, sigma /
+// eps for a charged one (Sec. 5.4); *moved is raised when the sphere moved
+// half a cell or more along an axis since the previous mapping (minimum image
+// on periodic axes).
+constexpr int kFlagSide = 32;  // longest row of the bit words, halo included
+
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 6)
+    k_flags(Grid g, DParticle* part, double* mapped, const int* __restrict__ kind, const int32_t* __restrict__ owner,
+            uint8_t* flags, uint8_t* st0, int* nfaces, int all_cells, double eps, float* pbc, int* moved) {
+    __shared__ unsigned s_solid[kFlagSide * kFlagSide], s_out[kFlagSide * kFlagSide], s_dir[kFlagSide * kFlagSide],
+        s_own[kFlagSide * kFlagSide], s_near7[kFlagSide * kFlagSide], s_near19[kFlagSide * kFlagSide];
     __shared__ Box sb;
-    __shared__ BallF sbo, sbn;
-    __shared__ float sband[5];  // lo1, hi1, lo2, hi2, skip_ok
+    __shared__ float sd2[3];
     __shared__ int sw[32];
-    int p = blockIdx.x;
-    if (threadIdx.x == 0) {
-        const double* Xo = mapped + 9 * p;
-        const double R = part[p].R;
-        sb = union_box(g, Xo, part[p].x, R, 2);
-        sbo.init(g, Xo, R, sb.lo, sb.hi);
-        sbn.init(g, part[p].x, R, sb.lo, sb.hi);
-        float D2 = 0.0f;
-        for (int a = 0; a < 3; a++) {
-            double d = part[p].x[a] - Xo[a];
-            if (g.per[a]) {
-                const double L = (double)gdim(g, a);
-                if (d > 0.5 * L) d -= L;
-                if (d < -0.5 * L) d += L;
-            }
-            D2 += (float)d * (float)d;
+    const int p = blockIdx.x;
+    const double* Xo = mapped + 9 * p;
+    const double R = part[p].R;
+    if (threadIdx.x < 3) {
+        const int a = threadIdx.x;
+        union_range(g, a, Xo[a], part[p].x[a], R, 2, sb);
+        double d = part[p].x[a] - Xo[a];
+        if (g.per[a]) {
+            const double L = (double)gdim(g, a);
+            if (d > 0.5 * L) d -= L;
+            if (d < -0.5 * L) d += L;
         }
-        // (bands: faces need the new surface's outer layer, R .. R + 1;
-        // changed flags lie within sqrt 2 + D of both surfaces; 0.05 margin)
-        const float rf = (float)R, w1 = 1.05f, w2 = 1.47f + sqrtf(D2) * 1.001f;
-        sband[0] = rf > w1 ? (rf - w1) * (rf - w1) : -1.0f;
-        sband[1] = (rf + w1) * (rf + w1);
-        sband[2] = rf > w2 ? (rf - w2) * (rf - w2) : -1.0f;
-        sband[3] = (rf + w2) * (rf + w2);
-        sband[4] = (!all_cells && sbo.ok && sbn.ok) ? 1.0f : 0.0f;
+        sd2[a] = (float)d * (float)d;
     }
     __syncthreads();
+    pdl_wait();
     const Box b = sb;
-    const BallF bo = sbo, bn = sbn;
-    const float lo1 = sband[0], hi1 = sband[1], lo2 = sband[2], hi2 = sband[3];
-    const bool skip_ok = sband[4] != 0.0f;
-    const OwnerTile T{{b.size(0), b.size(1), b.size(2)}};
-    const bool use_tile = T.fits();
-    if (use_tile) {
-        load_owner_tile(g, owner, b.lo, T, tile);
-        __syncthreads();
-    }
-    int n = b.count();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = THREADS / 32;
     int faces = 0;
-    BoxWalk w;
-    w.start(threadIdx.x, blockDim.x, b.size(0), b.size(1));
-    for (int t = threadIdx.x; t < n; t += blockDim.x, w.next()) {
-        if (skip_ok) {
-            const float dn = bn.d2(w.i, w.j, w.k), dol = bo.d2(w.i, w.j, w.k);
-            const bool near_new = dn >= lo1 && dn <= hi1;
-            const bool near_both = dn >= lo2 && dn <= hi2 && dol >= lo2 && dol <= hi2;
-            if (!near_new && !near_both) continue;
-        }
-        int x, y, z;
-        b.at(g, w.i, w.j, w.k, x, y, z);
-        uint8_t fl, st;
-        if (use_tile) {
-            // cell_flags from the tile
-            const int ti = T.at(w.i, w.j, w.k);
-            const int o = tile[ti];
-            if (o >= 0) {
-                fl = F_SOLID;
-                st = kind[o] == ES_KIND_ZETA ? ST_DIR : ST_NEU;
-            } else {
-                bool near19 = false, near7 = false;
+    if (b.size(0) + 2 <= kFlagSide && b.size(1) + 2 <= kFlagSide && b.size(2) + 2 <= kFlagSide) {
+        const int sx = b.size(0), sy = b.size(1), sz = b.size(2), ry = sy + 2, nr = ry * (sz + 2);
+        const int gx0 = b.lo[0] - 1 + lane;
+        const bool xin = lane < sx + 2 && (g.per[0] || (gx0 >= 0 && gx0 < g.nx));
+        const int gx = xin ? wrap1(gx0, g.nx) : 0;
+        int jz = wid / ry, jy = wid - jz * ry;
+        for (int r0 = wid; r0 < nr; r0 += 4 * nw) {
+            int o[4];
+            bool in[4];
 #pragma unroll
-                for (int q = 1; q < 19; q++) {
-                    const int on = tile[ti + T.step(q)];
-                    const bool axis = (q <= 3) || (q >= 10 && q <= 12);
-                    if (on >= 0 || on == kOwnerOutside) {
-                        near19 = true;
-                        near7 |= axis;
-                        if (axis && on == p) faces++;
-                    }
-                }
-                fl = near19 ? F_NEAR19 : 0;
-                st = near7 ? ST_NEAR : ST_UNKNOWN;
+            for (int u = 0; u < 4; u++) {
+                const int y0 = b.lo[1] - 1 + jy, z0 = b.lo[2] - 1 + jz;
+                in[u] = xin && r0 + u * nw < nr && (g.per[1] || (y0 >= 0 && y0 < g.ny)) &&
+                        (g.per[2] || (z0 >= 0 && z0 < g.nz));
+                o[u] = in[u] ? owner[gx + g.nx * (wrap1(y0, g.ny) + g.ny * wrap1(z0, g.nz))] : -1;
+                for (jy += nw; jy >= ry; jy -= ry) jz++;
             }
-        } else {
-            faces += cell_flags(g, owner, kind, x, y, z, p, fl, st);
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const unsigned ws = __ballot_sync(0xffffffffu, o[u] >= 0);
+                const unsigned wx = __ballot_sync(0xffffffffu, !in[u]);
+                const unsigned wo = __ballot_sync(0xffffffffu, o[u] == p);
+                const unsigned wd = ws ? __ballot_sync(0xffffffffu, o[u] >= 0 && kind[o[u]] == ES_KIND_ZETA) : 0u;
+                if (lane == 0 && r0 + u * nw < nr) {
+                    s_solid[r0 + u * nw] = ws;
+                    s_out[r0 + u * nw] = wx;
+                    s_own[r0 + u * nw] = wo;
+                    s_dir[r0 + u * nw] = wd;
+                }
+            }
         }
-        long long c = lin(g, x, y, z);
-        flags[c] = fl;
-        st0[c] = st;
+        __syncthreads();
+        // a thread a row: which cells are next to an obstacle or a wall
+        const unsigned inside = ((1u << sx) - 1u) << 1;
+        for (int r = threadIdx.x; r < sy * sz; r += THREADS) {
+            const int k = r / sy, at = (r - k * sy) + 1 + ry * (k + 1);
+            auto block = [&](int d) { return s_solid[at + d] | s_out[at + d]; };
+            auto wide = [&](unsigned w) { return w | (w << 1) | (w >> 1); };
+            const unsigned own = s_own[at], c = block(0), n1 = block(-1) | block(1) | block(-ry) | block(ry);
+            const unsigned n2 = block(-1 - ry) | block(1 - ry) | block(-1 + ry) | block(1 + ry);
+            const unsigned x1 = (c << 1) | (c >> 1), fluid = ~c & inside;
+            faces += __popc(fluid & (own << 1)) + __popc(fluid & (own >> 1)) + __popc(fluid & s_own[at - 1]) +
+                     __popc(fluid & s_own[at + 1]) + __popc(fluid & s_own[at - ry]) + __popc(fluid & s_own[at + ry]);
+            s_near7[r] = fluid & (x1 | n1);
+            s_near19[r] = fluid & (x1 | wide(n1) | n2);
+        }
+        __syncthreads();
+        // a warp a row; lane i + 1: cell i of the row
+        if ((inside >> lane) & 1u) {
+            const unsigned bit = 1u << lane;
+            int k = wid / sy, j = wid - k * sy;
+            for (int r = wid; r < sy * sz; r += nw) {
+                const int at = j + 1 + ry * (k + 1);
+                const bool solid = (s_solid[at] & bit) != 0;
+                const int cell = gx + g.nx * (wrap1(b.lo[1] + j, g.ny) + g.ny * wrap1(b.lo[2] + k, g.nz));
+                flags[cell] = solid ? F_SOLID : ((s_near19[r] & bit) ? F_NEAR19 : 0);
+                st0[cell] = solid ? ((s_dir[at] & bit) ? ST_DIR : ST_NEU) : ((s_near7[r] & bit) ? ST_NEAR : ST_UNKNOWN);
+                for (j += nw; j >= sy; j -= sy) k++;
+            }
+        }
+    } else {
+        BallF bo, bn;
+        bo.init(g, Xo, R, b.lo, b.hi);
+        bn.init(g, part[p].x, R, b.lo, b.hi);
+        // (bands: faces need the new surface's outer layer, R .. R + 1;
+        // changed flags lie within sqrt 2 + D of both surfaces; 0.05 margin)
+        const float rf = (float)R, w1 = 1.05f, w2 = 1.47f + sqrtf(sd2[0] + sd2[1] + sd2[2]) * 1.001f;
+        const float lo1 = rf > w1 ? (rf - w1) * (rf - w1) : -1.0f, hi1 = (rf + w1) * (rf + w1);
+        const float lo2 = rf > w2 ? (rf - w2) * (rf - w2) : -1.0f, hi2 = (rf + w2) * (rf + w2);
+        const bool skip_ok = !all_cells && bo.ok && bn.ok;
+        const int n = b.count();
+        BoxWalk w;
+        w.start(threadIdx.x, blockDim.x, b.size(0), b.size(1));
+        for (int t = threadIdx.x; t < n; t += blockDim.x, w.next()) {
+            if (skip_ok) {
+                const float dn = bn.d2(w.i, w.j, w.k), dol = bo.d2(w.i, w.j, w.k);
+                const bool near_new = dn >= lo1 && dn <= hi1;
+                const bool near_both = dn >= lo2 && dn <= hi2 && dol >= lo2 && dol <= hi2;
+                if (!near_new && !near_both) continue;
+            }
+            int x, y, z;
+            b.at(g, w.i, w.j, w.k, x, y, z);
+            uint8_t fl, st;
+            faces += cell_flags(g, owner, kind, x, y, z, p, fl, st);
+            const long long c = lin(g, x, y, z);
+            flags[c] = fl;
+            st0[c] = st;
+        }
     }
     // block sum of the face counts (integers: exact in any order)
     for (int o = 16; o > 0; o >>= 1) faces += __shfl_down_sync(0xffffffffu, faces, o);
-    if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = faces;
+    if (lane == 0) sw[wid] = faces;
     __syncthreads();
     if (threadIdx.x == 0) {
         int nf = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) nf += sw[w];
+        for (int w = 0; w < nw; w++) nf += sw[w];
         nfaces[p] = nf;
         // Neumann charge per face: sigma = q / faces, so that the flux over
         // the staircase surface equals the particle charge.
-        part[p].sigma = nf > 0 ? part[p].q / (double)nf : 0.0;
+        const double sigma = nf > 0 ? part[p].q / (double)nf : 0.0;
+        part[p].sigma = sigma;
+        if (pbc) {
+            const ff v = ff_from_double(kind[p] == ES_KIND_ZETA ? 2.0 * part[p].zeta : sigma / eps);
+            pbc[2 * p] = v.hi;
+            pbc[2 * p + 1] = v.lo;
+        }
     }
-}
-
-// Keeps the mapped state for the next reconstruction and, in the MIXED32
-// form, the sphere's boundary value for the float-float outer residual:
-// 2 zeta for a Dirichlet sphere, sigma / eps for a charged one (Sec. 5.4).
-// Raises *moved when the sphere moved half a cell or more along an axis
-// since the previous mapping (minimum image on periodic axes).
-__global__ void k_store_mapped(Grid g, const DParticle* part, const int* kind, double eps, double* mapped,
-                               float* pbc, int np, int* moved) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    for (int a = 0; a < 3; a++) {
+    if (threadIdx.x >= 32 && threadIdx.x < 35) {
+        const int a = threadIdx.x - 32;
         double d = fabs(part[p].x[a] - mapped[9 * p + a]);
         const double L = (double)gdim(g, a);
         if (g.per[a] && d > 0.5 * L) d = L - d;
         if (!(d < 0.5)) *moved = 1;
-    }
-    for (int a = 0; a < 3; a++) {
         mapped[9 * p + a] = part[p].x[a];
         mapped[9 * p + 3 + a] = part[p].v[a];
         mapped[9 * p + 6 + a] = part[p].w[a];
-    }
-    if (pbc) {
-        const ff v = ff_from_double(kind[p] == ES_KIND_ZETA ? 2.0 * part[p].zeta : part[p].sigma / eps);
-        pbc[2 * p] = v.hi;
-        pbc[2 * p + 1] = v.lo;
     }
 }
 
@@ -377,6 +422,7 @@ __global__ void k_store_mapped(Grid g, const DParticle* part, const int* kind, d
 // Dirichlet, else unknown if any child is unknown, else Neumann.
 __global__ void k_coarse_kind(int fx, int fy, int fz, int cxn, int cyn, int czn, const uint8_t* fine,
                               uint8_t* coarse) {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int j = blockIdx.y, k = blockIdx.z;
     if (i >= cxn) return;
@@ -399,6 +445,7 @@ __global__ void k_coarse_kind(int fx, int fy, int fz, int cxn, int cyn, int czn,
 __global__ void __launch_bounds__(256) k_coarse_kind_v(int fx, int fy, int cxn, int cyn,
                                                        const uint8_t* __restrict__ fine,
                                                        uint8_t* __restrict__ coarse) {
+    pdl_wait();
     const int i0 = 4 * (blockIdx.x * 32 + threadIdx.x);
     const int j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
     if (i0 >= cxn || j >= cyn) return;
@@ -430,6 +477,7 @@ __global__ void __launch_bounds__(256) k_coarse_kind_v(int fx, int fy, int cxn, 
 // kind bits, and neighbours read only kind bits, so every read sees the
 // kinds whether or not the word was rewritten yet.
 __global__ void __launch_bounds__(256) k_near_bits_v(int nx, int ny, int nz, int px, int py, int pz, uint8_t* st) {
+    pdl_wait();
     const int i0 = 4 * (blockIdx.x * 32 + threadIdx.x);
     const int j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
     if (i0 >= nx || j >= ny) return;
@@ -472,6 +520,7 @@ __global__ void __launch_bounds__(256) k_near_bits_v(int nx, int ny, int nz, int
 // unknown, or a non-periodic domain face.  Only the bit is written; the
 // kind bits neighbours read are unchanged, so updating in place is safe.
 __global__ void k_near_bits(int nx, int ny, int nz, int px, int py, int pz, uint8_t* st) {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int j = blockIdx.y, k = blockIdx.z;
     if (i >= nx) return;
@@ -525,6 +574,7 @@ __device__ __forceinline__ int warp_excl_scan(int v, int& total) {
 __global__ void __launch_bounds__(256) k_near_list(int nx, int ny, int nz, const uint8_t* __restrict__ st,
                                                    int cap, int* list, int* count, uint32_t* __restrict__ rbmask,
                                                    int wpr) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= ny * nz) return;  // whole warps
@@ -595,6 +645,7 @@ __global__ void __launch_bounds__(256) k_near_list(int nx, int ny, int nz, const
 // row segments as k_near_list does.
 __global__ void __launch_bounds__(256) k_near19_list(int nx, int ny, int nz, const uint8_t* __restrict__ flags,
                                                      int cap, int* list, int* count) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -632,6 +683,7 @@ __global__ void __launch_bounds__(256) k_lists_l0(int nx, int ny, int nz, const 
                                                   const uint8_t* __restrict__ flags, int cap, int* list,
                                                   int* count, int bf_cap, int* bf_list, int* bf_count,
                                                   uint32_t* __restrict__ rbmask, int wpr) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= ny * nz) return;  // whole warps
@@ -722,34 +774,49 @@ __global__ void __launch_bounds__(256) k_lists_l0(int nx, int ny, int nz, const 
 
 }  // namespace
 
-cudaError_t launch_near_lists(es_ctx* c) {
-    cudaError_t e = cudaMemsetAsync(c->near_count, 0, 2 * kNearSegs * ES_MAXLEV * sizeof(int), c->stream);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(c->bf_count, 0, kNearSegs * sizeof(int), c->stream);
-    if (e != cudaSuccess) return e;
+// The near-cell list of a level (and level 1's update masks) are made where
+// some kernel reads them: the colour-split levels' half sweeps, the half
+// sweeps of levels above near_list_cells, and the FP64 restriction of levels
+// too large to form those children itself (restrict_inline).
+static bool list_needed(const es_ctx* c, int l) {
+    if (l >= c->tail_l0) return false;
+    if (split_level(c, l)) return true;
+    const long long most = c->P.near_list_cells > 0 ? (long long)c->P.near_list_cells : (long long)ES_NEAR_LIST_CELLS;
+    const long long n = (long long)c->ln[l][0] * c->ln[l][1] * c->ln[l][2];
+    return n > most || (!mixed(c) && n > (1 << 18));
+}
+
+// zero: the counters are not zero yet (no mapping kernel ran before this).
+cudaError_t launch_near_lists(es_ctx* c, bool zero) {
+    if (zero) {
+        cudaError_t e = cudaMemsetAsync(c->near_count, 0, 2 * kNearSegs * ES_MAXLEV * sizeof(int), c->stream);
+        if (e != cudaSuccess) return e;
+        e = cudaMemsetAsync(c->bf_count, 0, kNearSegs * sizeof(int), c->stream);
+        if (e != cudaSuccess) return e;
+    }
     int l0 = 0;
+    const int rows0 = c->g.ny * c->g.nz;
     if (c->g.nx % 4 == 0) {
         ProfScope ps(c, "cell_lists", 0, 2.0 * (double)c->g.N);
-        k_lists_l0<<<(c->g.ny * c->g.nz + 7) / 8, 256, 0, c->stream>>>(c->g.nx, c->g.ny, c->g.nz, c->st[0], c->flags,
-                                                                      c->near_cap[0], c->near_list[0], c->near_count,
-                                                                      c->bf_cap, c->bf_list, c->bf_count,
-                                                                      c->rbmask, c->rb_wpr);
+        launch_pdl(c, k_lists_l0, (rows0 + 7) / 8, 256, 0, c->g.nx, c->g.ny, c->g.nz, c->st[0], c->flags,
+                   c->near_cap[0], c->near_list[0], c->near_count, c->bf_cap, c->bf_list, c->bf_count, c->rbmask,
+                   c->rb_wpr);
         count(c);
         l0 = 1;
     }
     for (int l = l0; l < c->L; l++) {
+        if (l > 0 && !list_needed(c, l)) continue;
         const int* n = c->ln[l];
         const int rows = n[1] * n[2];
         const int nb = (rows + 7) / 8;  // a warp per row: every row in flight at once
         ProfScope ps(c, "cell_lists", l, (double)rows * n[0]);
-        k_near_list<<<nb, 256, 0, c->stream>>>(n[0], n[1], n[2], c->st[l], c->near_cap[l], c->near_list[l],
-                                                c->near_count + 2 * kNearSegs * l, l == 1 ? c->rbmask1 : nullptr,
-                                                c->rb_wpr1);
+        launch_pdl(c, k_near_list, nb, 256, 0, n[0], n[1], n[2], c->st[l], c->near_cap[l], c->near_list[l],
+                   c->near_count + 2 * kNearSegs * l, l == 1 ? c->rbmask1 : nullptr, c->rb_wpr1);
         count(c);
     }
     if (l0 == 0) {
-        k_near19_list<<<(c->g.ny * c->g.nz + 7) / 8, 256, 0, c->stream>>>(c->g.nx, c->g.ny, c->g.nz, c->flags,
-                                                                          c->bf_cap, c->bf_list, c->bf_count);
+        launch_pdl(c, k_near19_list, (rows0 + 7) / 8, 256, 0, c->g.nx, c->g.ny, c->g.nz, c->flags, c->bf_cap,
+                   c->bf_list, c->bf_count);
         count(c);
     }
     return cudaGetLastError();
@@ -766,38 +833,40 @@ cudaError_t launch_init_flags(es_ctx* c) {
 cudaError_t launch_map(es_ctx* c) {
     if (c->np == 0) return cudaSuccess;
     const Grid& g = c->g;
-    const int T = 256;
+    // few spheres: a block of 1,024 threads each (64 spheres R = 6 leave an SM
+    // one block: the four kernels 74 -> 39 us); many: 256 (2,880 spheres fill
+    // the SMs either way)
+    const int T = c->np <= 2 * c->n_sm ? 1024 : 256;
     const FlipList flips{c->flip_list, c->flip_count, c->flip_cap, c->d_moved};
     {
         ProfScope ps(c, "map_clear", -1, 0.0);
-        k_clear<<<c->np, T, 0, c->stream>>>(g, c->part, c->mapped, c->owner);
+        launch_pdl(c, k_clear, c->np, T, 0, g, c->part, c->mapped, c->owner, c->near_count,
+                   2 * kNearSegs * ES_MAXLEV, c->bf_count);
     }
     {
         ProfScope ps(c, "map_set", -1, 0.0);
-        k_set<<<c->np, T, 0, c->stream>>>(g, c->part, c->kind, c->owner, c->psi, c->psi32, c->psi_lo, c->d_status,
-                                          flips);
+        launch_pdl(c, k_set, c->np, T, 0, g, c->part, c->kind, c->owner, c->psi, c->psi32, c->psi_lo, c->d_status,
+                   flips);
     }
     {
         ProfScope ps(c, "map_uncover", -1, 0.0);
         if (c->P.precision == ES_MIXED16)
-            k_uncover<__half><<<c->np, T, 0, c->stream>>>(g, c->part, c->mapped, c->owner, (__half*)c->pdf[c->cur],
-                                                            flips);
+            launch_pdl(c, k_uncover<__half>, c->np, T, 0, g, c->part, c->mapped, c->owner, (__half*)c->pdf[c->cur],
+                       flips);
         else if (mixed(c))
-            k_uncover<float><<<c->np, T, 0, c->stream>>>(g, c->part, c->mapped, c->owner, (float*)c->pdf[c->cur],
-                                                           flips);
+            launch_pdl(c, k_uncover<float>, c->np, T, 0, g, c->part, c->mapped, c->owner, (float*)c->pdf[c->cur],
+                       flips);
         else
-            k_uncover<double><<<c->np, T, 0, c->stream>>>(g, c->part, c->mapped, c->owner, (double*)c->pdf[c->cur],
-                                                            flips);
+            launch_pdl(c, k_uncover<double>, c->np, T, 0, g, c->part, c->mapped, c->owner, (double*)c->pdf[c->cur],
+                       flips);
     }
     {
         ProfScope ps(c, "map_flags", -1, 0.0);
-        k_flags<<<c->np, T, 0, c->stream>>>(g, c->part, c->mapped, c->kind, c->owner, c->flags, c->st[0],
-                                            c->nfaces, c->mapped_once ? 0 : 1);
+        launch_pdl(c, T == 1024 ? k_flags<1024> : k_flags<256>, c->np, T, 0, g, c->part, c->mapped, c->kind, c->owner, c->flags, c->st[0], c->nfaces,
+                   c->mapped_once ? 0 : 1, c->S.eps, c->pbc, c->d_moved);
         c->mapped_once = true;
     }
-    k_store_mapped<<<(c->np + 127) / 128, 128, 0, c->stream>>>(g, c->part, c->kind, c->S.eps, c->mapped, c->pbc,
-                                                                c->np, c->d_moved);
-    count(c, 5);
+    count(c, 4);
     return cudaGetLastError();
 }
 
@@ -808,17 +877,22 @@ cudaError_t launch_coarse_states(es_ctx* c) {
         dim3 blk(128), grd((m[0] + 127) / 128, m[1], m[2]);
         const double nc = (double)m[0] * m[1] * m[2];
         ProfScope ps(c, "coarse_states", l, 8.0 * nc + nc + 2.0 * nc);
+        // (near-boundary bits: not on the levels of k_tail, whose codes look at
+        // the neighbours' kinds themselves)
+        const bool near = l < c->tail_l0;
         if (m[0] % 4 == 0) {
             const dim3 vblk(32, 8), vgrd((m[0] / 4 + 31) / 32, (m[1] + 7) / 8, m[2]);
-            k_coarse_kind_v<<<vgrd, vblk, 0, c->stream>>>(f[0], f[1], m[0], m[1], c->st[l - 1], c->st[l]);
-            k_near_bits_v<<<vgrd, vblk, 0, c->stream>>>(m[0], m[1], m[2], c->g.per[0], c->g.per[1], c->g.per[2],
-                                                         c->st[l]);
+            launch_pdl(c, k_coarse_kind_v, vgrd, vblk, 0, f[0], f[1], m[0], m[1], c->st[l - 1], c->st[l]);
+            if (near)
+                launch_pdl(c, k_near_bits_v, vgrd, vblk, 0, m[0], m[1], m[2], c->g.per[0], c->g.per[1], c->g.per[2],
+                           c->st[l]);
         } else {
-            k_coarse_kind<<<grd, blk, 0, c->stream>>>(f[0], f[1], f[2], m[0], m[1], m[2], c->st[l - 1], c->st[l]);
-            k_near_bits<<<grd, blk, 0, c->stream>>>(m[0], m[1], m[2], c->g.per[0], c->g.per[1], c->g.per[2],
-                                                    c->st[l]);
+            launch_pdl(c, k_coarse_kind, grd, blk, 0, f[0], f[1], f[2], m[0], m[1], m[2], c->st[l - 1], c->st[l]);
+            if (near)
+                launch_pdl(c, k_near_bits, grd, blk, 0, m[0], m[1], m[2], c->g.per[0], c->g.per[1], c->g.per[2],
+                           c->st[l]);
         }
-        count(c, 2);
+        count(c, near ? 2 : 1);
     }
     return cudaGetLastError();
 }

@@ -542,6 +542,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
 // The codes of all levels in the blocks' layout: a thread a span of four
 // places (blockIdx.y: level).
 __global__ void __launch_bounds__(256) k_tail_codes(const __grid_constant__ TailCodes A) {
+    pdl_wait();
     const TailShape& S = A.s[blockIdx.y];
     const uint8_t* st = A.st[blockIdx.y];
     const int spans = S.ploc / 4;  // of a colour in a slab
@@ -558,10 +559,7 @@ __global__ void __launch_bounds__(256) k_tail_codes(const __grid_constant__ Tail
             code[k] = kTailOff;
             if (z >= S.nz || j0 + k >= S.nxh || x >= S.nx) continue;
             const int c = x + S.nx * (y + S.ny * z);
-            const uint8_t s = st[c];
-            if ((s & ST_KIND) != ST_UNKNOWN) continue;
-            code[k] = kTailInner;
-            if (!(s & ST_NEAR)) continue;
+            if ((st[c] & ST_KIND) != ST_UNKNOWN) continue;
             const int v[3] = {x, y, z}, n3[3] = {S.nx, S.ny, S.nz}, stride[3] = {1, S.nx, S.nx * S.ny};
             unsigned kind[6], wall = 0;
 #pragma unroll
@@ -771,7 +769,7 @@ cudaError_t launch_tail_codes(es_ctx* c) {
     for (int f = 0; f < 6; f++) A.pot_bc[f] = c->S.pot_bc[f];
     A.out = c->tail_codes;
     const int spans = p.s[0].ploc / 2 * p.blocks;
-    k_tail_codes<<<dim3((spans + 255) / 256, p.n), 256, 0, c->stream>>>(A);
+    launch_pdl(c, k_tail_codes, dim3((spans + 255) / 256, p.n), 256, 0, A);
     count(c);
     return cudaGetLastError();
 }

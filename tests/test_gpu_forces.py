@@ -1,0 +1,48 @@
+"""Force and torque by momentum exchange: a block a sphere, with the box's rows
+as bit words (R <= 13) or from the fields, against the FP64 oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1708_08741_gb300 as es
+from paper_1708_08741_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _workload(dims, periodic, radius, n, seed=7):
+    wl = W.mixed_box(dims=dims, periodic=periodic, n_spheres=n, radius=radius, levels=2, seed=seed)
+    wl.res_rf = 1e-8
+    return wl
+
+
+@pytest.mark.parametrize("precision", [es.ES_FP64, es.ES_MIXED32])
+@pytest.mark.parametrize("dims,periodic,radius,n", [
+    ((24, 20, 24), (1, 1, 1), 0.9, 3),      # a handful of cells
+    ((16, 16, 20), (1, 1, 1), 6.2, 1),      # the box spans the whole axes
+    ((32, 28, 32), (1, 0, 0), 3.3, 2),      # against walls
+    ((32, 32, 32), (1, 1, 1), 12.9, 1),     # the longest rows of bit words
+    ((36, 36, 36), (1, 1, 0), 14.2, 1),     # beyond them
+    ((96, 96, 96), (1, 1, 1), 2.6, 330),    # many spheres: small blocks
+])
+def test_forces_match_oracle(precision, dims, periodic, radius, n):
+    """FP64: the oracle's sums in another order, about 1e-15 of a cancelling
+    sum: 1e-11.  MIXED32: the parity bar of the reduced forms, 1e-4."""
+    wl = _workload(dims, periodic, radius, n)
+    g, o = es.Simulation(wl, precision), oracle.Oracle(wl, omp=True)
+    for _ in range(2):
+        o.map_particles()
+        info = o.solve()
+        o.body_force()
+        o.lbm_step()
+        Fo, To = o.forces()
+        o.advance()
+        g.map_particles()
+        g.solve(forced_cycles=info["cycles"] if precision == es.ES_FP64 else -1)
+        g.lbm_step()
+        F, T = g.forces()
+        g.advance()
+    tol = 1e-11 if precision == es.ES_FP64 else 1e-4
+    assert np.linalg.norm(F - Fo) <= tol * np.linalg.norm(Fo)
+    assert np.linalg.norm(T - To) <= tol * max(np.linalg.norm(To), radius * np.linalg.norm(Fo) * 0.1)
+    g.close()
