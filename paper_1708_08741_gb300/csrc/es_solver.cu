@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(kRedThreads) k_outer_residual(Grid g, Solver s
                                                                 const int* __restrict__ kind,
                                                                 double* __restrict__ r_out,
                                                                 double* __restrict__ partial) {
+    pdl_wait();
     __shared__ double sh[32];
     double acc = 0.0;
     const int nx = g.nx, ny = g.ny, nxy = g.nx * g.ny;
@@ -355,6 +356,7 @@ __global__ void __launch_bounds__(256) k_outer_residual_near_ff(Grid g, ff diag0
                                                                 const int* __restrict__ list,
                                                                 const int* __restrict__ count, int cap,
                                                                 float* __restrict__ r_out, M m) {
+    pdl_wait();
     // blockIdx.y: list segment
     const int n = count[blockIdx.y];
     const int* seg = list + (size_t)blockIdx.y * cap;
@@ -404,6 +406,7 @@ __global__ void __launch_bounds__(256, 2) k_outer_residual_ff(Grid g, ff diag0, 
                                                            double* __restrict__ partial, int zc, Tile tl,
                                                            const int* __restrict__ gate) {
     static_assert(!SPLIT || W == 4, "the split store takes 4-cell spans");
+    pdl_wait();
     if (gate && *gate == 0) return;  // (uniform over the grid: the patched residual runs instead)
     __shared__ float swarp[8];
     const int half = (int)(g.N >> 1);
@@ -539,12 +542,39 @@ __global__ void __launch_bounds__(256, 2) k_outer_residual_ff(Grid g, ff diag0, 
     }
 }
 
-__global__ void k_finalize_norm(const double* partial, int n, double* out) {
+// Where a residual norm goes: to the device and, with the status word, into
+// pinned host memory, which the host reads once the stream has drained (two
+// copies less on the way to the host).
+struct NormOut {
+    double* norm;
+    double* h_norm;
+    const int* status;
+    int* h_status;
+    int *moved, *flips;  // cleared for the next mapping (or null)
+    __device__ __forceinline__ void put(double v) const {
+        norm[0] = v;
+        if (moved) {
+            *moved = 0;
+            *flips = 0;
+        }
+        *(volatile double*)h_norm = v;
+        *(volatile int*)h_status = *(const volatile int*)status;
+        __threadfence_system();
+    }
+};
+
+NormOut norm_out(const es_ctx* c, bool clear) {
+    return NormOut{c->d_norm, c->h_norm, c->d_status, c->h_status, clear ? c->d_moved : nullptr,
+                   clear ? c->flip_count : nullptr};
+}
+
+__global__ void __launch_bounds__(1024) k_finalize_norm(const double* partial, int n, NormOut out) {
     __shared__ double sh[32];
+    pdl_wait();
     double v = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) v += partial[i];
     double tot = block_sum(v, sh);
-    if (threadIdx.x == 0) out[0] = sqrt(tot);
+    if (threadIdx.x == 0) out.put(sqrt(tot));
 }
 
 template <class T>
@@ -2233,6 +2263,7 @@ __global__ void __launch_bounds__(256, 2) k_residual_update_rb(Level<float> L, f
                                                                const float* __restrict__ near_res, int half,
                                                                double* __restrict__ partial, int zc, Tile tl,
                                                                float* __restrict__ psi_hi, float* __restrict__ psi_lo) {
+    pdl_wait();
     __shared__ float swarp[8];
     const int nx = L.nx, ny = L.ny, nz = L.nz, nxh = nx >> 1;
     int X0, y;
@@ -2708,6 +2739,7 @@ __global__ void k_zero(T* p, int n) {
 // psi += e at unknown cells (FP64 form).
 __global__ void k_correct(int N, const uint8_t* __restrict__ st0, const double* __restrict__ e,
                           double* __restrict__ psi) {
+    pdl_wait();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     if ((st0[c] & ST_KIND) != ST_UNKNOWN) return;
@@ -2723,6 +2755,7 @@ template <class E, bool SPLIT = false>
 __global__ void k_correct_ff(int N, const uint8_t* __restrict__ st0, const E* __restrict__ e,
                              float* __restrict__ psi_hi, float* __restrict__ psi_lo, EAcc<float, E> A,
                              int nx = 0, int ny = 0) {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int N4 = N >> 2;
     if (i == N4 - 1 || (N4 == 0 && i == 0))
@@ -2824,6 +2857,7 @@ __global__ void __launch_bounds__(128) k_body_force(Grid g, Solver s, P Ex, P Ey
                                                     const DParticle* __restrict__ part, const int* __restrict__ kind,
                                                     const uint8_t* __restrict__ st0, const float2* __restrict__ pbc,
                                                     WallF wall2, S* __restrict__ fb) {
+    pdl_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= g.nx) return;
@@ -2956,6 +2990,7 @@ __global__ void __launch_bounds__(256) k_body_force_near(Grid g, Solver s, float
                                                          const int* __restrict__ list,
                                                          const int* __restrict__ count, int cap,
                                                          float* __restrict__ fb) {
+    pdl_wait();
     const int n = count[blockIdx.y];
     const int* seg = list + (size_t)blockIdx.y * cap;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -3466,6 +3501,7 @@ __global__ void __launch_bounds__(256) k_flip_patch(Grid g, ff diag0, WallFF wal
                                                     const int* __restrict__ flips, const int* __restrict__ nflips,
                                                     int cap, float* __restrict__ r_out, M m,
                                                     const int* __restrict__ gate) {
+    pdl_wait();
     if (*gate != 0) return;
     const int n = *nflips < cap ? *nflips : cap;
     const int nx = g.nx, ny = g.ny, nz = g.nz;
@@ -3497,6 +3533,7 @@ __global__ void __launch_bounds__(256) k_flip_patch(Grid g, ff diag0, WallFF wal
 // instead.
 __global__ void __launch_bounds__(256) k_rhs_norm_rb(Grid g, const float* __restrict__ r, int zc, Tile tl,
                                                      double* __restrict__ partial, const int* __restrict__ gate) {
+    pdl_wait();
     if (*gate != 0) return;
     __shared__ float swarp[8];
     const int half = (int)(g.N >> 1);
@@ -3536,15 +3573,24 @@ __global__ void __launch_bounds__(256) k_rhs_norm_rb(Grid g, const float* __rest
 // V-cycle: psi += e there, r -= A e there and on the ring one cell further
 // out, and the residual norm is updated by the change of r^2 over those
 // cells.  The V-cycles then start from that residual (none when it is
-// already below the tolerance).  Cells of the region carry bit 7 of their
-// flag byte, ring cells bit 6, while the kernel runs.  Flipped cells closer
-// than 2 kLocalR + 4 cells (Chebyshev, periodic images) form one cluster
-// (k_local_clusters); one block corrects each cluster, and no two clusters'
-// boxes share or touch a cell, so the blocks need no order; the norm takes
-// their changes of r^2 in cluster order (k_local_norm).  gate: 1 when the
-// full residual ran (a sphere moved far or the flip list overflowed); more
-// than kLocalFlips flips leave the V-cycles alone, and a cluster whose
-// region overflows its share of the scratch keeps its residual.
+// already below the tolerance).  Flipped cells closer than 2 kLocalR + 4 cells
+// (Chebyshev, periodic images) form one cluster (the norm's kernel finds
+// them); one block corrects each cluster, and no two clusters' boxes share or
+// touch a cell, so the blocks need no order; the norm takes their changes of
+// r^2 in cluster order (k_local_norm).  gate: 1 when the full residual ran (a
+// sphere moved far or the flip list overflowed); more than kLocalFlips flips
+// leave the V-cycles alone, and a cluster whose region overflows its share of
+// the scratch keeps its residual.
+//
+// A cluster whose box has up to kBoxCells cells (a flip has 19^3 = 6,859; two
+// flips up to six cells apart fit) is solved in shared memory: p with a halo
+// of zeros, x and r for the box, and a code byte a cell, so that a neighbour
+// outside the region needs no test.  The dot products are summed in
+// float-float and the quotients formed in FP32, the precision in which they
+// are used: their FP64 sums and, above all, the FP64 divisions of 1,024
+// threads took the FP64 pipe 20 us of every iteration (a solve's start with
+// its local correction at 512^3: 0.86 ms before, 0.42 ms now; 128^3: 178 us,
+// 80 us).  Larger clusters keep their vectors in global memory.
 constexpr int kLocalR = 8;
 constexpr int kLocalFlips = 16;
 constexpr int kLocalIters = 40;
@@ -3552,11 +3598,12 @@ constexpr int kLocalCap = kLocalFlips * (2 * kLocalR + 3) * (2 * kLocalR + 3) * 
 static_assert(kLocalCap == kLocalCells, "the scratch sized at creation");
 constexpr int kLocalThreads = 1024;
 constexpr int kLocalBox = (2 * kLocalR + 3) * (2 * kLocalR + 3) * (2 * kLocalR + 3);  // scratch cells a flip
+constexpr int kBoxCells = 25 * 25 * 25;
+constexpr size_t kBoxSmem = ((size_t)27 * 27 * 27 + 2 * (size_t)kBoxCells) * 4 + kBoxCells + 64;
 
-// The clusters of the flipped cells, built by one thread: flips in cluster
-// order, the cluster starts, the scratch base of each cluster (kLocalBox
-// cells per flip), the cluster count, and room for each cluster's change of
-// the squared norm.
+// The clusters of the flipped cells: flips in cluster order, the cluster
+// starts, the scratch base of each cluster (kLocalBox cells per flip), the
+// cluster count, and room for each cluster's change of the squared norm.
 struct LocalMeta {
     int n;
     int start[kLocalFlips + 1];
@@ -3567,66 +3614,314 @@ struct LocalMeta {
 
 static_assert(sizeof(LocalMeta) <= 1024, "the cluster table's allocation");
 
-__global__ void k_local_clusters(Grid g, const int* __restrict__ flips, const int* __restrict__ nflips, int fcap,
-                                 const int* __restrict__ gate, LocalMeta* meta) {
-    if (threadIdx.x != 0) return;
+// One warp, a lane a flip; clusters in the order of their first flip, a
+// cluster's flips in list order.
+__device__ void local_clusters(const Grid& g, const int* flips, const int* nflips, int fcap, const int* gate,
+                               LocalMeta* meta) {
+    const int lane = threadIdx.x & 31;
     const int nf = *nflips;
-    meta->n = 0;
+    if (lane == 0) meta->n = 0;
     if (*gate != 0 || nf <= 0 || nf > kLocalFlips || nf > fcap) return;
-    int cl[kLocalFlips];
-    for (int i = 0; i < nf; i++) cl[i] = i;
-    auto root = [&](int i) {
-        while (cl[i] != i) i = cl[i];
-        return i;
+    const int c = lane < nf ? flips[lane] : 0;
+    const int px = c % g.nx, py = (c / g.nx) % g.ny, pz = c / (g.nx * g.ny);
+    unsigned touch = 0;  // the flips within 2 kLocalR + 3 of this lane's
+    auto dist = [](int a, int b, int n, int per) {
+        const int d = abs(a - b);
+        return per && n - d < d ? n - d : d;
     };
-    const int n3[3] = {g.nx, g.ny, g.nz};
-    for (int i = 0; i < nf; i++)
-        for (int j = i + 1; j < nf; j++) {
-            const int a = flips[i], b = flips[j];
-            const int pa[3] = {a % g.nx, (a / g.nx) % g.ny, a / (g.nx * g.ny)};
-            const int pb[3] = {b % g.nx, (b / g.nx) % g.ny, b / (g.nx * g.ny)};
-            int d = 0;
-            for (int k = 0; k < 3; k++) {
-                int dk = abs(pa[k] - pb[k]);
-                if (g.per[k] && n3[k] - dk < dk) dk = n3[k] - dk;
-                d = max(d, dk);
-            }
-            if (d <= 2 * kLocalR + 3) {
-                const int ri = root(i), rj = root(j);
-                if (ri != rj) cl[max(ri, rj)] = min(ri, rj);
-            }
+    for (int j = 0; j < nf; j++) {
+        const int qx = __shfl_sync(0xffffffffu, px, j), qy = __shfl_sync(0xffffffffu, py, j),
+                  qz = __shfl_sync(0xffffffffu, pz, j);
+        if (dist(px, qx, g.nx, g.per[0]) <= 2 * kLocalR + 3 && dist(py, qy, g.ny, g.per[1]) <= 2 * kLocalR + 3 &&
+            dist(pz, qz, g.nz, g.per[2]) <= 2 * kLocalR + 3)
+            touch |= 1u << j;
+    }
+    int label = lane < nf ? lane : 32;
+    for (bool more = true; more;) {
+        int best = label;
+        for (int j = 0; j < nf; j++) {
+            const int lj = __shfl_sync(0xffffffffu, label, j);
+            if (lane < nf && ((touch >> j) & 1u) && lj < best) best = lj;
         }
+        more = __any_sync(0xffffffffu, best != label);
+        label = best;
+    }
     int n = 0, at = 0;
     for (int r = 0; r < nf; r++) {
-        if (root(r) != r) continue;
-        meta->start[n] = at;
-        meta->base[n] = at * kLocalBox;
-        for (int i = 0; i < nf; i++)
-            if (root(i) == r) meta->flip[at++] = flips[i];
-        meta->delta[n] = 0.0;
+        const unsigned m = __ballot_sync(0xffffffffu, label == r);
+        if (!m) continue;
+        if (lane == 0) {
+            meta->start[n] = at;
+            meta->base[n] = at * kLocalBox;
+            meta->delta[n] = 0.0;
+        }
+        if ((m >> lane) & 1u) meta->flip[at + __popc(m & ((1u << lane) - 1u))] = c;
+        at += __popc(m);
         n++;
     }
-    meta->start[n] = at;
-    meta->n = n;
+    if (lane == 0) {
+        meta->start[n] = at;
+        meta->n = n;
+    }
+}
+
+// The norm of a patched residual (k_finalize_norm), and the flips' clusters.
+__global__ void __launch_bounds__(1024) k_finalize_clusters(const double* partial, int n, double* norm, Grid g,
+                                                            const int* flips, const int* nflips, int fcap,
+                                                            const int* gate, LocalMeta* meta) {
+    __shared__ double sh[32];
+    pdl_wait();
+    if (threadIdx.x >= 992) local_clusters(g, flips, nflips, fcap, gate, meta);
+    double v = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) v += partial[i];
+    double tot = block_sum(v, sh);
+    if (threadIdx.x == 0) norm[0] = sqrt(tot);
 }
 
 // The residual norm after the local correction: the clusters' changes of
 // r^2 in cluster order.
-__global__ void k_local_norm(const LocalMeta* __restrict__ meta, double* norm) {
-    if (threadIdx.x != 0 || meta->n == 0) return;
-    double n2 = norm[0] * norm[0];
-    for (int c = 0; c < meta->n; c++) n2 += meta->delta[c];
-    norm[0] = sqrt(n2 > 0.0 ? n2 : 0.0);
+__global__ void k_local_norm(const LocalMeta* __restrict__ meta, NormOut out) {
+    pdl_wait();
+    if (threadIdx.x != 0) return;
+    double v = out.norm[0];
+    if (meta->n > 0) {
+        double n2 = v * v;
+        for (int c = 0; c < meta->n; c++) n2 += meta->delta[c];
+        v = sqrt(n2 > 0.0 ? n2 : 0.0);
+    }
+    out.put(v);
 }
 
-__device__ __forceinline__ double block_sum_all(double v, double* sh) {
-    v = block_sum(v, sh);
+// Sum over the block of one float-float value a thread, to every thread
+// (fixed order).  kLocalThreads threads.
+__device__ __forceinline__ ff block_ff_sum(ff v, float2* sh) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const ff u = {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+        v = ff_add(v, u);
+    }
     __syncthreads();
-    if (threadIdx.x == 0) sh[0] = v;
+    if (lane == 0) sh[wid] = make_float2(v.hi, v.lo);
     __syncthreads();
-    v = sh[0];
-    __syncthreads();
+    const float2 q = sh[lane];
+    v = {q.x, q.y};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const ff u = {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+        v = ff_add(v, u);
+    }
     return v;
+}
+
+// acc += a b, exactly up to the float-float sum
+__device__ __forceinline__ void ff_dot(ff_acc& acc, float a, float b) {
+    const float p = __fmul_rn(a, b);
+    acc.add(p, __fmaf_rn(a, b, -p));
+}
+
+// The box of a cluster that is solved in shared memory: origin (ring
+// included), extents; false when it is too large, or does not fit a periodic
+// axis.
+struct LocalCube {
+    int lo[3], n[3];
+    __device__ bool find(const Level<float>& L, const int* flips, int nf) {
+        const int n3[3] = {L.nx, L.ny, L.nz};
+        const int p0[3] = {flips[0] % L.nx, (flips[0] / L.nx) % L.ny, flips[0] / (L.nx * L.ny)};
+        int mn[3] = {0, 0, 0}, mx[3] = {0, 0, 0};
+        for (int f = 1; f < nf; f++) {
+            const int c = flips[f];
+            const int p[3] = {c % L.nx, (c / L.nx) % L.ny, c / (L.nx * L.ny)};
+#pragma unroll
+            for (int a = 0; a < 3; a++) {
+                int d = p[a] - p0[a];
+                if (L.per[a]) {
+                    if (2 * d > n3[a]) d -= n3[a];
+                    if (2 * d < -n3[a]) d += n3[a];
+                }
+                mn[a] = min(mn[a], d);
+                mx[a] = max(mx[a], d);
+            }
+        }
+        int vol = 1, halo = 1;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            n[a] = mx[a] - mn[a] + 2 * kLocalR + 3;
+            lo[a] = p0[a] + mn[a] - kLocalR - 1;
+            if (n[a] > 64 || (L.per[a] && n[a] > n3[a])) return false;
+            vol *= n[a];
+            halo *= n[a] + 2;
+        }
+        return vol <= kBoxCells && halo <= 27 * 27 * 27;
+    }
+};
+
+// The cluster in its box, in shared memory.  Every thread owns the box cells
+// threadIdx.x + k kLocalThreads throughout.
+__device__ __forceinline__ void local_solve_box(const Level<float>& L, const uint8_t* __restrict__ st,
+                                                const int* flips, int nf, const LocalCube& Q, float* r, float* psi_hi,
+                                                float* psi_lo, int half, float* sm, float2* sh, double* delta) {
+    const RbMap rb{half};
+    const int bx = Q.n[0], by = Q.n[1], bz = Q.n[2], vol = bx * by * bz;
+    const int hx = bx + 2, hxy = hx * (by + 2), hvol = hxy * (bz + 2);
+    float* P = sm;             // with a halo
+    float* X = P + hvol;
+    float* R = X + vol;
+    uint8_t* C = (uint8_t*)(R + vol);  // bit 7 region, bit 6 ring, low bits 6 + diagonal shift
+    const int n3[3] = {L.nx, L.ny, L.nz};
+    const float inv_h2 = 1.0f / L.h2;
+    auto cell = [&](const BoxWalk& w, int (&g)[3]) {
+        const int l[3] = {w.i, w.j, w.k};
+        bool ok = true;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            int v = Q.lo[a] + l[a];
+            if (v < 0 || v >= n3[a]) {
+                if (!L.per[a]) ok = false;
+                v = v < 0 ? v + n3[a] : v - n3[a];
+            }
+            g[a] = v;
+        }
+        return ok;
+    };
+    auto place = [&](const BoxWalk& w) { return (w.i + 1) + hx * (w.j + 1) + hxy * (w.k + 1); };
+    for (int t = threadIdx.x; t < hvol; t += kLocalThreads) P[t] = 0.0f;
+    __syncthreads();
+    BoxWalk w0;
+    w0.start(threadIdx.x, kLocalThreads, bx, by);
+    ff_acc rr_a{0.0f, 0.0f}, old_a{0.0f, 0.0f};
+    {
+        BoxWalk w = w0;
+        for (int t = threadIdx.x; t < vol; t += kLocalThreads, w.next()) {
+            int g[3];
+            unsigned code = 0;
+            float v = 0.0f;
+            if (cell(w, g)) {
+                const int c = g[0] + L.nx * (g[1] + L.ny * g[2]);
+                const uint8_t s = st[c];
+                int dist = 1 << 20;
+                for (int f = 0; f < nf; f++) {
+                    const int cf = flips[f];
+                    const int pf[3] = {cf % L.nx, (cf / L.nx) % L.ny, cf / (L.nx * L.ny)};
+                    int d = 0;
+#pragma unroll
+                    for (int a = 0; a < 3; a++) {
+                        int da = abs(g[a] - pf[a]);
+                        if (L.per[a] && n3[a] - da < da) da = n3[a] - da;
+                        d = max(d, da);
+                    }
+                    dist = min(dist, d);
+                }
+                if ((s & ST_KIND) == ST_UNKNOWN && dist <= kLocalR + 1) {
+                    int shift = 0;
+                    if (s & ST_NEAR) {
+                        int nb[6];
+                        const unsigned fc = near_faces(L, st, g[0], g[1], g[2], nb);
+#pragma unroll
+                        for (int k = 0; k < 6; k++) {
+                            const unsigned f = (fc >> (2 * k)) & 3u;
+                            shift += f == 0u ? 0 : (f == 1u ? 1 : -1);
+                        }
+                    }
+                    code = (dist <= kLocalR ? 0x80u : 0x40u) | (unsigned)(6 + shift);
+                    v = r[rb(c, (g[0] + g[1] + g[2]) & 1)];
+                    ff_dot(old_a, v, v);
+                    if (code & 0x80u) {
+                        P[place(w)] = v;
+                        ff_dot(rr_a, v, v);
+                    }
+                }
+            }
+            C[t] = (uint8_t)code;
+            X[t] = 0.0f;
+            R[t] = v;
+        }
+    }
+    auto apply = [&](int at, unsigned code) {  // (A p) h^2; 0 outside the region counts as no neighbour
+        const float pv = P[at];
+        float off = P[at - 1];
+        off += P[at + 1];
+        off += P[at - hx];
+        off += P[at + hx];
+        off += P[at - hxy];
+        off += P[at + hxy];
+        return (L.diag0 + (float)((int)(code & 15u) - 6)) * pv - off;
+    };
+    ff rr = block_ff_sum(rr_a.value(), sh);
+    const ff old_sq = block_ff_sum(old_a.value(), sh);
+    const float rr0 = rr.hi;
+    for (int it = 0; it < kLocalIters && rr.hi > 1e-6f * rr0 && rr.hi > 0.0f; it++) {
+        ff_acc pq_a{0.0f, 0.0f};
+        {
+            BoxWalk w = w0;
+            for (int t = threadIdx.x; t < vol; t += kLocalThreads, w.next()) {
+                const unsigned code = C[t];
+                if (!(code & 0x80u)) continue;
+                const int at = place(w);
+                ff_dot(pq_a, P[at], apply(at, code) * inv_h2);
+            }
+        }
+        const ff pq = block_ff_sum(pq_a.value(), sh);
+        if (!(pq.hi > 0.0f)) break;  // (uniform)
+        const float alpha = __fdiv_rn(rr.hi, pq.hi);
+        ff_acc rn_a{0.0f, 0.0f};
+        {
+            BoxWalk w = w0;
+            for (int t = threadIdx.x; t < vol; t += kLocalThreads, w.next()) {
+                const unsigned code = C[t];
+                if (!(code & 0x80u)) continue;
+                const int at = place(w);
+                X[t] += alpha * P[at];
+                const float v = R[t] - alpha * (apply(at, code) * inv_h2);
+                R[t] = v;
+                ff_dot(rn_a, v, v);
+            }
+        }
+        const ff rn = block_ff_sum(rn_a.value(), sh);  // (also: every thread is done reading p)
+        const float beta = __fdiv_rn(rn.hi, rr.hi);
+        {
+            BoxWalk w = w0;
+            for (int t = threadIdx.x; t < vol; t += kLocalThreads, w.next())
+                if (C[t] & 0x80u) {
+                    const int at = place(w);
+                    P[at] = R[t] + beta * P[at];
+                }
+        }
+        __syncthreads();
+        rr = rn;
+    }
+    // psi += e on the region; r -= A e on the region and the ring, with e in p's place
+    {
+        BoxWalk w = w0;
+        for (int t = threadIdx.x; t < vol; t += kLocalThreads, w.next())
+            if (C[t] & 0x80u) {
+                int g[3];
+                cell(w, g);
+                const int c = g[0] + L.nx * (g[1] + L.ny * g[2]);
+                P[place(w)] = X[t];
+                const ff v = ff_add_f({psi_hi[c], psi_lo[c]}, X[t]);
+                psi_hi[c] = v.hi;
+                psi_lo[c] = v.lo;
+            }
+    }
+    __syncthreads();
+    ff_acc new_a{0.0f, 0.0f};
+    {
+        BoxWalk w = w0;
+        for (int t = threadIdx.x; t < vol; t += kLocalThreads, w.next()) {
+            const unsigned code = C[t];
+            if (!code) continue;
+            int g[3];
+            cell(w, g);
+            float* rp = r + rb(g[0] + L.nx * (g[1] + L.ny * g[2]), (g[0] + g[1] + g[2]) & 1);
+            const float v = *rp - apply(place(w), code) * inv_h2;
+            *rp = v;
+            ff_dot(new_a, v, v);
+        }
+    }
+    const ff new_sq = block_ff_sum(new_a.value(), sh);
+    if (threadIdx.x == 0)
+        *delta = ((double)new_sq.hi + (double)new_sq.lo) - ((double)old_sq.hi + (double)old_sq.lo);
 }
 
 // Visits the cells of the boxes of radius rb around the flipped cells
@@ -3663,23 +3958,13 @@ __device__ __forceinline__ void local_boxes(const Level<float>& L, const int* fl
     }
 }
 
-__global__ void __launch_bounds__(kLocalThreads) k_local_solve(Level<float> L, const uint8_t* __restrict__ st,
-                                                               uint8_t* flags, LocalMeta* meta, float* r, float* e,
-                                                               float* p, float* psi_hi, float* psi_lo, int* list_all,
-                                                               float* rl_all, float* ec_all, float* q_all,
-                                                               int half) {
-    __shared__ int s_n[2];
-    __shared__ int s_over;
-    __shared__ double sh[32];
-    const int cluster = blockIdx.x;
-    if (cluster >= meta->n) return;  // (uniform over the block)
-    const int f0 = meta->start[cluster], nf = meta->start[cluster + 1] - f0;
-    const int* flips = meta->flip + f0;
+// A larger cluster: cells in a list, vectors in global memory.  Cells of the
+// region carry bit 7 of their flag byte, ring cells bit 6, meanwhile.
+__device__ __noinline__ void local_solve_list(const Level<float>& L, const uint8_t* __restrict__ st, uint8_t* flags,
+                                              const int* flips, int nf, float* r, float* e, float* p, float* psi_hi,
+                                              float* psi_lo, int* list, float* rl, float* ec, float* q, int half,
+                                              int* s_n, int& s_over, float2* sh, double* delta) {
     const int cap = nf * kLocalBox;  // this cluster's share of the scratch
-    int* list = list_all + meta->base[cluster];
-    float* rl = rl_all + meta->base[cluster];
-    float* ec = ec_all + meta->base[cluster];
-    float* q = q_all + meta->base[cluster];
     const RbMap rb{half};
     const int nx = L.nx, ny = L.ny;
     const float inv_h2 = 1.0f / L.h2;
@@ -3719,23 +4004,23 @@ __global__ void __launch_bounds__(kLocalThreads) k_local_solve(Level<float> L, c
             p[rb(cc, cl)] = 0.0f;
         }
         __syncthreads();
-        double rr = 0.0, old_sq = 0.0;
+        ff_acc rr_a{0.0f, 0.0f}, old_a{0.0f, 0.0f};
         for (int i = threadIdx.x; i < nt; i += blockDim.x) {
             const int cc = list[i];
             const float v = r[rb(cc, col(cc))];
-            old_sq += (double)v * v;
+            ff_dot(old_a, v, v);
             if (i < ni) {
                 rl[i] = v;
                 ec[i] = 0.0f;
                 p[rb(cc, col(cc))] = v;
-                rr += (double)v * v;
+                ff_dot(rr_a, v, v);
             }
         }
-        rr = block_sum_all(rr, sh);
-        old_sq = block_sum_all(old_sq, sh);
-        const double rr0 = rr;
-        for (int it = 0; it < kLocalIters && rr > 1e-6 * rr0 && rr > 0.0; it++) {
-            double pq = 0.0;
+        ff rr = block_ff_sum(rr_a.value(), sh);
+        const ff old_sq = block_ff_sum(old_a.value(), sh);
+        const float rr0 = rr.hi;
+        for (int it = 0; it < kLocalIters && rr.hi > 1e-6f * rr0 && rr.hi > 0.0f; it++) {
+            ff_acc pq_a{0.0f, 0.0f};
             for (int i = threadIdx.x; i < ni; i += blockDim.x) {
                 const int cc = list[i];
                 const int x = cc % nx, y = (cc / nx) % ny, z = cc / (nx * ny);
@@ -3745,20 +4030,20 @@ __global__ void __launch_bounds__(kLocalThreads) k_local_solve(Level<float> L, c
                 const float pv = p[rb(cc, col(cc))];
                 const float qv = (dg * pv - off) * inv_h2;
                 q[i] = qv;
-                pq += (double)pv * qv;
+                ff_dot(pq_a, pv, qv);
             }
-            pq = block_sum_all(pq, sh);
-            if (!(pq > 0.0)) break;
-            const double alpha = rr / pq;
-            double rn = 0.0;
+            const ff pq = block_ff_sum(pq_a.value(), sh);
+            if (!(pq.hi > 0.0f)) break;
+            const float alpha = __fdiv_rn(rr.hi, pq.hi);
+            ff_acc rn_a{0.0f, 0.0f};
             for (int i = threadIdx.x; i < ni; i += blockDim.x) {
                 const int cc = list[i];
-                ec[i] += (float)alpha * p[rb(cc, col(cc))];
-                rl[i] -= (float)alpha * q[i];
-                rn += (double)rl[i] * rl[i];
+                ec[i] += alpha * p[rb(cc, col(cc))];
+                rl[i] -= alpha * q[i];
+                ff_dot(rn_a, rl[i], rl[i]);
             }
-            rn = block_sum_all(rn, sh);  // (also: every thread is done reading p)
-            const float beta = (float)(rn / rr);
+            const ff rn = block_ff_sum(rn_a.value(), sh);  // (also: every thread is done reading p)
+            const float beta = __fdiv_rn(rn.hi, rr.hi);
             for (int i = threadIdx.x; i < ni; i += blockDim.x) {
                 const int cc = list[i];
                 float* pp = p + rb(cc, col(cc));
@@ -3778,7 +4063,7 @@ __global__ void __launch_bounds__(kLocalThreads) k_local_solve(Level<float> L, c
         __syncthreads();
         // r -= A e on the region and the ring (e = 0 beyond the region: a
         // neighbour counts only if it carries the region's bit)
-        double new_sq = 0.0;
+        ff_acc new_a{0.0f, 0.0f};
         for (int i = threadIdx.x; i < nt; i += blockDim.x) {
             const int cc = list[i];
             const int x = cc % nx, y = (cc / nx) % ny, z = cc / (nx * ny);
@@ -3806,14 +4091,37 @@ __global__ void __launch_bounds__(kLocalThreads) k_local_solve(Level<float> L, c
             float* rp = r + rb(cc, col(cc));
             const float rv = *rp - (dg * ev - off) * inv_h2;
             *rp = rv;
-            new_sq += (double)rv * rv;
+            ff_dot(new_a, rv, rv);
         }
-        new_sq = block_sum_all(new_sq, sh);
-        if (threadIdx.x == 0) meta->delta[cluster] = new_sq - old_sq;
+        const ff new_sq = block_ff_sum(new_a.value(), sh);
+        if (threadIdx.x == 0)
+            *delta = ((double)new_sq.hi + (double)new_sq.lo) - ((double)old_sq.hi + (double)old_sq.lo);
     }
     __syncthreads();
     // clear the bits (every box cell: also those an overflow left unlisted)
     local_boxes(L, flips, nf, kLocalR + 1, [&](int cc, int) { atomicAnd(word(cc), ~(0xC0u << (8 * (cc & 3)))); });
+}
+
+__global__ void __launch_bounds__(kLocalThreads) k_local_solve(Level<float> L, const uint8_t* __restrict__ st,
+                                                               uint8_t* flags, LocalMeta* meta, float* r, float* e,
+                                                               float* p, float* psi_hi, float* psi_lo, int* list_all,
+                                                               float* rl_all, float* ec_all, float* q_all,
+                                                               int half) {
+    extern __shared__ __align__(16) float lsm[];
+    __shared__ int s_n[2];
+    __shared__ int s_over;
+    __shared__ float2 sh[32];
+    pdl_wait();
+    const int cluster = blockIdx.x;
+    if (cluster >= meta->n) return;  // (uniform over the block)
+    const int f0 = meta->start[cluster], nf = meta->start[cluster + 1] - f0, base = meta->base[cluster];
+    const int* flips = meta->flip + f0;
+    LocalCube Q;
+    if (Q.find(L, flips, nf))
+        local_solve_box(L, st, flips, nf, Q, r, psi_hi, psi_lo, half, lsm, sh, &meta->delta[cluster]);
+    else
+        local_solve_list(L, st, flags, flips, nf, r, e, p, psi_hi, psi_lo, list_all + base, rl_all + base,
+                         ec_all + base, q_all + base, half, s_n, s_over, sh, &meta->delta[cluster]);
 }
 
 }  // namespace
@@ -3861,63 +4169,59 @@ cudaError_t launch_outer_residual(es_ctx* c, bool patch) {
         // patch: the full residual only if the mapping flagged a sphere that
         // moved half a cell or more (the gate), else the patched one
         const int* gate = patch ? c->d_moved : nullptr;
+        const float2* pbc = (const float2*)c->pbc;
+        const float *ph = c->psi32, *pl = c->psi_lo;
+        const uint8_t* st = c->st[0];
+        const int *nl = c->near_list[0], *nc = c->near_count;
+        const int32_t* own = c->owner;
         if (c->rb0) {
             // r goes to the colour-split right-hand side of the finest level
             const RbMap rb{(int)(c->g.N / 2)};
-            k_outer_residual_near_ff<RbMap><<<ngrd, 256, 0, c->stream>>>(
-                c->g, d0, wall, mask, c->psi32, c->psi_lo, c->st[0], c->owner, (const float2*)c->pbc,
-                c->near_list[0], c->near_count, c->near_cap[0], r, rb);
-            k_outer_residual_ff<4, true><<<grd, kTileThreads, 0, c->stream>>>(c->g, d0, c->psi32, c->psi_lo, c->st[0],
-                                                                               r, c->partial, zc, tl, gate);
+            launch_pdl(c, k_outer_residual_near_ff<RbMap>, ngrd, 256, 0, c->g, d0, wall, mask, ph, pl, st, own, pbc, nl,
+                       nc, c->near_cap[0], r, rb);
+            launch_pdl(c, k_outer_residual_ff<4, true>, grd, kTileThreads, 0, c->g, d0, ph, pl, st, r, c->partial, zc,
+                       tl, gate);
             if (patch) {
-                k_flip_patch<RbMap><<<2 * c->n_sm, 256, 0, c->stream>>>(
-                    c->g, d0, wall, mask, c->psi32, c->psi_lo, c->st[0], c->owner, (const float2*)c->pbc,
-                    c->flip_list, c->flip_count, c->flip_cap, r, rb, c->d_moved);
-                k_rhs_norm_rb<<<grd, kTileThreads, 0, c->stream>>>(c->g, r, zc, tl, c->partial, c->d_moved);
+                launch_pdl(c, k_flip_patch<RbMap>, 2 * c->n_sm, 256, 0, c->g, d0, wall, mask, ph, pl, st, own, pbc,
+                           (const int*)c->flip_list, (const int*)c->flip_count, c->flip_cap, r, rb,
+                           (const int*)c->d_moved);
+                launch_pdl(c, k_rhs_norm_rb, grd, kTileThreads, 0, c->g, (const float*)r, zc, tl, c->partial,
+                           (const int*)c->d_moved);
                 count(c, 2);
             }
         } else {
-            k_outer_residual_near_ff<NatMap><<<ngrd, 256, 0, c->stream>>>(
-                c->g, d0, wall, mask, c->psi32, c->psi_lo, c->st[0], c->owner, (const float2*)c->pbc,
-                c->near_list[0], c->near_count, c->near_cap[0], r, NatMap{});
-            if (W == 4)
-                k_outer_residual_ff<4, false><<<grd, kTileThreads, 0, c->stream>>>(
-                    c->g, d0, c->psi32, c->psi_lo, c->st[0], r, c->partial, zc, tl, nullptr);
-            else
-                k_outer_residual_ff<1, false><<<grd, kTileThreads, 0, c->stream>>>(
-                    c->g, d0, c->psi32, c->psi_lo, c->st[0], r, c->partial, zc, tl, nullptr);
+            launch_pdl(c, k_outer_residual_near_ff<NatMap>, ngrd, 256, 0, c->g, d0, wall, mask, ph, pl, st, own, pbc,
+                       nl, nc, c->near_cap[0], r, NatMap{});
+            launch_pdl(c, W == 4 ? k_outer_residual_ff<4, false> : k_outer_residual_ff<1, false>, grd, kTileThreads, 0,
+                       c->g, d0, ph, pl, st, r, c->partial, zc, tl, (const int*)nullptr);
         }
-        k_finalize_norm<<<1, 1024, 0, c->stream>>>(c->partial, gx * gy * gz, c->d_norm);
+        // (the last kernel clears the flag of far moves and the flip list: the
+        // mapping raises and fills them from here on)
         count(c, 3);
         if (patch && c->local_list) {
             // the local correction around the flipped cells (k_local_solve), one block a cluster
             LocalMeta* meta = (LocalMeta*)c->local_meta;
-            k_local_clusters<<<1, 32, 0, c->stream>>>(c->g, c->flip_list, c->flip_count, c->flip_cap, c->d_moved,
-                                                      meta);
-            k_local_solve<<<kLocalFlips, kLocalThreads, 0, c->stream>>>(
-                level_desc<float>(c, 0), c->st[0], c->flags, meta, r, (float*)c->e[0], (float*)c->e2[0],
-                c->psi32, c->psi_lo, c->local_list, c->local_f, c->local_f + kLocalCap, c->local_f + 2 * kLocalCap,
-                (int)(c->g.N / 2));
-            k_local_norm<<<1, 32, 0, c->stream>>>(meta, c->d_norm);
-            count(c, 3);
+            launch_pdl(c, k_finalize_clusters, 1, 1024, 0, (const double*)c->partial, gx * gy * gz, c->d_norm, c->g,
+                       (const int*)c->flip_list, (const int*)c->flip_count, c->flip_cap, (const int*)c->d_moved, meta);
+            cudaError_t err = cudaFuncSetAttribute(k_local_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)kBoxSmem);
+            if (err != cudaSuccess) return err;
+            launch_pdl(c, k_local_solve, kLocalFlips, kLocalThreads, kBoxSmem, level_desc<float>(c, 0), st, c->flags,
+                       meta, r, (float*)c->e[0], (float*)c->e2[0], c->psi32, c->psi_lo, c->local_list, c->local_f,
+                       c->local_f + kLocalCap, c->local_f + 2 * kLocalCap, (int)(c->g.N / 2));
+            launch_pdl(c, k_local_norm, 1, 32, 0, (const LocalMeta*)meta, norm_out(c, true));
+            count(c, 2);
+        } else {
+            launch_pdl(c, k_finalize_norm, 1, 1024, 0, (const double*)c->partial, gx * gy * gz, norm_out(c, true));
         }
-        // (the mapping raises the flag again when a sphere moves far, and
-        // lists the cells that flip from here on)
-        cudaError_t err = cudaMemsetAsync(c->d_moved, 0, sizeof(int), c->stream);
-        if (err == cudaSuccess) err = cudaMemsetAsync(c->flip_count, 0, sizeof(int), c->stream);
-        if (err != cudaSuccess) return err;
         return cudaGetLastError();
     }
     const double k2 = c->S.kappa * c->S.kappa;
-    if (c->P.phi_t > 0.0)
-        k_outer_residual<true><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            c->g, c->S, diag0, k2, c->P.phi_t, c->dk, c->psi, c->st[0], c->owner, c->part, c->kind,
-            (double*)c->rhs[0], c->partial);
-    else
-        k_outer_residual<false><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            c->g, c->S, diag0, k2, 0.0, nullptr, c->psi, c->st[0], c->owner, c->part, c->kind,
-            (double*)c->rhs[0], c->partial);
-    k_finalize_norm<<<1, 1024, 0, c->stream>>>(c->partial, c->red_blocks, c->d_norm);
+    launch_pdl(c, c->P.phi_t > 0.0 ? k_outer_residual<true> : k_outer_residual<false>, c->red_blocks, kRedThreads, 0,
+               c->g, c->S, diag0, k2, c->P.phi_t, c->dk, (const double*)c->psi, (const uint8_t*)c->st[0],
+               (const int32_t*)c->owner, (const DParticle*)c->part, (const int*)c->kind, (double*)c->rhs[0],
+               c->partial);
+    launch_pdl(c, k_finalize_norm, 1, 1024, 0, (const double*)c->partial, c->red_blocks, norm_out(c, false));
     count(c, 2);
     return cudaGetLastError();
 }
@@ -3987,18 +4291,15 @@ cudaError_t launch_correct(es_ctx* c) {
     if (mixed(c)) {
         const int n4 = (N >> 2) > 0 ? (N >> 2) : 1;
         if (c->P.mg_storage == ES_MG_FP16)
-            k_correct_ff<__half><<<(n4 + 255) / 256, 256, 0, c->stream>>>(
-                N, c->st[0], (const __half*)c->e[0], c->psi32, c->psi_lo,
-                EAcc<float, __half>{c->e_scale, 1.0f / c->e_scale});
-        else if (c->rb0)
-            k_correct_ff<float, true><<<(n4 + 255) / 256, 256, 0, c->stream>>>(
-                N, c->st[0], (const float*)c->e[0], c->psi32, c->psi_lo, EAcc<float, float>{1.0f, 1.0f}, c->g.nx,
-                c->g.ny);
+            launch_pdl(c, k_correct_ff<__half>, (n4 + 255) / 256, 256, 0, N, (const uint8_t*)c->st[0],
+                       (const __half*)c->e[0], c->psi32, c->psi_lo,
+                       EAcc<float, __half>{c->e_scale, 1.0f / c->e_scale}, 0, 0);
         else
-            k_correct_ff<float><<<(n4 + 255) / 256, 256, 0, c->stream>>>(
-                N, c->st[0], (const float*)c->e[0], c->psi32, c->psi_lo, EAcc<float, float>{1.0f, 1.0f});
+            launch_pdl(c, c->rb0 ? k_correct_ff<float, true> : k_correct_ff<float>, (n4 + 255) / 256, 256, 0, N,
+                       (const uint8_t*)c->st[0], (const float*)c->e[0], c->psi32, c->psi_lo,
+                       EAcc<float, float>{1.0f, 1.0f}, c->g.nx, c->g.ny);
     } else {
-        k_correct<<<(N + 255) / 256, 256, 0, c->stream>>>(N, c->st[0], (const double*)c->e[0], c->psi);
+        launch_pdl(c, k_correct, (N + 255) / 256, 256, 0, N, (const uint8_t*)c->st[0], (const double*)c->e[0], c->psi);
     }
     count(c);
     return cudaGetLastError();
@@ -4014,24 +4315,20 @@ cudaError_t launch_residual_update(es_ctx* c, bool correct) {
     ProfScope ps(c, correct ? "residual_update_correct" : "residual_update", -1, (double)N * (correct ? 29.0 : 13.0));
     float* scratch = (float*)c->e2[0];
     const dim3 ngrd(near_grid_x(c), 2 * kNearSegs);
-    k_near_residual<float, float, RbMap><<<ngrd, 256, 0, c->stream>>>(
-        L, c->st[0], (const float*)c->rhs[0], (const float*)c->e[0], c->near_list[0], c->near_count,
-        c->near_cap[0], 1.0f / L.h2, scratch, EAcc<float, float>{1.0f, 1.0f}, RbMap{N / 2});
+    launch_pdl(c, k_near_residual<float, float, RbMap>, ngrd, 256, 0, L, (const uint8_t*)c->st[0],
+               (const float*)c->rhs[0], (const float*)c->e[0], (const int*)c->near_list[0],
+               (const int*)c->near_count, c->near_cap[0], 1.0f / L.h2, scratch, EAcc<float, float>{1.0f, 1.0f},
+               RbMap{N / 2});
     const Tile tl = plane_tile(L.nx / 8, L.ny);
     dim3 grd = tile_grid(tl, L.nx / 8, L.ny, 1);
     const int gx = grd.x, gy = grd.y;
     int gz, zc;
     res_march_grid(c, gx, gy, L.nz, gz, zc);
     grd.z = gz;
-    if (correct)
-        k_residual_update_rb<true><<<grd, kTileThreads, 0, c->stream>>>(
-            L, 1.0f / L.h2, c->st[0], (float*)c->rhs[0], (const float*)c->e[0], scratch, N / 2, c->partial, zc, tl,
-            c->psi32, c->psi_lo);
-    else
-        k_residual_update_rb<false><<<grd, kTileThreads, 0, c->stream>>>(
-            L, 1.0f / L.h2, c->st[0], (float*)c->rhs[0], (const float*)c->e[0], scratch, N / 2, c->partial, zc, tl,
-            nullptr, nullptr);
-    k_finalize_norm<<<1, 1024, 0, c->stream>>>(c->partial, gx * gy * gz, c->d_norm);
+    launch_pdl(c, correct ? k_residual_update_rb<true> : k_residual_update_rb<false>, grd, kTileThreads, 0, L,
+               1.0f / L.h2, (const uint8_t*)c->st[0], (float*)c->rhs[0], (const float*)c->e[0], (const float*)scratch,
+               N / 2, c->partial, zc, tl, correct ? c->psi32 : nullptr, correct ? c->psi_lo : nullptr);
+    launch_pdl(c, k_finalize_norm, 1, 1024, 0, (const double*)c->partial, gx * gy * gz, norm_out(c, false));
     count(c, 3);
     return cudaGetLastError();
 }
@@ -4065,9 +4362,10 @@ cudaError_t launch_body_force_near(es_ctx* c) {
     WallF wall2;
     for (int f = 0; f < 6; f++) wall2.v2[f] = (float)(2.0 * c->S.pot_val[f]);
     ProfScope ps(c, "body_force_near", -1, 0.0);
-    k_body_force_near<<<dim3(near_grid_x(c), kNearSegs), 256, 0, c->stream>>>(
-        g, c->S, (float)E[0], (float)E[1], (float)E[2], (float)k2e, c->psi32, c->owner, c->st[0],
-        (const float2*)c->pbc, wall2, c->bf_list, c->bf_count, c->bf_cap, (float*)c->fb);
+    launch_pdl(c, k_body_force_near, dim3(near_grid_x(c), kNearSegs), 256, 0, g, c->S, (float)E[0], (float)E[1],
+               (float)E[2], (float)k2e, (const float*)c->psi32, (const int32_t*)c->owner, (const uint8_t*)c->st[0],
+               (const float2*)c->pbc, wall2, (const int*)c->bf_list, (const int*)c->bf_count, c->bf_cap,
+               (float*)c->fb);
     count(c);
     return cudaGetLastError();
 }
@@ -4095,15 +4393,15 @@ cudaError_t launch_body_force_full(es_ctx* c) {
     }
     ProfScope ps(c, "body_force", -1, (double)g.N * (s + 1.0 + 3.0 * s));
     if (mixed(c))
-        k_body_force<float, float><<<grd, blk, 0, c->stream>>>(g, c->S, (float)E[0], (float)E[1], (float)E[2],
-                                                               (float)k2e, 0.0f, c->psi32, c->flags, c->owner, c->part,
-                                                               c->kind, c->st[0], (const float2*)c->pbc, wall2,
-                                                               (float*)c->fb);
+        launch_pdl(c, k_body_force<float, float>, grd, blk, 0, g, c->S, (float)E[0], (float)E[1], (float)E[2],
+                   (float)k2e, 0.0f, (const float*)c->psi32, (const uint8_t*)c->flags, (const int32_t*)c->owner,
+                   (const DParticle*)c->part, (const int*)c->kind, (const uint8_t*)c->st[0], (const float2*)c->pbc,
+                   wall2, (float*)c->fb);
     else
-        k_body_force<double, double><<<grd, blk, 0, c->stream>>>(g, c->S, E[0], E[1], E[2], k2e, c->P.phi_t,
-                                                                 c->psi, c->flags,
-                                                                 c->owner, c->part, c->kind, c->st[0], nullptr,
-                                                                 wall2, (double*)c->fb);
+        launch_pdl(c, k_body_force<double, double>, grd, blk, 0, g, c->S, E[0], E[1], E[2], k2e, c->P.phi_t,
+                   (const double*)c->psi, (const uint8_t*)c->flags, (const int32_t*)c->owner,
+                   (const DParticle*)c->part, (const int*)c->kind, (const uint8_t*)c->st[0], (const float2*)nullptr,
+                   wall2, (double*)c->fb);
     count(c);
     return cudaGetLastError();
 }

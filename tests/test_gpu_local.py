@@ -1,0 +1,55 @@
+"""The local correction at a solve's start: clusters solved in shared memory
+(one flip, flips close together) and in global memory (boxes too large, or
+longer than a periodic axis), against a start without it."""
+import numpy as np
+import pytest
+
+import paper_1708_08741_gb300 as es
+from paper_1708_08741_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _spheres(dims, periodic, x, levels):
+    n = len(x)
+    wl = W.Workload(name="local", dims=dims, periodic=periodic, tau=1.0, kappa=0.3, eps=1.0, E_ext=(1e-3, 0.0, 0.0),
+                    levels=levels, res_rf=1e-8, coarse_sweeps=16, max_cycles=200)
+    return W._set_particles(wl, np.array(x, dtype=float), np.full(n, 4.2), np.array([i % 2 for i in range(n)]),
+                            np.ones(n), np.full(n, 1.3))
+
+
+@pytest.mark.parametrize("dims,periodic,x,levels", [
+    ((64, 64, 64), (1, 1, 1), [(31.37, 32.11, 30.83)], 3),
+    ((64, 64, 64), (1, 1, 1), [(1.37, 62.11, 0.83)], 3),                         # across the periodic faces
+    ((64, 48, 56), (1, 0, 0), [(31.37, 6.11, 50.2)], 3),                         # against walls
+    ((64, 64, 64), (1, 1, 1), [(20.37, 32.11, 30.83), (34.1, 30.7, 33.9)], 3),   # a chain of flips
+    ((16, 48, 48), (1, 1, 1), [(7.37, 24.11, 22.83)], 2),                        # the box exceeds the x axis
+])
+def test_local_correction(dims, periodic, x, levels):
+    """Both solves end below 1e-8 of the first residual, so the potentials
+    differ by at most 2e-8 cond(A) < 2e-8 (12 + kappa^2) / kappa^2 = 2.7e-6."""
+    wl = _spheres(dims, periodic, x, levels)
+    sims = [es.Simulation(wl, es.ES_MIXED32, overrides=dict(fast_update_cells=f)) for f in (1, 2 ** 31 - 1)]
+    for s in sims:
+        s.map_particles()
+        s.solve()
+    own = sims[0].field(es.FIELD_OWNER)
+    rng = np.random.Generator(np.random.PCG64(3))
+    flipped = 0
+    for _ in range(6):
+        wl.x = wl.x + rng.uniform(-0.04, 0.04, wl.x.shape)
+        info = []
+        for s in sims:
+            s.set_particles(wl.x, wl.v, wl.w)
+            s.map_particles()
+            info.append(s.solve())
+        new = sims[0].field(es.FIELD_OWNER)
+        flipped += int(((new >= 0) != (own >= 0)).sum())
+        own = new
+        np.testing.assert_array_equal(own, sims[1].field(es.FIELD_OWNER))
+        a, b = (s.field(es.FIELD_PSI) for s in sims)
+        assert np.linalg.norm(a - b) <= 2.7e-6 * np.linalg.norm(b)
+        assert info[0]["r0"] <= info[1]["r0"] * (1 + 1e-3)
+    assert flipped > 0
+    for s in sims:
+        s.close()
