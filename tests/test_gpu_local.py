@@ -44,12 +44,14 @@ def test_local_correction(dims, periodic, x, levels):
             s.map_particles()
             info.append(s.solve())
         new = sims[0].field(es.FIELD_OWNER)
-        flipped += int(((new >= 0) != (own >= 0)).sum())
+        now = int(((new >= 0) != (own >= 0)).sum())
+        flipped += now
         own = new
         np.testing.assert_array_equal(own, sims[1].field(es.FIELD_OWNER))
         a, b = (s.field(es.FIELD_PSI) for s in sims)
         assert np.linalg.norm(a - b) <= 2.7e-6 * np.linalg.norm(b)
-        assert info[0]["r0"] <= info[1]["r0"] * (1 + 1e-3)
+        if now:  # (else each solve starts from its own last residual)
+            assert info[0]["r0"] <= info[1]["r0"] * (1 + 1e-3)
     assert flipped > 0
     for s in sims:
         s.close()
