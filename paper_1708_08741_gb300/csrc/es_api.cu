@@ -376,7 +376,7 @@ int es_create_with_allocator(const es_params* params, const es_particle* parts, 
         c->st[l] = (uint8_t*)A(Nl);
         c->e[l] = A(Nl * (l == 0 && c->P.mg_storage == ES_MG_FP16 ? 2 : s));
         c->e2[l] = A(Nl * s);
-        {
+        if (mixed(c)) {  // (the FP64 kernels read states only)
             const long long rows = (long long)c->ln[l][1] * c->ln[l][2];
             // a segment holds one colour of rows = seg (mod kNearSegs)
             c->near_cap[l] = (int)(((rows + kNearSegs - 1) / kNearSegs) * ((c->ln[l][0] + 1) / 2));
@@ -386,6 +386,7 @@ int es_create_with_allocator(const es_params* params, const es_particle* parts, 
     }
     c->part = (DParticle*)A(np1 * sizeof(DParticle));
     c->partf = mixed(c) ? (float*)A(np1 * 12 * sizeof(float)) : nullptr;
+    c->pbd = mixed(c) ? nullptr : (double*)A(np1 * 8);
     c->pbc = mixed(c) ? (float*)A(np1 * 2 * sizeof(float)) : nullptr;
     c->mapped = (double*)A(np1 * 9 * 8);
     c->kind = (int*)A(np1 * 4);
@@ -459,6 +460,7 @@ int es_create_with_allocator(const es_params* params, const es_particle* parts, 
     if (e == cudaSuccess && c->psi32) e = cudaMemsetAsync(c->psi32, 0, N * 4, c->stream);
     if (e == cudaSuccess && c->psi_lo) e = cudaMemsetAsync(c->psi_lo, 0, N * 4, c->stream);
     if (e == cudaSuccess && c->dk) e = cudaMemsetAsync(c->dk, 0, N * 8, c->stream);
+    if (e == cudaSuccess && c->pbd) e = cudaMemsetAsync(c->pbd, 0, np1 * 8, c->stream);
     if (e == cudaSuccess && c->pbc) e = cudaMemsetAsync(c->pbc, 0, np1 * 2 * sizeof(float), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->fb, 0, 3 * N * s, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->F, 0, np1 * 3 * 8, c->stream);

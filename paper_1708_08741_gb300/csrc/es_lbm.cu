@@ -1424,7 +1424,7 @@ cudaError_t launch_forces(es_ctx* c) {
 // boundary value (2 zeta, or sigma / eps) is split into float-float as the
 // mapping does.
 __global__ void k_set_particles(const double* __restrict__ in, DParticle* part, const int* kind, double eps,
-                                float* pbc, float* __restrict__ pf, int np) {
+                                double* pbd, float* pbc, float* __restrict__ pf, int np) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np) return;
     const double* s = in + 12 * p;
@@ -1439,8 +1439,10 @@ __global__ void k_set_particles(const double* __restrict__ in, DParticle* part, 
     d.zeta = s[9];
     d.q = s[10];
     d.qeff = s[11];
+    const double bv = kind[p] == ES_KIND_ZETA ? 2.0 * d.zeta : d.sigma / eps;
+    if (pbd) pbd[p] = bv;
     if (pbc) {
-        const ff v = ff_from_double(kind[p] == ES_KIND_ZETA ? 2.0 * d.zeta : d.sigma / eps);
+        const ff v = ff_from_double(bv);
         pbc[2 * p] = v.hi;
         pbc[2 * p + 1] = v.lo;
     }
@@ -1448,7 +1450,7 @@ __global__ void k_set_particles(const double* __restrict__ in, DParticle* part, 
 
 cudaError_t launch_set_particles(es_ctx* c) {
     if (c->np == 0) return cudaSuccess;
-    k_set_particles<<<blocks_for(c->np, 128), 128, 0, c->stream>>>(c->pstage, c->part, c->kind, c->S.eps, c->pbc,
+    k_set_particles<<<blocks_for(c->np, 128), 128, 0, c->stream>>>(c->pstage, c->part, c->kind, c->S.eps, c->pbd, c->pbc,
                                                                    c->partf, c->np);
     count(c);
     return cudaGetLastError();

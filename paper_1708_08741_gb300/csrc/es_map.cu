@@ -274,7 +274,7 @@ constexpr int kFlagSide = 32;  // longest row of the bit words, halo included
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 6)
     k_flags(Grid g, DParticle* part, double* mapped, const int* __restrict__ kind, const int32_t* __restrict__ owner,
-            uint8_t* flags, uint8_t* st0, int* nfaces, int all_cells, double eps, float* pbc, int* moved) {
+            uint8_t* flags, uint8_t* st0, int* nfaces, int all_cells, double eps, double* pbd, float* pbc, int* moved) {
     __shared__ unsigned s_solid[kFlagSide * kFlagSide], s_out[kFlagSide * kFlagSide], s_dir[kFlagSide * kFlagSide],
         s_own[kFlagSide * kFlagSide], s_near7[kFlagSide * kFlagSide], s_near19[kFlagSide * kFlagSide];
     __shared__ Box sb;
@@ -400,8 +400,10 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 6)
         // the staircase surface equals the particle charge.
         const double sigma = nf > 0 ? part[p].q / (double)nf : 0.0;
         part[p].sigma = sigma;
+        const double bv = kind[p] == ES_KIND_ZETA ? 2.0 * part[p].zeta : sigma / eps;
+        if (pbd) pbd[p] = bv;
         if (pbc) {
-            const ff v = ff_from_double(kind[p] == ES_KIND_ZETA ? 2.0 * part[p].zeta : sigma / eps);
+            const ff v = ff_from_double(bv);
             pbc[2 * p] = v.hi;
             pbc[2 * p + 1] = v.lo;
         }
@@ -775,19 +777,19 @@ __global__ void __launch_bounds__(256) k_lists_l0(int nx, int ny, int nz, const 
 }  // namespace
 
 // The near-cell list of a level (and level 1's update masks) are made where
-// some kernel reads them: the colour-split levels' half sweeps, the half
-// sweeps of levels above near_list_cells, and the FP64 restriction of levels
-// too large to form those children itself (restrict_inline).
+// some kernel reads them: the colour-split levels' half sweeps, and those of
+// levels above near_list_cells.
 static bool list_needed(const es_ctx* c, int l) {
     if (l >= c->tail_l0) return false;
     if (split_level(c, l)) return true;
     const long long most = c->P.near_list_cells > 0 ? (long long)c->P.near_list_cells : (long long)ES_NEAR_LIST_CELLS;
-    const long long n = (long long)c->ln[l][0] * c->ln[l][1] * c->ln[l][2];
-    return n > most || (!mixed(c) && n > (1 << 18));
+    return (long long)c->ln[l][0] * c->ln[l][1] * c->ln[l][2] > most;
 }
 
 // zero: the counters are not zero yet (no mapping kernel ran before this).
+// The FP64 kernels read states only.
 cudaError_t launch_near_lists(es_ctx* c, bool zero) {
+    if (!mixed(c)) return cudaSuccess;
     if (zero) {
         cudaError_t e = cudaMemsetAsync(c->near_count, 0, 2 * kNearSegs * ES_MAXLEV * sizeof(int), c->stream);
         if (e != cudaSuccess) return e;
@@ -863,7 +865,7 @@ cudaError_t launch_map(es_ctx* c) {
     {
         ProfScope ps(c, "map_flags", -1, 0.0);
         launch_pdl(c, T == 1024 ? k_flags<1024> : k_flags<256>, c->np, T, 0, g, c->part, c->mapped, c->kind, c->owner, c->flags, c->st[0], c->nfaces,
-                   c->mapped_once ? 0 : 1, c->S.eps, c->pbc, c->d_moved);
+                   c->mapped_once ? 0 : 1, c->S.eps, c->pbd, c->pbc, c->d_moved);
         c->mapped_once = true;
     }
     count(c, 4);

@@ -93,102 +93,6 @@ struct Level {
     T diag0;  // 6 + kappa^2 h_l^2
 };
 
-// Fine-level face contribution for the FP64 outer residual: adds the centre
-// adjustment to diag and the boundary value to b, or returns the index of an
-// unknown neighbour (>= 0).
-__device__ __forceinline__ int fine_face(const Grid& g, const Solver& s, const int32_t* owner,
-                                         const DParticle* part, const int* kind, int x, int y, int z, int a,
-                                         int side, double& diag, double& b) {
-    int d[3] = {0, 0, 0};
-    d[a] = side;
-    long long nb;
-    if (!neighbour(g, x, y, z, d[0], d[1], d[2], nb)) {
-        int face = 2 * a + (side > 0 ? 1 : 0);
-        if (s.pot_bc[face] == ES_POT_DIRICHLET) {
-            diag += 1.0;
-            b += 2.0 * s.pot_val[face];
-        } else {
-            diag -= 1.0;
-        }
-        return -1;
-    }
-    int o = owner[nb];
-    if (o < 0) return (int)nb;
-    if (kind[o] == ES_KIND_ZETA) {
-        diag += 1.0;
-        b += 2.0 * part[o].zeta;
-    } else {
-        diag -= 1.0;
-        b += part[o].sigma / s.eps;
-    }
-    return -1;
-}
-
-// r = b - A psi on the unknowns (FP64 form), stored as the V-cycle
-// right-hand side, and per-block partial sums of r^2.  Blocks stride over
-// rows (y, z); threads over x.  PB: the nonlinear Poisson-Boltzmann form
-// (Eq. SPBE): the screening term kappa^2 psi of A psi becomes
-// kappa^2 phi_t sinh(psi / phi_t), and the kernel also leaves the shift of
-// the stencil's centre entry linearised about psi, kappa^2 (cosh(psi /
-// phi_t) - 1), for the sweeps of this iteration (Sec. 5.3: the stencils are
-// re-set at the start of every iteration).
-template <bool PB>
-__global__ void __launch_bounds__(kRedThreads) k_outer_residual(Grid g, Solver s, double diag0, double k2,
-                                                                double phi_t, double* __restrict__ dk,
-                                                                const double* __restrict__ psi,
-                                                                const uint8_t* __restrict__ st0,
-                                                                const int32_t* __restrict__ owner,
-                                                                const DParticle* __restrict__ part,
-                                                                const int* __restrict__ kind,
-                                                                double* __restrict__ r_out,
-                                                                double* __restrict__ partial) {
-    pdl_wait();
-    __shared__ double sh[32];
-    double acc = 0.0;
-    const int nx = g.nx, ny = g.ny, nxy = g.nx * g.ny;
-    const int rows = g.ny * g.nz;
-    for (int row = blockIdx.x; row < rows; row += gridDim.x) {
-        const int y = row % ny, z = row / ny;
-        const int base = row * nx;
-        const int ym = (y == 0 ? ny - 1 : y - 1) - y, yp = (y == ny - 1 ? 0 : y + 1) - y;
-        const int zm = (z == 0 ? g.nz - 1 : z - 1) - z, zp = (z == g.nz - 1 ? 0 : z + 1) - z;
-        for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-            const int c = base + x;
-            const uint8_t st = st0[c];
-            double r = 0.0;
-            if ((st & ST_KIND) == ST_UNKNOWN) {
-                if (!(st & ST_NEAR)) {
-                    const int xm = (x == 0 ? nx - 1 : x - 1) - x, xp = (x == nx - 1 ? 0 : x + 1) - x;
-                    double off = psi[c + xm];
-                    off += psi[c + xp];
-                    off += psi[c + ym * nx];
-                    off += psi[c + yp * nx];
-                    off += psi[c + zm * nxy];
-                    off += psi[c + zp * nxy];
-                    r = off - diag0 * psi[c];
-                } else {
-                    double diag = diag0, b = 0.0, off = 0.0;
-                    for (int a = 0; a < 3; a++)
-                        for (int side = -1; side <= 1; side += 2) {
-                            int nb = fine_face(g, s, owner, part, kind, x, y, z, a, side, diag, b);
-                            if (nb >= 0) off += psi[nb];
-                        }
-                    r = b - (diag * psi[c] - off);
-                }
-                if constexpr (PB) {
-                    const double pc = psi[c], u = pc / phi_t;
-                    r += k2 * pc - k2 * phi_t * sinh(u);
-                    dk[c] = k2 * (cosh(u) - 1.0);
-                }
-                acc += r * r;
-            }
-            r_out[c] = r;
-        }
-    }
-    double tot = block_sum(acc, sh);
-    if (threadIdx.x == 0) partial[blockIdx.x] = tot;
-}
-
 // Stores natural cells c .. c+3 (c % 4 == 0, cell c of colour col) of a
 // float field in the colour-split layout (cells c, c+2 of colour col sit at
 // c/2, c/2+1 of half col; cells c+1, c+3 at the same places of the other).
@@ -1787,6 +1691,252 @@ __global__ void __launch_bounds__(32 * (kRbRows + 1), sizeof(T) == 4 ? 2 : 1) k_
     asm volatile("cp.async.wait_all;\n" ::);
 }
 
+// --- FP64 kernels of the fine levels and the outer residual ---
+//
+// All four (half sweep, restriction, outer residual, body force) are bound by
+// the FP64 pipe, which gives a warp's instruction two lanes a cycle and SM
+// whatever its lanes do, and a division some twenty of them.  So a warp with
+// near-boundary cells runs the same FP64 instructions as any other: the faces
+// that do not enter the sum are replaced by +0 (exact) with integer selects,
+// the diagonal diag0 + k, k = #Dirichlet - #Neumann faces (Sec. 5.4), and its
+// reciprocal come from a table, and only the state bytes of the neighbours
+// are loaded in addition.  One thread has one cell of the colour (or one
+// coarse cell), so that no lane is spent on the other colour.  A half sweep is
+// 7 such instructions a warp (14 us of pipe at 128^3, 110 us at 256^3).
+// Channel of 64 spheres, 128^3, four-cell spans with branches and divisions /
+// so (event times, 3 us of bracket): half sweep 45 / 21 us, 64^3 18 / 8 us,
+// restriction 55 / 23, outer residual 76 / 47, body force 156 / 128, V-cycle
+// 727 / 372 us; 256^3, 512 spheres: V-cycle 2,840 / 1,820 us.
+
+struct DiagTab {
+    double d[13], inv[13];  // diag0 + (k - 6) and its reciprocal
+};
+
+__device__ __forceinline__ int near_shift(unsigned code) {  // #Dirichlet - #Neumann + 6
+    return __popc(code & 0x555u) - __popc(code & 0xAAAu) + 6;
+}
+
+// Sum of the neighbours' values face by face, those of code != 0 left out.
+__device__ __forceinline__ double face_sum(unsigned code, bool any, const double (&v)[6]) {
+    double w[6];
+#pragma unroll
+    for (int k = 0; k < 6; k++) w[k] = v[k];
+    if (any) {
+#pragma unroll
+        for (int k = 0; k < 6; k++)
+            if ((code >> (2 * k)) & 3u) w[k] = 0.0;
+    }
+    double o = w[0];
+#pragma unroll
+    for (int k = 1; k < 6; k++) o += w[k];
+    return o;
+}
+
+// The six neighbours of a cell, every axis wrapped (beyond a wall the cell is
+// a near-boundary cell, and the value is left out).
+__device__ __forceinline__ void wrapped_nb(const Level<double>& L, int x, int y, int z, int (&nb)[6]) {
+    const int nx = L.nx, nxy = L.nx * L.ny;
+    const int c = x + nx * (y + L.ny * z);
+    nb[0] = x == 0 ? c + nx - 1 : c - 1;
+    nb[1] = x == nx - 1 ? c - nx + 1 : c + 1;
+    nb[2] = y == 0 ? c + nxy - nx : c - nx;
+    nb[3] = y == L.ny - 1 ? c - nxy + nx : c + nx;
+    nb[4] = z == 0 ? c + (L.nz - 1) * nxy : c - nxy;
+    nb[5] = z == L.nz - 1 ? c - (L.nz - 1) * nxy : c + nxy;
+}
+
+// One red (colour 0) or black (1) Gauss-Seidel / SOR half sweep: a thread has
+// the pair (2t, 2t+1) of a row and updates its cell of the colour.  first != 0:
+// the iterate starts at zero (neighbours are not read, and everything the
+// sweep does not update is zeroed).  (The neighbours'
+// states loaded in any case, ahead of the wait for the kernel before this
+// one, gave the same times at 32^3 .. 256^3.)
+__global__ void __launch_bounds__(kTileThreads) k_smooth_d(Level<double> L, const __grid_constant__ DiagTab D,
+                                                           const uint8_t* __restrict__ st,
+                                                           const double* __restrict__ rhs, double* __restrict__ e,
+                                                           int colour, int first, double omega, Tile tl) {
+    int t, y;
+    const int z = blockIdx.z;
+    bool on = tile_at(tl, (L.nx + 1) / 2, L.ny, threadIdx.x, t, y);
+    const int par = (colour + y + z) & 1;
+    const int row = L.nx * (y + L.ny * z);
+    int x = 2 * t + par, xo = 2 * t + 1 - par;
+    const bool other = on && xo < L.nx;
+    if (x >= L.nx) {  // odd extent: the last pair has one cell
+        on = false;
+        x = 2 * t;
+    }
+    const int c = row + x;
+    const unsigned s = st[c];
+    const bool upd = on && (s & ST_KIND) == ST_UNKNOWN;
+    const bool near = upd && (s & ST_NEAR);
+    int nb[6];
+    unsigned code = 0;
+    const bool any = __any_sync(0xffffffffu, near);
+    pdl_wait();
+    const double r = rhs[c];
+    wrapped_nb(L, x, y, z, nb);
+    double v[6], o = 0.0;
+    if (!first) {
+#pragma unroll
+        for (int k = 0; k < 6; k++) v[k] = e[nb[k]];
+    }
+    if (any) {
+        code = near_faces(L, st, x, y, z, nb);
+        code = near ? code : 0u;
+    }
+    if (!first) o = face_sum(code, any, v);
+    double inv = D.inv[6];
+    if (any) inv = D.inv[near_shift(code)];
+    double gs = (L.h2 * r + o) * inv;
+    if (omega != 1.0) gs = first ? omega * gs : (1.0 - omega) * e[c] + omega * gs;
+    if (upd)
+        e[c] = gs;
+    else if (first && on)
+        e[c] = 0.0;
+    if (first && other) e[row + xo] = 0.0;
+}
+
+// Residual at the unknown cells and its restriction, the mean of the 8
+// children (children that are not unknowns contribute 0); one thread per
+// coarse cell.  RED: after a Gauss-Seidel black half sweep the black residuals
+// vanish (they are rounding), so the red children alone are summed.
+template <bool RED>
+__global__ void __launch_bounds__(kTileThreads) k_restrict_d(Level<double> L, const __grid_constant__ DiagTab D,
+                                                             double inv_h2, const uint8_t* __restrict__ st,
+                                                             const double* __restrict__ rhs,
+                                                             const double* __restrict__ e, int cnx, int cny,
+                                                             const uint8_t* __restrict__ cst,
+                                                             double* __restrict__ crhs, Tile tl) {
+    pdl_wait();
+    int i, j;
+    const int k = blockIdx.z;
+    const bool on = tile_at(tl, cnx, cny, threadIdx.x, i, j);
+    double sum = 0.0;
+#pragma unroll
+    for (int dk = 0; dk < 2; dk++)
+#pragma unroll
+        for (int dj = 0; dj < 2; dj++) {
+            double part = 0.0;
+#pragma unroll
+            for (int di = 0; di < 2; di++) {
+                if (RED && ((di + dj + dk) & 1)) continue;
+                const int x = 2 * i + di, y = 2 * j + dj, z = 2 * k + dk;
+                const int c = x + L.nx * (y + L.ny * z);
+                int nb[6];
+                wrapped_nb(L, x, y, z, nb);
+                double v[6];
+#pragma unroll
+                for (int f = 0; f < 6; f++) v[f] = e[nb[f]];
+                const double ec = e[c], r = rhs[c];
+                const unsigned s = st[c];
+                const bool unk = (s & ST_KIND) == ST_UNKNOWN, near = unk && (s & ST_NEAR);
+                const bool any = __any_sync(0xffffffffu, near);
+                unsigned code = 0;
+                if (any) {
+                    code = near_faces(L, st, x, y, z, nb);
+                    code = near ? code : 0u;
+                }
+                const double o = face_sum(code, any, v);
+                const double dg = any ? D.d[near_shift(code)] : L.diag0;
+                double res = r - (dg * ec - o) * inv_h2;
+                if (!unk) res = 0.0;
+                part = (RED || di == 0) ? res : part + res;
+            }
+            sum = (dj | dk) ? sum + part : part;
+        }
+    if (on) {
+        const int C = i + cnx * (j + cny * k);
+        crhs[C] = (cst[C] & ST_KIND) == ST_UNKNOWN ? sum * 0.125 : 0.0;
+    }
+}
+
+// Boundary values 2 v of the Dirichlet walls (0: zero flux).
+struct WallD {
+    double v2[6];
+};
+
+// r = b - A psi on the unknowns, stored as the V-cycle right-hand side, and
+// per-block partial sums of r^2.  A warp takes 32 cells of a row, the blocks
+// stride over them.  pbd: the spheres' boundary values (2 zeta, or sigma /
+// eps).  PB: the nonlinear Poisson-Boltzmann form (Eq. SPBE): the screening
+// term kappa^2 psi of A psi becomes kappa^2 phi_t sinh(psi / phi_t), and the
+// kernel also leaves the shift of the stencil's centre entry linearised about
+// psi, kappa^2 (cosh(psi / phi_t) - 1), for the sweeps of this iteration
+// (Sec. 5.3: the stencils are re-set at the start of every iteration).
+template <bool PB>
+__global__ void __launch_bounds__(kRedThreads) k_outer_residual(Level<double> L, const __grid_constant__ DiagTab D,
+                                                                const __grid_constant__ WallD wall, double k2,
+                                                                double phi_t, double* __restrict__ dk,
+                                                                const double* __restrict__ psi,
+                                                                const uint8_t* __restrict__ st0,
+                                                                const int32_t* __restrict__ owner,
+                                                                const double* __restrict__ pbd,
+                                                                double* __restrict__ r_out,
+                                                                double* __restrict__ partial) {
+    pdl_wait();
+    __shared__ double sh[32];
+    double acc = 0.0;
+    const int nx = L.nx, ny = L.ny;
+    const int chunks = (nx + 31) >> 5, lane = threadIdx.x & 31;
+    const int n = chunks * ny * L.nz;
+    constexpr int kWarps = kRedThreads / 32;
+    for (int w = blockIdx.x * kWarps + (threadIdx.x >> 5); w < n; w += gridDim.x * kWarps) {
+        const int row = w / chunks, z = row / ny, y = row - z * ny;
+        int x = 32 * (w - row * chunks) + lane;
+        const bool on = x < nx;
+        if (!on) x = nx - 1;
+        const int c = row * nx + x;
+        int nb[6];
+        wrapped_nb(L, x, y, z, nb);
+        double v[6];
+#pragma unroll
+        for (int f = 0; f < 6; f++) v[f] = psi[nb[f]];
+        const double pc = psi[c];
+        const unsigned s = st0[c];
+        const bool unk = on && (s & ST_KIND) == ST_UNKNOWN, near = unk && (s & ST_NEAR);
+        const bool any = __any_sync(0xffffffffu, near);
+        unsigned code = 0;
+        if (any) {
+            code = near_faces(L, st0, x, y, z, nb);
+            code = near ? code : 0u;
+        }
+        const double o = face_sum(code, any, v);
+        double r;
+        if (any) {
+            double bv[6];
+#pragma unroll
+            for (int f = 0; f < 6; f++) {
+                const int a = f >> 1, q = a == 0 ? x : (a == 1 ? y : z);
+                const int edge = (f & 1) ? (a == 0 ? nx : (a == 1 ? ny : L.nz)) - 1 : 0;
+                const bool bd = (code >> (2 * f)) & 3u;
+                if (bd && !(q == edge && !L.per[a]))
+                    bv[f] = pbd[owner[nb[f]]];
+                else
+                    bv[f] = bd ? wall.v2[f] : 0.0;
+            }
+            double b = bv[0];
+#pragma unroll
+            for (int f = 1; f < 6; f++) b += bv[f];
+            r = b - (D.d[near_shift(code)] * pc - o);
+        } else {
+            r = o - L.diag0 * pc;
+        }
+        if constexpr (PB) {
+            if (unk) {
+                const double u = pc / phi_t;
+                r += k2 * pc - k2 * phi_t * sinh(u);
+                dk[c] = k2 * (cosh(u) - 1.0);
+            }
+        }
+        if (!unk) r = 0.0;
+        acc += r * r;
+        if (on) r_out[c] = r;
+    }
+    const double tot = block_sum(acc, sh);
+    if (threadIdx.x == 0) partial[blockIdx.x] = tot;
+}
+
 // Residual of level l at its unknown cells, restricted to level l+1 as the
 // mean of the 8 children (children that are not unknowns contribute 0).
 template <class T>
@@ -1977,8 +2127,8 @@ __global__ void __launch_bounds__(256) k_near_residual(Level<T> L, const uint8_t
 // (dk, dj, di) of the scalar kernel.
 // SPLIT: e and rhs of this level in the colour-split layout (float).
 // INLINE_NEAR: near-boundary children load their neighbours' state bytes
-// here; else they come from k_near_residual, run just before (see
-// restrict_inline).
+// here; else they come from k_near_residual, run just before (levels above
+// near_list_cells).
 template <class T, class E, bool INLINE_NEAR, bool SPLIT = false>
 __global__ void __launch_bounds__(256) k_restrict_v(Level<T> L, T inv_diag0, T inv_h2, const uint8_t* __restrict__ st,
                                                     const T* __restrict__ rhs, const E* __restrict__ e,
@@ -2805,27 +2955,10 @@ __global__ void k_join_psi(int N, const float* __restrict__ hi, const float* __r
 
 // --- EDL field and body force (Sec. 5.6) ---
 
-// Value across face (a, side) of unknown cell c for a D3Q7 central
-// difference: neighbour value, or the boundary value extrapolated from the
-// cell (Dirichlet: 2 v - psi_c; Neumann: psi_c + sigma/eps; wall: psi_c).
-template <class P>
-__device__ __forceinline__ P face_value(const Grid& g, const Solver& s, const P* psi, const int32_t* owner,
-                                        const DParticle* part, const int* kind, int x, int y, int z, P pc, int a,
-                                        int side) {
-    int d[3] = {0, 0, 0};
-    d[a] = side;
-    long long nb;
-    if (!neighbour(g, x, y, z, d[0], d[1], d[2], nb)) {
-        int face = 2 * a + (side > 0 ? 1 : 0);
-        return s.pot_bc[face] == ES_POT_DIRICHLET ? (P)(2.0 * s.pot_val[face]) - pc : pc;
-    }
-    int o = owner[nb];
-    if (o < 0) return psi[nb];
-    if (kind[o] == ES_KIND_ZETA) return (P)(2.0 * part[o].zeta) - pc;
-    return pc + (P)(part[o].sigma / s.eps);
-}
-
-// The same ghost values in FP32 for the reduced forms: the sphere's
+// Ghost values for the D3Q7 central difference at an unknown cell next to a
+// boundary, FP32, for the reduced forms: neighbour value, or the boundary
+// value extrapolated from the cell (Dirichlet: 2 v - psi_c; Neumann: psi_c +
+// sigma / eps; zero-flux wall: psi_c): the sphere's
 // boundary value (2 zeta or sigma / eps) comes from its float-float record
 // (high part), a Dirichlet wall's 2 * value from wall2.
 struct WallF {
@@ -2848,15 +2981,15 @@ __device__ __forceinline__ float face_value_f(const Grid& g, const Solver& s, co
 }
 
 // f_b = rho_e (E_ext - grad psi), rho_e = -kappa^2 eps psi (Eq. ChrgDensDHA),
-// computed in the type P of the potential it reads (double, or the float
-// high part of psi in the reduced forms) and stored in the type S of f_b.
-template <class S, class P>
-__global__ void __launch_bounds__(128) k_body_force(Grid g, Solver s, P Ex, P Ey, P Ez, P k2e, P phi_t,
-                                                    const P* __restrict__ psi, const uint8_t* __restrict__ flags,
-                                                    const int32_t* __restrict__ owner,
-                                                    const DParticle* __restrict__ part, const int* __restrict__ kind,
-                                                    const uint8_t* __restrict__ st0, const float2* __restrict__ pbc,
-                                                    WallF wall2, S* __restrict__ fb) {
+// reduced forms on rows that are no multiple of four cells, from the float
+// high part of psi.
+__global__ void __launch_bounds__(128) k_body_force_f(Grid g, Solver s, float Ex, float Ey, float Ez, float k2e,
+                                                      const float* __restrict__ psi,
+                                                      const uint8_t* __restrict__ flags,
+                                                      const int32_t* __restrict__ owner,
+                                                      const uint8_t* __restrict__ st0,
+                                                      const float2* __restrict__ pbc, WallF wall2,
+                                                      float* __restrict__ fb) {
     pdl_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -2864,57 +2997,114 @@ __global__ void __launch_bounds__(128) k_body_force(Grid g, Solver s, P Ex, P Ey
     const int nx = g.nx, nxy = g.nx * g.ny;
     const int c = x + nx * (y + g.ny * z);
     const uint8_t fl = flags[c];
-    P f0 = (P)0, f1 = (P)0, f2 = (P)0;
+    float f0 = 0.0f, f1 = 0.0f, f2 = 0.0f;
     if (!(fl & F_SOLID)) {
-        const P pc = psi[c];
-        P g0, g1, g2;
+        const float pc = psi[c];
+        float g0 = 0.0f, g1 = 0.0f, g2 = 0.0f;
         if (!(fl & F_NEAR19)) {
             // isotropic D3Q19 gradient (1/c_s^2) sum_q w_q psi(x + e_q) e_q,
             // taken pairwise: 3 w_q (psi(x + e_q) - psi(x - e_q)) e_q
             const int dx[3] = {(x == 0 ? nx - 1 : x - 1) - x, 0, (x == nx - 1 ? 0 : x + 1) - x};
             const int dy[3] = {((y == 0 ? g.ny - 1 : y - 1) - y) * nx, 0, ((y == g.ny - 1 ? 0 : y + 1) - y) * nx};
             const int dz[3] = {((z == 0 ? g.nz - 1 : z - 1) - z) * nxy, 0, ((z == g.nz - 1 ? 0 : z + 1) - z) * nxy};
-            g0 = (P)0;
-            g1 = (P)0;
-            g2 = (P)0;
 #pragma unroll
             for (int q = 1; q <= 9; q++) {
                 const int op = dx[1 + cx(q)] + dy[1 + cy(q)] + dz[1 + cz(q)];
                 const int om = dx[1 - cx(q)] + dy[1 - cy(q)] + dz[1 - cz(q)];
-                const P d = (P)(3.0 * wq(q)) * (psi[c + op] - psi[c + om]);
+                const float d = (float)(3.0 * wq(q)) * (psi[c + op] - psi[c + om]);
                 if (cx(q)) g0 += cx(q) > 0 ? d : -d;
                 if (cy(q)) g1 += cy(q) > 0 ? d : -d;
                 if (cz(q)) g2 += cz(q) > 0 ? d : -d;
             }
-        } else if constexpr (sizeof(P) == 4) {
+        } else {
             g0 = 0.5f * (face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 0, 1) -
                          face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 0, -1));
             g1 = 0.5f * (face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 1, 1) -
                          face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 1, -1));
             g2 = 0.5f * (face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 2, 1) -
                          face_value_f(g, s, wall2, psi, owner, st0, pbc, x, y, z, pc, 2, -1));
-        } else {
-            g0 = (P)0.5 * (face_value<P>(g, s, psi, owner, part, kind, x, y, z, pc, 0, 1) -
-                           face_value<P>(g, s, psi, owner, part, kind, x, y, z, pc, 0, -1));
-            g1 = (P)0.5 * (face_value<P>(g, s, psi, owner, part, kind, x, y, z, pc, 1, 1) -
-                           face_value<P>(g, s, psi, owner, part, kind, x, y, z, pc, 1, -1));
-            g2 = (P)0.5 * (face_value<P>(g, s, psi, owner, part, kind, x, y, z, pc, 2, 1) -
-                           face_value<P>(g, s, psi, owner, part, kind, x, y, z, pc, 2, -1));
         }
-        // (phi_t > 0: the nonlinear Poisson-Boltzmann charge density)
-        const P rho_e = phi_t > (P)0 ? -k2e * phi_t * sinh(pc / phi_t) : -k2e * pc;
+        const float rho_e = -k2e * pc;
         f0 = rho_e * (Ex - g0);
         f1 = rho_e * (Ey - g1);
         f2 = rho_e * (Ez - g2);
     }
-    fb[c] = (S)f0;
-    fb[(long long)g.N + c] = (S)f1;
-    fb[2LL * g.N + c] = (S)f2;
+    fb[c] = f0;
+    fb[(long long)g.N + c] = f1;
+    fb[2LL * g.N + c] = f2;
+}
+
+// The same in FP64 (see the FP64 kernels above).  Interior fluid cells take
+// the isotropic D3Q19 gradient (1/c_s^2) sum_q w_q psi(x + e_q) e_q as nine
+// differences of opposite neighbours, 1/12 (2 d_axis + sum of four diagonal
+// ones) a component, so 28 FP64 instructions a warp; cells with a non-fluid
+// D3Q19 neighbour the D3Q7 central difference with ghost values, the boundary
+// value extrapolated from the cell (Dirichlet: 2 v - psi_c; Neumann: psi_c +
+// sigma / eps; zero-flux wall: psi_c).
+__global__ void __launch_bounds__(128) k_body_force_d(Level<double> L, double Ex, double Ey, double Ez, double k2e,
+                                                      double phi_t, const double* __restrict__ psi,
+                                                      const uint8_t* __restrict__ flags,
+                                                      const int32_t* __restrict__ owner,
+                                                      const uint8_t* __restrict__ st0,
+                                                      const double* __restrict__ pbd,
+                                                      const __grid_constant__ WallD wall, double* __restrict__ fb,
+                                                      Tile tl) {
+    pdl_wait();
+    int x, y;
+    const int z = blockIdx.z;
+    if (!tile_at(tl, L.nx, L.ny, threadIdx.x, x, y)) return;
+    const int nx = L.nx, ny = L.ny, nz = L.nz, nxy = nx * ny;
+    const int c = x + nx * (y + ny * z);
+    const unsigned fl = flags[c];
+    double f0 = 0.0, f1 = 0.0, f2 = 0.0;
+    if (!(fl & F_SOLID)) {
+        const double pc = psi[c];
+        double d0, d1, d2, scale;  // gradient = scale d
+        if (!(fl & F_NEAR19)) {
+            const int xm = (x == 0 ? nx - 1 : x - 1) - x, xp = (x == nx - 1 ? 0 : x + 1) - x;
+            const int ym = ((y == 0 ? ny - 1 : y - 1) - y) * nx, yp = ((y == ny - 1 ? 0 : y + 1) - y) * nx;
+            const int zm = ((z == 0 ? nz - 1 : z - 1) - z) * nxy, zp = ((z == nz - 1 ? 0 : z + 1) - z) * nxy;
+            const double* p = psi + c;
+            const double ax = p[xp] - p[xm], ay = p[yp] - p[ym], az = p[zp] - p[zm];
+            const double xya = p[xp + yp] - p[xm + ym], xyb = p[xp + ym] - p[xm + yp];
+            const double xza = p[xp + zp] - p[xm + zm], xzb = p[xp + zm] - p[xm + zp];
+            const double yza = p[yp + zp] - p[ym + zm], yzb = p[yp + zm] - p[ym + zp];
+            d0 = 2.0 * ax + ((xya + xyb) + (xza + xzb));
+            d1 = 2.0 * ay + ((xya - xyb) + (yza + yzb));
+            d2 = 2.0 * az + ((xza - xzb) + (yza - yzb));
+            scale = 1.0 / 12.0;
+        } else {
+            int nb[6];
+            const unsigned code = near_faces(L, st0, x, y, z, nb);
+            double v[6];
+#pragma unroll
+            for (int f = 0; f < 6; f++) {
+                const unsigned k = (code >> (2 * f)) & 3u;
+                const int a = f >> 1, q = a == 0 ? x : (a == 1 ? y : z);
+                const int edge = (f & 1) ? (a == 0 ? nx : (a == 1 ? ny : nz)) - 1 : 0;
+                const bool wl = q == edge && !L.per[a];
+                v[f] = k == 0u ? psi[nb[f]] : (wl ? wall.v2[f] : pbd[owner[nb[f]]]);
+                if (k) v[f] += k == (unsigned)ST_DIR ? -pc : pc;
+            }
+            d0 = v[1] - v[0];
+            d1 = v[3] - v[2];
+            d2 = v[5] - v[4];
+            scale = 0.5;
+        }
+        // (phi_t > 0: the nonlinear Poisson-Boltzmann charge density)
+        const double rho_e = phi_t > 0.0 ? -k2e * phi_t * sinh(pc / phi_t) : -k2e * pc;
+        f0 = rho_e * (Ex - scale * d0);
+        f1 = rho_e * (Ey - scale * d1);
+        f2 = rho_e * (Ez - scale * d2);
+    }
+    fb[c] = f0;
+    fb[(long long)L.nx * ny * nz + c] = f1;
+    fb[2LL * L.nx * ny * nz + c] = f2;
 }
 
 // Body force of the reduced forms, 4-cell spans (16-byte loads of the nine
 // rows the D3Q19 gradient touches).  Interior fluid cells take the
-// isotropic gradient (Eq. ElPotGradComp, pairwise as in k_body_force);
+// isotropic gradient (Eq. ElPotGradComp, pairwise as in k_body_force_f);
 // obstacle cells get 0; cells with a non-fluid D3Q19 neighbour are written
 // again right after by k_body_force_near with the D3Q7 ghost-value gradient.
 __global__ void __launch_bounds__(256) k_body_force_v(Grid g, float Ex, float Ey, float Ez, float k2e,
@@ -3046,6 +3236,21 @@ Level<T> level_desc(const es_ctx* c, int l) {
     return L;
 }
 
+DiagTab diag_tab(const Level<double>& L) {
+    DiagTab t;
+    for (int k = 0; k < 13; k++) {
+        t.d[k] = L.diag0 + (k - 6);
+        t.inv[k] = 1.0 / t.d[k];
+    }
+    return t;
+}
+
+WallD wall_values(const es_ctx* c) {
+    WallD w;
+    for (int f = 0; f < 6; f++) w.v2[f] = c->S.pot_bc[f] == ES_POT_DIRICHLET ? 2.0 * c->S.pot_val[f] : 0.0;
+    return w;
+}
+
 // Shared memory of the staged finest-level half sweep (0: not staged).
 size_t bulk_smem_bytes(const es_ctx* c) {
     const int nxh = c->ln[0][0] / 2;
@@ -3074,18 +3279,6 @@ size_t coarse_smem_bytes(const es_ctx* c, size_t tsize) {
 // pass over the near-cell list.
 long long inline_near_cells(const es_ctx* c) {
     return c->P.near_list_cells > 0 ? (long long)c->P.near_list_cells : (long long)ES_NEAR_LIST_CELLS;
-}
-
-// Whether the restriction of a natural level of Nl cells forms its
-// near-boundary children itself (saving the launch of k_near_residual and its
-// serial chain of loads) or takes them from that pass.  FP64: the pass packs
-// those cells into full warps, and a warp costs the FP64 pipe the same
-// whatever its lanes do, so from 2^18 cells on the pass wins (16^3 .. 32^3:
-// 23 -> 18 us inline, 64^3 the same, 128^3 54 -> 68 us).
-template <class T>
-bool restrict_inline(const es_ctx* c, int Nl) {
-    const long long most = inline_near_cells(c);
-    return Nl <= (sizeof(T) == 8 && most > (1 << 18) ? (1 << 18) : most);
 }
 
 // Launch shape of the fused sweep: 128 x 12 output tiles, and the z extent
@@ -3268,7 +3461,17 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
                 return;
             }
         }
-        if (vec) {
+        if constexpr (kNative && std::is_same<T, double>::value) {
+            const Tile pt = plane_tile((L.nx + 1) / 2, L.ny);
+            for (int col = 0; col < 2; col++) {
+                const int fs = first && col == 0;
+                ProfScope ps(c, "smooth_half", l, fs ? b_first : b_half);
+                launch_pdl(c, k_smooth_d, tile_grid(pt, (L.nx + 1) / 2, L.ny, L.nz),
+                           kTileThreads, 0, L, diag_tab(L), st, rhs, e, col, fs, omega, pt);
+            }
+            count(c, 2);
+            return;
+        } else if (vec) {
             const NearWork nwl{st, c->near_list[l], c->near_count + 2 * kNearSegs * l, c->near_cap[l]};
             if (Nl <= inline_near_cells(c)) {
                 {
@@ -3294,7 +3497,7 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
             count(c, 2);
             return;
         }
-        if constexpr (kNative) {
+        if constexpr (kNative && std::is_same<T, float>::value) {
             {
                 ProfScope ps(c, "smooth_half", l, first ? b_first : b_half);
                 launch_pdl(c, k_smooth<T>, half, blk, 0, L, st, rhs, e, 0, first, omega, (const T*)nullptr);
@@ -3352,7 +3555,14 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
     const double b_grid = nl * (es + ts + 1.0) + nc * (ts + 1.0);
     {
         ProfScope ps_r(c, "restrict", l, b_grid);
-        if (vec) {
+        if constexpr (std::is_same<T, double>::value) {
+            const Tile rt = plane_tile(m[0], m[1]);
+            const bool red = c->P.omega == 1.0 && c->P.nu1 >= 1;
+            launch_pdl(c, red ? k_restrict_d<true> : k_restrict_d<false>, tile_grid(rt, m[0], m[1], m[2]),
+                       kTileThreads, 0, L, diag_tab(L), 1.0 / L.h2, st, rhs, e, m[0], m[1], c->st[l + 1],
+                       (T*)c->rhs[l + 1], rt);
+            count(c);
+        } else if (vec) {
             const Tile rt = plane_tile(m[0] / 2, m[1]);
             const dim3 rgrd = tile_grid(rt, m[0] / 2, m[1], m[2]);
             bool done = false;
@@ -3384,7 +3594,7 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
                 }
             }
             if (!done) {
-                const bool inl = restrict_inline<T>(c, Nl);
+                const bool inl = Nl <= inline_near_cells(c);
                 T* scratch = (T*)c->e2[l];  // (the fused sweep's second iterate; free between sweeps)
                 if (!inl) {
                     launch_pdl(c, k_near_residual<T, E>, dim3(near_grid_x(c), 2 * kNearSegs), 256, 0, L, st, rhs, e,
@@ -4217,9 +4427,10 @@ cudaError_t launch_outer_residual(es_ctx* c, bool patch) {
         return cudaGetLastError();
     }
     const double k2 = c->S.kappa * c->S.kappa;
+    const Level<double> L0 = level_desc<double>(c, 0);
     launch_pdl(c, c->P.phi_t > 0.0 ? k_outer_residual<true> : k_outer_residual<false>, c->red_blocks, kRedThreads, 0,
-               c->g, c->S, diag0, k2, c->P.phi_t, c->dk, (const double*)c->psi, (const uint8_t*)c->st[0],
-               (const int32_t*)c->owner, (const DParticle*)c->part, (const int*)c->kind, (double*)c->rhs[0],
+               L0, diag_tab(L0), wall_values(c), k2, c->P.phi_t, c->dk, (const double*)c->psi,
+               (const uint8_t*)c->st[0], (const int32_t*)c->owner, (const double*)c->pbd, (double*)c->rhs[0],
                c->partial);
     launch_pdl(c, k_finalize_norm, 1, 1024, 0, (const double*)c->partial, c->red_blocks, norm_out(c, false));
     count(c, 2);
@@ -4393,15 +4604,15 @@ cudaError_t launch_body_force_full(es_ctx* c) {
     }
     ProfScope ps(c, "body_force", -1, (double)g.N * (s + 1.0 + 3.0 * s));
     if (mixed(c))
-        launch_pdl(c, k_body_force<float, float>, grd, blk, 0, g, c->S, (float)E[0], (float)E[1], (float)E[2],
-                   (float)k2e, 0.0f, (const float*)c->psi32, (const uint8_t*)c->flags, (const int32_t*)c->owner,
-                   (const DParticle*)c->part, (const int*)c->kind, (const uint8_t*)c->st[0], (const float2*)c->pbc,
-                   wall2, (float*)c->fb);
-    else
-        launch_pdl(c, k_body_force<double, double>, grd, blk, 0, g, c->S, E[0], E[1], E[2], k2e, c->P.phi_t,
-                   (const double*)c->psi, (const uint8_t*)c->flags, (const int32_t*)c->owner,
-                   (const DParticle*)c->part, (const int*)c->kind, (const uint8_t*)c->st[0], (const float2*)nullptr,
-                   wall2, (double*)c->fb);
+        launch_pdl(c, k_body_force_f, grd, blk, 0, g, c->S, (float)E[0], (float)E[1], (float)E[2], (float)k2e,
+                   (const float*)c->psi32, (const uint8_t*)c->flags, (const int32_t*)c->owner,
+                   (const uint8_t*)c->st[0], (const float2*)c->pbc, wall2, (float*)c->fb);
+    else {
+        const Tile tl = plane_tile(g.nx, g.ny, 128);
+        launch_pdl(c, k_body_force_d, tile_grid(tl, g.nx, g.ny, g.nz), 128, 0, level_desc<double>(c, 0), E[0], E[1],
+                   E[2], k2e, c->P.phi_t, (const double*)c->psi, (const uint8_t*)c->flags, (const int32_t*)c->owner,
+                   (const uint8_t*)c->st[0], (const double*)c->pbd, wall_values(c), (double*)c->fb, tl);
+    }
     count(c);
     return cudaGetLastError();
 }
