@@ -35,15 +35,16 @@ constexpr int kRedThreads = 256;
 // shape then leaves up to half of the lanes idle; the shape with the fewest
 // blocks is taken, 32 x 8 where it is as good (512^3).  288 x 576 x 288, with
 // 32 x 8 / so: restriction 154 / 123 us, residual update 412 / 338 us,
-// prolongation 57 / 49 us.  The half sweeps keep 32 x 8: they are bound by
-// the latency of their near-boundary cells, and the fewer blocks cost as much
-// as the full lanes gain (98 / 96 us there, 12.1 / 14.4 us at 96^3).
+// prolongation 57 / 49 us.  The half sweeps of the colour-split levels take it
+// where at least six blocks an SM are left: 288 x 576 x 288, 32 x 8 / 36 x 7:
+// 92 / 84 us; 96^3, with 3 an SM, a V-cycle 150 / 155 us.
 struct Tile {
     int tw, th;
     unsigned inv;  // ceil(2^16 / tw): t / tw = (t inv) >> 16 for t < 256, tw <= 64
 };
 
 constexpr int kTileThreads = 256;
+constexpr Tile kTile32{32, 8, 2048};
 
 Tile plane_tile(int nspan, int nrows, int threads = kTileThreads) {
     Tile best{32, threads / 32, 2048};
@@ -1133,12 +1134,12 @@ template <class T>
 __global__ void __launch_bounds__(256, 4) k_smooth_rb(Level<T> L, T inv_diag0, const uint32_t* __restrict__ mask,
                                                       int wpr, const T* __restrict__ rhs, T* __restrict__ e,
                                                       int colour, int first, T omega, int half, NearWork nw,
-                                                      int zc) {
+                                                      int zc, Tile tl) {
     const int cc0 = near_first(nw, colour);
     pdl_wait();
-    const int i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (y < L.ny && i0 < (L.nx >> 1)) {
+    int span, y;
+    if (tile_at(tl, L.nx >> 3, L.ny, threadIdx.x, span, y)) {
+        const int i0 = 4 * span;
         const int z0 = (int)blockIdx.z * zc;
         const int z1 = z0 + zc < L.nz ? z0 + zc : L.nz;
         const uint32_t* mcol = mask + (size_t)colour * ((size_t)L.ny * L.nz * wpr);
@@ -3396,21 +3397,34 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
             if (split) {
                 // colour-split finest level: interior pass, then the colour's
                 // near-boundary cells from the list
-                // planes per block: up to 16, keeping about eight blocks per
-                // SM in all
-                // rows of at most half a block's width take a narrower, taller
-                // block, as long as every SM still gets about six (128^3,
-                // 16 spans: a V-cycle 272 -> 250 us; at 96^3, where four an
-                // SM would be left, 208 -> 215 us)
-                int bx = 32;
-                while (bx > 8 && L.nx / 8 <= bx / 2 &&
-                       (long long)((L.ny + 512 / bx - 1) / (512 / bx)) * L.nz >= 6LL * c->n_sm)
-                    bx /= 2;
-                const dim3 sblk(bx, 256 / bx);
-                const int gx = (L.nx / 8 + bx - 1) / bx, gy = (L.ny + 256 / bx - 1) / (256 / bx);
-                int zc = (int)((long long)gx * gy * L.nz / (8LL * c->n_sm));
-                zc = zc < 1 ? 1 : (zc > 16 ? 16 : zc);
-                const dim3 sgrd(gx, gy, (L.nz + zc - 1) / zc);
+                Tile tl = plane_tile(L.nx / 8, L.ny);
+                dim3 sgrd = tile_grid(tl, L.nx / 8, L.ny, 1);
+                if ((long long)sgrd.x * sgrd.y * L.nz < 6LL * c->n_sm) {
+                    tl = kTile32;
+                    sgrd = tile_grid(tl, L.nx / 8, L.ny, 1);
+                }
+                // planes per block: one, while that makes no more than 24
+                // blocks an SM; else the count of 3 to 16 whose blocks fill
+                // whole waves of the four that an SM holds best, each paying
+                // two planes of start-up (288 x 576 x 288: 16 planes 84 us a
+                // half sweep, 10 planes, 3.96 waves, 73; 256^3: 6 and 14
+                // planes 26.0 / 24.2; on 128^3 and less, where a plane is
+                // enough, several planes 8.9 -> 9.9 us)
+                int zc = (int)((long long)sgrd.x * sgrd.y * L.nz / (8LL * c->n_sm));
+                if (zc >= 3) {
+                    const long long cap = 4LL * c->n_sm;
+                    double best = 1e300;
+                    for (int zq = 3; zq <= 16 && zq <= L.nz; zq++) {
+                        const long long nb = (long long)sgrd.x * sgrd.y * ((L.nz + zq - 1) / zq);
+                        const double cost = (double)((nb + cap - 1) / cap) * (zq + 2);
+                        if (cost < best - 1e-9) {
+                            best = cost;
+                            zc = zq;
+                        }
+                    }
+                }
+                zc = zc < 1 ? 1 : zc;
+                sgrd.z = (L.nz + zc - 1) / zc;
                 const int* cnt = c->near_count + 2 * kNearSegs * l;
                 // per cell: the other colour's e in, the colour's e out, its
                 // rhs in (from zero: rhs in, e out), the mask bits; the
@@ -3454,8 +3468,8 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
                         launch_pdl(c, k_smooth_rb_bulk<T>, bgrd, 256, bsm, L, inv_diag0, rbmask, rb_wpr, rhs, e, col,
                                    fs, omega, rb.half, nw, bs, c->d_status);
                     else
-                        launch_pdl(c, k_smooth_rb<T>, sgrd, sblk, 0, L, inv_diag0, rbmask, rb_wpr, rhs, e, col, fs,
-                                   omega, rb.half, nw, zc);
+                        launch_pdl(c, k_smooth_rb<T>, sgrd, kTileThreads, 0, L, inv_diag0, rbmask, rb_wpr, rhs, e, col, fs,
+                                   omega, rb.half, nw, zc, tl);
                 }
                 count(c, 2);
                 return;
