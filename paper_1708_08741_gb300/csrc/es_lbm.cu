@@ -359,7 +359,6 @@ __device__ __forceinline__ void lbm_cell(const Grid& g, const Streams<S>& P, con
             }
             // moving bounce-back (Eq. LBMMovWall): the population sent from x
             // towards the surface cell returns with 2 w_q rho_0 (c_q . u_s)/c_s^2
-            f[q] = St::ld(opp(q), P.src[opp(q)][c]);
             if constexpr (sizeof(C) == 4) {
                 // FP32 form: lever arm from the float copy of the particle
                 const float* pf = partf + 12 * o;
@@ -376,8 +375,9 @@ __device__ __forceinline__ void lbm_cell(const Grid& g, const Streams<S>& P, con
                 const float u1 = pf[4] + (pf[8] * r[0] - pf[6] * r[2]);
                 const float u2 = pf[5] + (pf[6] * r[1] - pf[7] * r[0]);
                 const float cu = (float)cx(q) * u0 + (float)cy(q) * u1 + (float)cz(q) * u2;
-                f[q] += (float)(6.0 * wq(q)) * cu;
+                f[q] = St::ld(opp(q), P.src[opp(q)][c]) + (float)(6.0 * wq(q)) * cu;
             } else {
+                f[q] = St::ld(opp(q), P.src[opp(q)][c]);
                 many = many || (hit != 0u && o != o1);
                 if (hit == 0u) {
                     o1 = o;
