@@ -23,12 +23,16 @@
 //
 // What bounds it: a half sweep is one cluster barrier (480 cycles with its
 // release fence, whatever the cluster's size), one distributed-shared-memory
-// read (264 cycles) and the arithmetic (FP64: six 64-cycle operations in a
-// row).  Measured per half sweep, 16 blocks: FP32 0.16 us (16^3, one block,
-// no cluster barrier), 0.6 us (32^3), 2.3 us (64^3); FP64 0.9 us (16^3), 2.7 us
-// (32^3); a launch of its own took 2.7 to 5 us.  V-cycle with its correction and
-// residual, before / now: FP32 128^3 250 / 189 us, 96^3 208 / 168, 256^3
-// 526 / 507, 32^3 134 / 85; FP64 32^3 202 / 143, 128^3 1117 / 741 us.
+// read (264 cycles) and the arithmetic (FP64: four 64-cycle operations in a
+// row, and on 32^3 the FP64 pipe: six or seven instructions a warp at 17
+// cycles each).  Measured per half sweep, 16 blocks: FP32 0.16 us (16^3, one
+// block, no cluster barrier), 0.6 us (32^3), 2.3 us (64^3); FP64 0.84 us (16^3),
+// 2.6 us (32^3); a launch of its own took 2.7 to 5 us.  V-cycle with its
+// correction and residual, every level launched / with it: FP32 128^3 250 /
+// 170 us, 96^3 208 / 150, 256^3 526 / 485, 32^3 134 / 64; FP64 32^3 202 / 118 us.
+// Boundary planes pushed to the neighbours with an mbarrier each, in place of
+// the cluster barrier, were no faster (FP64 32^3 107 / 111 us a tail, FP32
+// 96^3 150 / 164 a V-cycle): that round trip is as long.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -270,6 +274,10 @@ __device__ __forceinline__ void tail_smooth(const TailLevel<T>& L, const Slab<T>
             r1.v[k] *= h2;
             i0.v[k] = inv[cd0.at(k) >> 12];
             i1.v[k] = inv[cd1.at(k) >> 12];
+            if (W == 1) {  // (FP64: an operation less in each half sweep's chain)
+                r0.v[k] *= i0.v[k];
+                r1.v[k] *= i1.v[k];
+            }
         }
         auto half = [&](const Around<T>& at, const Codes<T>& cd, const Span<T>& r, const Span<T>& id, T* e) {
             if (on) {
@@ -278,7 +286,7 @@ __device__ __forceinline__ void tail_smooth(const TailLevel<T>& L, const Slab<T>
                 if (!gs) c = ldspan(e);
 #pragma unroll
                 for (int k = 0; k < W; k++) {
-                    const T g = (r.v[k] + o.v[k]) * id.v[k];
+                    const T g = W == 1 ? o.v[k] * id.v[k] + r.v[k] : (r.v[k] + o.v[k]) * id.v[k];
                     c.v[k] = gs ? g : keep * c.v[k] + omega * g;
                 }
                 stspan(e, c);
@@ -685,7 +693,7 @@ cudaError_t tail_run(es_ctx* c, int warm) {
     A.nu2 = c->P.nu2;
     A.sweeps = c->P.coarse_sweeps;
     A.omega = (T)c->P.omega;
-    A.red_only = std::is_same<T, float>::value && c->P.omega == 1.0 && c->P.nu1 >= 1;
+    A.red_only = c->P.omega == 1.0 && c->P.nu1 >= 1;
     A.solo = p.solo;
     A.status = c->d_status;
     double cells = 0.0;
