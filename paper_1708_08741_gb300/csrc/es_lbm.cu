@@ -730,9 +730,14 @@ __device__ __forceinline__ int force_cells_fields(const Grid& g, const int32_t* 
 // FP64 form.  The FP64 pipe (2 operations a clock and SM) bounds it, so a
 // cell's links share what they can: u_s . c_q = u_F . c_q with u_F = V + W x
 // r_F, since x_s = x_F + c_q and (W x c_q) . c_q = 0, and the torques add up to
-// r_F x sum m_q c_q, since c_q x c_q = 0; about five operations a link instead
-// of 35.  (A sphere R = 4 / 64 spheres R = 6: 62 / 133 us before, 32 / 48
-// now.)
+// r_F x sum m_q c_q, since c_q x c_q = 0.  A warp has links along all 18
+// directions, so a cell takes them by pairs without a branch: with b = 1 where
+// there is a link (f = 0 where not), m_q - m_-q = 2 [f_q - f_-q - 3 w_q (b_q +
+// b_-q) u_F . c_q]; 39 instructions for the 18 instead of 78.  The block's sums
+// exchange halves of the six components instead of adding all six at each of
+// five steps (8 instructions a warp, not 30), in the warps that have cells.
+// (A sphere R = 4 / 64 spheres R = 6: 62 / 133 us with a lever arm a link, 32
+// / 48 link by link, 23 / 35 now.)
 template <int T>
 __global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __restrict__ part,
                                                  const int32_t* __restrict__ owner, const uint8_t* __restrict__ flags,
@@ -754,7 +759,10 @@ __global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __rest
     const double X[3] = {P.x[0], P.x[1], P.x[2]}, V[3] = {P.v[0], P.v[1], P.v[2]}, Wv[3] = {P.w[0], P.w[1], P.w[2]};
     const size_t ps = (size_t)g.ps;
     double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    int active = 0;  // warps that have had cells
     auto consume = [&](int total) {
+        const int w = (total + 31) / 32;
+        active = w > active ? (w < T / 32 ? w : T / 32) : active;
         for (int i = threadIdx.x; i < total; i += T) {
             int v[3];
             bi.at(s_near[i], v);
@@ -765,22 +773,22 @@ __global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __rest
             const double r0 = cell_disp(g, 0, x, X[0]), r1 = cell_disp(g, 1, y, X[1]), r2 = cell_disp(g, 2, z, X[2]);
             const double u[3] = {V[0] + (Wv[1] * r2 - Wv[2] * r1), V[1] + (Wv[2] * r0 - Wv[0] * r2),
                                  V[2] + (Wv[0] * r1 - Wv[1] * r0)};
-            double d[3] = {0.0, 0.0, 0.0};
-            // six directions' populations in flight at a time
+            double d[3] = {0.0, 0.0, 0.0};  // half the sum of m_q c_q
+            // three pairs of populations in flight at a time
 #pragma unroll
-            for (int q0 = 1; q0 < 19; q0 += 6) {
-                double f[6];
+            for (int q0 = 1; q0 <= 9; q0 += 3) {
+                double f[3], h[3];
 #pragma unroll
-                for (int j = 0; j < 6; j++) f[j] = ((m >> (q0 + j)) & 1u) ? src[(q0 + j) * ps + c] : 0.0;
+                for (int j = 0; j < 3; j++) {
+                    f[j] = ((m >> (q0 + j)) & 1u) ? src[(q0 + j) * ps + c] : 0.0;
+                    h[j] = ((m >> (q0 + j + 9)) & 1u) ? src[(q0 + j + 9) * ps + c] : 0.0;
+                }
 #pragma unroll
-                for (int j = 0; j < 6; j++) {
+                for (int j = 0; j < 3; j++) {
                     const int q = q0 + j;
-                    if (!((m >> q) & 1u)) continue;
-                    double cu = 0.0;
-                    if (cx(q)) cu = cx(q) > 0 ? u[0] : -u[0];
-                    if (cy(q)) cu = cx(q) ? (cy(q) > 0 ? cu + u[1] : cu - u[1]) : (cy(q) > 0 ? u[1] : -u[1]);
-                    if (cz(q)) cu = cx(q) || cy(q) ? (cz(q) > 0 ? cu + u[2] : cu - u[2]) : (cz(q) > 0 ? u[2] : -u[2]);
-                    const double mq = 2.0 * f[j] - 6.0 * wq(q) * cu;
+                    const unsigned b0 = (m >> q) & 1u, b1 = (m >> (q + 9)) & 1u;
+                    const double k = (b0 & b1) ? -6.0 * wq(q) : ((b0 | b1) ? -3.0 * wq(q) : 0.0);
+                    const double mq = (f[j] - h[j]) + k * dot_c(q, u);
                     if (cx(q)) d[0] += cx(q) > 0 ? mq : -mq;
                     if (cy(q)) d[1] += cy(q) > 0 ? mq : -mq;
                     if (cz(q)) d[2] += cz(q) > 0 ? mq : -mq;
@@ -802,17 +810,37 @@ __global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __rest
             __syncthreads();
         }
     }
-    // block sums in a fixed order: warps, then one thread per component
+    // block sums in a fixed order: the warps that had cells (half a warp keeps
+    // three components, a quarter two of four, ...), then one thread per
+    // component
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid < active) {
+        const bool up = lane & 16, up2 = lane & 8, up3 = lane & 4;
+        double a3[4];
 #pragma unroll
-    for (int k = 0; k < 6; k++) {
-        for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
-        if ((threadIdx.x & 31) == 0) sh[k][threadIdx.x >> 5] = acc[k];
+        for (int k = 0; k < 3; k++) {
+            const double mine = up ? acc[k + 3] : acc[k], other = up ? acc[k] : acc[k + 3];
+            a3[k] = mine + __shfl_xor_sync(0xffffffffu, other, 16);
+        }
+        a3[3] = 0.0;
+        double a2[2];
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const double mine = up2 ? a3[k + 2] : a3[k], other = up2 ? a3[k] : a3[k + 2];
+            a2[k] = mine + __shfl_xor_sync(0xffffffffu, other, 8);
+        }
+        double a1 = (up3 ? a2[1] : a2[0]) + __shfl_xor_sync(0xffffffffu, up3 ? a2[0] : a2[1], 4);
+        a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
+        a1 += __shfl_xor_sync(0xffffffffu, a1, 1);
+        const int k = (up2 ? 2 : 0) + (up3 ? 1 : 0);
+        if ((lane & 3) == 0 && k < 3) sh[(up ? 3 : 0) + k][wid] = a1;
     }
     __syncthreads();
     if (threadIdx.x < 6) {
         const int k = threadIdx.x;
         double s = 0.0;
-        for (int w = 0; w < T / 32; w++) s += sh[k][w];
+        for (int w = 0; w < active; w++) s += sh[k][w];
+        s *= 2.0;
         const double E[3] = {Ex, Ey, Ez};
         if (k < 3)
             F[3 * p + k] = s + P.qeff * E[k];  // F_C = q E_ext (Sec. 5.6)
