@@ -243,6 +243,13 @@ __device__ __forceinline__ double dot_c(int q, const double (&u)[3]) {
     return t;
 }
 
+// The faces (bits as in lbm_cell) beyond which the source x - c_q lies of a
+// cell at all of them.
+__device__ __forceinline__ unsigned crossed(int q) {
+    return (cx(q) > 0 ? 1u : cx(q) < 0 ? 2u : 0u) | (cy(q) > 0 ? 4u : cy(q) < 0 ? 8u : 0u) |
+           (cz(q) > 0 ? 16u : cz(q) < 0 ? 32u : 0u);
+}
+
 // The electric body force evaluated inside the stream-collide (reduced
 // forms): psi (the float potential), E_ext and kappa^2 eps.
 struct FbPsi {
@@ -282,8 +289,17 @@ __device__ __forceinline__ Psi19 load_psi19(const float* __restrict__ p, const i
 // neighbours (body_force_iso, Sec. 5.6), so f_b makes no round trip through
 // HBM: the cell reads 4 bytes of psi (the neighbours' come from cache)
 // instead of 12 of stored f_b.  Cells next to obstacles or walls read the
-// stored field (their D3Q7 ghost-value gradient, k_body_force_near).
-template <class S, bool SLIP, bool FBPSI, bool EARLY, class C = typename Store<S>::C>
+// stored field (their D3Q7 ghost-value gradient, k_body_force_near).  PER:
+// every axis is periodic, so no source lies beyond a wall.  The near cells
+// take a tenth of the kernel at a few per cent of the cells, bound by the
+// instructions of 18 directions: their sources are the wrapped ones of the
+// pull, a wall six bits of the cell against the direction's constant ones
+// (instead of an index test and three wraps a direction), and a sphere's
+// state comes as two 16-byte loads and one more (instead of nine).  Without
+// PER the wall bits cost a register that spills at 48: 512^3 periodic 3.94 ms
+// against 3.79 (3.89 before), 288 x 576 x 288 with walls 1.48 (1.56 before);
+// FP16 256^3 444 -> 413 us, 96^3 55 -> 52 us.
+template <class S, bool SLIP, bool FBPSI, bool EARLY, bool PER, class C = typename Store<S>::C>
 __device__ __forceinline__ void lbm_cell(const Grid& g, const Streams<S>& P, const uint8_t* __restrict__ flags,
                                          const int32_t* __restrict__ owner, const DParticle* __restrict__ part,
                                          const float* __restrict__ partf, const C* __restrict__ fb, C ax, C ay,
@@ -336,14 +352,21 @@ __device__ __forceinline__ void lbm_cell(const Grid& g, const Streams<S>& P, con
         fy = fb[N + c] + ay;
         fz = fb[2u * N + c] + az;
         if constexpr (!EARLY) f[0] = St::ld(0, P.src[0][c]);
+        // the non-periodic faces that the cell lies at, two bits an axis
+        const unsigned wall =
+            PER ? 0u
+                : (g.per[0] ? 0u : (x == 0 ? 1u : 0u) | (x == nx - 1 ? 2u : 0u)) |
+                      (g.per[1] ? 0u : (y == 0 ? 4u : 0u) | (y == g.ny - 1 ? 8u : 0u)) |
+                      (g.per[2] ? 0u : (z == 0 ? 16u : 0u) | (z == g.nz - 1 ? 32u : 0u));
         unsigned hit = 0;  // FP64: directions whose source is an obstacle cell
         int o1 = -1;       // the first one's sphere
         int k0 = 0, k1 = 0, k2 = 0;
         bool many = false;
 #pragma unroll
         for (int q = 1; q < 19; q++) {
-            long long nb;
-            if (!neighbour(g, x, y, z, -cx(q), -cy(q), -cz(q), nb)) {
+            const int nb = c + sx[1 + cx(q)] + sy[1 + cy(q)] + sz[1 + cz(q)];
+            const int o = owner[nb];
+            if (!PER && (wall & crossed(q))) {
                 if constexpr (SLIP) {
                     const WallSrc w = wall_source(g, slip_faces, owner, x, y, z, q, c);
                     f[q] = St::ld(q, P.src[w.q][w.cell]);
@@ -352,7 +375,6 @@ __device__ __forceinline__ void lbm_cell(const Grid& g, const Streams<S>& P, con
                 }
                 continue;
             }
-            const int o = owner[nb];
             if (o < 0) {  // a fluid source: the value pulled above
                 if constexpr (!EARLY) f[q] = St::ld(q, P.src[q][nb]);
                 continue;
@@ -361,13 +383,15 @@ __device__ __forceinline__ void lbm_cell(const Grid& g, const Streams<S>& P, con
             // towards the surface cell returns with 2 w_q rho_0 (c_q . u_s)/c_s^2
             if constexpr (sizeof(C) == 4) {
                 // FP32 form: lever arm from the float copy of the particle
-                const float* pf = partf + 12 * o;
+                const float4* p4 = reinterpret_cast<const float4*>(partf + 12 * o);
+                const float4 pa = p4[0], pb = p4[1];
+                const float pf[9] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w, partf[12 * o + 8]};
                 float r[3] = {(float)x + 0.5f - (float)cx(q) - pf[0], (float)y + 0.5f - (float)cy(q) - pf[1],
                               (float)z + 0.5f - (float)cz(q) - pf[2]};
                 const float Lw[3] = {(float)g.nx, (float)g.ny, (float)g.nz};
 #pragma unroll
                 for (int a = 0; a < 3; a++)
-                    if (g.per[a]) {
+                    if (PER || g.per[a]) {
                         if (r[a] > 0.5f * Lw[a]) r[a] -= Lw[a];
                         if (r[a] < -0.5f * Lw[a]) r[a] += Lw[a];
                     }
@@ -443,7 +467,7 @@ __device__ __forceinline__ void lbm_cell(const Grid& g, const Streams<S>& P, con
 // (the reduced forms cap a thread at 48 registers, 1,280 threads per SM: with
 // the pull loads issued ahead of the flag test, 40 registers spill and 64
 // leave too few threads; both measured slower)
-template <class S, bool SLIP, bool FBPSI = false, class C = typename Store<S>::C>
+template <class S, bool SLIP, bool FBPSI, bool PER, class C = typename Store<S>::C>
 __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 3 : 5) k_lbm(Grid g, const Streams<S> P, const uint8_t* __restrict__ flags,
                                              const int32_t* __restrict__ owner, const DParticle* __restrict__ part,
                                              const float* __restrict__ partf, const C* __restrict__ fb, C ax, C ay,
@@ -452,7 +476,7 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 3 : 5) k_lbm(Grid g, con
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
     if (x >= g.nx || y >= g.ny) return;
-    lbm_cell<S, SLIP, FBPSI, true>(g, P, flags, owner, part, partf, fb, ax, ay, az, R, slip_faces, fp, x, y, z);
+    lbm_cell<S, SLIP, FBPSI, true, PER>(g, P, flags, owner, part, partf, fb, ax, ay, az, R, slip_faces, fp, x, y, z);
 }
 
 // Several resident runs stepped by one persistent launch (es_lbm_step_batch):
@@ -505,12 +529,12 @@ __global__ void __launch_bounds__(kBatchTileX * kBatchTileY, sizeof(S) == 8 ? 6 
         if (x >= R.g.nx || y >= R.g.ny) continue;
         if constexpr (std::is_same<typename Store<S>::C, float>::value) {
             if (R.lazy) {
-                lbm_cell<S, false, true, false>(R.g, R.P, R.flags, R.owner, R.part, R.partf, R.fb, R.ax, R.ay, R.az,
+                lbm_cell<S, false, true, false, false>(R.g, R.P, R.flags, R.owner, R.part, R.partf, R.fb, R.ax, R.ay, R.az,
                                          R.R, 0, R.fp, x, y, z);
                 continue;
             }
         }
-        lbm_cell<S, false, false, false>(R.g, R.P, R.flags, R.owner, R.part, R.partf, R.fb, R.ax, R.ay, R.az, R.R, 0, R.fp, x, y, z);
+        lbm_cell<S, false, false, false, false>(R.g, R.P, R.flags, R.owner, R.part, R.partf, R.fb, R.ax, R.ay, R.az, R.R, 0, R.fp, x, y, z);
     }
 }
 
@@ -1371,8 +1395,11 @@ cudaError_t launch_lbm(es_ctx* c) {
         // algorithmic bytes per cell: 19 populations in and out, f_b (3 C)
         // or psi (4) and the flag byte in
         ProfScope ps(c, "lbm", -1, (double)g.N * (38.0 * sizeof(S) + (lazy ? 4.0 : 3.0 * sizeof(C)) + 1.0));
+        const bool per = g.per[0] && g.per[1] && g.per[2];
         auto run = [&](auto slip, auto fused) {
-            launch_pdl(c, k_lbm<S, decltype(slip)::value, decltype(fused)::value>, grd, blk, 0, g, streams<S>(c),
+            constexpr bool SL = decltype(slip)::value, FB = decltype(fused)::value;
+            auto k = per ? k_lbm<S, false, FB, true> : k_lbm<S, SL, FB, false>;
+            launch_pdl(c, k, grd, blk, 0, g, streams<S>(c),
                        (const uint8_t*)c->flags, (const int32_t*)c->owner, (const DParticle*)c->part,
                        (const float*)c->partf, (const C*)c->fb, (C)a[0], (C)a[1], (C)a[2],
                        trt<C>(c->lambda_e, c->lambda_o), c->slip, fp);
