@@ -442,12 +442,13 @@ def kernel_table(prof, lbm_bytes, peak):
 
 
 # kernels that make up a V-cycle (per level)
-VCYCLE_KERNELS = ("smooth_half", "smooth_near", "smooth_fused", "restrict", "prolong", "coarse_solve")
-# floating-point operations of the stream-collide per interior fluid cell,
-# counted from k_lbm with an FMA as two: moments 45, modified velocity, u.u,
-# u.f and constants 23, rest population 10, nine TRT pairs with Luo forcing
-# 264 (axis pairs 28 each, diagonal pairs 30)
-LBM_FLOPS = 342
+VCYCLE_KERNELS = ("smooth_half", "smooth_near", "smooth_fused", "restrict", "prolong", "coarse_solve", "tail")
+# floating-point operations of the FP64 stream-collide per interior fluid
+# cell, counted from collide() with an FMA as two: pair sums and moments 39,
+# force, modified velocity, u.u, u.f and constants 26, rest population 3, the
+# vectors h and g 24, nine TRT pairs with Luo forcing 90 (axis pairs 8 each,
+# diagonal pairs 11)
+LBM_FLOPS = 182
 
 
 def vcycle_stats(prof, cycles):
