@@ -1369,7 +1369,8 @@ void dispatch_store(const es_ctx* c, Fn&& fn) {
 // The stream-collide's block shape (es_params.lbm_block; 0 = 32 x 4: a warp
 // per row segment and four rows a block, so that the rows y +- 1 of psi the
 // fused body force reads are mostly in the block's own L1; measured at 512^3
-// 3.95 ms against 4.14 ms for 128 x 1).
+// 3.79 ms against 3.85 for 32 x 2 and 64 x 2, 3.86 for 32 x 8, 4.09 for 128 x
+// 2).
 dim3 lbm_block(const es_ctx* c) {
     if (c->P.lbm_block[0] <= 0) return dim3(32, 4);
     return dim3(c->P.lbm_block[0], c->P.lbm_block[1] > 0 ? c->P.lbm_block[1] : 1);
