@@ -384,6 +384,9 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
     }
     for (int t = A.code_bytes + 16 * (int)threadIdx.x; t < A.smem_bytes; t += 16 * kTailThreads)
         *reinterpret_cast<uint4*>(smem + t) = make_uint4(0u, 0u, 0u, 0u);
+    // (these stores go through the generic proxy; the bulk copies below, which
+    // overwrite some of them, through the async one)
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (threadIdx.x == 0 && !bulk_wait(bar_at, 0)) late = 1;
     pdl_wait();
