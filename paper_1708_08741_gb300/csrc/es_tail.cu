@@ -654,9 +654,14 @@ bool tail_layout(const es_params& P, int l0, TailPlan& T) {
     return true;
 }
 
-// The finest level whose coarser ones all fit the cluster, or -1.
+// The finest level whose coarser ones all fit the cluster, or -1.  A cell of a
+// periodic axis of one cell is its own neighbour there, of its own colour,
+// which the colours' separate arrays do not hold in the neighbour's place:
+// such grids (one level) are launched.
 int tail_first(const es_params& P, TailPlan& T) {
     if (P.phi_t > 0.0 || P.smoother != ES_SMOOTH_TWO_PASS) return -1;
+    for (int a = 0; a < 3; a++)
+        if (P.periodic[a] && P.dims[a] == 1) return -1;
     const long long most = P.near_list_cells > 0 ? (long long)P.near_list_cells : (long long)ES_NEAR_LIST_CELLS;
     for (int l = P.mg_storage == ES_MG_FP16 ? 1 : 0; l < P.levels; l++) {
         if ((long long)(P.dims[0] >> l) * (P.dims[1] >> l) * (P.dims[2] >> l) > most) continue;

@@ -3,8 +3,10 @@ levels launched one by one (near_list_cells = 1 keeps every level out of it)."""
 import numpy as np
 import pytest
 
+import oracle
 import paper_1708_08741_gb300 as es
 from paper_1708_08741_gb300 import workloads as W
+from _pair import rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -61,4 +63,59 @@ def test_bulk_copied_right_hand_side(dims, levels):
         if ref is None:
             ref = psi
         np.testing.assert_array_equal(psi, ref)
+    sim.close()
+
+
+def _levels_in_cluster(sim):
+    """The levels of the cluster launches of one V-cycle."""
+    sim.profile_start()
+    sim.solve(forced_cycles=1)
+    return [r["level"] for r in sim.profile_stop() if r["name"] == "tail"]
+
+
+@pytest.mark.parametrize("precision", [es.ES_FP64, es.ES_MIXED32])
+@pytest.mark.parametrize("dims,axis", [((32, 32, 1), 0), ((64, 1, 1), 0), ((1, 32, 32), 1), ((1, 1, 40), 2),
+                                       ((36, 1, 20), 2)])
+def test_periodic_axis_of_one_cell(precision, dims, axis):
+    """A cell is its own neighbour along a periodic axis of one cell.  FP64: the
+    oracle's iteration up to the rounding of sums of seven terms, 1e-12 after
+    two cycles, and its cycle count.  MIXED32: below 1e-10 of the first residual
+    after one cycle more (FP32 reaches 1e-5 a cycle and more here), so the
+    potentials differ by at most 2e-10 (12 + kappa^2) / kappa^2 = 3e-8."""
+    bc, val = [0] * 6, [0.0] * 6
+    bc[2 * axis] = bc[2 * axis + 1] = 1
+    val[2 * axis], val[2 * axis + 1] = 0.7, -0.4
+    wl = W.Workload(name="thin", dims=list(dims), periodic=tuple(0 if a == axis else 1 for a in range(3)), tau=0.8,
+                    kappa=0.3, eps=1.0, E_ext=(0.0, 0.0, 0.0), levels=1, coarse_sweeps=400, res_rf=1e-10,
+                    max_cycles=200, pot_bc=tuple(bc), pot_val=tuple(val))
+    sim, o = es.Simulation(wl, precision), oracle.Oracle(wl)
+    sim.map_particles()
+    o.map_particles()
+    if precision == es.ES_FP64:
+        io, ig = o.solve(forced_cycles=2), sim.solve(forced_cycles=2)
+        assert rel_l2(sim.field(es.FIELD_PSI), o.field(oracle.FIELD_PSI)) < 1e-12
+        assert abs(ig["r0"] - io["r0"]) <= 1e-12 * io["r0"]
+        assert sim.solve()["cycles"] == o.solve()["cycles"]
+    else:
+        io = o.solve()
+        assert sim.solve(forced_cycles=io["cycles"] + 1)["r"] <= io["tol"]
+        assert rel_l2(sim.field(es.FIELD_PSI), o.field(oracle.FIELD_PSI)) < 3e-8
+    assert _levels_in_cluster(sim) == []
+    sim.close()
+
+
+@pytest.mark.parametrize("precision,dims,levels,lists,want", [
+    (es.ES_FP64, (32, 32, 32), 3, 0, [0]),
+    (es.ES_FP64, (64, 64, 64), 3, 0, [1]),
+    (es.ES_MIXED32, (64, 64, 64), 4, 0, [0]),
+    (es.ES_MIXED32, (96, 96, 48), 4, 0, [1]),
+    (es.ES_MIXED32, (64, 64, 64), 4, 1, []),
+])
+def test_levels_of_the_cluster_launch(precision, dims, levels, lists, want):
+    """The cluster launch runs, from the finest level that fits it on;
+    near_list_cells = 1 keeps every level out of it."""
+    wl = W.mixed_box(dims=dims, periodic=(1, 1, 1), levels=levels, n_spheres=3, radius=3.2)
+    sim = es.Simulation(wl, precision, overrides=dict(near_list_cells=lists))
+    sim.map_particles()
+    assert _levels_in_cluster(sim) == want
     sim.close()
