@@ -220,6 +220,9 @@ void tail_setup(es_ctx* c);
 bool tail_split(const es_ctx* c);
 cudaError_t launch_tail_codes(es_ctx* c);
 cudaError_t launch_tail(es_ctx* c, int warm);
+// how the kernel of the coarsest level divides by the diagonal: 0 k_coarse_lists
+// (tabulated inverses), 1 k_coarse_solve (quotients), 2 the half sweeps
+int coarse_divides(const es_ctx* c);
 cudaError_t launch_split_psi(es_ctx* c, const double* src);  // MIXED32: psi = src
 cudaError_t launch_join_psi(es_ctx* c, double* dst);         // MIXED32: dst = psi
 cudaError_t launch_correct(es_ctx* c);

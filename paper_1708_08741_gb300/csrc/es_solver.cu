@@ -4350,6 +4350,11 @@ __global__ void __launch_bounds__(kLocalThreads) k_local_solve(Level<float> L, c
 
 }  // namespace
 
+int coarse_divides(const es_ctx* c) {
+    const size_t t = mixed(c) ? sizeof(float) : sizeof(double);
+    return coarse_by_lists(c, t) ? 0 : (coarse_smem_bytes(c, t) <= 200 * 1024 ? 1 : 2);
+}
+
 // Grid of a marching residual pass over a level of nz planes with (gx, gy)
 // blocks per plane: zc planes per block, about eight blocks per SM in all
 // (up to 16 planes each), and no more blocks than partial-sum slots.

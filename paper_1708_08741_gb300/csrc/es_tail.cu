@@ -10,9 +10,10 @@
 // codes live in the blocks' shared memory, a block owns a slab of z planes of
 // every level and reads the planes next to it through distributed shared
 // memory, and cluster barriers separate the half sweeps instead of launches.
-// The arithmetic is the kernels' of es_solver.cu (a near-boundary cell
-// multiplies by the tabulated inverse of its diagonal, as the coarsest-level
-// kernels do).
+// The arithmetic is the kernels' of es_solver.cu; in FP32 with the same
+// operations in the same order, so that a reduced-form solve gives the bits of
+// the levels launched one by one (TailLevel::how).  In FP64 every cell
+// multiplies by the tabulated inverse of its diagonal, as k_smooth_d does.
 //
 // Layout in shared memory: per level the two colours apart, a row holding the
 // compact places x / 2 of its cells padded to a multiple of four, so that a
@@ -50,8 +51,9 @@ constexpr int kTailCluster = 16;          // most blocks of the cluster
 constexpr size_t kTailSmem = 220 * 1024;  // most dynamic shared memory of a block
 // A cell's code: the six faces as near_faces has them (two bits each) and in
 // the top four bits 6 + (faces that raise the diagonal) - (faces that lower it);
-// kTailOff: not an unknown cell.
-constexpr unsigned kTailOff = 0xFFFFu, kTailInner = 6u << 12;
+// kTailOff: not an unknown cell.  FP32: kTailOdd there means that the diagonal
+// formed face by face differs from diag0 plus that sum by rounding.
+constexpr unsigned kTailOff = 0xFFFFu, kTailInner = 6u << 12, kTailOdd = 13u;
 
 struct TailShape {
     int nx, ny, nz;
@@ -66,10 +68,23 @@ struct TailShape {
     unsigned mpw, mny, mzs;  // ceil(2^22 / d) of pw, ny, zs: t / d = (t m) >> 22 for t < 1024
 };
 
+// How the FP32 half sweeps divide by the diagonal: as k_coarse_lists (the
+// coarsest level), by a tabulated inverse; as k_smooth_v, interior cells by the
+// inverse of diag0 and near-boundary cells by a quotient; as k_smooth and
+// k_coarse_solve, every cell by a quotient.
+enum TailHow { kByTable, kNearQuotient, kQuotient };
+
 template <class T>
 struct TailLevel {
     TailShape s;
     T h2, inv_h2, diag0;
+    int how;       // TailHow (FP64: by table)
+    int red_only;  // the restriction takes the red residuals only
+    int pairs;     // and adds the two children of a fine row first (k_restrict_v)
+    // omega != 1, FP32: omega g enters the sum (1 - omega) e + omega g unrounded
+    // (else the other product does), at interior and at near-boundary cells, as
+    // in the level's kernels
+    int fuse_inner, fuse_near;
 };
 
 struct TailCodes {
@@ -77,6 +92,7 @@ struct TailCodes {
     const uint8_t* st[ES_MAXLEV];
     int n, blocks, bytes;  // levels, blocks, code bytes of a block
     int per[3], pot_bc[6];
+    float diag0[ES_MAXLEV];  // 0: no kTailOdd
     unsigned char* out;
 };
 
@@ -92,7 +108,6 @@ struct TailArgs {
     int warm;       // the iterate starts from out instead of zero
     int nu1, nu2, sweeps;
     T omega;
-    int red_only;   // the restriction takes the red residuals only
     int solo;       // the coarsest level belongs to block 0 alone
     int* status;
 };
@@ -132,6 +147,12 @@ struct Codes {
         }
     }
     __device__ __forceinline__ unsigned at(int k) const { return (w[k >> 1] >> (16 * (k & 1))) & 0xFFFFu; }
+    __device__ __forceinline__ bool odd() const {  // (a cell with kTailOdd)
+        bool any = false;
+#pragma unroll
+        for (int k = 0; k < kSpan<T>; k++) any |= (at(k) >> 12) == kTailOdd;
+        return any;
+    }
     __device__ __forceinline__ bool inner() const {
         if constexpr (kSpan<T> == 4)
             return w[0] == (kTailInner | (kTailInner << 16)) && w[1] == w[0];
@@ -210,6 +231,73 @@ struct Around {
     }
 };
 
+// The diagonal of a cell that is unknown, face by face as near_sums forms it
+// (in FP32 diag0 + 1 + 1 - 1 is not always diag0 + 1).
+__device__ __forceinline__ float code_diag(float diag0, unsigned c) {
+    float d = diag0;
+#pragma unroll
+    for (int f = 0; f < 6; f++) {
+        const unsigned u = (c >> (2 * f)) & 3u;
+        d += u == 0u ? 0.0f : (u == 1u ? 1.0f : -1.0f);
+    }
+    return d;
+}
+
+// The inverse diagonals of a span's cells (0 at those that are not unknown) and,
+// in FP32, the diagonals, from the level's tables.
+template <class T>
+struct Diagonals {
+    Span<T> y, d;
+    __device__ __forceinline__ Diagonals(const T* inv, const T* diag, const Codes<T>& cd) {
+#pragma unroll
+        for (int k = 0; k < kSpan<T>; k++) {
+            y.v[k] = inv[cd.at(k) >> 12];
+            if (sizeof(T) == 4) d.v[k] = diag[cd.at(k) >> 12];
+        }
+    }
+};
+
+// n over the diagonal for a span's cells (see TailHow).  The quotient comes
+// from the tabulated inverse y = RN(1 / d): n y is within two ulp of n / d, one
+// correction by the remainder n - q d brings it within one, and from there the
+// next gives the correctly rounded quotient (P. Markstein, Computation of
+// elementary functions on the IBM RISC System/6000 processor, IBM J. Res. Dev.
+// 34, 1990): the bits of a division at four multiply-adds a near-boundary cell
+// (a 192^3 solve from zero: 7 % over products alone, 13 % with divisions).
+template <class T>
+__device__ __forceinline__ Span<T> quotients(const TailLevel<T>& L, const Span<T>& n, const Diagonals<T>& D,
+                                             const Codes<T>& cd) {
+    Span<T> q;
+#pragma unroll
+    for (int k = 0; k < kSpan<T>; k++) q.v[k] = n.v[k] * D.y.v[k];
+    if constexpr (sizeof(T) == 4) {
+        if (L.how == kByTable || (L.how == kNearQuotient && cd.inner())) return q;
+#pragma unroll
+        for (int k = 0; k < kSpan<T>; k++) {
+            const float d = D.d.v[k], y = D.y.v[k];
+            float c = __fmaf_rn(__fmaf_rn(-q.v[k], d, n.v[k]), y, q.v[k]);
+            c = __fmaf_rn(__fmaf_rn(-c, d, n.v[k]), y, c);
+            if (L.how == kQuotient || cd.at(k) != kTailInner) q.v[k] = c;
+        }
+        if (cd.odd()) {
+#pragma unroll
+            for (int k = 0; k < kSpan<T>; k++)
+                if ((cd.at(k) >> 12) == kTailOdd) q.v[k] = n.v[k] / code_diag(L.diag0, cd.at(k));
+        }
+    }
+    return q;
+}
+
+// (1 - omega) e + omega g
+__device__ __forceinline__ double relaxed(const TailLevel<double>&, double omega, double e, double g, unsigned) {
+    return (1.0 - omega) * e + omega * g;
+}
+__device__ __forceinline__ float relaxed(const TailLevel<float>& L, float omega, float e, float g, unsigned c) {
+    const float keep = 1.0f - omega;
+    return c == kTailInner ? (L.fuse_inner ? __fmaf_rn(omega, g, __fmul_rn(keep, e)) : __fmaf_rn(keep, e, __fmul_rn(omega, g)))
+                           : (L.fuse_near ? __fmaf_rn(omega, g, __fmul_rn(keep, e)) : __fmaf_rn(keep, e, __fmul_rn(omega, g)));
+}
+
 // The sums of the unknown neighbours of a span's cells, in the order x left,
 // right, y-1, y+1, z-1, z+1 (FP64: the three pairs first, which takes two of
 // the seven 64-cycle operations off the chain).
@@ -254,12 +342,12 @@ __device__ __forceinline__ Span<T> neighbour_sums(const T* e, const Around<T>& a
 // thread has at most one span of a colour, what the sweeps do not change --
 // the addresses, codes, inverse diagonals and h^2 r -- stays in registers.
 template <class T>
-__device__ __forceinline__ void tail_smooth(const TailLevel<T>& L, const Slab<T>& s, const T* inv, int sweeps, T omega,
-                                            bool solo, cg::cluster_group& cl) {
+__device__ __forceinline__ void tail_smooth(const TailLevel<T>& L, const Slab<T>& s, const T* inv, const T* diag,
+                                            int sweeps, T omega, bool solo, cg::cluster_group& cl) {
     constexpr int W = kSpan<T>;
     const TailShape& S = L.s;
     const bool gs = omega == (T)1;
-    const T h2 = L.h2, keep = (T)1 - omega;
+    const T h2 = L.h2;
     if (sweeps == 0) return;
     if (S.ny * S.zs <= S.rpi) {
         const bool on = s.row0 < s.nrows;
@@ -267,28 +355,31 @@ __device__ __forceinline__ void tail_smooth(const TailLevel<T>& L, const Slab<T>
         const Around<T> at0(S, s, 0, row, y, lz), at1(S, s, 1, row, y, lz);
         const int own = row * S.nxp + s.j0;
         const Codes<T> cd0(s.code + own), cd1(s.code + S.ploc + own);
-        Span<T> r0 = ldspan(s.r + own), r1 = ldspan(s.r + S.ploc + own), i0, i1;
+        Span<T> r0 = ldspan(s.r + own), r1 = ldspan(s.r + S.ploc + own);
+        const Diagonals<T> i0(inv, diag, cd0), i1(inv, diag, cd1);
 #pragma unroll
         for (int k = 0; k < W; k++) {
             r0.v[k] *= h2;  // (exact: a power of two)
             r1.v[k] *= h2;
-            i0.v[k] = inv[cd0.at(k) >> 12];
-            i1.v[k] = inv[cd1.at(k) >> 12];
             if (W == 1) {  // (FP64: an operation less in each half sweep's chain)
-                r0.v[k] *= i0.v[k];
-                r1.v[k] *= i1.v[k];
+                r0.v[k] *= i0.y.v[k];
+                r1.v[k] *= i1.y.v[k];
             }
         }
-        auto half = [&](const Around<T>& at, const Codes<T>& cd, const Span<T>& r, const Span<T>& id, T* e) {
+        auto half = [&](const Around<T>& at, const Codes<T>& cd, const Span<T>& r, const Diagonals<T>& id, T* e) {
             if (on) {
                 const Span<T> o = neighbour_sums<T>(s.e, at, cd);
-                Span<T> c;
+                Span<T> c, g;
                 if (!gs) c = ldspan(e);
+                if constexpr (W == 1) {
+                    g.v[0] = o.v[0] * id.y.v[0] + r.v[0];
+                } else {
 #pragma unroll
-                for (int k = 0; k < W; k++) {
-                    const T g = W == 1 ? o.v[k] * id.v[k] + r.v[k] : (r.v[k] + o.v[k]) * id.v[k];
-                    c.v[k] = gs ? g : keep * c.v[k] + omega * g;
+                    for (int k = 0; k < W; k++) g.v[k] = r.v[k] + o.v[k];
+                    g = quotients<T>(L, g, id, cd);
                 }
+#pragma unroll
+                for (int k = 0; k < W; k++) c.v[k] = gs ? g.v[k] : relaxed(L, omega, c.v[k], g.v[k], cd.at(k));
                 stspan(e, c);
             }
             if (solo)
@@ -309,13 +400,13 @@ __device__ __forceinline__ void tail_smooth(const TailLevel<T>& L, const Slab<T>
             const Codes<T> cd(s.code + own);
             const Span<T> r = ldspan(s.r + own);
             const Span<T> o = neighbour_sums<T>(s.e, Around<T>(S, s, colour, row, y, lz), cd);
-            Span<T> c;
+            Span<T> c, g;
             if (!gs) c = ldspan(s.e + own);
 #pragma unroll
-            for (int k = 0; k < W; k++) {
-                const T g = (h2 * r.v[k] + o.v[k]) * inv[cd.at(k) >> 12];
-                c.v[k] = gs ? g : keep * c.v[k] + omega * g;
-            }
+            for (int k = 0; k < W; k++) g.v[k] = h2 * r.v[k] + o.v[k];
+            g = quotients<T>(L, g, Diagonals<T>(inv, diag, cd), cd);
+#pragma unroll
+            for (int k = 0; k < W; k++) c.v[k] = gs ? g.v[k] : relaxed(L, omega, c.v[k], g.v[k], cd.at(k));
             stspan(s.e + own, c);
         });
         if (solo)
@@ -435,7 +526,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
         const TailShape& S = L.s;
         const TailShape& M = A.lv[l + 1].s;
         const Slab<T> s(S, smem, cl, rank);
-        tail_smooth<T>(L, s, inv_tab[l], A.nu1, A.omega, false, cl);
+        tail_smooth<T>(L, s, inv_tab[l], diag_tab[l], A.nu1, A.omega, false, cl);
         // restriction: the mean of the 8 children's residuals (with red_only
         // the black ones count as 0); the children of a coarse cell share a slab
         // (an even number of planes), the coarse cell may be another block's.
@@ -459,19 +550,22 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
                         const int own = colour * S.ploc + row * S.nxp + s.j0;
 #pragma unroll
                         for (int k = 0; k < W; k++) res[d][k] = (T)0;
-                        if (A.red_only && colour) continue;
+                        if (L.red_only && colour) continue;
                         const Codes<T> cd(s.code + own);
                         const Span<T> o = neighbour_sums<T>(s.e, Around<T>(S, s, colour, row, y, lz), cd);
                         const Span<T> r = ldspan(s.r + own), e = ldspan(s.e + own);
 #pragma unroll
                         for (int k = 0; k < W; k++) {
                             const unsigned c = cd.at(k);
-                            if (c != kTailOff)
-                                res[d][k] = r.v[k] - (diag_tab[l][c >> 12] * e.v[k] - o.v[k]) * L.inv_h2;
+                            T dg = diag_tab[l][c >> 12];
+                            if constexpr (W == 4)
+                                if ((c >> 12) == kTailOdd) dg = code_diag(L.diag0, c);
+                            if (c != kTailOff) res[d][k] = r.v[k] - (dg * e.v[k] - o.v[k]) * L.inv_h2;
                         }
                     }
 #pragma unroll
-                    for (int k = 0; k < W; k++) sum[k] += res[0][k] + res[1][k];
+                    for (int k = 0; k < W; k++)
+                        sum[k] = L.pairs ? sum[k] + (res[0][k] + res[1][k]) : (sum[k] + res[0][k]) + res[1][k];
                 }
                 const int Z = (s.z0 >> 1) + Zl, owner = slab_owner(M, Z);
                 T* out = cl.map_shared_rank(cr, owner) + M.nxp * (Y + M.ny * (Z - owner * M.zs));
@@ -486,7 +580,8 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
     {
         const TailLevel<T>& L = A.lv[A.n - 1];
         if (!A.solo || rank == 0)
-            tail_smooth<T>(L, Slab<T>(L.s, smem, cl, rank), inv_tab[A.n - 1], A.sweeps, A.omega, A.solo != 0, cl);
+            tail_smooth<T>(L, Slab<T>(L.s, smem, cl, rank), inv_tab[A.n - 1], diag_tab[A.n - 1], A.sweeps, A.omega,
+                           A.solo != 0, cl);
         if (A.solo) cl.sync();
     }
     for (int l = A.n - 2; l >= 0; l--) {
@@ -513,7 +608,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
                 stspan(s.e + i, v);
             });
         cl.sync();
-        tail_smooth<T>(L, s, inv_tab[l], A.nu2, A.omega, false, cl);
+        tail_smooth<T>(L, s, inv_tab[l], diag_tab[l], A.nu2, A.omega, false, cl);
     }
     {
         const TailShape& S = A.lv[0].s;
@@ -592,6 +687,9 @@ __global__ void __launch_bounds__(256) k_tail_codes(const __grid_constant__ Tail
                 cd |= u << (2 * f);
                 dk += u == 0u ? 0 : (u == 1u ? 1 : -1);
             }
+            if (A.diag0[blockIdx.y] > 0.0f &&
+                code_diag(A.diag0[blockIdx.y], cd) != A.diag0[blockIdx.y] + (float)(dk - 6))
+                dk = (int)kTailOdd;
             code[k] = cd | ((unsigned)dk << 12);
         }
         *reinterpret_cast<uint2*>(A.out + (size_t)block * A.bytes + S.c + 2 * (size_t)(colour * S.ploc + 4 * i)) =
@@ -688,7 +786,25 @@ cudaError_t tail_run(es_ctx* c, int warm) {
     A.n = p.n;
     for (int l = 0; l < p.n; l++) {
         const double h = (double)(1 << (l0 + l));
-        A.lv[l] = TailLevel<T>{p.s[l], (T)(h * h), (T)(1.0 / (h * h)), (T)(6.0 + c->S.kappa * c->S.kappa * h * h)};
+        TailLevel<T>& L = A.lv[l];
+        L = TailLevel<T>{p.s[l], (T)(h * h), (T)(1.0 / (h * h)), (T)(6.0 + c->S.kappa * c->S.kappa * h * h)};
+        L.how = kByTable;
+        L.red_only = c->P.omega == 1.0 && c->P.nu1 >= 1;
+        L.pairs = 1;
+        L.fuse_inner = L.fuse_near = 0;
+        if (sizeof(T) == 4) {
+            // what the level's kernels do when it is launched by itself
+            const bool spans = p.s[l].nx % 4 == 0;
+            L.how = spans ? kNearQuotient : kQuotient;
+            if (l + 1 < p.n || coarse_divides(c) == 2) {
+                L.fuse_inner = !spans;                         // (k_smooth)
+                L.fuse_near = !spans || split_level(c, l0 + l);  // (near_gs)
+            } else {
+                L.how = coarse_divides(c) == 0 ? kByTable : kQuotient;
+            }
+            L.red_only = L.red_only && spans;
+            L.pairs = spans;
+        }
     }
     A.codes = c->tail_codes;
     A.code_bytes = p.code_bytes;
@@ -701,7 +817,6 @@ cudaError_t tail_run(es_ctx* c, int warm) {
     A.nu2 = c->P.nu2;
     A.sweeps = c->P.coarse_sweeps;
     A.omega = (T)c->P.omega;
-    A.red_only = c->P.omega == 1.0 && c->P.nu1 >= 1;
     A.solo = p.solo;
     A.status = c->d_status;
     double cells = 0.0;
@@ -780,6 +895,9 @@ cudaError_t launch_tail_codes(es_ctx* c) {
     for (int l = 0; l < p.n; l++) {
         A.s[l] = p.s[l];
         A.st[l] = c->st[c->tail_l0 + l];
+        const double h = (double)(1 << (c->tail_l0 + l));
+        const bool table = l + 1 == p.n && coarse_divides(c) == 0;  // (k_coarse_lists takes the sum's inverse)
+        A.diag0[l] = mixed(c) && !table ? (float)(6.0 + c->S.kappa * c->S.kappa * h * h) : 0.0f;
     }
     for (int a = 0; a < 3; a++) A.per[a] = c->g.per[a];
     for (int f = 0; f < 6; f++) A.pot_bc[f] = c->S.pot_bc[f];
