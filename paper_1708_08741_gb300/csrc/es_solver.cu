@@ -3810,11 +3810,11 @@ __global__ void __launch_bounds__(256) k_rhs_norm_rb(Grid g, const float* __rest
 // flips up to six cells apart fit) is solved in shared memory: p with a halo
 // of zeros, x and r for the box, and a code byte a cell, so that a neighbour
 // outside the region needs no test.  The dot products are summed in
-// float-float and the quotients formed in FP32, the precision in which they
-// are used: their FP64 sums and, above all, the FP64 divisions of 1,024
-// threads took the FP64 pipe 20 us of every iteration (a solve's start with
-// its local correction at 512^3: 0.86 ms before, 0.42 ms now; 128^3: 178 us,
-// 80 us).  Larger clusters keep their vectors in global memory.
+// float-float and the quotients formed from both parts and rounded once, so
+// that alpha and beta are the FP32 values of FP64 sums and quotients: those
+// took the FP64 pipe 20 us of every iteration (the patched starts of seven
+// solves, mean, 512^3: 0.80 ms with them, 0.41 ms so; 128^3: 105 us, 54 us).
+// Larger clusters keep their vectors in global memory.
 constexpr int kLocalR = 8;
 constexpr int kLocalFlips = 16;
 constexpr int kLocalIters = 40;
@@ -3916,6 +3916,14 @@ __global__ void k_local_norm(const LocalMeta* __restrict__ meta, NormOut out) {
     out.put(v);
 }
 
+// The dot products of the local correction: exact products, float-float sums
+// (FP64 sums of 1,024 threads take the FP64 pipe longer than everything else
+// there).
+__device__ __forceinline__ void ff_dot(ff_acc& acc, float a, float b) {
+    const float p = __fmul_rn(a, b);
+    acc.add(p, __fmaf_rn(a, b, -p));
+}
+
 // Sum over the block of one float-float value a thread, to every thread
 // (fixed order).  kLocalThreads threads.
 __device__ __forceinline__ ff block_ff_sum(ff v, float2* sh) {
@@ -3938,10 +3946,32 @@ __device__ __forceinline__ ff block_ff_sum(ff v, float2* sh) {
     return v;
 }
 
-// acc += a b, exactly up to the float-float sum
-__device__ __forceinline__ void ff_dot(ff_acc& acc, float a, float b) {
-    const float p = __fmul_rn(a, b);
-    acc.add(p, __fmaf_rn(a, b, -p));
+// The power of two that brings the block's largest |v| to between 1 and 2: the
+// correction works on the residual times it, so that neither the squares nor
+// their low parts leave FP32's range.
+__device__ __forceinline__ float block_scale(float v, float2* sh) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(v)));
+    __syncthreads();
+    if (lane == 0) sh[wid].x = __uint_as_float(m);
+    __syncthreads();
+    m = __reduce_max_sync(0xffffffffu, __float_as_uint(sh[lane].x)) >> 23;
+    return m == 0 ? 1.0f : __uint_as_float(m < 253u ? (254u - m) << 23 : 1u << 23);
+}
+
+// a / b rounded once to FP32: the leading parts' quotient, and the remainder's
+// (to 2^-46 before that rounding, so the FP32 value of an FP64 quotient).
+__device__ __forceinline__ float ff_quotient(ff a, ff b) {
+    const float q = __fdiv_rn(a.hi, b.hi);
+    const float r = __fadd_rn(__fmaf_rn(-q, b.hi, a.hi), __fmaf_rn(-q, b.lo, a.lo));
+    return __fadd_rn(q, __fdiv_rn(r, b.hi));
+}
+
+// a > 1e-6 b, in FP64 where the leading parts are close
+__device__ __forceinline__ bool ff_above(ff a, ff b) {
+    const float lim = 1e-6f * b.hi;
+    if (fabsf(a.hi - lim) > 1e-5f * lim) return a.hi > lim;
+    return (double)a.hi + (double)a.lo > 1e-6 * ((double)b.hi + (double)b.lo);
 }
 
 // The box of a cluster that is solved in shared memory: origin (ring
@@ -3980,6 +4010,15 @@ struct LocalCube {
     }
 };
 
+// The diagonal at a near-boundary cell.
+__device__ __noinline__ float local_diag(const Level<float>& L, const uint8_t* __restrict__ st, int x, int y, int z) {
+    int nb[6];
+    const float none[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    float dg, off;
+    near_sums(near_faces(L, st, x, y, z, nb), L.diag0, none, dg, off);
+    return dg;
+}
+
 // The cluster in its box, in shared memory.  Every thread owns the box cells
 // threadIdx.x + k kLocalThreads throughout.
 __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uint8_t* __restrict__ st,
@@ -3991,7 +4030,8 @@ __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uin
     float* P = sm;             // with a halo
     float* X = P + hvol;
     float* R = X + vol;
-    uint8_t* C = (uint8_t*)(R + vol);  // bit 7 region, bit 6 ring, low bits 6 + diagonal shift
+    uint8_t* C = (uint8_t*)(R + vol);  // bit 7 region, bit 6 ring, low bits 6 + diagonal shift (kOdd: see diagonal)
+    constexpr unsigned kOdd = 13;
     const int n3[3] = {L.nx, L.ny, L.nz};
     const float inv_h2 = 1.0f / L.h2;
     auto cell = [&](const BoxWalk& w, int (&g)[3]) {
@@ -4009,11 +4049,19 @@ __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uin
         return ok;
     };
     auto place = [&](const BoxWalk& w) { return (w.i + 1) + hx * (w.j + 1) + hxy * (w.k + 1); };
+    // the diagonal as near_sums forms it, face by face: where that is not diag0
+    // plus the shift (rounding), from the faces again
+    auto diagonal = [&](const BoxWalk& w, unsigned code) {
+        if ((code & 15u) != kOdd) return L.diag0 + (float)((int)(code & 15u) - 6);
+        int g[3];
+        cell(w, g);
+        return local_diag(L, st, g[0], g[1], g[2]);
+    };
     for (int t = threadIdx.x; t < hvol; t += kLocalThreads) P[t] = 0.0f;
     __syncthreads();
     BoxWalk w0;
     w0.start(threadIdx.x, kLocalThreads, bx, by);
-    ff_acc rr_a{0.0f, 0.0f}, old_a{0.0f, 0.0f};
+    float most = 0.0f;
     {
         BoxWalk w = w0;
         for (int t = threadIdx.x; t < vol; t += kLocalThreads, w.next()) {
@@ -4037,23 +4085,19 @@ __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uin
                     dist = min(dist, d);
                 }
                 if ((s & ST_KIND) == ST_UNKNOWN && dist <= kLocalR + 1) {
-                    int shift = 0;
+                    unsigned low = 6;
                     if (s & ST_NEAR) {
                         int nb[6];
                         const unsigned fc = near_faces(L, st, g[0], g[1], g[2], nb);
-#pragma unroll
-                        for (int k = 0; k < 6; k++) {
-                            const unsigned f = (fc >> (2 * k)) & 3u;
-                            shift += f == 0u ? 0 : (f == 1u ? 1 : -1);
-                        }
+                        low = (unsigned)near_shift(fc);
+                        const float none[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+                        float dg, off;
+                        near_sums(fc, L.diag0, none, dg, off);
+                        if (dg != L.diag0 + (float)((int)low - 6)) low = kOdd;
                     }
-                    code = (dist <= kLocalR ? 0x80u : 0x40u) | (unsigned)(6 + shift);
+                    code = (dist <= kLocalR ? 0x80u : 0x40u) | low;
                     v = r[rb(c, (g[0] + g[1] + g[2]) & 1)];
-                    ff_dot(old_a, v, v);
-                    if (code & 0x80u) {
-                        P[place(w)] = v;
-                        ff_dot(rr_a, v, v);
-                    }
+                    most = fmaxf(most, fabsf(v));
                 }
             }
             C[t] = (uint8_t)code;
@@ -4061,7 +4105,22 @@ __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uin
             R[t] = v;
         }
     }
-    auto apply = [&](int at, unsigned code) {  // (A p) h^2; 0 outside the region counts as no neighbour
+    const float sc = block_scale(most, sh), isc = 1.0f / sc;
+    ff_acc rr_a{0.0f, 0.0f}, old_a{0.0f, 0.0f};
+    {
+        BoxWalk w = w0;
+        for (int t = threadIdx.x; t < vol; t += kLocalThreads, w.next()) {
+            const float v = sc * R[t];
+            R[t] = v;
+            ff_dot(old_a, v, v);  // (0 at cells that take no part)
+            if (C[t] & 0x80u) {
+                P[place(w)] = v;
+                ff_dot(rr_a, v, v);
+            }
+        }
+    }
+    // (A p) h^2; 0 outside the region counts as no neighbour
+    auto apply = [&](const BoxWalk& w, int at, unsigned code) {
         const float pv = P[at];
         float off = P[at - 1];
         off += P[at + 1];
@@ -4069,12 +4128,12 @@ __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uin
         off += P[at + hx];
         off += P[at - hxy];
         off += P[at + hxy];
-        return (L.diag0 + (float)((int)(code & 15u) - 6)) * pv - off;
+        return diagonal(w, code) * pv - off;
     };
     ff rr = block_ff_sum(rr_a.value(), sh);
     const ff old_sq = block_ff_sum(old_a.value(), sh);
-    const float rr0 = rr.hi;
-    for (int it = 0; it < kLocalIters && rr.hi > 1e-6f * rr0 && rr.hi > 0.0f; it++) {
+    const ff rr0 = rr;
+    for (int it = 0; it < kLocalIters && ff_above(rr, rr0) && rr.hi > 0.0f; it++) {
         ff_acc pq_a{0.0f, 0.0f};
         {
             BoxWalk w = w0;
@@ -4082,12 +4141,12 @@ __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uin
                 const unsigned code = C[t];
                 if (!(code & 0x80u)) continue;
                 const int at = place(w);
-                ff_dot(pq_a, P[at], apply(at, code) * inv_h2);
+                ff_dot(pq_a, P[at], apply(w, at, code) * inv_h2);
             }
         }
         const ff pq = block_ff_sum(pq_a.value(), sh);
         if (!(pq.hi > 0.0f)) break;  // (uniform)
-        const float alpha = __fdiv_rn(rr.hi, pq.hi);
+        const float alpha = ff_quotient(rr, pq);
         ff_acc rn_a{0.0f, 0.0f};
         {
             BoxWalk w = w0;
@@ -4096,13 +4155,13 @@ __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uin
                 if (!(code & 0x80u)) continue;
                 const int at = place(w);
                 X[t] += alpha * P[at];
-                const float v = R[t] - alpha * (apply(at, code) * inv_h2);
+                const float v = R[t] - alpha * (apply(w, at, code) * inv_h2);
                 R[t] = v;
                 ff_dot(rn_a, v, v);
             }
         }
         const ff rn = block_ff_sum(rn_a.value(), sh);  // (also: every thread is done reading p)
-        const float beta = __fdiv_rn(rn.hi, rr.hi);
+        const float beta = ff_quotient(rn, rr);
         {
             BoxWalk w = w0;
             for (int t = threadIdx.x; t < vol; t += kLocalThreads, w.next())
@@ -4122,8 +4181,9 @@ __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uin
                 int g[3];
                 cell(w, g);
                 const int c = g[0] + L.nx * (g[1] + L.ny * g[2]);
-                P[place(w)] = X[t];
-                const ff v = ff_add_f({psi_hi[c], psi_lo[c]}, X[t]);
+                const float x = isc * X[t];
+                P[place(w)] = x;
+                const ff v = ff_add_f({psi_hi[c], psi_lo[c]}, x);
                 psi_hi[c] = v.hi;
                 psi_lo[c] = v.lo;
             }
@@ -4138,14 +4198,15 @@ __device__ __forceinline__ void local_solve_box(const Level<float>& L, const uin
             int g[3];
             cell(w, g);
             float* rp = r + rb(g[0] + L.nx * (g[1] + L.ny * g[2]), (g[0] + g[1] + g[2]) & 1);
-            const float v = *rp - apply(place(w), code) * inv_h2;
+            const float v = *rp - apply(w, place(w), code) * inv_h2;
             *rp = v;
-            ff_dot(new_a, v, v);
+            ff_dot(new_a, sc * v, sc * v);
         }
     }
     const ff new_sq = block_ff_sum(new_a.value(), sh);
     if (threadIdx.x == 0)
-        *delta = ((double)new_sq.hi + (double)new_sq.lo) - ((double)old_sq.hi + (double)old_sq.lo);
+        *delta = (((double)new_sq.hi + (double)new_sq.lo) - ((double)old_sq.hi + (double)old_sq.lo)) *
+                 ((double)isc * (double)isc);
 }
 
 // Visits the cells of the boxes of radius rb around the flipped cells
@@ -4222,16 +4283,18 @@ __device__ __noinline__ void local_solve_list(const Level<float>& L, const uint8
     const int ni = min(s_n[0], cap), nt = min(s_n[1], cap);
     if (!s_over) {
         // e = p = 0 on the listed cells (the ring keeps 0: A restricted to the region)
+        float most = 0.0f;
         for (int i = threadIdx.x; i < nt; i += blockDim.x) {
             const int cc = list[i], cl = col(cc);
             e[rb(cc, cl)] = 0.0f;
             p[rb(cc, cl)] = 0.0f;
+            most = fmaxf(most, fabsf(r[rb(cc, cl)]));
         }
-        __syncthreads();
+        const float sc = block_scale(most, sh), isc = 1.0f / sc;  // (also: p is zeroed)
         ff_acc rr_a{0.0f, 0.0f}, old_a{0.0f, 0.0f};
         for (int i = threadIdx.x; i < nt; i += blockDim.x) {
             const int cc = list[i];
-            const float v = r[rb(cc, col(cc))];
+            const float v = sc * r[rb(cc, col(cc))];
             ff_dot(old_a, v, v);
             if (i < ni) {
                 rl[i] = v;
@@ -4242,8 +4305,8 @@ __device__ __noinline__ void local_solve_list(const Level<float>& L, const uint8
         }
         ff rr = block_ff_sum(rr_a.value(), sh);
         const ff old_sq = block_ff_sum(old_a.value(), sh);
-        const float rr0 = rr.hi;
-        for (int it = 0; it < kLocalIters && rr.hi > 1e-6f * rr0 && rr.hi > 0.0f; it++) {
+        const ff rr0 = rr;
+        for (int it = 0; it < kLocalIters && ff_above(rr, rr0) && rr.hi > 0.0f; it++) {
             ff_acc pq_a{0.0f, 0.0f};
             for (int i = threadIdx.x; i < ni; i += blockDim.x) {
                 const int cc = list[i];
@@ -4258,7 +4321,7 @@ __device__ __noinline__ void local_solve_list(const Level<float>& L, const uint8
             }
             const ff pq = block_ff_sum(pq_a.value(), sh);
             if (!(pq.hi > 0.0f)) break;
-            const float alpha = __fdiv_rn(rr.hi, pq.hi);
+            const float alpha = ff_quotient(rr, pq);
             ff_acc rn_a{0.0f, 0.0f};
             for (int i = threadIdx.x; i < ni; i += blockDim.x) {
                 const int cc = list[i];
@@ -4267,7 +4330,7 @@ __device__ __noinline__ void local_solve_list(const Level<float>& L, const uint8
                 ff_dot(rn_a, rl[i], rl[i]);
             }
             const ff rn = block_ff_sum(rn_a.value(), sh);  // (also: every thread is done reading p)
-            const float beta = __fdiv_rn(rn.hi, rr.hi);
+            const float beta = ff_quotient(rn, rr);
             for (int i = threadIdx.x; i < ni; i += blockDim.x) {
                 const int cc = list[i];
                 float* pp = p + rb(cc, col(cc));
@@ -4279,6 +4342,7 @@ __device__ __noinline__ void local_solve_list(const Level<float>& L, const uint8
         // psi += e on the region; e in place for the residual
         for (int i = threadIdx.x; i < ni; i += blockDim.x) {
             const int cc = list[i];
+            ec[i] *= isc;
             e[rb(cc, col(cc))] = ec[i];
             const ff v = ff_add_f({psi_hi[cc], psi_lo[cc]}, ec[i]);
             psi_hi[cc] = v.hi;
@@ -4315,11 +4379,12 @@ __device__ __noinline__ void local_solve_list(const Level<float>& L, const uint8
             float* rp = r + rb(cc, col(cc));
             const float rv = *rp - (dg * ev - off) * inv_h2;
             *rp = rv;
-            ff_dot(new_a, rv, rv);
+            ff_dot(new_a, sc * rv, sc * rv);
         }
         const ff new_sq = block_ff_sum(new_a.value(), sh);
         if (threadIdx.x == 0)
-            *delta = ((double)new_sq.hi + (double)new_sq.lo) - ((double)old_sq.hi + (double)old_sq.lo);
+            *delta = (((double)new_sq.hi + (double)new_sq.lo) - ((double)old_sq.hi + (double)old_sq.lo)) *
+                     ((double)isc * (double)isc);
     }
     __syncthreads();
     // clear the bits (every box cell: also those an overflow left unlisted)

@@ -55,3 +55,67 @@ def test_local_correction(dims, periodic, x, levels):
     assert flipped > 0
     for s in sims:
         s.close()
+
+
+CLUSTERS = [  # solved in shared memory; and, on a short axis, from the list in global memory
+    ((64, 64, 64), (1, 1, 1), [(31.37, 32.11, 30.83)], 3),
+    ((16, 48, 48), (1, 1, 1), [(7.37, 24.11, 22.83)], 2),
+]
+
+
+def _moves(wl, sims, n):
+    """The solves' records of n small moves of the spheres; True where a cell flipped."""
+    rng = np.random.Generator(np.random.PCG64(3))
+    for s in sims:
+        s.map_particles()
+        s.solve()
+    own = sims[0].field(es.FIELD_OWNER)
+    for _ in range(n):
+        wl.x = wl.x + rng.uniform(-0.04, 0.04, wl.x.shape)
+        info = []
+        for s in sims:
+            s.set_particles(wl.x, wl.v, wl.w)
+            s.map_particles()
+            info.append(s.solve())
+        new = sims[0].field(es.FIELD_OWNER)
+        yield bool(((new >= 0) != (own >= 0)).any()), info
+        own = new
+
+
+@pytest.mark.parametrize("dims,periodic,x,levels", CLUSTERS)
+def test_scaled_problem_gives_scaled_bits(dims, periodic, x, levels):
+    """The solve is linear and its sums hold their range: surface potentials and
+    charges times 2^-40 give the potential times 2^-40 to the last bit (the
+    squares of the residuals, below 1e-45 then, are out of FP32's range)."""
+    wl = [_spheres(dims, periodic, x, levels) for _ in range(2)]
+    wl[1].zeta, wl[1].q = wl[1].zeta * 2.0 ** -40, wl[1].q * 2.0 ** -40
+    sims = [es.Simulation(w, es.ES_MIXED32, overrides=dict(fast_update_cells=1)) for w in wl]
+    flips = 0
+    for flipped, info in _moves(wl[0], sims, 6):
+        flips += flipped
+        assert info[0]["cycles"] == info[1]["cycles"]
+        np.testing.assert_array_equal(sims[1].field(es.FIELD_PSI) * 2.0 ** 40, sims[0].field(es.FIELD_PSI))
+    assert flips > 0
+    for s in sims:
+        s.close()
+
+
+@pytest.mark.parametrize("dims,periodic,x,levels", CLUSTERS)
+def test_reported_residual_after_the_correction(dims, periodic, x, levels):
+    """The first residual of a solve that corrects locally, kept by the change of
+    r^2 over the clusters, against the residual of its potential formed in full:
+    within the 1 % of the tolerance that the carried residual may drift by.  At a
+    tolerance of 1e-3 of the first solve's residual (a flip leaves some 3e-2)
+    the correction does without V-cycles, and a start without it needs them."""
+    wl = _spheres(dims, periodic, x, levels)
+    wl.res_rf = 1e-3
+    sims = [es.Simulation(wl, es.ES_MIXED32, overrides=dict(fast_update_cells=f)) for f in (1, 2 ** 31 - 1)]
+    spared = 0
+    for flipped, info in _moves(wl, sims, 6):
+        if flipped and info[0]["cycles"] == 0:
+            full = sims[0].solve(forced_cycles=0)["r0"]
+            assert abs(full - info[0]["r0"]) <= 0.01 * info[0]["tol"]
+            spared += info[1]["cycles"] > 0
+    assert spared > 0
+    for s in sims:
+        s.close()
