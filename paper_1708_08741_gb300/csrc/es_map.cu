@@ -82,12 +82,16 @@ __device__ void union_range(const Grid& g, int a, double xo, double xn, double R
 // Cells whose state flipped since the last solve (obstacle <-> fluid) go to
 // a short list for the patched residual at the next solve's start
 // (k_flip_patch); when it is full the next solve forms the residual in full.
+// Only a colour-split finest level is patched: other contexts have no list
+// (their solves would never empty it, and its counter would run past the
+// integers' range).  Once the next residual is a full one nothing is added.
 struct FlipList {
-    int* cells;
+    int* cells;  // null: no list
     int* count;
     int cap;
-    int* full;  // set when a cell did not fit
+    int* full;  // set when a cell did not fit, or a sphere moved far
     __device__ __forceinline__ void add(long long c) const {
+        if (!cells || *(const volatile int*)full != 0) return;
         const int i = atomicAdd(count, 1);
         if (i < cap)
             cells[i] = (int)c;
@@ -839,7 +843,7 @@ cudaError_t launch_map(es_ctx* c) {
     // one block: the four kernels 74 -> 39 us); many: 256 (2,880 spheres fill
     // the SMs either way)
     const int T = c->np <= 2 * c->n_sm ? 1024 : 256;
-    const FlipList flips{c->flip_list, c->flip_count, c->flip_cap, c->d_moved};
+    const FlipList flips{c->rb0 ? c->flip_list : nullptr, c->flip_count, c->flip_cap, c->d_moved};
     {
         ProfScope ps(c, "map_clear", -1, 0.0);
         launch_pdl(c, k_clear, c->np, T, 0, g, c->part, c->mapped, c->owner, c->near_count,

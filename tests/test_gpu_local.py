@@ -119,3 +119,40 @@ def test_reported_residual_after_the_correction(dims, periodic, x, levels):
     assert spared > 0
     for s in sims:
         s.close()
+
+
+@pytest.mark.parametrize("precision,dims", [(es.ES_MIXED32, (96, 96, 96)), (es.ES_MIXED32, (84, 84, 84)),
+                                            (es.ES_FP64, (64, 64, 64))])
+def test_many_mappings_between_solves(precision, dims):
+    """Spheres mapped to and fro until more cells have flipped than the list of
+    flipped cells holds (2^16): the next solve ends where one does whose
+    context was mapped there once, both below 1e-10 of the first residual, so
+    within 2e-10 (12 + kappa^2) / kappa^2 = 2.7e-8.  (84: not colour-split,
+    FP64: neither keeps a list.)"""
+    wl = W.mixed_box(dims=dims, periodic=(1, 1, 1), levels=2, n_spheres=60 if dims[0] > 64 else 20, radius=4.2)
+    wl.v[:] = 0.0
+    wl.w[:] = 0.0
+    x0 = wl.x.copy()
+    sims = [es.Simulation(wl, precision, overrides=dict(fast_update_cells=1)) for _ in range(2)]
+    for s in sims:
+        s.map_particles()
+        s.solve(forced_cycles=3)
+    own = sims[0].field(es.FIELD_OWNER) >= 0
+    flips = 0
+    for k in range(1, 61):
+        sims[0].set_particles(x0 + (0.4 if k % 2 else 0.0), wl.v, wl.w)
+        sims[0].map_particles()
+        if k in (1, 2):
+            new = sims[0].field(es.FIELD_OWNER) >= 0
+            flips += 30 * int((new != own).sum())
+            own = new
+    assert flips > (1 << 16) or precision == es.ES_FP64
+    for s in sims:
+        s.set_particles(x0 + 0.1, wl.v, wl.w)
+        s.map_particles()
+        s.solve()
+    np.testing.assert_array_equal(sims[0].field(es.FIELD_OWNER), sims[1].field(es.FIELD_OWNER))
+    a, b = (s.field(es.FIELD_PSI) for s in sims)
+    assert np.linalg.norm(a - b) <= 2.7e-8 * np.linalg.norm(b)
+    for s in sims:
+        s.close()
