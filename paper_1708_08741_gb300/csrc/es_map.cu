@@ -845,9 +845,17 @@ cudaError_t launch_map(es_ctx* c) {
     const int T = c->np <= 2 * c->n_sm ? 1024 : 256;
     const FlipList flips{c->rb0 ? c->flip_list : nullptr, c->flip_count, c->flip_cap, c->d_moved};
     {
+        // (k_clear reads the mapped states ahead of its wait, and a mapping of
+        // one FP64 level without k_tail ends with the kernel that stores them:
+        // two such mappings in a row are not overlapped)
+        const bool ahead = mixed(c) || c->L > 1 || c->tail_l0 < c->L;
         ProfScope ps(c, "map_clear", -1, 0.0);
-        launch_pdl(c, k_clear, c->np, T, 0, g, c->part, c->mapped, c->owner, c->near_count,
-                   2 * kNearSegs * ES_MAXLEV, c->bf_count);
+        if (ahead)
+            launch_pdl(c, k_clear, c->np, T, 0, g, c->part, c->mapped, c->owner, c->near_count,
+                       2 * kNearSegs * ES_MAXLEV, c->bf_count);
+        else
+            k_clear<<<c->np, T, 0, c->stream>>>(g, c->part, c->mapped, c->owner, c->near_count,
+                                                2 * kNearSegs * ES_MAXLEV, c->bf_count);
     }
     {
         ProfScope ps(c, "map_set", -1, 0.0);

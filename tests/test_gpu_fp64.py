@@ -38,3 +38,26 @@ def test_fp64_cycle_and_body_force(dims, periodic, levels, nu1, nu2, omega):
     fb = p.g.field(es.FIELD_FB)
     assert rel_l2(fb[:, fluid], p.o.field(oracle.FIELD_FB)[:, fluid]) < 1e-12
     assert np.all(fb[:, ~fluid] == 0.0)
+
+
+@pytest.mark.parametrize("dims,levels,lists", [((24, 20, 28), 1, 1), ((40, 36, 44), 1, 0), ((24, 20, 28), 1, 0),
+                                               ((24, 20, 28), 2, 0)])
+def test_mappings_in_a_row(dims, levels, lists):
+    """Mappings that follow each other at once, with and without a move between:
+    the oracle's owners every time (whole numbers).  One level
+    with and without the cluster launch (40 x 36 x 44 is too large for it)."""
+    wl = W.mixed_box(dims=dims, periodic=(1, 1, 0), levels=levels, n_spheres=3, radius=3.2)
+    p = Pair(wl, lib_overrides=dict(near_list_cells=lists))
+    rng = np.random.Generator(np.random.PCG64(5))
+    for k in range(12):
+        for _ in range(1 + k % 3):
+            p.g.map_particles()
+        p.o.map_particles()
+        np.testing.assert_array_equal(p.g.field(es.FIELD_OWNER), p.o.owner())
+        x = wl.x + rng.uniform(-0.3, 0.3, wl.x.shape)
+        p.g.set_particles(x, wl.v, wl.w)
+        p.o.set_particles(x, wl.v, wl.w)
+        p.g.map_particles()
+        p.g.map_particles()
+        p.o.map_particles()
+        np.testing.assert_array_equal(p.g.field(es.FIELD_OWNER), p.o.owner())
