@@ -751,6 +751,30 @@ __device__ __forceinline__ int force_cells_fields(const Grid& g, const int32_t* 
     return total;
 }
 
+// Half the force and torque of the links m of cell (x, y, z), link by link.
+__device__ __noinline__ void force_links_each(const Grid& g, const DParticle& P, unsigned m, int x, int y, int z,
+                                              const double* __restrict__ src, size_t ps, double (&acc)[6]) {
+    const int c = x + g.nx * (y + g.ny * z);
+    for (; m; m &= m - 1u) {
+        const int q = __ffs(m) - 1;
+        int v[3];
+        dir_of(q, v);
+        const int bx = wrap_coord(x + v[0], g.nx), by = wrap_coord(y + v[1], g.ny), bz = wrap_coord(z + v[2], g.nz);
+        const double r0 = cell_disp(g, 0, bx, P.x[0]), r1 = cell_disp(g, 1, by, P.x[1]), r2 = cell_disp(g, 2, bz, P.x[2]);
+        double us[3];
+        surface_velocity(g, P.x, P.v, P.w, bx, by, bz, us);
+        const double w = (q <= 3 || (q >= 10 && q <= 12)) ? 1.0 / 18.0 : 1.0 / 36.0;
+        const double mq = src[q * ps + c] - 3.0 * w * (v[0] * us[0] + v[1] * us[1] + v[2] * us[2]);
+        const double d0 = mq * v[0], d1 = mq * v[1], d2 = mq * v[2];
+        acc[0] += d0;
+        acc[1] += d1;
+        acc[2] += d2;
+        acc[3] += r1 * d2 - r2 * d1;
+        acc[4] += r2 * d0 - r0 * d2;
+        acc[5] += r0 * d1 - r1 * d0;
+    }
+}
+
 // FP64 form.  The FP64 pipe (2 operations a clock and SM) bounds it, so a
 // cell's links share what they can: u_s . c_q = u_F . c_q with u_F = V + W x
 // r_F, since x_s = x_F + c_q and (W x c_q) . c_q = 0, and the torques add up to
@@ -797,6 +821,18 @@ __global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __rest
             const double r0 = cell_disp(g, 0, x, X[0]), r1 = cell_disp(g, 1, y, X[1]), r2 = cell_disp(g, 2, z, X[2]);
             const double u[3] = {V[0] + (Wv[1] * r2 - Wv[2] * r1), V[1] + (Wv[2] * r0 - Wv[0] * r2),
                                  V[2] + (Wv[0] * r1 - Wv[1] * r0)};
+            // a sphere that moved since its mapping may have a fluid cell past
+            // half a periodic axis whose surface cells are not: then each
+            // link has its own lever arm, at its surface cell's nearest image
+            const double r3[3] = {r0, r1, r2};
+            const int n3[3] = {g.nx, g.ny, g.nz};
+            bool past = false;
+#pragma unroll
+            for (int a = 0; a < 3; a++) past |= g.per[a] && fabsf((float)r3[a]) + 1.01f > 0.5f * (float)n3[a];
+            if (past) {
+                force_links_each(g, P, m, x, y, z, src, ps, acc);
+                continue;
+            }
             double d[3] = {0.0, 0.0, 0.0};  // half the sum of m_q c_q
             // three pairs of populations in flight at a time
 #pragma unroll
@@ -964,6 +1000,21 @@ __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
             isum[0] += S0;
             isum[1] += S1;
             isum[2] += S2;
+            bool past = false;  // (see k_forces)
+#pragma unroll
+            for (int a = 0; a < 3; a++) past |= image(v[a] + 1, a) - image(v[a] - 1, a) != 2;
+            if (past) {
+                for (unsigned l = m; l; l &= l - 1u) {
+                    const int q = __ffs(l) - 1, w = (q <= 3 || (q >= 10 && q <= 12)) ? 2 : 1;
+                    int k[3];
+                    dir_of(q, k);
+                    const int s0 = image(v[0] + k[0], 0), s1 = image(v[1] + k[1], 1), s2 = image(v[2] + k[2], 2);
+                    isum[3] += w * (s1 * k[2] - s2 * k[1]);
+                    isum[4] += w * (s2 * k[0] - s0 * k[2]);
+                    isum[5] += w * (s0 * k[1] - s1 * k[0]);
+                }
+                continue;
+            }
             isum[3] += u1 * S2 - u2 * S1;
             isum[4] += u2 * S0 - u0 * S2;
             isum[5] += u0 * S1 - u1 * S0;

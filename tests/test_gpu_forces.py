@@ -46,3 +46,32 @@ def test_forces_match_oracle(precision, dims, periodic, radius, n):
     assert np.linalg.norm(F - Fo) <= tol * np.linalg.norm(Fo)
     assert np.linalg.norm(T - To) <= tol * max(np.linalg.norm(To), radius * np.linalg.norm(Fo) * 0.1)
     g.close()
+
+
+@pytest.mark.parametrize("precision", [es.ES_FP64, es.ES_MIXED32])
+@pytest.mark.parametrize("dims,periodic,radius,shift", [
+    ((16, 16, 20), (1, 1, 1), 6.9, (0.4, -0.3, 0.2)),  # a box as long as two axes allow
+    ((16, 24, 16), (1, 0, 1), 6.8, (-0.4, 0.1, 0.45)),
+    ((32, 32, 32), (1, 1, 1), 14.4, (0.3, 0.3, -0.4)),  # rows beyond the bit words
+])
+def test_forces_of_a_sphere_moved_since_its_mapping(precision, dims, periodic, radius, shift):
+    """Momentum exchange with the links of the last mapping and the present centre:
+    each surface cell is taken at its own nearest image, also where its fluid
+    cell lies past half the axis.  Tolerances as above."""
+    wl = _workload(dims, periodic, radius, 1)
+    wl.x = np.array([[d / 2.0 + 0.2 for d in dims]])
+    wl.v, wl.w = np.array([[0.02, -0.01, 0.015]]), np.array([[0.01, 0.02, -0.015]])
+    g, o = es.Simulation(wl, precision), oracle.Oracle(wl)
+    for s in (o, g):
+        s.map_particles()
+        s.solve(forced_cycles=1)
+    o.body_force()
+    for s in (o, g):
+        s.lbm_step()
+        s.set_particles(wl.x + np.array([shift]), wl.v, wl.w)
+    Fo, To = o.forces()
+    F, T = g.forces()
+    tol = 1e-11 if precision == es.ES_FP64 else 1e-4
+    assert np.linalg.norm(F - Fo) <= tol * np.linalg.norm(Fo)
+    assert np.linalg.norm(T - To) <= tol * max(np.linalg.norm(To), radius * np.linalg.norm(Fo) * 0.1)
+    g.close()
