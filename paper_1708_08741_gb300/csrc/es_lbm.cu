@@ -549,9 +549,10 @@ __global__ void __launch_bounds__(kBatchTileX * kBatchTileY, sizeof(S) == 8 ? 6 
 //  * finds the cells with links a whole row at a time by shifts of those
 //    words, and lists them (a prefix sum: in the order of their box index);
 //  * then works on that list only.
-// Boxes whose rows exceed 32 cells (R > 13) look every cell's neighbours up
-// in the fields, 256 cells at a time.  Fixed order: deterministic.
+// Boxes whose rows exceed 32 cells (R > 13) look the cells near the sphere's
+// surface up in the fields (force_cells_fields).  Fixed order: deterministic.
 constexpr int kForceChunk = 256;   // cells of a chunk (see k_forces_f32)
+constexpr int kForceEach = 8;      // cells a thread looks up in the fields at a time
 constexpr int kForceLinks = 4608;  // links held at once: at least one chunk's 18 x 256
 constexpr int kForceSide = 32;     // longest row (halo included) of the bit words
 constexpr int kForceChunks = (kForceSide - 2) * (kForceSide - 2) * (kForceSide - 2) / kForceChunk + 1;
@@ -729,26 +730,60 @@ __device__ __forceinline__ int force_cells(const Grid& g, const int32_t* __restr
     return total;
 }
 
-// The cells with links among the box's cells t0 .. t0 + 255, from the fields.
+// The cells with links among the box's cells t0 .. t0 + kForceEach T - 1, from
+// the fields, a thread a run of kForceEach of them.  A link runs from a fluid
+// cell to a cell of p within sqrt 2, and p's cells are those within R of its
+// centre at the last mapping, so only cells between R - 1 and R + 1.5 of that
+// centre are looked up (FP32 distances; the bounds are far outside their
+// rounding): a tenth of the box.  (One sphere R = 16 / R = 24: reduced forms
+// 971 / 3,020 us looking at every cell 256 at a time, 278 / 796 so; FP64 1,128 /
+// 3,410 and 326 / 809.)
 template <int T>
 __device__ __forceinline__ int force_cells_fields(const Grid& g, const int32_t* __restrict__ owner,
                                                   const uint8_t* __restrict__ flags, int p, ForceBox& B,
-                                                  const BoxIndex& bi, int t0, int n, int* s_near, unsigned* s_mask) {
-    const int t = t0 + (int)threadIdx.x;
-    unsigned m = 0;
-    if (threadIdx.x < kForceChunk && t < n) {
-        int v[3];
-        bi.at(t, v);
-        m = force_links_fields(g, owner, flags, p, B.lo[0] + v[0], B.lo[1] + v[1], B.lo[2] + v[2]);
+                                                  const BallF& ball, bool shell, float R, const BoxIndex& bi, int t0,
+                                                  int n, int* s_near, unsigned* s_mask) {
+    const float rin = R - 1.0f, rout = R + 1.5f, in2 = rin > 0.0f ? rin * rin : -1.0f, out2 = rout * rout;
+    const int first = t0 + (int)threadIdx.x * kForceEach;
+    unsigned m[kForceEach];
+    int cnt = 0, v[3];
+    bi.at(first < n ? first : 0, v);
+#pragma unroll
+    for (int u = 0; u < kForceEach; u++) {
+        m[u] = 0;
+        if (first + u < n) {
+            const float d2 = shell ? ball.d2(v[0], v[1], v[2]) : in2;
+            if (d2 >= in2 && d2 <= out2)
+                m[u] = force_links_fields(g, owner, flags, p, B.lo[0] + v[0], B.lo[1] + v[1], B.lo[2] + v[2]);
+        }
+        cnt += m[u] != 0;
+        if (++v[0] == B.n[0]) {
+            v[0] = 0;
+            if (++v[1] == B.n[1]) {
+                v[1] = 0;
+                v[2]++;
+            }
+        }
     }
     int total;
-    const int at = block_excl<T>(m ? 1 : 0, B.warp, total);
-    if (m) {
-        s_near[at] = t;
-        s_mask[at] = m;
-    }
+    int at = block_excl<T>(cnt, B.warp, total);
+#pragma unroll
+    for (int u = 0; u < kForceEach; u++)
+        if (m[u]) {
+            s_near[at] = first + u;
+            s_mask[at++] = m[u];
+        }
     __syncthreads();
     return total;
+}
+
+// The mapped centre's ball relative to the box, for that (every thread calls).
+__device__ __forceinline__ bool force_ball(const Grid& g, const double* __restrict__ X, double R, const ForceBox& B,
+                                           BallF& ball) {
+    const int hi[3] = {B.lo[0] + B.n[0] - 1, B.lo[1] + B.n[1] - 1, B.lo[2] + B.n[2] - 1};
+    ball.init_by_axis(g, X, R, B.lo, hi);
+    __syncthreads();
+    return ball.all_ok();
 }
 
 // Half the force and torque of the links m of cell (x, y, z), link by link.
@@ -785,14 +820,16 @@ __device__ __noinline__ void force_links_each(const Grid& g, const DParticle& P,
 // exchange halves of the six components instead of adding all six at each of
 // five steps (8 instructions a warp, not 30), in the warps that have cells.
 // (A sphere R = 4 / 64 spheres R = 6: 62 / 133 us with a lever arm a link, 32
-// / 48 link by link, 23 / 35 now.)
+// / 48 link by link, 23 / 37 now.)
 template <int T>
 __global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __restrict__ part,
                                                  const int32_t* __restrict__ owner, const uint8_t* __restrict__ flags,
                                                  const double* __restrict__ src, double Ex, double Ey, double Ez,
-                                                 double* F, double* T_out, int cells) {
+                                                 const double* __restrict__ mapped, double* F, double* T_out,
+                                                 int cells) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ ForceBox B;
+    __shared__ BallF ball;
     __shared__ double sh[6][32];
     unsigned* own = (unsigned*)dyn;
     unsigned* fluid = own + kForceSide * kForceSide;
@@ -865,8 +902,9 @@ __global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __rest
     if (force_by_rows(B)) {
         consume(force_cells<T>(g, owner, p, B, bi, own, fluid, s_near, s_mask));
     } else {
-        for (int t0 = 0; t0 < n; t0 += kForceChunk) {
-            consume(force_cells_fields<T>(g, owner, flags, p, B, bi, t0, n, s_near, s_mask));
+        const bool shell = force_ball(g, mapped + 9 * p, P.R, B, ball);
+        for (int t0 = 0; t0 < n; t0 += kForceEach * T) {
+            consume(force_cells_fields<T>(g, owner, flags, p, B, ball, shell, (float)P.R, bi, t0, n, s_near, s_mask));
             __syncthreads();
         }
     }
@@ -929,10 +967,11 @@ template <class S, int T>
 __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
     k_forces_f32(Grid g, const DParticle* __restrict__ part, const int32_t* __restrict__ owner,
                  const uint8_t* __restrict__ flags, const S* __restrict__ src, double Ex, double Ey, double Ez,
-                 double* F, double* T_out, int cells) {
+                 const double* __restrict__ mapped, double* F, double* T_out, int cells) {
     using St = Store<S>;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ ForceBox B;
+    __shared__ BallF ball;
     __shared__ float s_X[3], s_V[3], s_W[3];
     __shared__ double s_off[3], s_qeff;
     __shared__ int s_int[6], s_first[kForceChunks], s_count[kForceChunks];
@@ -1110,8 +1149,11 @@ __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
         const int total = force_cells<T>(g, owner, p, B, bi, own, fluid, s_near, s_mask);
         consume(total, 0, (n + kForceChunk - 1) / kForceChunk);
     } else {
-        for (int t0 = 0; t0 < n; t0 += kForceChunk)
-            consume(force_cells_fields<T>(g, owner, flags, p, B, bi, t0, n, s_near, s_mask), t0, 1);
+        const float R = (float)part[p].R;
+        const bool shell = force_ball(g, mapped + 9 * p, part[p].R, B, ball);
+        for (int t0 = 0; t0 < n; t0 += kForceEach * T)
+            consume(force_cells_fields<T>(g, owner, flags, p, B, ball, shell, R, bi, t0, n, s_near, s_mask), t0,
+                    kForceEach * T / kForceChunk);
     }
     // block sum of the six FP32 partials in float-float (fixed order)
     if (threadIdx.x < kForceChunk) {
@@ -1552,13 +1594,16 @@ cudaError_t run_forces(es_ctx* c, int src, double rmax) {
     // they number less than the volume between R - 1.9 and R + 2.4
     const double r = rmax < 13.5 ? rmax : 13.5, ro = r + 2.4, ri = r > 1.9 ? r - 1.9 : 0.0;
     const int room = (int)(4.19 * (ro * ro * ro - ri * ri * ri)) + 32;
-    const int cells = room < kForceChunk ? kForceChunk : (room + 7) / 8 * 8;
+    // (and for a pass over the fields of a larger one)
+    const int least = rmax > 12.0 ? kForceEach * T : kForceChunk;
+    const int cells = room < least ? least : (room + 7) / 8 * 8;
     auto launch = [&](auto* kernel, size_t lists, size_t most) -> cudaError_t {
         // (the attribute belongs to the kernel: the most any context needs)
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
         if (e != cudaSuccess) return e;
         launch_pdl(c, kernel, c->np, T, lists, c->g, (const DParticle*)c->part, (const int32_t*)c->owner,
-                   (const uint8_t*)c->flags, (const S*)c->pdf[src], E[0], E[1], E[2], c->F, c->T, cells);
+                   (const uint8_t*)c->flags, (const S*)c->pdf[src], E[0], E[1], E[2], (const double*)c->mapped,
+                   c->F, c->T, cells);
         return cudaGetLastError();
     };
     const size_t words = (size_t)2 * kForceSide * kForceSide * 4, list = (size_t)cells * 8, most = 12 * 1024 * 8;

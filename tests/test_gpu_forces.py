@@ -75,3 +75,35 @@ def test_forces_of_a_sphere_moved_since_its_mapping(precision, dims, periodic, r
     assert np.linalg.norm(F - Fo) <= tol * np.linalg.norm(Fo)
     assert np.linalg.norm(T - To) <= tol * max(np.linalg.norm(To), radius * np.linalg.norm(Fo) * 0.1)
     g.close()
+
+
+@pytest.mark.parametrize("precision", [es.ES_FP64, es.ES_MIXED32])
+@pytest.mark.parametrize("n_small,big", [(0, 16.0), (340, 16.0), (340, 13.1)])
+def test_forces_from_the_fields(precision, n_small, big):
+    """A sphere whose rows are beyond the bit words, alone (1,024 threads a block)
+    and among many small ones (256); tolerances as above."""
+    dims = (88, 80, 72)
+    wl = _workload(dims, (1, 1, 1), 2.6, 1)
+    c = np.array([44.3, 40.1, 35.8])
+    grid = np.array([(x, y, z) for x in range(4, 88, 8) for y in range(4, 80, 8) for z in range(4, 72, 8)], dtype=float)
+    grid = grid[np.linalg.norm(grid - c, axis=1) > big + 5.0][:n_small]
+    assert len(grid) == n_small
+    n = 1 + n_small
+    rng = np.random.Generator(np.random.PCG64(2))
+    W._set_particles(wl, np.vstack([c[None], grid + 0.3]), np.array([big] + [2.6] * n_small),
+                     np.array([i % 2 for i in range(n)]), np.ones(n), np.full(n, 1.3))
+    wl.v, wl.w = rng.uniform(-0.02, 0.02, (n, 3)), rng.uniform(-0.01, 0.01, (n, 3))
+    g, o = es.Simulation(wl, precision), oracle.Oracle(wl, omp=True)
+    for s in (o, g):
+        s.map_particles()
+        s.solve(forced_cycles=1)
+    o.body_force()
+    for s in (o, g):
+        s.lbm_step()
+    Fo, To = o.forces()
+    F, T = g.forces()
+    tol = 1e-11 if precision == es.ES_FP64 else 1e-4
+    for k in (slice(0, 1), slice(1, n)):  # the large one, and the others
+        assert np.linalg.norm(F[k] - Fo[k]) <= tol * np.linalg.norm(Fo[k])
+        assert np.linalg.norm(T[k] - To[k]) <= tol * max(np.linalg.norm(To[k]), 2.6 * np.linalg.norm(Fo[k]) * 0.1)
+    g.close()
