@@ -75,8 +75,9 @@ __device__ void union_range(const Grid& g, int a, double xo, double xn, double R
 }
 
 // GB300 runs FP64 arithmetic at a small fraction of the FP32 rate, so the
-// per-sphere kernels form their FP64 set-up (box, FP32 ball) once per block
-// in thread 0 and share it; per cell they work in integers and FP32 and
+// per-sphere kernels form their FP64 set-up (box, FP32 ball) an axis a thread
+// and share it (k_flags forms the balls of large spheres in every thread, which
+// its loop over the box outweighs); per cell they work in integers and FP32 and
 // fall back to the FP64 cell-in-sphere test only where FP32 cannot decide.
 
 // Cells whose state flipped since the last solve (obstacle <-> fluid) go to
