@@ -1295,9 +1295,33 @@ __global__ void __launch_bounds__(256) k_moments(long long N, long long ps, cons
 // force of an interior cell is formed from psi as the stream-collide forms
 // it (cells next to obstacles read the stored field, obstacle cells have
 // none), so the whole field is neither stored nor read back.
+//
+// Sums that are not finite (a diverged state) are formed again in FP64: TwoSum
+// makes NaN of an infinity.
 struct Accel3 {
     ff a[3];  // - accel / 2
 };
+
+// Density or velocity of cell c in FP64; h: f_b plus the acceleration, halved.
+template <class S, bool RHO>
+__device__ __noinline__ void moments_fp64(const S* __restrict__ f, size_t ps, size_t N, int c, double h0, double h1,
+                                          double h2, double* __restrict__ out) {
+    double r = 0.0, j[3] = {0.0, 0.0, 0.0};
+    for (int q = 0; q < 19; q++) {
+        const double v = Store<S>::to_f(q, f[q * ps + c]);
+        r += v;
+        j[0] += cx(q) * v;
+        j[1] += cy(q) * v;
+        j[2] += cz(q) * v;
+    }
+    if (RHO) {
+        out[c] = r;
+    } else {
+        out[c] = j[0] - h0;
+        out[N + c] = j[1] - h1;
+        out[2 * N + c] = j[2] - h2;
+    }
+}
 
 template <class S, bool RHO, bool FBPSI>
 __global__ void __launch_bounds__(256) k_moments_ff(Grid g, const S* __restrict__ f, const float* __restrict__ fb,
@@ -1330,6 +1354,8 @@ __global__ void __launch_bounds__(256) k_moments_ff(Grid g, const S* __restrict_
             v = s.value();
         }
         out[c] = 1.0 + widen(v);
+        const float t = __fadd_rn(v.hi, v.lo);
+        if (!(__fsub_rn(t, t) == 0.0f)) moments_fp64<S, true>(f, g.ps, 0, c, 0.0, 0.0, 0.0, out);
     } else {
         ff_acc s[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, d[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
 #pragma unroll
@@ -1347,7 +1373,7 @@ __global__ void __launch_bounds__(256) k_moments_ff(Grid g, const S* __restrict_
         }
         const size_t N = (size_t)g.N;
         float b[3];
-        bool stored = true;
+        bool stored = true, bad = false;
         if constexpr (FBPSI) {
             const uint8_t fl = flags[c];
             stored = (fl & (F_SOLID | F_NEAR19)) == F_NEAR19;
@@ -1373,7 +1399,12 @@ __global__ void __launch_bounds__(256) k_moments_ff(Grid g, const S* __restrict_
                 v = s[a].value();
             v = ff_add(ff_add_f(v, -0.5f * b[a]), acc.a[a]);
             out[a * N + c] = widen(v);
+            const float t = __fadd_rn(v.hi, v.lo);
+            bad |= !(__fsub_rn(t, t) == 0.0f);
         }
+        if (bad)
+            moments_fp64<S, false>(f, g.ps, N, c, 0.5 * b[0] - widen(acc.a[0]), 0.5 * b[1] - widen(acc.a[1]),
+                                   0.5 * b[2] - widen(acc.a[2]), out);
     }
 }
 

@@ -28,3 +28,28 @@ def test_moments_match_populations(precision, dims, periodic):
     np.testing.assert_allclose(u, want, rtol=0, atol=4e-15)
     np.testing.assert_allclose(rho, f.sum(0), rtol=0, atol=4e-15)
     sim.close()
+
+
+@pytest.mark.parametrize("precision", [es.ES_FP64, es.ES_MIXED32, es.ES_MIXED16])
+def test_moments_of_infinite_populations(precision):
+    """A diverged state reads back as the FP64 sums of its populations would:
+    infinities keep their sign, opposite ones give NaN."""
+    wl = W.mixed_box(dims=(24, 20, 16), periodic=(1, 1, 1), levels=2)
+    sim = es.Simulation(wl, precision)
+    sim.step()
+    f = sim.field(es.FIELD_PDF)
+    c, _ = es.lattice()
+    east, west = (next(q for q in range(19) if tuple(c[q]) == v) for v in ((1, 0, 0), (-1, 0, 0)))
+    cells = [(1, 2, 3), (4, 5, 6), (7, 8, 9)]
+    f[(east,) + cells[0]] = np.inf
+    f[(west,) + cells[1]] = np.inf
+    f[(east,) + cells[2]], f[(west,) + cells[2]] = np.inf, -np.inf
+    sim.set_field(es.FIELD_PDF, f)
+    rho, u = sim.field(es.FIELD_RHO), sim.field(es.FIELD_U)
+    assert rho[cells[0]] == np.inf and rho[cells[1]] == np.inf and np.isnan(rho[cells[2]])
+    assert u[0][cells[0]] == np.inf and u[0][cells[1]] == -np.inf and u[0][cells[2]] == np.inf
+    rest = np.ones(rho.shape, dtype=bool)
+    for k in cells:
+        rest[k] = False
+    assert np.isfinite(rho[rest]).all() and np.isfinite(u[:, rest]).all()
+    sim.close()
