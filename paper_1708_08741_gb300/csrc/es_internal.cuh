@@ -288,6 +288,14 @@ inline bool split_level(const es_ctx* c, int l) { return (l == 0 && c->rb0) || (
 // separate launches over all SMs (32^3: 2.7 us against 5; 64^3 would be bound
 // by the pipes at about 20 us, against 15 launched).
 constexpr long long kTailCells32 = 1 << 18, kTailCells64 = 40 * 1024;
+// A block has whole planes, so a flat level leaves most of the 16 idle: no block
+// may have more cells than that makes of a full cluster, and of the coarsest
+// level, which takes most of the sweeps, no more than these, where the block
+// needs as long as a launched half sweep (FP32 2.0 us, FP64 2.4).  32 sweeps of
+// 128 x 128 x 4 in FP32: 220 us in four blocks, 150 launched; 64 x 64 x 8 in
+// FP64: 330 us in eight, 160 launched; 64^3 with spheres: 253 in 16, 231.
+constexpr long long kTailBlock32 = kTailCells32 / 16, kTailBlock64 = kTailCells64 / 16;
+constexpr long long kTailLast32 = 10 * 1024, kTailLast64 = 2 * 1024;
 
 constexpr int kFlipCap = 1 << 16;
 // cells of the local correction's region and ring: at most 16 flipped cells, boxes of radius 9

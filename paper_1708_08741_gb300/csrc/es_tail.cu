@@ -728,6 +728,9 @@ bool tail_layout(const es_params& P, int l0, TailPlan& T) {
         // a block (the coarsest level has none)
         S.zs = l + 1 < T.n ? 2 * ((S.nz / 2 + T.blocks - 1) / T.blocks)
                            : (T.solo ? S.nz : (S.nz + T.blocks - 1) / T.blocks);
+        const long long block = (long long)S.nx * S.ny * S.zs;  // cells of a slab
+        if (block > (ts == 8 ? kTailBlock64 : kTailBlock32)) return false;
+        if (l + 1 == T.n && block > (ts == 8 ? kTailLast64 : kTailLast32)) return false;
         S.plane = S.nxp * S.ny;
         if ((long long)S.zs * S.plane * (2 * ts + 2) * 2 > (long long)kTailSmem) return false;
         S.ploc = S.zs * S.plane;

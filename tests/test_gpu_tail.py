@@ -144,3 +144,37 @@ def test_cluster_levels_give_the_same_bits(dims, periodic, levels, nu1, nu2, ome
         out.append(sim.field(es.FIELD_PSI))
         sim.close()
     np.testing.assert_array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("precision,dims,levels,want", [
+    (es.ES_MIXED32, (64, 160, 16), 1, [0]),    # 10,240 cells of the coarsest level in each of 16 blocks
+    (es.ES_MIXED32, (64, 168, 16), 1, []),
+    (es.ES_MIXED32, (128, 128, 4), 1, []),     # four blocks
+    (es.ES_MIXED32, (128, 128, 16), 2, [1]),   # 64 x 64 x 8
+    (es.ES_MIXED32, (64, 64, 64), 2, [0]),     # above it 16,384 a block
+    (es.ES_MIXED32, (64, 72, 56), 2, [1]),
+    (es.ES_FP64, (32, 64, 16), 1, [0]),        # 2,048 cells
+    (es.ES_FP64, (32, 66, 16), 1, []),
+    (es.ES_FP64, (64, 64, 8), 1, []),
+    (es.ES_FP64, (40, 32, 24), 2, [0]),        # above it 2,560
+    (es.ES_FP64, (40, 36, 24), 2, [1]),
+])
+def test_flat_levels_are_launched(precision, dims, levels, want):
+    """Which levels the cluster takes by the cells of a block's planes; the same
+    V-cycle either way: the bits in FP32, 1e-12 in FP64 (as above)."""
+    wl = W.Workload(name="flat", dims=list(dims), periodic=(1, 1, 1), tau=0.8, kappa=0.3, eps=1.0,
+                    E_ext=(0.0, 0.0, 0.0), levels=levels, coarse_sweeps=12)
+    psi0 = W.random_fields(dims[0] * dims[1] * dims[2], 5).reshape(dims[::-1])
+    out = []
+    for lists in (0, 1):
+        sim = es.Simulation(wl, precision, overrides=dict(near_list_cells=lists))
+        sim.map_particles()
+        assert _levels_in_cluster(sim) == (want if lists == 0 else [])
+        sim.set_field(es.FIELD_PSI, psi0)
+        sim.solve(forced_cycles=2)
+        out.append(sim.field(es.FIELD_PSI))
+        sim.close()
+    if precision == es.ES_FP64:
+        assert rel_l2(out[0], out[1]) < 1e-12
+    else:
+        np.testing.assert_array_equal(out[0], out[1])
