@@ -123,13 +123,15 @@ typedef struct {
     int fine_layout;    /* ES_LAYOUT_AUTO (0, default) or ES_LAYOUT_NATURAL: storage of
                            the finest level's multigrid correction and right-hand
                            side (see below); both give the same iteration          */
-    int near_list_cells; /* multigrid levels (dims[0] % 4 == 0 on the level) with more
-                           cells than this smooth their near-boundary cells in
-                           separate passes over per-colour cell lists, the others
-                           inside the smoothing kernel; the same sweep either way.
-                           0 selects the default ES_NEAR_LIST_CELLS; < 0 is
-                           ES_EINVAL.  (The colour-split finest level always uses
-                           the lists.)                                             */
+    int near_list_cells; /* reduced forms: multigrid levels (dims[0] % 4 == 0 on the
+                           level) with more cells than this smooth their near-boundary
+                           cells in separate passes over per-colour cell lists, the
+                           others inside the smoothing kernel; the same sweep either
+                           way.  (The colour-split finest level always uses the
+                           lists.)  All forms: only levels of at most this many cells
+                           may go to the one launch of the coarse levels, so a small
+                           value keeps every level out of it.  0 selects the default
+                           ES_NEAR_LIST_CELLS; < 0 is ES_EINVAL.                    */
     int sweep_staging;  /* colour-split finest level, rows of up to 512 cells:
                            ES_STAGE_REGISTERS (0, default) each thread loads its
                            neighbours' rows into registers, marching through z
@@ -395,7 +397,9 @@ int es_alu_peak(int precision, double* gflops);
 /* Number of CUDA kernels this context has launched so far (telemetry). */
 uint64_t es_kernel_launches(const es_ctx* ctx);
 
-/* Device bytes a context with these parameters and n particles will hold. */
+/* Device bytes that a context with these parameters and n particles holds at
+ * most.  (ES_FP64: the near-cell lists, 4 bytes a cell of every level, are
+ * counted but not allocated, since no FP64 kernel reads them.) */
 size_t es_device_bytes(const es_params* params, int n);
 
 /* Message of the last failure on ctx (or of the last failed es_create when
