@@ -283,19 +283,24 @@ inline int near_grid_x(const es_ctx* c) {
 inline bool split_level(const es_ctx* c, int l) { return (l == 0 && c->rb0) || (l == 1 && c->rb1); }
 
 // Levels of up to this many cells (and what follows them) go to k_tail: in
-// FP32 what the shared memory of 16 blocks holds (64^3: a half sweep 2.3 us
-// there, about 4 launched); in FP64 what 16 SMs' FP64 pipes finish sooner than
-// separate launches over all SMs (32^3: 2.7 us against 5; 64^3 would be bound
-// by the pipes at about 20 us, against 15 launched).
-constexpr long long kTailCells32 = 1 << 18, kTailCells64 = 40 * 1024;
+// FP32 what the shared memory of 16 blocks holds (64^3 as the first of four
+// levels: 105 us a V-cycle, 108 with the cluster from 32^3 on; 128^3 184 / 187,
+// 256^3 508 / 514); in FP64 what 16 SMs' FP64 pipes finish sooner than separate
+// launches over all SMs (32^3 in it / launched: 117 / 109 us a V-cycle, 32
+// sweeps of it as the coarsest level 201 / 154; 24^3 97 / 95 and 157 / 149).
+constexpr long long kTailCells32 = 1 << 18, kTailCells64 = 16 * 1024;
 // A block has whole planes, so a flat level leaves most of the 16 idle: no block
-// may have more cells than that makes of a full cluster, and of the coarsest
-// level, which takes most of the sweeps, no more than these, where the block
-// needs as long as a launched half sweep (FP32 2.0 us, FP64 2.4).  32 sweeps of
+// may have more cells than that makes of a full cluster, and in FP32, of the
+// coarsest level, which takes most of the sweeps, no more than the last, where
+// the block needs as long as a launched half sweep (about 2 us); a coarsest level
+// that a single block would solve otherwise is not refused.  32 sweeps of
 // 128 x 128 x 4 in FP32: 220 us in four blocks, 150 launched; 64 x 64 x 8 in
 // FP64: 330 us in eight, 160 launched; 64^3 with spheres: 253 in 16, 231.
 constexpr long long kTailBlock32 = kTailCells32 / 16, kTailBlock64 = kTailCells64 / 16;
-constexpr long long kTailLast32 = 10 * 1024, kTailLast64 = 2 * 1024;
+constexpr long long kTailLast32 = 10 * 1024, kTailLast64 = kTailBlock64;
+// Shared memory up to which one block solves the coarsest level (k_coarse_lists,
+// k_coarse_solve).
+constexpr int kCoarseSmem = 200 * 1024;
 
 constexpr int kFlipCap = 1 << 16;
 // cells of the local correction's region and ring: at most 16 flipped cells, boxes of radius 9

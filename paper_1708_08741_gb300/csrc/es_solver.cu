@@ -3267,7 +3267,7 @@ size_t coarse_cells(const es_ctx* c) { return (size_t)c->ln[c->L - 1][0] * c->ln
 
 bool coarse_by_lists(const es_ctx* c, size_t tsize) {
     const int* m = c->ln[c->L - 1];
-    return m[0] <= 256 && m[1] <= 256 && m[2] <= 256 && coarse_cells(c) * (3 * tsize + 4) <= 200 * 1024;
+    return m[0] <= 256 && m[1] <= 256 && m[2] <= 256 && coarse_cells(c) * (3 * tsize + 4) <= kCoarseSmem;
 }
 
 size_t coarse_smem_bytes(const es_ctx* c, size_t tsize) {
@@ -3542,7 +3542,7 @@ cudaError_t vcycle_impl(es_ctx* c, int l, int warm) {
         }
         if (l == c->L - 1) {
             size_t sm = coarse_smem_bytes(c, sizeof(T));
-            if (sm <= 200 * 1024) {
+            if (sm <= kCoarseSmem) {
                 ProfScope ps(c, "coarse_solve", l, nl * (2.0 * ts + 1.0));
                 if (coarse_by_lists(c, sizeof(T)))
                     launch_pdl(c, k_coarse_lists<T>, 1, 1024, sm, L, st, rhs, e, c->P.coarse_sweeps, omega);
@@ -3697,9 +3697,9 @@ void set_bulk_smem(es_ctx* c) {
 template <class T>
 void set_coarse_smem(const es_ctx* c) {
     size_t sm = coarse_smem_bytes(c, sizeof(T));
-    if (sm > 48 * 1024 && sm <= 200 * 1024) {
-        cudaFuncSetAttribute(k_coarse_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_coarse_lists<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (sm > 48 * 1024 && sm <= kCoarseSmem) {
+        cudaFuncSetAttribute(k_coarse_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoarseSmem);
+        cudaFuncSetAttribute(k_coarse_lists<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoarseSmem);
     }
 }
 
@@ -4417,7 +4417,7 @@ __global__ void __launch_bounds__(kLocalThreads) k_local_solve(Level<float> L, c
 
 int coarse_divides(const es_ctx* c) {
     const size_t t = mixed(c) ? sizeof(float) : sizeof(double);
-    return coarse_by_lists(c, t) ? 0 : (coarse_smem_bytes(c, t) <= 200 * 1024 ? 1 : 2);
+    return coarse_by_lists(c, t) ? 0 : (coarse_smem_bytes(c, t) <= kCoarseSmem ? 1 : 2);
 }
 
 // Grid of a marching residual pass over a level of nz planes with (gx, gy)

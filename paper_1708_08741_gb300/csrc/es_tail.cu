@@ -729,8 +729,12 @@ bool tail_layout(const es_params& P, int l0, TailPlan& T) {
         S.zs = l + 1 < T.n ? 2 * ((S.nz / 2 + T.blocks - 1) / T.blocks)
                            : (T.solo ? S.nz : (S.nz + T.blocks - 1) / T.blocks);
         const long long block = (long long)S.nx * S.ny * S.zs;  // cells of a slab
-        if (block > (ts == 8 ? kTailBlock64 : kTailBlock32)) return false;
-        if (l + 1 == T.n && block > (ts == 8 ? kTailLast64 : kTailLast32)) return false;
+        const bool last = l + 1 == T.n;
+        // (a coarsest level that one block would hold otherwise, k_coarse_solve,
+        // is here in any case)
+        if (!(last && Nc * (2 * ts + 1) <= kCoarseSmem) &&
+            block > (ts == 8 ? (last ? kTailLast64 : kTailBlock64) : (last ? kTailLast32 : kTailBlock32)))
+            return false;
         S.plane = S.nxp * S.ny;
         if ((long long)S.zs * S.plane * (2 * ts + 2) * 2 > (long long)kTailSmem) return false;
         S.ploc = S.zs * S.plane;

@@ -105,8 +105,8 @@ def test_periodic_axis_of_one_cell(precision, dims, axis):
 
 
 @pytest.mark.parametrize("precision,dims,levels,lists,want", [
-    (es.ES_FP64, (32, 32, 32), 3, 0, [0]),
-    (es.ES_FP64, (64, 64, 64), 3, 0, [1]),
+    (es.ES_FP64, (32, 32, 32), 3, 0, [1]),
+    (es.ES_FP64, (24, 20, 28), 2, 0, [0]),
     (es.ES_MIXED32, (64, 64, 64), 4, 0, [0]),
     (es.ES_MIXED32, (96, 96, 48), 4, 0, [1]),
     (es.ES_MIXED32, (64, 64, 64), 4, 1, []),
@@ -153,11 +153,13 @@ def test_cluster_levels_give_the_same_bits(dims, periodic, levels, nu1, nu2, ome
     (es.ES_MIXED32, (128, 128, 16), 2, [1]),   # 64 x 64 x 8
     (es.ES_MIXED32, (64, 64, 64), 2, [0]),     # above it 16,384 a block
     (es.ES_MIXED32, (64, 72, 56), 2, [1]),
-    (es.ES_FP64, (32, 64, 16), 1, [0]),        # 2,048 cells
-    (es.ES_FP64, (32, 66, 16), 1, []),
+    (es.ES_FP64, (32, 32, 16), 1, [0]),        # 1,024 cells
+    (es.ES_FP64, (32, 34, 16), 1, []),
     (es.ES_FP64, (64, 64, 8), 1, []),
-    (es.ES_FP64, (40, 32, 24), 2, [0]),        # above it 2,560
-    (es.ES_FP64, (40, 36, 24), 2, [1]),
+    (es.ES_FP64, (16, 32, 32), 2, [0]),
+    (es.ES_FP64, (20, 28, 28), 2, [1]),        # (1,120)
+    (es.ES_FP64, (96, 80, 12), 2, [1]),        # 48 x 40 x 6: one block would solve it
+    (es.ES_FP64, (64, 64, 2), 1, [0]),
 ])
 def test_flat_levels_are_launched(precision, dims, levels, want):
     """Which levels the cluster takes by the cells of a block's planes; the same
