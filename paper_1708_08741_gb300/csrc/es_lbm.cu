@@ -960,7 +960,7 @@ __global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __rest
 //    c_q over a cell's links, sum S and sum rel x S (rel: the cell's
 //    coordinates relative to the box, minimum image), from which sum 2 w_q c_q
 //    and sum 2 w_q (x_s - X) x c_q follow in FP64 at the end (c_q x c_q = 0).
-// (2,880 spheres R = 5 / 64 spheres R = 6: 277 / 102 us before, 216 / 25
+// (2,880 spheres R = 5 / 64 spheres R = 6: 277 / 102 us before, 221 / 25
 // now: a sphere R = 6 did not fit the owner tile and looked every cell's
 // neighbours up one by one, and every link made four shared-memory atomics.)
 template <class S, int T>

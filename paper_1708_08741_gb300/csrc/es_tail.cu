@@ -26,11 +26,13 @@
 // release fence, whatever the cluster's size), one distributed-shared-memory
 // read (264 cycles) and the arithmetic (FP64: four 64-cycle operations in a
 // row, and on 32^3 the FP64 pipe: six or seven instructions a warp at 17
-// cycles each).  Measured per half sweep, 16 blocks: FP32 0.16 us (16^3, one
-// block, no cluster barrier), 0.6 us (32^3), 2.3 us (64^3); FP64 0.84 us (16^3),
-// 2.6 us (32^3); a launch of its own took 2.7 to 5 us.  V-cycle with its
-// correction and residual, every level launched / with it: FP32 128^3 250 /
-// 170 us, 96^3 208 / 150, 256^3 526 / 485, 32^3 134 / 64; FP64 32^3 202 / 118 us.
+// cycles each).  Measured per half sweep, 16 blocks: FP32 0.45 us (16^3, one
+// block, no cluster barrier), 0.72 us (32^3), 1.7 us (48^3), 3.1 us (64^3); FP64
+// 0.82 us (16^3), 2.75 us (32^3, now launched: 2.3 us); a launch of its own takes
+// 1.8 us and more on such levels, and some 3 us next to obstacles.  V-cycle with
+// its correction and residual, every level launched (when this was made) / with
+// it: FP32 128^3 250 / 183 us, 96^3 208 / 141, 256^3 526 / 508, 32^3 134 / 69;
+// FP64 32^3 202 / 109 us (16^3 and 8^3 in it).
 // Boundary planes pushed to the neighbours with an mbarrier each, in place of
 // the cluster barrier, were no faster (FP64 32^3 107 / 111 us a tail, FP32
 // 96^3 150 / 164 a V-cycle): that round trip is as long.
