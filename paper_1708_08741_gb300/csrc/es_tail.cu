@@ -26,13 +26,13 @@
 // release fence, whatever the cluster's size), one distributed-shared-memory
 // read (264 cycles) and the arithmetic (FP64: four 64-cycle operations in a
 // row, and on 32^3 the FP64 pipe: six or seven instructions a warp at 17
-// cycles each).  Measured per half sweep, 16 blocks: FP32 0.45 us (16^3, one
-// block, no cluster barrier), 0.72 us (32^3), 1.7 us (48^3), 3.1 us (64^3); FP64
-// 0.82 us (16^3), 2.75 us (32^3, now launched: 2.3 us); a launch of its own takes
-// 1.8 us and more on such levels, and some 3 us next to obstacles.  V-cycle with
-// its correction and residual, every level launched (when this was made) / with
-// it: FP32 128^3 250 / 183 us, 96^3 208 / 141, 256^3 526 / 508, 32^3 134 / 69;
-// FP64 32^3 202 / 109 us (16^3 and 8^3 in it).
+// cycles each).  Measured per half sweep, 16 blocks: FP32 0.18 us (8^3) and 0.42
+// (16^3, one block, no cluster barrier), 0.62 us (32^3), 1.6 us (48^3), 2.8 us
+// (64^3); FP64 0.82 us (16^3); a launch of its own takes 1.8 us and more on such
+// levels, and some 3 us next to obstacles.  V-cycle with its correction and
+// residual, every level launched (when this was made) / with it: FP32 128^3
+// 250 / 185 us, 96^3 208 / 139, 256^3 526 / 508, 32^3 134 / 62; FP64 32^3 202 /
+// 109 us (16^3 and 8^3 in it).
 // Boundary planes pushed to the neighbours with an mbarrier each, in place of
 // the cluster barrier, were no faster (FP64 32^3 107 / 111 us a tail, FP32
 // 96^3 150 / 164 a V-cycle): that round trip is as long.
@@ -53,9 +53,10 @@ constexpr int kTailCluster = 16;          // most blocks of the cluster
 constexpr size_t kTailSmem = 220 * 1024;  // most dynamic shared memory of a block
 // A cell's code: the six faces as near_faces has them (two bits each) and in
 // the top four bits 6 + (faces that raise the diagonal) - (faces that lower it);
-// kTailOff: not an unknown cell.  FP32: kTailOdd there means that the diagonal
-// formed face by face differs from diag0 plus that sum by rounding.
-constexpr unsigned kTailOff = 0xFFFFu, kTailInner = 6u << 12, kTailOdd = 13u;
+// kTailOff: not an unknown cell.  FP32, levels that divide: kTailOdd there means
+// that the diagonal formed face by face differs from diag0 plus that sum by
+// rounding, kTailEven a near-boundary cell whose sum is 0 (6: interior ones).
+constexpr unsigned kTailOff = 0xFFFFu, kTailInner = 6u << 12, kTailOdd = 13u, kTailEven = 14u;
 
 struct TailShape {
     int nx, ny, nz;
@@ -81,6 +82,7 @@ struct TailLevel {
     TailShape s;
     T h2, inv_h2, diag0;
     int how;       // TailHow (FP64: by table)
+    int odd;       // kTailOdd may occur
     int red_only;  // the restriction takes the red residuals only
     int pairs;     // and adds the two children of a fine row first (k_restrict_v)
     // omega != 1, FP32: omega g enters the sum (1 - omega) e + omega g unrounded
@@ -94,7 +96,7 @@ struct TailCodes {
     const uint8_t* st[ES_MAXLEV];
     int n, blocks, bytes;  // levels, blocks, code bytes of a block
     int per[3], pot_bc[6];
-    float diag0[ES_MAXLEV];  // 0: no kTailOdd
+    float diag0[ES_MAXLEV];  // 0: no kTailOdd, kTailEven
     unsigned char* out;
 };
 
@@ -149,12 +151,6 @@ struct Codes {
         }
     }
     __device__ __forceinline__ unsigned at(int k) const { return (w[k >> 1] >> (16 * (k & 1))) & 0xFFFFu; }
-    __device__ __forceinline__ bool odd() const {  // (a cell with kTailOdd)
-        bool any = false;
-#pragma unroll
-        for (int k = 0; k < kSpan<T>; k++) any |= (at(k) >> 12) == kTailOdd;
-        return any;
-    }
     __device__ __forceinline__ bool inner() const {
         if constexpr (kSpan<T> == 4)
             return w[0] == (kTailInner | (kTailInner << 16)) && w[1] == w[0];
@@ -235,7 +231,7 @@ struct Around {
 
 // The diagonal of a cell that is unknown, face by face as near_sums forms it
 // (in FP32 diag0 + 1 + 1 - 1 is not always diag0 + 1).
-__device__ __forceinline__ float code_diag(float diag0, unsigned c) {
+__device__ __noinline__ float code_diag(float diag0, unsigned c) {
     float d = diag0;
 #pragma unroll
     for (int f = 0; f < 6; f++) {
@@ -245,59 +241,85 @@ __device__ __forceinline__ float code_diag(float diag0, unsigned c) {
     return d;
 }
 
-// The inverse diagonals of a span's cells (0 at those that are not unknown) and,
-// in FP32, the diagonals, from the level's tables.
+// A level's tables, by the top four bits of a code: inverse diagonals (0 at cells
+// that are not unknown), diagonals, and in FP32 the inverses again at the cells
+// that take the quotient (else 0).
 template <class T>
-struct Diagonals {
-    Span<T> y, d;
-    __device__ __forceinline__ Diagonals(const T* inv, const T* diag, const Codes<T>& cd) {
-#pragma unroll
-        for (int k = 0; k < kSpan<T>; k++) {
-            y.v[k] = inv[cd.at(k) >> 12];
-            if (sizeof(T) == 4) d.v[k] = diag[cd.at(k) >> 12];
-        }
-    }
+struct Tables {
+    const T *inv, *diag, *cor;
 };
 
-// n over the diagonal for a span's cells (see TailHow).  The quotient comes
-// from the tabulated inverse y = RN(1 / d): n y is within two ulp of n / d, one
-// correction by the remainder n - q d brings it within one, and from there the
-// next gives the correctly rounded quotient (P. Markstein, Computation of
-// elementary functions on the IBM RISC System/6000 processor, IBM J. Res. Dev.
-// 34, 1990): the bits of a division at four multiply-adds a near-boundary cell
-// (a 192^3 solve from zero: 7 % over products alone, 13 % with divisions).
+// The inverse diagonals of a span's cells.
 template <class T>
-__device__ __forceinline__ Span<T> quotients(const TailLevel<T>& L, const Span<T>& n, const Diagonals<T>& D,
-                                             const Codes<T>& cd) {
+__device__ __forceinline__ Span<T> inverses(const Tables<T>& B, const Codes<T>& cd) {
+    Span<T> y;
+#pragma unroll
+    for (int k = 0; k < kSpan<T>; k++) y.v[k] = B.inv[cd.at(k) >> 12];
+    return y;
+}
+
+// (Rare paths are calls: the kernel's time on the smallest levels is also that of
+// fetching its instructions.)
+__device__ __noinline__ Span<float> odd_diagonals(float diag0, Span<float> d, Codes<float> cd) {
+    for (int k = 0; k < kSpan<float>; k++)
+        if ((cd.at(k) >> 12) == kTailOdd) d.v[k] = code_diag(diag0, cd.at(k));
+    return d;
+}
+__device__ __noinline__ Span<float> odd_inverses(Span<float> d, Span<float> y, Codes<float> cd) {
+    for (int k = 0; k < kSpan<float>; k++)
+        if ((cd.at(k) >> 12) == kTailOdd) y.v[k] = __fdiv_rn(1.0f, d.v[k]);
+    return y;
+}
+__device__ __noinline__ Span<float> odd_quotients(float diag0, Span<float> n, Span<float> q, Codes<float> cd) {
+    for (int k = 0; k < kSpan<float>; k++)
+        if ((cd.at(k) >> 12) == kTailOdd) q.v[k] = n.v[k] / code_diag(diag0, cd.at(k));
+    return q;
+}
+
+// n over the diagonal for a span's cells (see TailHow).  The quotient comes
+// from the tabulated inverse y = RN(1 / d): q = RN(n y) is within 1.5 ulp of n / d
+// (within one unless n < d), and q + (n - q d) y then rounds to n / d (P.
+// Markstein, Computation of elementary functions on the IBM RISC System/6000
+// processor, IBM J. Res. Dev. 34, 1990, for a q within one ulp; beyond it n / d
+// would have to lie within 1.5 2^-23 ulp of a midpoint, which puts n and d
+// within three ulp of 2, where it does not; 8e9 pairs tried).  So the bits of a
+// division for two multiply-adds a near-boundary cell.
+template <class T>
+__device__ __forceinline__ Span<T> quotients(const TailLevel<T>& L, int how, int odd, const Tables<T>& B,
+                                             const Span<T>& n, const Span<T>& y, const Codes<T>& cd) {
     Span<T> q;
 #pragma unroll
-    for (int k = 0; k < kSpan<T>; k++) q.v[k] = n.v[k] * D.y.v[k];
+    for (int k = 0; k < kSpan<T>; k++) q.v[k] = n.v[k] * y.v[k];
     if constexpr (sizeof(T) == 4) {
-        if (L.how == kByTable || (L.how == kNearQuotient && cd.inner())) return q;
+        if (how == kByTable || (how == kNearQuotient && cd.inner())) return q;
 #pragma unroll
         for (int k = 0; k < kSpan<T>; k++) {
-            const float d = D.d.v[k], y = D.y.v[k];
-            float c = __fmaf_rn(__fmaf_rn(-q.v[k], d, n.v[k]), y, q.v[k]);
-            c = __fmaf_rn(__fmaf_rn(-c, d, n.v[k]), y, c);
-            if (L.how == kQuotient || cd.at(k) != kTailInner) q.v[k] = c;
+            const unsigned i = cd.at(k) >> 12;
+            const T cor = how == kNearQuotient && i == 6u ? (T)0 : y.v[k];  // (as Tables::cor)
+            q.v[k] = __fmaf_rn(__fmaf_rn(-q.v[k], B.diag[i], n.v[k]), cor, q.v[k]);
         }
-        if (cd.odd()) {
-#pragma unroll
-            for (int k = 0; k < kSpan<T>; k++)
-                if ((cd.at(k) >> 12) == kTailOdd) q.v[k] = n.v[k] / code_diag(L.diag0, cd.at(k));
-        }
+        if (odd) q = odd_quotients(L.diag0, n, q, cd);
     }
     return q;
 }
 
 // (1 - omega) e + omega g
-__device__ __forceinline__ double relaxed(const TailLevel<double>&, double omega, double e, double g, unsigned) {
-    return (1.0 - omega) * e + omega * g;
+__device__ __forceinline__ Span<double> relaxed(const TailLevel<double>&, double omega, Span<double> e, Span<double> g,
+                                                const Codes<double>&) {
+    return {{(1.0 - omega) * e.v[0] + omega * g.v[0]}};
 }
-__device__ __forceinline__ float relaxed(const TailLevel<float>& L, float omega, float e, float g, unsigned c) {
+__device__ __noinline__ Span<float> relaxed_as(int inner, int near, float omega, Span<float> e, Span<float> g,
+                                               Codes<float> cd) {
     const float keep = 1.0f - omega;
-    return c == kTailInner ? (L.fuse_inner ? __fmaf_rn(omega, g, __fmul_rn(keep, e)) : __fmaf_rn(keep, e, __fmul_rn(omega, g)))
-                           : (L.fuse_near ? __fmaf_rn(omega, g, __fmul_rn(keep, e)) : __fmaf_rn(keep, e, __fmul_rn(omega, g)));
+    for (int k = 0; k < kSpan<float>; k++) {
+        const bool fuse = cd.at(k) == kTailInner ? inner : near;
+        e.v[k] = fuse ? __fmaf_rn(omega, g.v[k], __fmul_rn(keep, e.v[k])) : __fmaf_rn(keep, e.v[k], __fmul_rn(omega, g.v[k]));
+    }
+    return e;
+}
+__device__ __forceinline__ Span<float> relaxed(const TailLevel<float>& L, float omega, Span<float> e, Span<float> g,
+                                               const Codes<float>& cd) {
+    return relaxed_as(L.fuse_inner, L.fuse_near, omega, e, g, cd);
 }
 
 // The sums of the unknown neighbours of a span's cells, in the order x left,
@@ -339,61 +361,89 @@ __device__ __forceinline__ Span<T> neighbour_sums(const T* e, const Around<T>& a
     return o;
 }
 
-// `sweeps` red-black sweeps of a level; inv: the level's inverse diagonals
-// (inv[15] = 0 keeps e = 0 at cells that are not unknown).  Where every
-// thread has at most one span of a colour, what the sweeps do not change --
-// the addresses, codes, inverse diagonals and h^2 r -- stays in registers.
+// `sweeps` red-black sweeps of a level (B.inv[15] = 0 keeps e = 0 at cells that
+// are not unknown).  Where every thread has at most one span of a colour, what
+// the sweeps do not change -- the addresses, codes, diagonals, their inverses
+// and h^2 r -- stays in registers (FP32 32^3: a half sweep 0.62 us; with the
+// quotient's operands looked up in each of them 0.71, products alone 0.60).
 template <class T>
-__device__ __forceinline__ void tail_smooth(const TailLevel<T>& L, const Slab<T>& s, const T* inv, const T* diag,
+__device__ __forceinline__ void tail_smooth(const TailLevel<T>& L, const Slab<T>& s, const Tables<T>& B,
                                             int sweeps, T omega, bool solo, cg::cluster_group& cl) {
     constexpr int W = kSpan<T>;
     const TailShape& S = L.s;
     const bool gs = omega == (T)1;
     const T h2 = L.h2;
+    const int how = L.how, odd = L.odd;
     if (sweeps == 0) return;
-    if (S.ny * S.zs <= S.rpi) {
+    // (FP32: not with over-relaxation)
+    bool resident = S.ny * S.zs <= S.rpi;
+    if (resident) {
         const bool on = s.row0 < s.nrows;
         const int row = on ? s.row0 : 0, y = on ? s.y0 : 0, lz = on ? s.lz0 : 0;
         const Around<T> at0(S, s, 0, row, y, lz), at1(S, s, 1, row, y, lz);
         const int own = row * S.nxp + s.j0;
         const Codes<T> cd0(s.code + own), cd1(s.code + S.ploc + own);
         Span<T> r0 = ldspan(s.r + own), r1 = ldspan(s.r + S.ploc + own);
-        const Diagonals<T> i0(inv, diag, cd0), i1(inv, diag, cd1);
+        Span<T> i0 = inverses<T>(B, cd0), i1 = inverses<T>(B, cd1);
+        Span<T> d0, d1, c0, c1;  // (FP32: diagonals, and inverses where the quotient is taken)
+        bool other = false;
 #pragma unroll
         for (int k = 0; k < W; k++) {
             r0.v[k] *= h2;  // (exact: a power of two)
             r1.v[k] *= h2;
-            if (W == 1) {  // (FP64: an operation less in each half sweep's chain)
-                r0.v[k] *= i0.y.v[k];
-                r1.v[k] *= i1.y.v[k];
+            if constexpr (W == 1) {  // (FP64: an operation less in each half sweep's chain)
+                r0.v[k] *= i0.v[k];
+                r1.v[k] *= i1.v[k];
+            } else {
+                d0.v[k] = B.diag[cd0.at(k) >> 12];
+                d1.v[k] = B.diag[cd1.at(k) >> 12];
+                c0.v[k] = how == kByTable ? (T)0 : B.cor[cd0.at(k) >> 12];
+                c1.v[k] = how == kByTable ? (T)0 : B.cor[cd1.at(k) >> 12];
+                other |= (cd0.at(k) >> 12) == kTailOdd || (cd1.at(k) >> 12) == kTailOdd;
             }
         }
-        auto half = [&](const Around<T>& at, const Codes<T>& cd, const Span<T>& r, const Diagonals<T>& id, T* e) {
+        if constexpr (W == 4) {
+            resident = gs;
+            if (odd && __syncthreads_or(other)) {  // (rare)
+                d0 = odd_diagonals(L.diag0, d0, cd0);
+                d1 = odd_diagonals(L.diag0, d1, cd1);
+                i0 = odd_inverses(d0, i0, cd0);
+                i1 = odd_inverses(d1, i1, cd1);
+                c0 = odd_inverses(d0, c0, cd0);
+                c1 = odd_inverses(d1, c1, cd1);
+            }
+        }
+        auto half = [&](const Around<T>& at, const Codes<T>& cd, const Span<T>& r, const Span<T>& id,
+                        const Span<T>& dg, const Span<T>& cor, T* e) {
             if (on) {
                 const Span<T> o = neighbour_sums<T>(s.e, at, cd);
-                Span<T> c, g;
-                if (!gs) c = ldspan(e);
+                Span<T> g;
                 if constexpr (W == 1) {
-                    g.v[0] = o.v[0] * id.y.v[0] + r.v[0];
+                    g.v[0] = o.v[0] * id.v[0] + r.v[0];
+                    if (!gs) g = relaxed(L, omega, ldspan(e), g, cd);
                 } else {
+                    // (as quotients, all in registers and without a branch)
 #pragma unroll
-                    for (int k = 0; k < W; k++) g.v[k] = r.v[k] + o.v[k];
-                    g = quotients<T>(L, g, id, cd);
+                    for (int k = 0; k < W; k++) {
+                        const T n = r.v[k] + o.v[k];
+                        g.v[k] = n * id.v[k];
+                        g.v[k] = __fmaf_rn(__fmaf_rn(-g.v[k], dg.v[k], n), cor.v[k], g.v[k]);
+                    }
                 }
-#pragma unroll
-                for (int k = 0; k < W; k++) c.v[k] = gs ? g.v[k] : relaxed(L, omega, c.v[k], g.v[k], cd.at(k));
-                stspan(e, c);
+                stspan(e, g);
             }
             if (solo)
                 __syncthreads();
             else
                 cl.sync();
         };
-        for (int h = 0; h < sweeps; h++) {
-            half(at0, cd0, r0, i0, s.e + own);
-            half(at1, cd1, r1, i1, s.e + S.ploc + own);
+        if (resident) {
+            for (int h = 0; h < sweeps; h++) {
+                half(at0, cd0, r0, i0, d0, c0, s.e + own);
+                half(at1, cd1, r1, i1, d1, c1, s.e + S.ploc + own);
+            }
+            return;
         }
-        return;
     }
     for (int h = 0; h < 2 * sweeps; h++) {
         const int colour = h & 1;
@@ -402,14 +452,12 @@ __device__ __forceinline__ void tail_smooth(const TailLevel<T>& L, const Slab<T>
             const Codes<T> cd(s.code + own);
             const Span<T> r = ldspan(s.r + own);
             const Span<T> o = neighbour_sums<T>(s.e, Around<T>(S, s, colour, row, y, lz), cd);
-            Span<T> c, g;
-            if (!gs) c = ldspan(s.e + own);
+            Span<T> g;
 #pragma unroll
             for (int k = 0; k < W; k++) g.v[k] = h2 * r.v[k] + o.v[k];
-            g = quotients<T>(L, g, Diagonals<T>(inv, diag, cd), cd);
-#pragma unroll
-            for (int k = 0; k < W; k++) c.v[k] = gs ? g.v[k] : relaxed(L, omega, c.v[k], g.v[k], cd.at(k));
-            stspan(s.e + own, c);
+            g = quotients<T>(L, how, odd, B, g, inverses<T>(B, cd), cd);
+            if (!gs) g = relaxed(L, omega, ldspan(s.e + own), g, cd);
+            stspan(s.e + own, g);
         });
         if (solo)
             __syncthreads();
@@ -454,7 +502,7 @@ template <class T>
 __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ TailArgs<T> A) {
     constexpr int W = kSpan<T>;
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ T inv_tab[ES_MAXLEV][16], diag_tab[ES_MAXLEV][16];
+    __shared__ T inv_tab[ES_MAXLEV][16], diag_tab[ES_MAXLEV][16], cor_tab[sizeof(T) == 4 ? ES_MAXLEV : 1][16];
     __shared__ __align__(8) uint64_t bar;
     __shared__ int late;
     cg::cluster_group cl = cg::this_cluster();
@@ -471,9 +519,10 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
     }
     for (int t = threadIdx.x; t < 16 * A.n; t += kTailThreads) {
         const int l = t >> 4, k = t & 15;
-        const T d = A.lv[l].diag0 + (T)(k - 6);
+        const T d = A.lv[l].diag0 + (T)(k == (int)kTailEven ? 0 : k - 6), y = k == 15 ? (T)0 : (T)1 / d;
         diag_tab[l][k] = d;
-        inv_tab[l][k] = k == 15 ? (T)0 : (T)1 / d;
+        inv_tab[l][k] = y;
+        if constexpr (sizeof(T) == 4) cor_tab[l][k] = k == 6 && A.lv[l].how == kNearQuotient ? (T)0 : y;
     }
     for (int t = A.code_bytes + 16 * (int)threadIdx.x; t < A.smem_bytes; t += 16 * kTailThreads)
         *reinterpret_cast<uint4*>(smem + t) = make_uint4(0u, 0u, 0u, 0u);
@@ -483,6 +532,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
     __syncthreads();
     if (threadIdx.x == 0 && !bulk_wait(bar_at, 0)) late = 1;
     pdl_wait();
+    auto tables = [&](int l) { return Tables<T>{inv_tab[l], diag_tab[l], cor_tab[sizeof(T) == 4 ? l : 0]}; };
     {
         const TailShape& S = A.lv[0].s;
         const Slab<T> s(S, smem, cl, rank);
@@ -528,7 +578,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
         const TailShape& S = L.s;
         const TailShape& M = A.lv[l + 1].s;
         const Slab<T> s(S, smem, cl, rank);
-        tail_smooth<T>(L, s, inv_tab[l], diag_tab[l], A.nu1, A.omega, false, cl);
+        tail_smooth<T>(L, s, tables(l), A.nu1, A.omega, false, cl);
         // restriction: the mean of the 8 children's residuals (with red_only
         // the black ones count as 0); the children of a coarse cell share a slab
         // (an even number of planes), the coarse cell may be another block's.
@@ -582,8 +632,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
     {
         const TailLevel<T>& L = A.lv[A.n - 1];
         if (!A.solo || rank == 0)
-            tail_smooth<T>(L, Slab<T>(L.s, smem, cl, rank), inv_tab[A.n - 1], diag_tab[A.n - 1], A.sweeps, A.omega,
-                           A.solo != 0, cl);
+            tail_smooth<T>(L, Slab<T>(L.s, smem, cl, rank), tables(A.n - 1), A.sweeps, A.omega, A.solo != 0, cl);
         if (A.solo) cl.sync();
     }
     for (int l = A.n - 2; l >= 0; l--) {
@@ -610,7 +659,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
                 stspan(s.e + i, v);
             });
         cl.sync();
-        tail_smooth<T>(L, s, inv_tab[l], diag_tab[l], A.nu2, A.omega, false, cl);
+        tail_smooth<T>(L, s, tables(l), A.nu2, A.omega, false, cl);
     }
     {
         const TailShape& S = A.lv[0].s;
@@ -689,9 +738,10 @@ __global__ void __launch_bounds__(256) k_tail_codes(const __grid_constant__ Tail
                 cd |= u << (2 * f);
                 dk += u == 0u ? 0 : (u == 1u ? 1 : -1);
             }
-            if (A.diag0[blockIdx.y] > 0.0f &&
-                code_diag(A.diag0[blockIdx.y], cd) != A.diag0[blockIdx.y] + (float)(dk - 6))
-                dk = (int)kTailOdd;
+            if (A.diag0[blockIdx.y] > 0.0f && cd != 0u)
+                dk = code_diag(A.diag0[blockIdx.y], cd) != A.diag0[blockIdx.y] + (float)(dk - 6)
+                         ? (int)kTailOdd
+                         : (dk == 6 ? (int)kTailEven : dk);
             code[k] = cd | ((unsigned)dk << 12);
         }
         *reinterpret_cast<uint2*>(A.out + (size_t)block * A.bytes + S.c + 2 * (size_t)(colour * S.ploc + 4 * i)) =
@@ -798,18 +848,21 @@ cudaError_t tail_run(es_ctx* c, int warm) {
         TailLevel<T>& L = A.lv[l];
         L = TailLevel<T>{p.s[l], (T)(h * h), (T)(1.0 / (h * h)), (T)(6.0 + c->S.kappa * c->S.kappa * h * h)};
         L.how = kByTable;
+        L.odd = 0;
         L.red_only = c->P.omega == 1.0 && c->P.nu1 >= 1;
         L.pairs = 1;
         L.fuse_inner = L.fuse_near = 0;
         if (sizeof(T) == 4) {
             // what the level's kernels do when it is launched by itself
             const bool spans = p.s[l].nx % 4 == 0;
+            for (int k = -6; k <= 6; k++) L.odd |= (double)(T)((double)L.diag0 + k) != (double)L.diag0 + k;
             L.how = spans ? kNearQuotient : kQuotient;
             if (l + 1 < p.n || coarse_divides(c) == 2) {
                 L.fuse_inner = !spans;                         // (k_smooth)
                 L.fuse_near = !spans || split_level(c, l0 + l);  // (near_gs)
             } else {
                 L.how = coarse_divides(c) == 0 ? kByTable : kQuotient;
+                if (L.how == kByTable) L.odd = 0;
             }
             L.red_only = L.red_only && spans;
             L.pairs = spans;
