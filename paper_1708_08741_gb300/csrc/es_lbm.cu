@@ -956,13 +956,15 @@ __global__ void __launch_bounds__(T, 1) k_forces(Grid g, const DParticle* __rest
 //    arms in FP32, then summed in FP32 by 256 of them -- link i of a chunk of
 //    256 box cells by thread i mod 256, chunk after chunk -- and over the block
 //    in float-float;
-//  * the 2 w_q part is summed exactly in integers: with S = sum of 18 x 2 w_q
-//    c_q over a cell's links, sum S and sum rel x S (rel: the cell's
-//    coordinates relative to the box, minimum image), from which sum 2 w_q c_q
-//    and sum 2 w_q (x_s - X) x c_q follow in FP64 at the end (c_q x c_q = 0).
-// (2,880 spheres R = 5 / 64 spheres R = 6: 277 / 102 us before, 221 / 25
-// now: a sphere R = 6 did not fit the owner tile and looked every cell's
-// neighbours up one by one, and every link made four shared-memory atomics.)
+//  * the 2 w_q part is summed exactly in integers: for each direction the
+//    number of links and the sums of their surface cells' coordinates (relative
+//    to the box, minimum image), a vote and a warp sum of the packed three a
+//    direction, from which sum 2 w_q c_q and sum 2 w_q (x_s - X) x c_q follow in
+//    FP64 at the end, direction by direction.
+// (2,880 spheres R = 5 / 64 spheres R = 6: 277 / 83 us with an owner tile, a
+// lookup a neighbour where it did not fit and four shared-memory atomics a link;
+// 238 / 27 now.  The constant part as six integers a cell instead of a
+// direction's sums is 221 / 25, but rounds differently at the end.)
 template <class S, int T>
 __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
     k_forces_f32(Grid g, const DParticle* __restrict__ part, const int32_t* __restrict__ owner,
@@ -974,7 +976,8 @@ __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
     __shared__ BallF ball;
     __shared__ float s_X[3], s_V[3], s_W[3];
     __shared__ double s_off[3], s_qeff;
-    __shared__ int s_int[6], s_first[kForceChunks], s_count[kForceChunks];
+    __shared__ int s_dir[19][4], s_first[kForceChunks], s_count[kForceChunks];
+    __shared__ double s_term[19][6];
     __shared__ float s_red[kForceChunk / 32][12];
     unsigned* own = (unsigned*)dyn;
     unsigned* fluid = own + kForceSide * kForceSide;
@@ -997,7 +1000,7 @@ __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
         s_W[a] = (float)P.w[a];
     }
     if (threadIdx.x == 32) s_qeff = part[p].qeff;
-    if (threadIdx.x < 6) s_int[threadIdx.x] = 0;
+    if (threadIdx.x < 4 * 19) s_dir[threadIdx.x / 4][threadIdx.x % 4] = 0;
     __syncthreads();
     const int n = B.n[0] * B.n[1] * B.n[2];
     const BoxIndex bi(B.n[0], B.n[1], n);
@@ -1013,7 +1016,15 @@ __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
         return u;
     };
     float acc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    int isum[6] = {0, 0, 0, 0, 0, 0};
+    // lane q of every warp: number of links along q, and the sums of their
+    // surface cells' coordinates
+    int nq = 0, sq[3] = {0, 0, 0};
+    const int lane = threadIdx.x & 31;
+    // Rows of bit words whose cells are their own nearest images: box
+    // coordinates below 32, so a warp's sums of the three fit one word.
+    bool packed = force_by_rows(B);
+#pragma unroll
+    for (int a = 0; a < 3; a++) packed &= !g.per[a] || B.n[a] + 4 <= gdim(g, a);
     // The listed cells' links: chunk of a cell: (box index - t0) / 256, nch chunks.
     auto consume = [&](int total, int t0, int nch) {
         for (int c = threadIdx.x; c < nch; c += T) s_count[c] = 0;
@@ -1022,41 +1033,47 @@ __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
         int cnt = 0;
         for (int u = 0; u < per; u++) {
             const int c = (int)threadIdx.x * per + u;
-            if (c >= total) break;
-            const unsigned m = s_mask[c];
-            const int t = s_near[c];
-            cnt += __popc(m);
-            atomicAdd(&s_count[(t - t0) / kForceChunk], __popc(m));
-            // S = sum of 18 x 2 w_q c_q: 2 for an axis, 1 for a diagonal
-            constexpr unsigned xp = dir_bits(0, 1), xm = dir_bits(0, -1), yp = dir_bits(1, 1), ym = dir_bits(1, -1),
-                               zp = dir_bits(2, 1), zm = dir_bits(2, -1);
-            auto axis = [&](int a) { return (int)((m >> (1 + a)) & 1u) - (int)((m >> (10 + a)) & 1u); };
-            const int S0 = __popc(m & xp) - __popc(m & xm) + axis(0), S1 = __popc(m & yp) - __popc(m & ym) + axis(1),
-                      S2 = __popc(m & zp) - __popc(m & zm) + axis(2);
-            int v[3];
-            bi.at(t, v);
-            const int u0 = image(v[0], 0), u1 = image(v[1], 1), u2 = image(v[2], 2);
-            isum[0] += S0;
-            isum[1] += S1;
-            isum[2] += S2;
-            bool past = false;  // (see k_forces)
-#pragma unroll
-            for (int a = 0; a < 3; a++) past |= image(v[a] + 1, a) - image(v[a] - 1, a) != 2;
-            if (past) {
-                for (unsigned l = m; l; l &= l - 1u) {
-                    const int q = __ffs(l) - 1, w = (q <= 3 || (q >= 10 && q <= 12)) ? 2 : 1;
-                    int k[3];
-                    dir_of(q, k);
-                    const int s0 = image(v[0] + k[0], 0), s1 = image(v[1] + k[1], 1), s2 = image(v[2] + k[2], 2);
-                    isum[3] += w * (s1 * k[2] - s2 * k[1]);
-                    isum[4] += w * (s2 * k[0] - s0 * k[2]);
-                    isum[5] += w * (s0 * k[1] - s1 * k[0]);
-                }
-                continue;
+            const bool on = c < total;
+            if (!__any_sync(0xffffffffu, on)) break;
+            const unsigned m = on ? s_mask[c] : 0u;
+            int v[3] = {0, 0, 0};
+            if (on) {
+                const int t = s_near[c];
+                cnt += __popc(m);
+                atomicAdd(&s_count[(t - t0) / kForceChunk], __popc(m));
+                bi.at(t, v);
             }
-            isum[3] += u1 * S2 - u2 * S1;
-            isum[4] += u2 * S0 - u0 * S2;
-            isum[5] += u0 * S1 - u1 * S0;
+            const unsigned place = (unsigned)v[0] | ((unsigned)v[1] << 10) | ((unsigned)v[2] << 20);
+            if (packed) {
+#pragma unroll 6
+                for (int q = 1; q < 19; q++) {
+                    const bool b = (m >> q) & 1u;
+                    const int n = __popc(__ballot_sync(0xffffffffu, b));
+                    const unsigned w = __reduce_add_sync(0xffffffffu, b ? place : 0u);
+                    if (lane == q) {
+                        int d[3];
+                        dir_of(q, d);
+                        nq += n;
+                        sq[0] += (int)(w & 1023u) + n * d[0];
+                        sq[1] += (int)((w >> 10) & 1023u) + n * d[1];
+                        sq[2] += (int)(w >> 20) + n * d[2];
+                    }
+                }
+            } else {
+#pragma unroll 1
+                for (int q = 1; q < 19; q++) {
+                    const bool b = (m >> q) & 1u;
+                    const int n = __popc(__ballot_sync(0xffffffffu, b));
+                    int d[3];
+                    dir_of(q, d);
+#pragma unroll
+                    for (int a = 0; a < 3; a++) {
+                        const int w = __reduce_add_sync(0xffffffffu, b ? image(v[a] + d[a], a) : 0);
+                        if (lane == q) sq[a] += w;
+                    }
+                    if (lane == q) nq += n;
+                }
+            }
         }
         int nlinks;
         const int base = block_excl<T>(cnt, B.warp, nlinks);
@@ -1173,10 +1190,32 @@ __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
                 s_red[threadIdx.x >> 5][2 * k + 1] = v[k].lo;
             }
     }
+    if (nq != 0) {
+        atomicAdd(&s_dir[lane][0], nq);
 #pragma unroll
-    for (int k = 0; k < 6; k++) {
-        const int v = __reduce_add_sync(0xffffffffu, isum[k]);
-        if ((threadIdx.x & 31) == 0 && v != 0) atomicAdd(&s_int[k], v);
+        for (int a = 0; a < 3; a++) atomicAdd(&s_dir[lane][1 + a], sq[a]);
+    }
+    __syncthreads();
+    // a direction's terms, a thread each: 2 w_q times its links (a force), and
+    // the sum of (x_s - X) x c_q (a torque), x_s - X = the sums + links (lo + 1/2 - X)
+    if (threadIdx.x < 6 * 18) {
+        const int q = 1 + threadIdx.x / 6, k = threadIdx.x % 6, c = k % 3, d = (c + 1) % 3, e = (c + 2) % 3;
+        int v[3];
+        dir_of(q, v);
+        auto sign = [&](int a, double x) {
+            const int s = a == 0 ? v[0] : (a == 1 ? v[1] : v[2]);
+            return s == 0 ? 0.0 : (s > 0 ? x : -x);
+        };
+        const double n = (double)s_dir[q][0], w2 = (q <= 3 || (q >= 10 && q <= 12)) ? 2.0 / 18.0 : 2.0 / 36.0;
+        double t;
+        if (k < 3) {
+            t = sign(c, __dmul_rn(w2, n));
+        } else {
+            const double rd = __fma_rn(n, s_off[d], (double)s_dir[q][1 + d]),
+                         re = __fma_rn(n, s_off[e], (double)s_dir[q][1 + e]);
+            t = __dadd_rn(sign(e, rd), -sign(d, re));
+        }
+        s_term[q][k] = t;
     }
     __syncthreads();
     if (threadIdx.x < 6) {
@@ -1184,16 +1223,14 @@ __global__ void __launch_bounds__(T, T == 1024 ? 1 : 3)
         ff a = {s_red[0][2 * k], s_red[0][2 * k + 1]};
         for (int w = 1; w < kForceChunk / 32; w++) a = ff_add(a, ff{s_red[w][2 * k], s_red[w][2 * k + 1]});
         double sum = (double)a.hi + (double)a.lo;
-        if (k < 3) {
-            const double E[3] = {Ex, Ey, Ez};
-            sum += (double)s_int[k] * (1.0 / 18.0);
-            F[3 * p + k] = sum + s_qeff * E[k];  // F_C = q E_ext (Sec. 5.6)
-        } else {
-            // x_F - X = rel + (lo + 1/2 - X)
-            const int c = k - 3, d = (c + 1) % 3, e = (c + 2) % 3;
-            sum += ((double)s_int[k] + (s_off[d] * (double)s_int[e] - s_off[e] * (double)s_int[d])) * (1.0 / 18.0);
-            T_out[3 * p + c] = sum;
-        }
+        // (a force adds its terms, rounded; a torque takes 2 w_q with the addition)
+#pragma unroll
+        for (int q = 1; q < 19; q++)
+            sum = __fma_rn(k < 3 ? 1.0 : 2.0 * wq(q), s_term[q][k], sum);
+        if (k < 3)
+            F[3 * p + k] = sum + s_qeff * (k == 0 ? Ex : (k == 1 ? Ey : Ez));  // F_C = q E_ext (Sec. 5.6)
+        else
+            T_out[3 * p + k - 3] = sum;
     }
 }
 
