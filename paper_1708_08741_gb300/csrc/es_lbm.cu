@@ -736,7 +736,7 @@ __device__ __forceinline__ int force_cells(const Grid& g, const int32_t* __restr
 // centre at the last mapping, so only cells between R - 1 and R + 1.5 of that
 // centre are looked up (FP32 distances; the bounds are far outside their
 // rounding): a tenth of the box.  (One sphere R = 16 / R = 24: reduced forms
-// 971 / 3,020 us looking at every cell 256 at a time, 278 / 796 so; FP64 1,128 /
+// 971 / 3,020 us looking at every cell 256 at a time, 311 / 878 so; FP64 1,128 /
 // 3,410 and 326 / 809.)
 template <int T>
 __device__ __forceinline__ int force_cells_fields(const Grid& g, const int32_t* __restrict__ owner,
